@@ -171,6 +171,10 @@ struct fsm_graph {
     double delta = 0.5;
     int32_t *by_rank = nullptr;
     int64_t *cls_off = nullptr;
+    // acceptance tables of the join kernel by stored size, made on first use
+    uint32_t *join_acc[FSM_JOIN_MAXL + 1] = {};
+    uint16_t *join_any[FSM_JOIN_MAXL + 1] = {};
+    int4 *vinfo = nullptr;
     int32_t *row_ptr = nullptr, *col = nullptr, *labels = nullptr, *rank = nullptr, *cls_size = nullptr,
             *end_off = nullptr;
     int64_t *piece_cnt = nullptr;
@@ -192,6 +196,7 @@ struct fsm_graph {
         g.pcol = col;
         g.pend = end_off;
         g.ppc = piece_cnt;
+        g.vinfo = vinfo;
         g.tri_off = tri_off;
         g.tri_bits = tri_bits;
         return g;
@@ -244,11 +249,44 @@ struct Miner {
     RunStats &rs;
     int V = FSM_EXPLORE_TV;   // exploration variant of this call (FSM_EXPLORE_*)
 
+    // Stored sizes up to 5 of two-vertex exploration with index-based keys are joined by
+    // fsm_join.cuh (its header has the times of both kernels: 1.8 to 14 times less); the ablations'
+    // key forms and sizes 6 and 7, whose acceptance tables would not fit, by fsm_extend.cuh.
+    bool joins(int L) const { return L <= FSM_JOIN_MAXL && (V == FSM_EXPLORE_TV || V == FSM_EXPLORE_TV_QUOTA); }
+
+    cudaError_t launch_pass(int pass, int L, const ExtArgs &A, int grid) {
+        if (joins(L)) return launch_join(pass, L, V, A, grid, st);
+        return pass == PASS_COUNT ? launch_extend_count(L, V, A, grid, st)
+             : pass == PASS_DOMAIN ? launch_extend_domain(L, V, A, grid, st)
+                                   : launch_extend_emit(L, V, A, grid, st);
+    }
+
+    // The join kernel's tables for stored size L, made once per graph handle.
+    void join_tables(int L) {
+        if (G->join_acc[L]) return;
+        size_t nacc = 0, nany = 0, ntmp = 0;
+        join_table_bytes(L, &nacc, &nany, &ntmp);
+        void *tmp = mem.get<char>((int64_t)ntmp);
+        void *acc = nullptr, *any = nullptr;
+        ck(cudaMallocAsync(&acc, nacc, st), "device allocation");
+        cudaError_t e = cudaMallocAsync(&any, nany, st);
+        if (e == cudaSuccess) e = launch_join_tables(L, (uint32_t *)acc, (uint16_t *)any, tmp, st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(st);   // later calls may run on another stream
+        if (e != cudaSuccess) {
+            cudaFreeAsync(acc, st);
+            if (any) cudaFreeAsync(any, st);
+            ck(e, "acceptance tables");
+        }
+        G->join_acc[L] = (uint32_t *)acc;
+        G->join_any[L] = (uint16_t *)any;
+        mem.release(tmp);
+    }
+
     int grid_for(int L, int pass) {
         int bps = 0;
-        cudaError_t e = pass == PASS_COUNT ? occupancy_extend_count(L, V, &bps)
+        cudaError_t e = joins(L) ? occupancy_join(pass, L, V, &bps)
+                      : pass == PASS_COUNT ? occupancy_extend_count(L, V, &bps)
                       : pass == PASS_DOMAIN ? occupancy_extend_domain(L, V, &bps)
-                      : pass == PASS_FUSED ? occupancy_extend_fused(L, &bps)
                                             : occupancy_extend_emit(L, V, &bps);
         ck(e, "occupancy query");
         if (bps < 1) bps = 1;
@@ -317,11 +355,7 @@ struct Miner {
         A.unit_base = base;
         A.chunk_ctr = ctr;
         auto launch_ext = [&]() {
-            cudaError_t e = pass == PASS_COUNT ? launch_extend_count(L, V, A, grid, st)
-                          : pass == PASS_DOMAIN ? launch_extend_domain(L, V, A, grid, st)
-                          : pass == PASS_FUSED ? launch_extend_fused(L, A, grid, st)
-                                                : launch_extend_emit(L, V, A, grid, st);
-            ck(e, "extension kernel");
+            ck(launch_pass(pass, L, A, grid), "extension kernel");
             rs.launches += 1;
             rs.pass_launches[L][pass] += 1;
         };
@@ -364,11 +398,7 @@ struct Miner {
                 if (total == 0) continue;
                 bytes(r);
                 int64_t chunk = chunk_for(L);
-                if (chunk <= 0) {   // as the kernel sizes it when the total stays on the device
-                    const int64_t per_unit = total / (r.ne * L);
-                    chunk = 256;
-                    while (chunk < 16384 && total / chunk > warps * 64 && chunk * 2 <= 16 * per_unit) chunk <<= 1;
-                }
+                if (chunk <= 0) chunk = join_chunk(total, r.ne * L, warps);   // as the kernel does when the total stays on the device
                 A.e0 = r.e0;
                 A.ne = r.ne;
                 A.total = total;
@@ -450,8 +480,7 @@ struct Miner {
             A.nchunks = (total + chunk - 1) / chunk;
             ck(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), st), "memset");
             ck(cudaEventRecord(a, st), "event record");
-            ck(pass == PASS_COUNT ? launch_extend_count(L, V, A, grid, st) : launch_extend_domain(L, V, A, grid, st),
-               "extension kernel");
+            ck(launch_pass(pass, L, A, grid), "extension kernel");
             ck(cudaEventRecord(b, st), "event record");
             ck(cudaEventSynchronize(b), "event sync");
             float ms = 0.f;
@@ -497,6 +526,17 @@ struct Miner {
         A.debug = G->debug;
         A.time_limit_ns = (uint64_t)G->time_limit_ms * 1000000ull;
         A.time_start = G->stats + 4;
+        unsigned long long *lf = nullptr;
+        if (joins(L)) {
+            join_tables(L);
+            A.acc = G->join_acc[L];
+            A.any = G->join_any[L];
+            if (piece_freq) {
+                lf = mem.get<unsigned long long>(3 * 4096);
+                ck(launch_label_masks(piece_freq, lf, st), "label masks");
+                A.lf = lf;
+            }
+        }
         if (V == FSM_EXPLORE_TV_QUOTA) {
             // Section 5: size-3 matching (l = 1) draws match_quota candidates per vertex; every
             // join draws join_quota^2 pieces per key group and, joining edges, join_quota edges
@@ -535,8 +575,9 @@ struct Miner {
             while (cap < 4 * G->qp_hint[L] && cap < ((int64_t)1 << 30)) cap <<= 1;
         unsigned long long *keys = nullptr, *qcount = nullptr, *used = nullptr, *ptop = nullptr, *ckeys = nullptr,
                            *coff = nullptr;
-        long long *soff = nullptr;
+        uint32_t *soff = nullptr;
         uint32_t *pool = nullptr;
+        int shift = 0;   // bitmap offsets are 32-bit, in units of 1 << shift words
         unsigned long long pool_words = 0;
         bool fused = final && G->fused && V == FSM_EXPLORE_TV && !sampled && K <= 7;
         if (fused) {
@@ -555,6 +596,7 @@ struct Miner {
                 pool = (uint32_t *)pp;
                 mem.ptrs.push_back(pp);
                 ptop = mem.get<unsigned long long>(1);
+                while ((pool_words >> shift) >= 0xFFFFFFFEull) ++shift;
             }
         }
         auto release_pass1 = [&]() {
@@ -572,7 +614,7 @@ struct Miner {
             if (fused) {
                 ck(launch_fill_u64(ckeys, FSM_EMPTY_KEY, cap, st), "fill");
                 ck(cudaMemsetAsync(coff, 0, sizeof(unsigned long long) * cap, st), "memset");
-                ck(cudaMemsetAsync(soff, 0xff, sizeof(long long) * cap * 8, st), "memset");
+                ck(cudaMemsetAsync(soff, 0xff, sizeof(uint32_t) * cap * 8, st), "memset");
                 ck(cudaMemsetAsync(pool, 0, pool_words * 4, st), "memset");
                 ck(cudaMemsetAsync(ptop, 0, sizeof(unsigned long long), st), "memset");
             }
@@ -586,12 +628,13 @@ struct Miner {
                 // at most half full whenever that one is
                 ckeys = mem.get<unsigned long long>(cap);
                 coff = mem.get<unsigned long long>(cap);
-                soff = mem.get<long long>(cap * 8);
+                soff = mem.get<uint32_t>(cap * 8);
                 A.pat_lab = in.lab8;
                 A.code_keys = ckeys;
                 A.code_off = coff;
                 A.code_mask = (uint64_t)cap - 1;
-                A.slot_off = soff;
+                A.slot_off32 = soff;
+                A.off_shift = shift;
                 A.pool = pool;
                 A.pool_top = ptop;
                 A.pool_words = pool_words;
@@ -626,6 +669,7 @@ struct Miner {
                 // pool or pattern table too small: the one-pass level stopped early; count again
                 // in a clean count pass and fill the domains in a domain pass
                 fused = false;
+                shift = 0;
                 G->pool_hint[L] = 0;
                 rs.fused_fallbacks += 1;
                 release_pass1();
@@ -688,14 +732,19 @@ struct Miner {
         if (fused) {
             // every pattern has its orbit bitmaps in the pool already: MNI from there
             rs.live = np;
-            ck(launch_fused_support(K, plab, padj, orbit, np, ckeys, coff, (uint64_t)cap - 1, G->cls_size, pool, sigma,
-                                    st), "fused support");
+            ck(launch_fused_support(K, plab, padj, orbit, np, ckeys, coff, (uint64_t)cap - 1, G->cls_size, shift, pool,
+                                    sigma, st), "fused support");
             if (G->profile) rs.pass_bytes[L][PASS_FUSED] += rs.final_accepted * 4 * K;   // one bitmap word per position
         } else {
-            ck(launch_domain_sizes(K, plab, orbit, minorb, pcount, np, t_live, G->cls_size, live, words, st), "domain sizes");
-            ck(launch_scan_i64(words, woff, np * FSM_MAXK, stmp2, st), "domain scan");
+            int64_t nwords = 0;
+            for (shift = 0;; ++shift) {   // past 2^32 words, bitmaps start on multiples of 2, 4, ... words
+                ck(launch_domain_sizes(K, plab, orbit, minorb, pcount, np, t_live, G->cls_size, shift, live, words, st),
+                   "domain sizes");
+                ck(launch_scan_i64(words, woff, np * FSM_MAXK, stmp2, st), "domain scan");
+                nwords = d2h(woff + np * FSM_MAXK, st);
+                if (!joins(L) || (nwords >> shift) < 0xFFFFFFFEll) break;
+            }
             ck(launch_domain_offsets(words, woff, np * FSM_MAXK, doff, st), "domain offsets");
-            const int64_t nwords = d2h(woff + np * FSM_MAXK, st);
             dom = mem.get<uint32_t>(nwords);
             ck(cudaMemsetAsync(dom, 0, sizeof(uint32_t) * std::max<int64_t>(nwords, 1), st), "memset");
             // live pattern count (for statistics)
@@ -712,9 +761,11 @@ struct Miner {
             A.orbit = orbit;
             A.dom_off = doff;
             A.dom = dom;
-            sbase = mem.get<int64_t>(cap * FSM_MAXK);
-            ck(launch_slot_bases(K, slots, nq, qpat, qperm, live, orbit, doff, sbase, st), "slot bases");
+            if (joins(L)) soff = mem.get<uint32_t>(cap * 8); else sbase = mem.get<int64_t>(cap * FSM_MAXK);
+            ck(launch_slot_bases(K, slots, nq, qpat, qperm, live, orbit, doff, shift, sbase, soff, st), "slot bases");
             A.slot_base = sbase;
+            A.slot_off32 = soff;
+            A.off_shift = shift;
             A.stats = nullptr;
             if (rs.live > 0) {
                 tune_chunk(in, A);
@@ -797,6 +848,7 @@ struct Miner {
         const int ew = err_word();
         if (ew) fail_word(ew);
         if (sbase) mem.release(sbase);
+        if (lf) mem.release(lf);
         release_pass1();
         for (void *p : std::initializer_list<void *>{slots, nq_d, qpat, qperm, flag, ids, stmp, plab,
                                                      padj, orbit, minorb, pcount, live, words, woff, doff, stmp2, sigma,
@@ -1101,6 +1153,7 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
         dalloc((void **)&g->col, sizeof(int32_t) * nnz);
         dalloc((void **)&g->labels, sizeof(int32_t) * n);
         dalloc((void **)&g->rank, sizeof(int32_t) * n);
+        dalloc((void **)&g->vinfo, sizeof(int4) * n);
         dalloc((void **)&g->cls_size, sizeof(int32_t) * 64);
         dalloc((void **)&g->end_off, sizeof(int32_t) * nnz);
         dalloc((void **)&g->piece_cnt, sizeof(int64_t) * n);
@@ -1114,7 +1167,7 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
         ck(launch_validate(g->dg(), num_labels, g->err, st), "validate");
         const int ew = d2h(g->err, st);
         if (ew) fail(FSM_EINVAL, "malformed CSR: rows must be sorted, symmetric, without self-loops or duplicates, labels in range");
-        ck(launch_prepare(g->dg(), g->piece_cnt, g->end_off, g->rank, g->cls_size, st), "prepare");
+        ck(launch_prepare(g->dg(), g->piece_cnt, g->end_off, g->rank, g->cls_size, g->vinfo, st), "prepare");
         {
             // Neighbour-adjacency matrices for the triangle test of centre pairs, for vertices
             // of degree >= dmin; dmin doubles until they fit the budget.
@@ -1466,9 +1519,13 @@ void fsm_free_graph(fsm_graph *g) {
     if (!g) return;
     cudaStream_t st = g->stream ? g->stream : g->own_stream;
     void *ps[] = {g->row_ptr, g->col, g->labels, g->rank, g->cls_size, g->end_off, g->piece_cnt, g->tri_off, g->tri_bits, g->err, g->stats,
-                  g->by_rank, g->cls_off};
+                  g->by_rank, g->cls_off, g->vinfo};
     for (void *p : ps)
         if (p) cudaFreeAsync(p, st);
+    for (int L = 0; L <= FSM_JOIN_MAXL; ++L) {
+        if (g->join_acc[L]) cudaFreeAsync(g->join_acc[L], st);
+        if (g->join_any[L]) cudaFreeAsync(g->join_any[L], st);
+    }
     if (st) cudaStreamSynchronize(st);
     if (g->own_stream) cudaStreamDestroy(g->own_stream);
     delete g;

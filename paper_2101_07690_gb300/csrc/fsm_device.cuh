@@ -53,6 +53,8 @@ struct DevGraph {
     // adjacency tests always use row_ptr / col.
     const int32_t *prow, *pcol, *pend;
     const int64_t *ppc;
+    // per vertex {row_ptr[v], row_ptr[v+1], label, rank}: one 16-byte read where a join needs them all
+    const int4 *vinfo;
     // Neighbour adjacency of high-degree vertices: for v with tri_off[v] >= 0, bit y of row x
     // (x < y < d(v)) of a d(v) x ceil(d(v)/32)-word matrix at word tri_off[v] of tri_bits says
     // whether the x-th and y-th neighbours of v are adjacent.  Indexed by positions in the
@@ -74,6 +76,12 @@ __device__ __forceinline__ bool is_adj(const DevGraph &g, int32_t u, int32_t w) 
         if (c < x) lo = mid + 1; else hi = mid;
     }
     return lo < end && __ldg(g.col + lo) == x;
+}
+
+// Words of the bitmap of a label class of n vertices, a whole number of 1 << shift words.
+FSM_HD int64_t bitmap_words(int64_t n, int shift) {
+    const int64_t w = (n + 31) / 32, a = (int64_t)1 << shift;
+    return (w + a - 1) & ~(a - 1);
 }
 
 // ---------------------------------------------------------------------------- pieces

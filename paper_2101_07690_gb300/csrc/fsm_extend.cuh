@@ -76,13 +76,22 @@ struct ExtArgs {
     unsigned long long *out_cursor;
     unsigned long long *stats;     // [0] joins tested, [1] joins accepted, [2] pieces enumerated
     // one-pass last level (PASS_FUSED): a table of canonical codes (packed by pack_code) with the
-    // pool word offset + 1 of each pattern's orbit bitmaps (0 = not yet claimed), and the bitmap
-    // word offset of every (key slot, local position), -1 until published
+    // pool word offset + 1 of each pattern's orbit bitmaps (0 = not yet claimed)
     const uint64_t *pat_lab;       // [P] 8 label bytes of the size-l patterns
     unsigned long long *code_keys; // [code_mask + 1], FSM_EMPTY_KEY when free
     unsigned long long *code_off;  // [code_mask + 1]
     uint64_t code_mask;
-    long long *slot_off;           // [cap * 8]
+    // one bitmap offset per (key slot, local position), [cap * 8], in units of 1 << off_shift words:
+    // written by the one-pass level (FSM_OFF_NONE until published), read by the domain pass of
+    // fsm_join.cuh (FSM_OFF_NONE: pattern without bitmaps)
+    uint32_t *slot_off32;
+    int off_shift;
+    // tables of fsm_join.cuh for this level size, and the size-3 frequencies as label masks: W[c][x]
+    // bit y (wedge of centre c, ends x, y), C[x][y] bit c (the same wedge by its centre) and
+    // T[x][y] bit z (triangle), 64 x 64 words each; NULL at level 1
+    const uint32_t *acc;
+    const uint16_t *any;
+    const unsigned long long *lf;
     uint32_t *pool;
     unsigned long long *pool_top;
     unsigned long long pool_words;
@@ -101,6 +110,16 @@ struct ExtArgs {
     const unsigned long long *time_start;   // the call's start on the device's global timer
     int *err;
 };
+
+// Pieces per work-stealing chunk of a pass of `total` pieces over `units` units on `warps` warps:
+// at least 64 chunks per warp, and at most about 16 units' pieces per chunk (a chunk over a few
+// units prepares them together).
+FSM_HD int64_t join_chunk(int64_t total, int64_t units, int64_t warps) {
+    const int64_t per_unit = total / (units > 0 ? units : 1);
+    int64_t chunk = 256;
+    while (chunk < 16384 && total / chunk > warps * 64 && chunk * 2 <= 16 * per_unit) chunk <<= 1;
+    return chunk;
+}
 
 __device__ __forceinline__ unsigned long long global_ns() {
     unsigned long long t;
@@ -215,34 +234,8 @@ FSM_HD bool dissect4_keeps(const int32_t (&gid)[4], const uint32_t (&adj)[4], in
 struct CountCache {
     unsigned long long key[8][FSM_WARP_SLOTS];
     unsigned long long cnt[8][FSM_WARP_SLOTS];
-    long long slot[8][FSM_WARP_SLOTS];   // global slot of the key, -1 until resolved (PASS_FUSED)
 };
-// PASS_COUNT launches allocate only key and cnt: more of the SM's shared storage stays L1.
-#define FSM_COUNT_SMEM (2 * 8 * FSM_WARP_SLOTS * sizeof(unsigned long long))
-
-// Count n more joins of key through the warp's table; returns the key's global slot (resolved
-// once per table entry; a race resolves it twice to the same value).
-__device__ __forceinline__ int64_t count_key_slot(const ExtArgs &A, CountCache *cc, uint64_t key, unsigned n) {
-    const int w = threadIdx.x >> 5;
-    uint32_t h = (uint32_t)mix64(key) & (FSM_WARP_SLOTS - 1);
-    for (int probe = 0; probe < FSM_SMEM_PROBES; ++probe) {
-        unsigned long long cur = cc->key[w][h];
-        if (cur == FSM_EMPTY_KEY) cur = atomicCAS(&cc->key[w][h], FSM_EMPTY_KEY, key);
-        if (cur == FSM_EMPTY_KEY || cur == key) {
-            atomicAdd(&cc->cnt[w][h], (unsigned long long)n);
-            long long s = ((volatile long long *)cc->slot[w])[h];
-            if (s < 0) {
-                s = qp_insert(A.qp, key, A.err);
-                ((volatile long long *)cc->slot[w])[h] = s;
-            }
-            return s;
-        }
-        h = (h + 1) & (FSM_WARP_SLOTS - 1);
-    }
-    int64_t slot = qp_insert(A.qp, key, A.err);
-    if (slot >= 0) atomicAdd(A.qp.count + slot, (unsigned long long)n);
-    return slot;
-}
+#define FSM_COUNT_SMEM sizeof(CountCache)
 
 __device__ __forceinline__ void count_key(const ExtArgs &A, CountCache *cc, uint64_t key, unsigned n) {
     const int w = threadIdx.x >> 5;
@@ -261,99 +254,22 @@ __device__ __forceinline__ void count_key(const ExtArgs &A, CountCache *cc, uint
 }
 
 // warp-synchronous: every lane of the warp calls it
-template <bool SLOTS>
 __device__ __forceinline__ void flush_warp_counts(const ExtArgs &A, CountCache *cc) {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     __syncwarp();
     for (int x = lane; x < FSM_WARP_SLOTS; x += 32) {
         const unsigned long long key = cc->key[w][x];
         if (key == FSM_EMPTY_KEY) continue;
-        int64_t slot = SLOTS ? cc->slot[w][x] : -1;
-        if (slot < 0) slot = qp_insert(A.qp, key, A.err);
+        const int64_t slot = qp_insert(A.qp, key, A.err);
         if (slot >= 0) atomicAdd(A.qp.count + slot, cc->cnt[w][x]);
         cc->key[w][x] = FSM_EMPTY_KEY;
         cc->cnt[w][x] = 0ull;
-        if (SLOTS) cc->slot[w][x] = -1;
     }
     __syncwarp();
 }
 
-// ---- one-pass last level: publication of per-slot bitmap offsets (gpu-scope release/acquire)
-__device__ __forceinline__ long long ld_acquire_s64(const long long *p) {
-    long long v;
-    asm volatile("ld.acquire.gpu.global.s64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ long long ld_relaxed_s64(const long long *p) {
-    long long v;
-    asm volatile("ld.relaxed.gpu.global.s64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_release_s64(long long *p, long long v) {
-    asm volatile("st.release.gpu.global.s64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ void st_relaxed_s64(long long *p, long long v) {
-    asm volatile("st.relaxed.gpu.global.s64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-
-// First sight of a quick pattern in the one-pass last level: canonicalise the graph its key
-// denotes, find or claim its pattern's entry in the code table, claim the pattern's orbit
-// bitmaps from the pool unless another lane already did (one CAS decides; a loser's pool words
-// stay unused), and publish the bitmap word offset of each local position -- position 0 last,
-// with release semantics, so a reader that sees it set sees the others.  Lanes racing on one key
-// compute and write the same values.  On a full table or pool the error word says so and nothing
-// is published; the host then runs the last level as two passes.
-struct ResolveArgs {
-    const uint64_t *pat_lab, *pat_adj;
-    const int32_t *cls_size;
-    unsigned long long *code_keys, *code_off, *pool_top;
-    uint64_t code_mask;
-    unsigned long long pool_words;
-    long long *slot_off;
-    int *err;
-    int explore, level;
-};
-
-static __device__ __noinline__ void resolve_slot(const ResolveArgs A, int64_t slot, uint64_t key) {
-    // K <= 7 here: the compact words of fsm_canon7.cuh
-    int K, lab[8], rep[8];
-    uint32_t adj[8];
-    key_graph7(A.explore, A.level, key, A.pat_lab, A.pat_adj, K, lab, adj);
-    unsigned long long clab;
-    uint32_t cadj, inv;
-    canonicalise7(K, lab, adj, clab, cadj, inv);
-    orbit_reps7(K, clab, cadj, rep);
-    int64_t pre[8], words = 0;
-    for (int c = 0; c < K; ++c) {
-        pre[c] = words;
-        if (rep[c] == c) words += ((int64_t)__ldg(A.cls_size + ((clab >> (8 * (7 - c))) & 0xff)) + 31) / 32;
-    }
-    const uint64_t pk = pack_code7(K, clab, cadj);
-    uint64_t h = mix64(pk) & A.code_mask;
-    int64_t ci = -1;
-    for (int probe = 0; probe < FSM_MAX_PROBES; ++probe) {
-        unsigned long long cur = __ldcg(A.code_keys + h);
-        if (cur == FSM_EMPTY_KEY) cur = atomicCAS(A.code_keys + h, FSM_EMPTY_KEY, pk);
-        if (cur == FSM_EMPTY_KEY || cur == pk) { ci = (int64_t)h; break; }
-        h = (h + 1) & A.code_mask;
-    }
-    if (ci < 0) { atomicOr(A.err, FSM_ERR_CODE_FULL); return; }
-    unsigned long long off = __ldcg(A.code_off + ci);
-    if (off == 0ull) {
-        const unsigned long long res = atomicAdd(A.pool_top, (unsigned long long)words);
-        if (res + (unsigned long long)words > A.pool_words) { atomicOr(A.err, FSM_ERR_POOL); return; }
-        const unsigned long long old = atomicCAS(A.code_off + ci, 0ull, res + 1ull);
-        off = old ? old : res + 1ull;
-    }
-    long long *so = A.slot_off + slot * 8;
-    for (int hh = K - 1; hh >= 0; --hh) {
-        const long long v = (long long)(off - 1ull) + pre[rep[(inv >> (3 * hh)) & 7]];
-        if (hh) st_relaxed_s64(so + hh, v); else st_release_s64(so, v);
-    }
-}
-
 // One accepted join: act according to PASS.
-// Per-lane memory of bitmap words already set (PASS_DOMAIN, PASS_FUSED): the last word of a piece
+// Per-lane memory of bitmap words already set (PASS_DOMAIN): the last word of a piece
 // vertex with its bits, and per position of s the last bitmap offset set for it (valid within
 // one unit: s and so its vertices' ranks are fixed there; -1 after a unit change).
 struct DomCache {
@@ -370,60 +286,6 @@ __device__ __forceinline__ void accept(const ExtArgs &A, CountCache *cc, DomCach
         const unsigned grp = __match_any_sync(act, key);
         const int lane = threadIdx.x & 31;
         if (lane == __ffs(grp) - 1) count_key(A, cc, key, __popc(grp));
-        return;
-    }
-    if (PASS == PASS_FUSED) {
-        // count the key (warp-aggregated), then set its orbits' bits as the domain pass does
-        const unsigned act = __activemask();
-        const unsigned grp = __match_any_sync(act, key);
-        const int lane = threadIdx.x & 31;
-        const int leader = __ffs(grp) - 1;
-        // the leader counts the key, resolves it on first sight, and reads its offsets once; the
-        // lanes of the group receive them by shuffle
-        long long off[K];
-#pragma unroll
-        for (int h = 0; h < K; ++h) off[h] = -1;
-        if (lane == leader) {
-            const long long slot = count_key_slot(A, cc, key, __popc(grp));
-            if (slot >= 0) {
-                const long long *so = A.slot_off + slot * 8;
-                long long o0 = ld_acquire_s64(so);
-                if (o0 < 0) {
-                    const ResolveArgs R{A.pat_lab, A.pat_adj, A.cls_size, A.code_keys, A.code_off, A.pool_top,
-                                        A.code_mask, A.pool_words, A.slot_off, A.err, A.explore, A.level};
-                    resolve_slot(R, slot, key);
-                    o0 = ld_acquire_s64(so);
-                }
-                if (o0 >= 0) {
-                    off[0] = o0;
-#pragma unroll
-                    for (int h = 1; h < K; ++h) off[h] = ld_relaxed_s64(so + h);
-                }
-            }
-        }
-#pragma unroll
-        for (int h = 0; h < K; ++h) off[h] = __shfl_sync(grp, off[h], leader);
-        // table overflow (the pass is repeated with a larger table), or pool or code table full
-        // (the level is redone in two passes): nothing to set
-        if (off[0] < 0) return;
-#pragma unroll
-        for (int h = 0; h < L; ++h) {
-            if (off[h] == dc.soff[h]) continue;
-            dc.soff[h] = off[h];
-            uint32_t *w = A.pool + off[h] + (rk[h] >> 5);
-            const uint32_t bit = 1u << (rk[h] & 31);
-            if (!(__ldcg(w) & bit)) atomicOr(w, bit);
-        }
-#pragma unroll
-        for (int h = L; h < K; ++h) {
-            const int32_t r = __ldg(A.g.rank + gid[h]);
-            uint32_t *w = A.pool + off[h] + (r >> 5);
-            const uint32_t bit = 1u << (r & 31);
-            if (w == dc.w && (dc.bits & bit)) continue;
-            atomicOr(w, bit);
-            if (w != dc.w) { dc.w = w; dc.bits = 0; }
-            dc.bits |= bit;
-        }
         return;
     }
     int64_t slot = qp_find(A.qp, key);
@@ -891,13 +753,12 @@ __global__ void __launch_bounds__(256, ExtMinBlocks<PASS>::value) extend_kernel(
     dc.bits = 0u;
     __shared__ uint32_t mask_s[8 * (L > 1 ? L - 1 : 1) * FSM_MASK_WORDS];   // per warp, see below
     extern __shared__ unsigned long long dyn_smem[];   // CountCache in PASS_COUNT launches
-    constexpr bool counts = PASS == PASS_COUNT || PASS == PASS_FUSED;
+    constexpr bool counts = PASS == PASS_COUNT;
     CountCache *cc = counts ? reinterpret_cast<CountCache *>(dyn_smem) : nullptr;
     if (counts) {
         for (int x = threadIdx.x; x < 8 * FSM_WARP_SLOTS; x += blockDim.x) {
             cc->key[x / FSM_WARP_SLOTS][x % FSM_WARP_SLOTS] = FSM_EMPTY_KEY;
             cc->cnt[x / FSM_WARP_SLOTS][x % FSM_WARP_SLOTS] = 0ull;
-            if (PASS == PASS_FUSED) cc->slot[x / FSM_WARP_SLOTS][x % FSM_WARP_SLOTS] = -1;
         }
         __syncthreads();
     }
@@ -905,25 +766,17 @@ __global__ void __launch_bounds__(256, ExtMinBlocks<PASS>::value) extend_kernel(
     if (total < 0) {
         // device-resident size: no host round trip between the prefix sum and this launch
         total = __ldg(A.unit_base + nunits);
-        if (chunk <= 0) {
-            // at least 64 chunks per warp, and at most about 16 units' pieces per chunk (a chunk
-            // over at most 32 small units builds their cross masks)
-            const int64_t warps = (int64_t)gridDim.x * (blockDim.x >> 5);
-            const int64_t per_unit = total / (nunits > 0 ? nunits : 1);
-            chunk = 256;
-            while (chunk < 16384 && total / chunk > warps * 64 && chunk * 2 <= 16 * per_unit) chunk <<= 1;
-        }
+        if (chunk <= 0) chunk = join_chunk(total, nunits, (int64_t)gridDim.x * (blockDim.x >> 5));
         nchunks = (total + chunk - 1) / chunk;
     }
     if (A.stats && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(A.stats + 2, (unsigned long long)total);
     for (;;) {
         unsigned long long c = 0;
         if (lane == 0) {
-            // stop early when the call ran out of time, when an overflowing count pass is to be
-            // repeated with a larger table, or when a one-pass level is to be redone in two passes
+            // stop early when the call ran out of time or when an overflowing count pass is to be
+            // repeated with a larger table
             const int ew = *(volatile int *)A.err;
-            bool stop = (ew & FSM_ERR_TIMEOUT) || (PASS == PASS_COUNT && (ew & FSM_ERR_QP_OVERFLOW)) ||
-                        (PASS == PASS_FUSED && ew);
+            bool stop = (ew & FSM_ERR_TIMEOUT) || (PASS == PASS_COUNT && (ew & FSM_ERR_QP_OVERFLOW));
             if (!stop && A.time_limit_ns && global_ns() - __ldcg(A.time_start) > A.time_limit_ns) {
                 atomicOr(A.err, FSM_ERR_TIMEOUT);
                 stop = true;
@@ -1034,7 +887,7 @@ __global__ void __launch_bounds__(256, ExtMinBlocks<PASS>::value) extend_kernel(
                     S[p] = __ldg(A.fv + (int64_t)p * A.fN + e);
                     SL[p] = __ldg(A.g.labels + S[p]);
                     SR[p] = make_int2(__ldg(A.g.row_ptr + S[p]), __ldg(A.g.row_ptr + S[p] + 1));
-                    RK[p] = (PASS == PASS_DOMAIN || PASS == PASS_FUSED) ? __ldg(A.g.rank + S[p]) : 0;
+                    RK[p] = PASS == PASS_DOMAIN ? __ldg(A.g.rank + S[p]) : 0;
                 }
                 pid = __ldg(A.fpid + e);
                 srows = L >= 2 ? __ldg(A.pat_adj + pid) : 0ull;
@@ -1073,7 +926,7 @@ __global__ void __launch_bounds__(256, ExtMinBlocks<PASS>::value) extend_kernel(
                 do_piece<L, PASS, V>(A, S, SL, SR, srows, pid, i, q - ub, tl, cc, dc, lmk, lstride, RK, cpos, ecur, qab,
                                      qc);
         }
-        if (counts) flush_warp_counts<PASS == PASS_FUSED>(A, cc);
+        if (counts) flush_warp_counts(A, cc);
     }
 
     // per-warp totals, one atomic per warp
@@ -1089,13 +942,12 @@ __global__ void __launch_bounds__(256, ExtMinBlocks<PASS>::value) extend_kernel(
     }
 }
 
-// Host launchers, one translation unit per pass.  V picks the exploration variant
-// (FSM_EXPLORE_*); the fused pass exists for two-vertex exploration with index-based keys only.
+// Host launchers, one translation unit per pass.  V picks the exploration variant (FSM_EXPLORE_*).
+// Two-vertex exploration with index-based keys comes here for stored sizes 6 and 7 only: smaller
+// ones are joined by fsm_join.cuh.
 cudaError_t launch_extend_count(int L, int V, const ExtArgs &A, int grid, cudaStream_t st);
 cudaError_t launch_extend_domain(int L, int V, const ExtArgs &A, int grid, cudaStream_t st);
 cudaError_t launch_extend_emit(int L, int V, const ExtArgs &A, int grid, cudaStream_t st);
-cudaError_t launch_extend_fused(int L, const ExtArgs &A, int grid, cudaStream_t st);
-cudaError_t occupancy_extend_fused(int L, int *blocks_per_sm);
 cudaError_t occupancy_extend_count(int L, int V, int *blocks_per_sm);
 cudaError_t occupancy_extend_domain(int L, int V, int *blocks_per_sm);
 cudaError_t occupancy_extend_emit(int L, int V, int *blocks_per_sm);
@@ -1109,5 +961,13 @@ cudaError_t occupancy_extend_quota(int pass, int L, int *blocks_per_sm);
 // size 7 -> 9 (count and domain passes of the method's own form)
 cudaError_t launch_extend_l7(int pass, const ExtArgs &A, int grid, cudaStream_t st);
 cudaError_t occupancy_extend_l7(int pass, int *blocks_per_sm);
+// fsm_join.cuh: V = FSM_EXPLORE_TV or FSM_EXPLORE_TV_QUOTA, L <= FSM_JOIN_MAXL, any pass (the
+// one-pass level with FSM_EXPLORE_TV only)
+#define FSM_JOIN_MAXL 5
+cudaError_t launch_join(int pass, int L, int V, const ExtArgs &A, int grid, cudaStream_t st);
+cudaError_t occupancy_join(int pass, int L, int V, int *blocks_per_sm);
+// its tables for stored size L: bytes of each, and the kernels that fill them (tmp: join_tmp_bytes)
+void join_table_bytes(int L, size_t *acc, size_t *any, size_t *tmp);
+cudaError_t launch_join_tables(int L, uint32_t *acc, uint16_t *any, void *tmp, cudaStream_t st);
 
 } // namespace fsm

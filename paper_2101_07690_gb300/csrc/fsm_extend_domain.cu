@@ -8,11 +8,6 @@ cudaError_t launch_extend_domain(int L, int V, const ExtArgs &A, int grid, cudaS
     if (V == FSM_EXPLORE_TV_EDGELIST) return launch_extend_edgelist(PASS_DOMAIN, L, A, grid, st);
     if (V == FSM_EXPLORE_TV_QUOTA) return launch_extend_quota(PASS_DOMAIN, L, A, grid, st);
     switch (L) {
-    case 1: extend_kernel<1, PASS_DOMAIN><<<grid, 256, 0, st>>>(A); break;
-    case 2: extend_kernel<2, PASS_DOMAIN><<<grid, 256, 0, st>>>(A); break;
-    case 3: extend_kernel<3, PASS_DOMAIN><<<grid, 256, 0, st>>>(A); break;
-    case 4: extend_kernel<4, PASS_DOMAIN><<<grid, 256, 0, st>>>(A); break;
-    case 5: extend_kernel<5, PASS_DOMAIN><<<grid, 256, 0, st>>>(A); break;
     case 6: extend_kernel<6, PASS_DOMAIN><<<grid, 256, 0, st>>>(A); break;
     case 7: return launch_extend_l7(PASS_DOMAIN, A, grid, st);
     default: return cudaErrorInvalidValue;
@@ -25,11 +20,6 @@ cudaError_t occupancy_extend_domain(int L, int V, int *blocks_per_sm) {
     if (V == FSM_EXPLORE_TV_EDGELIST) return occupancy_extend_edgelist(PASS_DOMAIN, L, blocks_per_sm);
     if (V == FSM_EXPLORE_TV_QUOTA) return occupancy_extend_quota(PASS_DOMAIN, L, blocks_per_sm);
     switch (L) {
-    case 1: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, extend_kernel<1, PASS_DOMAIN>, 256, 0);
-    case 2: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, extend_kernel<2, PASS_DOMAIN>, 256, 0);
-    case 3: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, extend_kernel<3, PASS_DOMAIN>, 256, 0);
-    case 4: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, extend_kernel<4, PASS_DOMAIN>, 256, 0);
-    case 5: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, extend_kernel<5, PASS_DOMAIN>, 256, 0);
     case 6: return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, extend_kernel<6, PASS_DOMAIN>, 256, 0);
     case 7: return occupancy_extend_l7(PASS_DOMAIN, blocks_per_sm);
     default: return cudaErrorInvalidValue;

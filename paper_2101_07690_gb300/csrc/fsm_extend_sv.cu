@@ -6,11 +6,11 @@
 namespace fsm {
 
 cudaError_t launch_extend_sv(int pass, int L, const ExtArgs &A, int grid, cudaStream_t st) {
-    return launch_variant<FSM_EXPLORE_SV, 6>(pass, L, A, grid, st);
+    return launch_variant<FSM_EXPLORE_SV, 1, 6>(pass, L, A, grid, st);
 }
 
 cudaError_t occupancy_extend_sv(int pass, int L, int *blocks_per_sm) {
-    return occupancy_variant<FSM_EXPLORE_SV, 6>(pass, L, blocks_per_sm);
+    return occupancy_variant<FSM_EXPLORE_SV, 1, 6>(pass, L, blocks_per_sm);
 }
 
 } // namespace fsm

@@ -1,0 +1,1064 @@
+// fsm_join.cuh -- the two-vertex extension kernel for stored levels of size l <= 5 (l -> l+2,
+// k <= 7; two-vertex exploration with index-based quick patterns, exact, rate-sampled or under
+// Section 5's quotas).  fsm_extend.cuh states the work of a join and holds the kernel of the other
+// forms; this one does the same joins in another order of steps.
+//
+// What bounds a level is the number of candidate pieces times the instructions each costs (DRAM
+// and L2 are nearly idle), so the steps are ordered by what they reject per instruction, and every
+// step runs with full warps:
+//
+//   tables     Whether smallest-vertex-first dissection (Algorithm 1) returns exactly (t, s) depends
+//              only on the relative order of the l + 2 ids and on the edges among them.  With s
+//              sorted by id, that is: the class of s (rank of the key vertex, edges of s in id
+//              order), the piece's form, the slots of its two new vertices a and b (how many ids of
+//              s lie below each), whether b > a, and the cross-edge subset.  `acc` holds one bit per
+//              combination (all 2^(2(l-1)) subsets of a row side by side), `any` the OR over
+//              subsets and forms for one new vertex's slot against the other's.
+//   segments   A unit's pieces are rows of sorted lists: centre row y (anchor b = y-th neighbour of
+//              v, partners a = the neighbours before it) and end list a (anchor a, partners b in
+//              N(a)).  One lane prepares one row: the slots its anchor allows its partner cut the
+//              row to a range (a row with none costs nothing more).
+//   filter     Lanes then walk the surviving ranges side by side: one coalesced list read, the
+//              partner's slot by l comparisons, one bit test.  Survivors go to a per-warp queue.
+//   joins      Full warps take 32 survivors: labels and ranks (one 16-byte read per vertex), the
+//              size-3 frequency of the piece, cross edges (a shared-memory Bloom filter of each
+//              list of s, misses are certain, hits are verified by binary search), joining-point
+//              pruning (Section 4.5) as cross bits that must or must not be set, then the subsets
+//              that are left and accepted by `acc`.
+//   accept     Keys go through one open-addressed table per block in shared memory that also holds
+//              each key's bitmap offsets; it is flushed between chunks when it fills.
+//
+// One launch on a GB300, the extension kernel before and this one (same graph and output):
+//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms ->  77.7 ms
+//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms -> 283 ms
+//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms ->  18.5 ms
+//   5 -> 7, count, ST 8 quotas, 6.0e8 pieces, 1.2e8 joins:          248 ms ->  60.6 ms
+//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms ->  8.1 ms
+#pragma once
+#include "fsm_extend.cuh"
+
+namespace fsm {
+
+// forms of a piece, by the order (a, b) in which its two non-key vertices are kept
+enum { FORM_CENTRE = 0, FORM_END = 1, FORM_TRI = 2 };
+// rows of `any`: centre rows that stand for the wedge only / for wedge and triangle, end lists
+// for the wedge only / for the wedge and, when b > a, the triangle
+enum { ANY_C = 0, ANY_CT = 1, ANY_E = 2, ANY_ET = 3 };
+
+// Geometry of the tables and of a warp's shared storage for stored size L.
+template <int L> struct JoinGeo {
+    static constexpr int K = L + 2;
+    static constexpr int O = L - 1;                  // vertices of s other than the key vertex
+    static constexpr int SUBS = 1 << (2 * O);        // cross-edge subsets
+    static constexpr int W = SUBS > 32 ? SUBS / 32 : 1;
+    static constexpr int EB = L * (L - 1) / 2;       // edge bits of s, pairs (0,1), (0,2), ... in id order
+    static constexpr int CLS = L << EB;              // class = rank of v << EB | edge bits
+    static constexpr int SL = L + 1;                 // slots of a new vertex
+    static constexpr int ROWS = 3 * SL * SL * 2;     // ((form * SL + slot a) * SL + slot b) * 2 + (b > a)
+    static constexpr int64_t ACC_WORDS = (int64_t)CLS * ROWS * W;
+    static constexpr int64_t ANY_ENTRIES = (int64_t)CLS * 4 * SL;   // (class * 4 + ANY_*) * SL + anchor slot
+};
+
+// Is the join accepted (edge-induced graph given by class, form, slots and cross subset)?  Vertices
+// are renamed by id order; sub bit r: a next to the r-th other vertex of s (in id order), bit
+// O + r: b next to it.
+template <int L>
+FSM_HD bool join_accepted(int cls, int form, int sa, int sb, int bgt, uint32_t sub) {
+    constexpr int K = L + 2, O = L - 1;
+    if (sa != sb && (sb > sa) != (bgt != 0)) return false;   // no such order
+    if (form != FORM_END && !bgt) return false;              // centre pieces and triangles keep a < b
+    if constexpr (L == 1) {
+        return sa == 1 && sb == 1;   // size-3 subgraphs are made at their smallest vertex
+    } else {
+        const int rv = cls >> JoinGeo<L>::EB;
+        int pos[L];
+        uint32_t adj[K];
+        int32_t gid[K];
+        for (int h = 0; h < K; ++h) { adj[h] = 0; gid[h] = h; }
+        for (int t = 0; t < L; ++t) pos[t] = t + (sa <= t) + (sb <= t);
+        const int pa = sa + (bgt ? 0 : 1), pb = sb + (bgt ? 1 : 0);
+        auto link = [&](int x, int y) { adj[x] |= 1u << y; adj[y] |= 1u << x; };
+        int bit = 0;
+        for (int t = 0; t < L; ++t)
+            for (int u = t + 1; u < L; ++u, ++bit)
+                if ((cls >> bit) & 1) link(pos[t], pos[u]);
+        uint32_t ms = 0;
+        for (int t = 0; t < L; ++t) ms |= 1u << pos[t];
+        if (!mask_connected(ms, adj, K)) return false;       // no stored embedding has this class
+        link(pos[rv], pa);
+        if (form != FORM_END) link(pos[rv], pb);
+        if (form != FORM_CENTRE) link(pa, pb);
+        for (int r = 0; r < O; ++r) {
+            const int t = r + (r >= rv);
+            if ((sub >> r) & 1u) link(pos[t], pa);
+            if ((sub >> (O + r)) & 1u) link(pos[t], pb);
+        }
+        uint32_t lm = 0;
+        int jn = -1;
+        dissect3(K, gid, adj, lm, jn);
+        return jn == pos[rv] && lm == ((1u << pos[rv]) | (1u << pa) | (1u << pb));
+    }
+}
+
+// survivors of the filter wait here until 32 are there
+#define FSM_JOIN_QUEUE 64
+// shared words per warp for the Bloom filters of a batch of units
+#define FSM_JOIN_BLOOM 512
+// slots of a block's key table
+#define FSM_JOIN_SLOTS 512
+#define FSM_JOIN_PROBES 8
+#define FSM_OFF_NONE 0xFFFFFFFFu     // key whose pattern has no bitmaps
+#define FSM_OFF_PENDING 0xFFFFFFFEu  // offsets not yet known (never a valid offset)
+
+// A batch's units in shared memory: UW words each.
+template <int L, bool QUOTA> struct UnitRec {
+    static constexpr int O = L - 1;
+    static constexpr int U = L <= 3 ? 16 : 8;        // units per batch
+    static constexpr int RP = 0, D = 1, PID = 2, META = 3, CLS = 4, OLAB = 5, OPP = 6, SEG = 7, SLO = 8, RLO = 9,
+                         RHI = 11, NC = 13, SS = 15, BND = SS + L, RK = BND + L, OB = RK + L, OE = OB + O, OK = OE + O,
+                         QA = OK + 6 * O, END = QA + (QUOTA ? 6 : 0);
+    static constexpr int UW = END | 1;               // odd stride: lanes on different units hit different banks
+};
+
+template <int L, int PASS, bool QUOTA> struct JoinSmem {
+    using R = UnitRec<L, QUOTA>;
+    static constexpr int K = L + 2;
+    static constexpr bool COUNTS = PASS == PASS_COUNT || PASS == PASS_FUSED;
+    static constexpr bool OFFS = PASS == PASS_DOMAIN || PASS == PASS_FUSED;
+    static constexpr int NS = PASS == PASS_EMIT ? 0 : FSM_JOIN_SLOTS;
+    unsigned long long key[NS ? NS : 1];
+    uint32_t cnt[COUNTS ? NS : 1];
+    uint32_t off[OFFS ? K : 1][OFFS ? NS : 1];
+    int load, flag, done;
+    uint32_t unit[8][R::U * R::UW];
+    uint32_t bloom[8][FSM_JOIN_BLOOM];
+    uint32_t qa[8][FSM_JOIN_QUEUE], qb[8][FSM_JOIN_QUEUE];
+    uint8_t qm[8][FSM_JOIN_QUEUE];
+    uint32_t sg_base[8][32], sg_anchor[8][32], sg_info[8][32];
+};
+
+__device__ __forceinline__ int32_t sorted_has(const int32_t *col, int32_t lo, int32_t end, int32_t x) {
+    int32_t hi = end;
+    while (lo < hi) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (__ldg(col + mid) < x) lo = mid + 1; else hi = mid;
+    }
+    return lo < end && __ldg(col + lo) == x;
+}
+
+__device__ __forceinline__ int32_t below(const int32_t *a, int32_t n, int32_t x) {
+    int32_t lo = 0, hi = n;
+    while (lo < hi) {
+        const int32_t mid = (lo + hi) >> 1;
+        if (__ldg(a + mid) < x) lo = mid + 1; else hi = mid;
+    }
+    return lo;
+}
+
+// Largest u in [lo, hi] with base[u] <= x (base[lo] <= x), by the whole warp: 32 probes per step,
+// so a prefix of millions of units takes five dependent reads instead of over twenty.
+__device__ __forceinline__ int64_t warp_last_le(const int64_t *base, int64_t lo, int64_t hi, int64_t x) {
+    const int lane = threadIdx.x & 31;
+    while (lo < hi) {
+        const int64_t step = (hi - lo + 31) >> 5;
+        const int64_t p = lo + (int64_t)(lane + 1) * step;
+        const bool le = p <= hi && __ldg(base + p) <= x;
+        const int c = __popc(__ballot_sync(0xffffffffu, le));   // base is nondecreasing: a prefix of the lanes
+        lo += (int64_t)c * step;
+        hi = min(hi, lo + step - 1);
+    }
+    return lo;
+}
+
+__device__ __forceinline__ unsigned long long rec_u64(const uint32_t *r, int w) {
+    return (unsigned long long)r[w] | ((unsigned long long)r[w + 1] << 32);
+}
+__device__ __forceinline__ void rec_put64(uint32_t *r, int w, unsigned long long x) {
+    r[w] = (uint32_t)x;
+    r[w + 1] = (uint32_t)(x >> 32);
+}
+
+// Row y of the centre pairs that holds pair number q: rows y < c hold y pairs, later rows c
+// (c = d when every pair is enumerated).
+__device__ __forceinline__ int32_t centre_row(int64_t q, int32_t c, int32_t d) {
+    const int64_t nt = (int64_t)c * (c - 1) / 2;
+    if (q < nt) {
+        int32_t y = (int32_t)((1.0f + sqrtf(1.0f + 8.0f * (float)q)) * 0.5f);
+        while ((int64_t)y * (y - 1) / 2 > q) --y;
+        while ((int64_t)(y + 1) * y / 2 <= q) ++y;
+        return y;
+    }
+    const int64_t r = q - nt;
+    return c + (int32_t)(r <= 0xffffffffll ? (int64_t)((uint32_t)r / (uint32_t)c) : r / c);
+}
+__device__ __forceinline__ int64_t centre_row_start(int32_t y, int32_t c) {
+    return y <= c ? (int64_t)y * (y - 1) / 2 : (int64_t)c * (c - 1) / 2 + (int64_t)(y - c) * c;
+}
+// the end list of the unit's key vertex that holds end piece number q
+__device__ __forceinline__ int32_t end_row(const int32_t *pend, int32_t d, int64_t q) {
+    int32_t lo = 0, hi = d - 1;
+    while (lo < hi) {
+        const int32_t mid = (lo + hi + 1) >> 1;
+        if ((int64_t)__ldg(pend + mid) <= q) lo = mid; else hi = mid - 1;
+    }
+    return lo;
+}
+
+// ---- one-pass last level: publication of a key slot's bitmap offsets (gpu-scope release/acquire)
+__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t *p) {
+    uint32_t v;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ void st_release_u32(uint32_t *p, uint32_t v) {
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+__device__ __forceinline__ void st_relaxed_u32(uint32_t *p, uint32_t v) {
+    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+// First sight of a quick pattern in the one-pass last level: canonicalise the graph its key
+// denotes, find or claim its pattern's entry in the code table, claim the pattern's orbit
+// bitmaps from the pool unless another lane already did (one CAS decides; a loser's pool words
+// stay unused), and publish the bitmap offset of each local position -- position 0 last, with
+// release semantics, so a reader that sees it set sees the others.  Lanes racing on one key
+// compute and write the same values.  On a full table or pool the error word says so and nothing
+// is published; the host then runs the last level as two passes.
+struct ResolveArgs {
+    const uint64_t *pat_lab, *pat_adj;
+    const int32_t *cls_size;
+    unsigned long long *code_keys, *code_off, *pool_top;
+    uint64_t code_mask;
+    unsigned long long pool_words;
+    uint32_t *slot_off;
+    int shift;
+    int *err;
+    int explore, level;
+};
+
+static __device__ __noinline__ void resolve_slot(const ResolveArgs A, int64_t slot, uint64_t key) {
+    // K <= 7 here: the compact words of fsm_canon7.cuh
+    int K, lab[8], rep[8];
+    uint32_t adj[8];
+    key_graph7(A.explore, A.level, key, A.pat_lab, A.pat_adj, K, lab, adj);
+    unsigned long long clab;
+    uint32_t cadj, inv;
+    canonicalise7(K, lab, adj, clab, cadj, inv);
+    orbit_reps7(K, clab, cadj, rep);
+    int64_t pre[8], words = 0;
+    for (int c = 0; c < K; ++c) {
+        pre[c] = words;
+        if (rep[c] == c)
+            words += bitmap_words(__ldg(A.cls_size + ((clab >> (8 * (7 - c))) & 0xff)), A.shift);
+    }
+    const uint64_t pk = pack_code7(K, clab, cadj);
+    uint64_t h = mix64(pk) & A.code_mask;
+    int64_t ci = -1;
+    for (int probe = 0; probe < FSM_MAX_PROBES; ++probe) {
+        unsigned long long cur = __ldcg(A.code_keys + h);
+        if (cur == FSM_EMPTY_KEY) cur = atomicCAS(A.code_keys + h, FSM_EMPTY_KEY, pk);
+        if (cur == FSM_EMPTY_KEY || cur == pk) { ci = (int64_t)h; break; }
+        h = (h + 1) & A.code_mask;
+    }
+    if (ci < 0) { atomicOr(A.err, FSM_ERR_CODE_FULL); return; }
+    unsigned long long off = __ldcg(A.code_off + ci);
+    if (off == 0ull) {
+        const unsigned long long res = atomicAdd(A.pool_top, (unsigned long long)words);
+        if (res + (unsigned long long)words > A.pool_words) { atomicOr(A.err, FSM_ERR_POOL); return; }
+        const unsigned long long old = atomicCAS(A.code_off + ci, 0ull, res + 1ull);
+        off = old ? old : res + 1ull;
+    }
+    uint32_t *so = A.slot_off + slot * 8;
+    for (int hh = K - 1; hh >= 0; --hh) {
+        const uint32_t v = (uint32_t)(((long long)(off - 1ull) + pre[rep[(inv >> (3 * hh)) & 7]]) >> A.shift);
+        if (hh) st_relaxed_u32(so + hh, v); else st_release_u32(so, v);
+    }
+}
+
+// Offsets (in units of 1 << off_shift words) of a key's bitmaps from the global tables: the domain
+// pass's table, or in the one-pass level the published slot, resolved on first sight.
+template <int K, int PASS>
+__device__ __forceinline__ bool key_offsets(const ExtArgs &A, uint64_t key, int64_t slot, uint32_t (&off)[K]) {
+    if (PASS == PASS_DOMAIN) {
+        const uint32_t *sb = A.slot_off32 + slot * 8;
+#pragma unroll
+        for (int h = 0; h < K; ++h) off[h] = __ldg(sb + h);
+        return true;
+    }
+    const uint32_t *so = A.slot_off32 + slot * 8;
+    uint32_t o0 = ld_acquire_u32(so);
+    if (o0 == FSM_OFF_NONE) {   // not yet published
+        const ResolveArgs R{A.pat_lab, A.pat_adj, A.cls_size, A.code_keys, A.code_off, A.pool_top,
+                            A.code_mask, A.pool_words, A.slot_off32, A.off_shift, A.err, A.explore, A.level};
+        resolve_slot(R, slot, key);
+        o0 = ld_acquire_u32(so);
+        if (o0 == FSM_OFF_NONE) return false;   // a table or the pool is full: the error word says so
+    }
+    off[0] = o0;
+#pragma unroll
+    for (int h = 1; h < K; ++h) off[h] = ld_relaxed_u32(so + h);
+    return true;
+}
+
+template <int L, int PASS, bool QUOTA>
+struct Joiner {
+    using G = JoinGeo<L>;
+    using R = UnitRec<L, QUOTA>;
+    using SM = JoinSmem<L, PASS, QUOTA>;
+    static constexpr int K = L + 2, O = L - 1, SL = L + 1;
+
+    const ExtArgs &A;
+    SM &sm;
+    const int w, lane;
+    int qn = 0;                       // survivors waiting
+    int lb = 5;                       // log2 bits of one Bloom filter of this batch
+    bool tfe;                         // triangles are made from end lists (see take)
+    unsigned long long tested = 0, accepted = 0;
+
+    __device__ __forceinline__ Joiner(const ExtArgs &a, SM &s)
+        : A(a), sm(s), w(threadIdx.x >> 5), lane(threadIdx.x & 31),
+          // An end piece v-a-b with b next to v closes the triangle {v, a, b}; taking it there, once
+          // (a < b), costs one Bloom probe on a survivor, where testing every surviving centre pair
+          // costs a search.  Kept pieces (sampling) and numbered candidates (quotas) are defined with
+          // the triangle at the centre pair, and vertex-induced centre pairs need the test anyway.
+          tfe(!QUOTA && a.mode == 0 && !a.sampled) {}
+
+    __device__ __forceinline__ uint32_t *rec(int j) { return sm.unit[w] + j * R::UW; }
+
+    // x in the list of the t-th smallest vertex of unit j's s?  A clear Bloom bit is a certain no.
+    __device__ __forceinline__ bool maybe(int j, int t, int32_t x) const {
+        const uint32_t h = ((uint32_t)x * 0x9E3779B1u) >> (32 - lb);
+        return (sm.bloom[w][((j * L + t) << (lb - 5)) + (h >> 5)] >> (h & 31)) & 1u;
+    }
+
+    // ---- the block's key table
+    __device__ __forceinline__ int table_find(uint64_t key) {
+        uint32_t h = ((uint32_t)key * 0x9E3779B1u) ^ ((uint32_t)(key >> 32) * 0x85EBCA77u);
+        h = (h ^ (h >> 15)) & (FSM_JOIN_SLOTS - 1);
+#pragma unroll 1
+        for (int p = 0; p < FSM_JOIN_PROBES; ++p) {
+            unsigned long long cur = ((volatile unsigned long long *)sm.key)[h];
+            if (cur == FSM_EMPTY_KEY) {
+                cur = atomicCAS(&sm.key[h], FSM_EMPTY_KEY, (unsigned long long)key);
+                if (cur == FSM_EMPTY_KEY) {
+                    if (atomicAdd(&sm.load, 1) >= FSM_JOIN_SLOTS * 3 / 4) sm.flag = 1;
+                    return (int)h;
+                }
+            }
+            if (cur == key) return (int)h;
+            h = (h + 1) & (FSM_JOIN_SLOTS - 1);
+        }
+        sm.flag = 1;
+        return -1;
+    }
+
+    __device__ __forceinline__ void set_bits(const uint32_t (&off)[K], const uint32_t *r, uint32_t ra, uint32_t rb, bool swap) {
+        uint32_t *base = PASS == PASS_DOMAIN ? A.dom : A.pool;
+        uint32_t *wd[K];
+        uint32_t bit[K], old[K];
+#pragma unroll
+        for (int h = 0; h < K; ++h) {
+            const uint32_t rk = h < L ? r[R::RK + (h < L ? h : 0)] : ((h == L) != swap ? ra : rb);
+            wd[h] = base + ((uint64_t)off[h] << A.off_shift) + (rk >> 5);
+            bit[h] = 1u << (rk & 31);
+        }
+        // read first: most bits are set already, and the reads of one join overlap
+#pragma unroll
+        for (int h = 0; h < K; ++h) old[h] = __ldcg(wd[h]);
+#pragma unroll
+        for (int h = 0; h < K; ++h)
+            if (!(old[h] & bit[h])) atomicOr(wd[h], bit[h]);
+    }
+
+    // One accepted join of this lane (not warp-synchronous).
+    __device__ __forceinline__ void accept(const uint32_t *r, uint64_t key, int32_t a, int32_t b, uint32_t ra, uint32_t rb,
+                                           bool swap) {
+        if constexpr (PASS == PASS_COUNT) {
+            const int e = table_find(key);
+            if (e >= 0) { atomicAdd(&sm.cnt[e], 1u); return; }
+            const int64_t slot = qp_insert(A.qp, key, A.err);
+            if (slot >= 0) atomicAdd(A.qp.count + slot, 1ull);
+        } else if constexpr (PASS == PASS_FUSED || PASS == PASS_DOMAIN) {
+            const int e = table_find(key);
+            uint32_t off[K];
+            off[0] = FSM_OFF_PENDING;
+            if (e >= 0) {
+                if (PASS == PASS_FUSED) atomicAdd(&sm.cnt[e], 1u);
+                off[0] = ((volatile uint32_t *)sm.off[0])[e];
+                if (off[0] != FSM_OFF_PENDING) {
+#pragma unroll
+                    for (int h = 1; h < K; ++h) off[h] = ((volatile uint32_t *)sm.off[h])[e];
+                }
+            }
+            if (off[0] == FSM_OFF_PENDING) {
+                int64_t slot;
+                if (PASS == PASS_DOMAIN) {
+                    slot = qp_find(A.qp, key);
+                    if (slot < 0) { atomicOr(A.err, FSM_ERR_QP_MISSING); return; }
+                } else {
+                    slot = qp_insert(A.qp, key, A.err);
+                    if (slot < 0) return;
+                    if (e < 0) atomicAdd(A.qp.count + slot, 1ull);
+                }
+                if (!key_offsets<K, PASS>(A, key, slot, off)) return;
+                if (e >= 0) {   // lanes racing here write the same values; position 0 last
+#pragma unroll
+                    for (int h = 1; h < K; ++h) ((volatile uint32_t *)sm.off[h])[e] = off[h];
+                    __threadfence_block();
+                    ((volatile uint32_t *)sm.off[0])[e] = off[0];
+                }
+            }
+            if (off[0] == FSM_OFF_NONE) return;   // pattern without domains
+            set_bits(off, r, ra, rb, swap);
+        } else {
+            const int64_t slot = qp_find(A.qp, key);
+            if (slot < 0) { atomicOr(A.err, FSM_ERR_QP_MISSING); return; }
+            const int32_t nid = __ldg(A.newid + __ldg(A.qp.pattern + slot));
+            if (nid < 0) return;
+            const uint64_t perm = __ldg(A.qp.perm + slot);
+            const unsigned act = __activemask();
+            const int leader = __ffs(act) - 1;
+            unsigned long long base = 0;
+            if (lane == leader) base = atomicAdd(A.out_cursor, (unsigned long long)__popc(act));
+            base = __shfl_sync(act, base, leader);
+            const int64_t pos = (int64_t)base + __popc(act & ((1u << lane) - 1u));
+            if (pos >= A.out_N) { atomicOr(A.err, FSM_ERR_BOUNDS); return; }
+            const uint32_t meta = r[R::META];
+#pragma unroll
+            for (int t = 0; t < L; ++t) {
+                const int h = (int)(meta >> (12 + 3 * t)) & 7;   // canonical position of the t-th smallest
+                A.out_v[(int64_t)nib_get(perm, h) * A.out_N + pos] = (int32_t)r[R::SS + t];
+            }
+            A.out_v[(int64_t)nib_get(perm, L) * A.out_N + pos] = swap ? b : a;
+            A.out_v[(int64_t)nib_get(perm, L + 1) * A.out_N + pos] = swap ? a : b;
+            A.out_pid[pos] = nid;
+        }
+    }
+
+    // The last n (<= 32) survivors of the queue, one per lane; warp-synchronous.
+    __device__ __forceinline__ void take(int n) {
+        __syncwarp();
+        const bool on = lane < n;
+        const int q = qn - n + (on ? lane : 0);
+        const uint32_t m = sm.qm[w][q];
+        const int32_t a = (int32_t)sm.qa[w][q], b = (int32_t)sm.qb[w][q];
+        const int j = m & 15;
+        const bool centre = (m & 16) == 0;
+        const uint32_t *r = rec(j);
+        const uint32_t meta = r[R::META];
+        const int ki = meta & 7, rv = (meta >> 3) & 7, lv = (meta >> 6) & 63;
+        const int32_t v = (int32_t)r[R::SS + rv];
+        const int4 ia = __ldg(A.g.vinfo + a), ib = __ldg(A.g.vinfo + b);
+        const int la = ia.z, lb_ = ib.z;
+        uint32_t forms = 0;
+        if (on) {
+            if (centre) {
+                forms = 1u << FORM_CENTRE;
+                if (!tfe) {
+                    const bool shorter = ia.y - ia.x <= ib.y - ib.x;
+                    if (shorter ? sorted_has(A.g.col, ia.x, ia.y, b) : sorted_has(A.g.col, ib.x, ib.y, a))
+                        forms = A.mode == 1 ? 1u << FORM_TRI : forms | (1u << FORM_TRI);
+                }
+            } else {
+                forms = 1u << FORM_END;
+                if (tfe) {
+                    if (a < b && maybe(j, rv, b) && sorted_has(A.g.col, (int32_t)r[R::RP], (int32_t)(r[R::RP] + r[R::D]), b))
+                        forms |= 1u << FORM_TRI;
+                } else if (A.mode == 1 && sorted_has(A.g.col, ib.x, ib.y, v)) {
+                    forms = 0;   // vertex-induced: only the triangle
+                }
+            }
+        }
+        if (A.lf) {
+            // the piece's own size-3 pattern must be frequent
+            if ((forms & (1u << FORM_CENTRE)) && !((__ldg(A.lf + lv * 64 + la) >> lb_) & 1ull)) forms &= ~(1u << FORM_CENTRE);
+            if ((forms & (1u << FORM_END)) && !((__ldg(A.lf + la * 64 + lv) >> lb_) & 1ull)) forms &= ~(1u << FORM_END);
+            if ((forms & (1u << FORM_TRI)) && !((__ldg(A.lf + 8192 + lv * 64 + la) >> lb_) & 1ull)) forms &= ~(1u << FORM_TRI);
+        }
+        const bool ab = lab_id_less(la, a, lb_, b);
+        const bool va = lab_id_less(lv, v, la, a), vb = lab_id_less(lv, v, lb_, b);
+        auto piece = [&](int form, int &jpos) -> uint32_t {
+            if (form == FORM_CENTRE) {
+                jpos = 0;
+                return piece_index(PIECE_WEDGE, lv, ab ? la : lb_, ab ? lb_ : la);
+            }
+            if (form == FORM_END) {
+                jpos = vb ? 1 : 2;
+                return piece_index(PIECE_WEDGE, la, vb ? lv : lb_, vb ? lb_ : lv);
+            }
+            jpos = (va ? 0 : 1) + (vb ? 0 : 1);
+            return tri_index(lv, la, lb_);
+        };
+        if (A.piece_sel && forms) {
+            int jp;
+#pragma unroll
+            for (int f = 0; f < 3; ++f)
+                if ((forms >> f & 1u) && !__ldg(A.piece_sel + piece(f, jp))) forms &= ~(1u << f);
+        }
+        // cross edges, and the cross bits pruning forces off (no*) or on (must) -- a's for any
+        // form, b's for forms in which b is next to v (bv) or not (be)
+        uint32_t avail = 0, no_a = 0, must_a = 0, no_bv = 0, must_bv = 0, no_be = 0;
+        int sa = 0, sb = 0;
+        if (forms) {
+#pragma unroll
+            for (int t = 0; t < L; ++t) {
+                const int32_t x = (int32_t)r[R::SS + t];
+                sa += x < a;
+                sb += x < b;
+            }
+#pragma unroll
+            for (int o = 0; o < O; ++o) {
+                const int t = o + (o >= rv);
+                const int32_t ob = (int32_t)r[R::OB + o], oe = (int32_t)r[R::OE + o];
+                if (maybe(j, t, a) && sorted_has(A.g.col, ob, oe, a)) avail |= 1u << o;
+                if (maybe(j, t, b) && sorted_has(A.g.col, ob, oe, b)) avail |= 1u << (O + o);
+                if (A.lf) {
+                    const unsigned long long k0 = rec_u64(r, R::OK + 6 * o), k1 = rec_u64(r, R::OK + 6 * o + 2),
+                                             k2 = rec_u64(r, R::OK + 6 * o + 4);
+                    must_a |= (uint32_t)(~(k0 >> la) & 1ull) << o;
+                    no_a |= (uint32_t)(~(k1 >> la) & 1ull) << o;
+                    must_bv |= (uint32_t)(~(k0 >> lb_) & 1ull) << (O + o);
+                    no_bv |= (uint32_t)(~(k1 >> lb_) & 1ull) << (O + o);
+                    no_be |= (uint32_t)(~(k2 >> lb_) & 1ull) << (O + o);
+                }
+            }
+        }
+        const uint32_t *rows = A.acc + ((int64_t)r[R::CLS] * G::ROWS + (sa * SL + sb) * 2 + (b > a)) * G::W;
+        int form = 0;
+        uint32_t must = 0, free_ = 0, cur = 0, sub = 0;
+        bool more = false;
+        const uint32_t *row = rows;
+        uint32_t roww = 0;
+        for (;;) {
+            bool have = false;
+            while (!have) {
+                if (!more) {
+                    if (!forms) break;
+                    form = __ffs(forms) - 1;
+                    forms &= forms - 1;
+                    const uint32_t no = no_a | (form == FORM_END ? no_be : no_bv);
+                    must = must_a | (form == FORM_END ? 0u : must_bv);
+                    if ((must & ~avail) || (must & no)) continue;
+                    if (A.mode == 0) {
+                        free_ = avail & ~no & ~must;
+                    } else {
+                        if (avail & no) continue;
+                        must = avail;   // vertex-induced: every cross edge
+                        free_ = 0;
+                    }
+                    cur = free_;
+                    more = true;
+                    row = rows + (int64_t)form * (SL * SL * 2) * G::W;
+                    if (G::W == 1) {
+                        roww = __ldg(row);
+                        if (!roww) { more = false; continue; }
+                    }
+                }
+                sub = cur | must;
+                ++tested;
+                have = ((G::W == 1 ? roww : __ldg(row + (sub >> 5))) >> (sub & 31)) & 1u;
+                if (cur == 0) more = false; else cur = (cur - 1) & free_;
+            }
+            if (!__any_sync(0xffffffffu, have)) break;
+            if (have) {
+                ++accepted;
+                int jpos;
+                const uint32_t pidx = piece(form, jpos);
+                const bool swap = form != FORM_END && !ab;   // the key's first new vertex is b
+                uint32_t cross = 0;
+                const uint32_t opp = r[R::OPP];
+#pragma unroll
+                for (int o = 0; o < O; ++o) {
+                    const int pp = (opp >> (3 * o)) & 7;
+                    cross |= ((sub >> o) & 1u) << (2 * pp + (swap ? 1 : 0));
+                    cross |= ((sub >> (O + o)) & 1u) << (2 * pp + (swap ? 0 : 1));
+                }
+                accept(r, make_key(r[R::PID], pidx, ki, jpos, cross, L), a, b, (uint32_t)ia.w, (uint32_t)ib.w, swap);
+            }
+        }
+        qn -= n;
+        __syncwarp();
+    }
+
+    // warp-synchronous: queue the survivors among the lanes' candidates, joining when 32 wait
+    __device__ __forceinline__ void push(bool ok, int32_t a, int32_t b, uint32_t m) {
+        const unsigned bal = __ballot_sync(0xffffffffu, ok);
+        if (ok) {
+            const int p = qn + __popc(bal & ((1u << lane) - 1u));
+            sm.qa[w][p] = (uint32_t)a;
+            sm.qb[w][p] = (uint32_t)b;
+            sm.qm[w][p] = (uint8_t)m;
+        }
+        qn += __popc(bal);
+        if (qn >= 32) take(32);
+    }
+
+    // Load units u0 .. u0 + nu - 1 (raw candidate range [q0, q1) of the chunk) into shared memory.
+    __device__ __forceinline__ void load_units(int64_t u0, int nu, int64_t q0, int64_t q1) {
+        const DevGraph &g = A.g;
+        uint32_t *r = rec(lane < nu ? lane : 0);
+        int nseg = 0;
+        if (lane < nu) {
+            const int64_t u = u0 + lane;
+            const int64_t e = A.e0 + u / L;
+            const int iu = (int)(u % L);
+            const int32_t pid = __ldg(A.fpid + e);
+            const uint64_t srows = L >= 2 ? __ldg(A.pat_adj + pid) : 0ull;
+            int32_t id[L];
+            int cp[L];
+#pragma unroll
+            for (int p = 0; p < L; ++p) { id[p] = __ldg(A.fv + (int64_t)p * A.fN + e); cp[p] = p; }
+            // sort by id, carrying canonical positions
+#pragma unroll
+            for (int x = 1; x < L; ++x)
+#pragma unroll
+                for (int y = L - 1; y >= x; --y)
+                    if (id[y] < id[y - 1]) {
+                        const int32_t ti = id[y]; id[y] = id[y - 1]; id[y - 1] = ti;
+                        const int tc = cp[y]; cp[y] = cp[y - 1]; cp[y - 1] = tc;
+                    }
+            int rv = 0, lv = 0;
+            int32_t v = 0;
+            int4 nfo[L];
+            uint32_t meta = (uint32_t)iu;
+#pragma unroll
+            for (int t = 0; t < L; ++t) {
+                nfo[t] = __ldg(g.vinfo + id[t]);
+                if (cp[t] == iu) { rv = t; v = id[t]; lv = nfo[t].z; }
+                meta |= (uint32_t)cp[t] << (12 + 3 * t);
+                r[R::SS + t] = (uint32_t)id[t];
+                r[R::RK + cp[t]] = (uint32_t)nfo[t].w;
+            }
+            meta |= ((uint32_t)rv << 3) | ((uint32_t)lv << 6);
+            uint32_t cls = (uint32_t)rv << G::EB;
+            int bit = 0;
+#pragma unroll
+            for (int t = 0; t < L; ++t)
+#pragma unroll
+                for (int t2 = t + 1; t2 < L; ++t2, ++bit)
+                    cls |= ((uint32_t)(srows >> (8 * cp[t] + cp[t2])) & 1u) << bit;
+            const int32_t rp = __ldg(g.prow + v), d = __ldg(g.prow + v + 1) - rp;
+            r[R::RP] = (uint32_t)rp;
+            r[R::D] = (uint32_t)d;
+            r[R::PID] = (uint32_t)pid;
+            r[R::META] = meta;
+            r[R::CLS] = cls;
+            uint32_t opp = 0;
+#pragma unroll
+            for (int t = 0; t < L; ++t) {
+                if (t == rv) continue;
+                const int o = t - (t > rv);
+                const int lo = nfo[t].z;
+                opp |= (uint32_t)(cp[t] < iu ? cp[t] : cp[t] - 1) << (3 * o);
+                r[R::OB + o] = (uint32_t)nfo[t].x;
+                r[R::OE + o] = (uint32_t)nfo[t].y;
+                if (A.lf) {
+                    // labels of a new vertex x with which {v, o, x} may be left as it is:
+                    // k0 x next to v only, k1 next to v and o, k2 next to o only
+                    const bool e1 = (srows >> (8 * iu + cp[t])) & 1ull;
+                    const unsigned long long k0 = e1 ? __ldg(A.lf + lv * 64 + lo) : ~0ull;
+                    const unsigned long long k1 = __ldg(A.lf + (e1 ? 8192 : 4096) + lv * 64 + lo);
+                    const unsigned long long k2 = e1 ? __ldg(A.lf + lo * 64 + lv) : ~0ull;
+                    rec_put64(r, R::OK + 6 * o, k0);
+                    rec_put64(r, R::OK + 6 * o + 2, k1);
+                    rec_put64(r, R::OK + 6 * o + 4, k2);
+                }
+            }
+            r[R::OPP] = opp;
+            int32_t cpos = d;
+#pragma unroll
+            for (int t = 0; t < L; ++t) {
+                const int32_t bd = below(g.pcol + rp, d, id[t]);
+                r[R::BND + t] = (uint32_t)bd;
+                if (L == 2 && t != rv) cpos = bd;
+            }
+            const int64_t nc = L == 2 ? centre_pairs(d, cpos) : (int64_t)d * (d - 1) / 2;
+            rec_put64(r, R::NC, (unsigned long long)nc);
+            const int64_t ub = __ldg(A.unit_base + u), ue = __ldg(A.unit_base + u + 1);
+            const int64_t lo = max(q0 - ub, (int64_t)0), hi = min(q1, ue) - ub;
+            rec_put64(r, R::RLO, (unsigned long long)lo);
+            rec_put64(r, R::RHI, (unsigned long long)hi);
+            if constexpr (QUOTA) {
+                // the unit's candidates before the quota cut (as the prefix kernel counted)
+                const int64_t c = nc + (__ldg(g.ppc + v) - (int64_t)d * (d - 1) / 2);
+                unsigned long long qa = 0, qb = 0, qc = 0;
+                if (A.quota > 0 && c > A.quota) {
+                    uint64_t x, y;
+                    quota_affine(quota_unit_hash(A.qseed, id, L, v), (uint64_t)c, x, y);
+                    qa = x;
+                    qb = y;
+                    qc = (unsigned long long)c;
+                }
+                rec_put64(r, R::QA, qa);
+                rec_put64(r, R::QA + 2, qb);
+                rec_put64(r, R::QA + 4, qc);
+                nseg = (int)(hi > lo ? hi - lo : 0);   // candidates of this unit in the chunk
+                r[R::SLO] = 0;
+            } else {
+                int s0 = 0, s1 = 0;
+                if (hi > lo) {
+                    s0 = lo <= 0 ? 0 : lo < nc ? centre_row(lo, cpos, d) : d + end_row(g.pend + rp, d, lo - nc);
+                    s1 = hi >= ue - ub ? 2 * d : hi - 1 < nc ? centre_row(hi - 1, cpos, d) + 1
+                                                             : d + end_row(g.pend + rp, d, hi - 1 - nc) + 1;
+                }
+                r[R::SLO] = (uint32_t)s0;
+                nseg = s1 - s0;
+            }
+        }
+        int inc = nseg;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, inc, o);
+            if (lane >= o) inc += y;
+        }
+        if (lane < nu) r[R::SEG] = (uint32_t)(inc - nseg);
+        total_seg = __shfl_sync(0xffffffffu, inc, 31);
+        // Bloom filters of the lists of s (of the key vertex only where triangles need it)
+        int bw = FSM_JOIN_BLOOM / (nu * L);
+        lb = 5 + (31 - __clz(bw));
+        __syncwarp();
+        for (int x = lane; x < FSM_JOIN_BLOOM; x += 32) sm.bloom[w][x] = 0u;
+        __syncwarp();
+        for (int j = 0; j < nu; ++j) {
+            const uint32_t *rj = rec(j);
+            const int rv = (rj[R::META] >> 3) & 7;
+#pragma unroll
+            for (int t = 0; t < L; ++t) {
+                int32_t x0, x1;
+                if (t == rv) {
+                    if (!tfe) continue;
+                    x0 = (int32_t)rj[R::RP];
+                    x1 = x0 + (int32_t)rj[R::D];
+                } else {
+                    const int o = t - (t > rv);
+                    x0 = (int32_t)rj[R::OB + o];
+                    x1 = (int32_t)rj[R::OE + o];
+                }
+                for (int32_t x = x0 + lane; x < x1; x += 32) {
+                    const uint32_t h = ((uint32_t)__ldg(g.col + x) * 0x9E3779B1u) >> (32 - lb);
+                    atomicOr(&sm.bloom[w][((j * L + t) << (lb - 5)) + (h >> 5)], 1u << (h & 31));
+                }
+            }
+        }
+        __syncwarp();
+    }
+    int total_seg = 0;
+
+    __device__ __forceinline__ int unit_of(int g, int nu) {
+        int lo = 0;
+#pragma unroll
+        for (int s = R::U / 2; s > 0; s >>= 1)
+            if (lo + s < nu && (int)rec(lo + s)[R::SEG] <= g) lo += s;
+        return lo;
+    }
+
+    // slots of a partner the row's anchor allows: bit (slot + (partner > anchor ? SL : 0))
+    __device__ __forceinline__ uint32_t allowed(const uint32_t *r, bool centre, int s) {
+        const int kind = centre ? (tfe ? ANY_C : ANY_CT) : (tfe ? ANY_ET : ANY_E);
+        return __ldg(A.any + ((int64_t)r[R::CLS] * 4 + kind) * SL + s);
+    }
+
+    // The candidates of the loaded units, row by row.
+    __device__ __forceinline__ void walk(int nu) {
+        const DevGraph &g = A.g;
+        for (int g0 = 0; g0 < total_seg; g0 += 32) {
+            int len = 0;
+            const int gi = g0 + lane;
+            if (gi < total_seg) {
+                const int j = unit_of(gi, nu);
+                const uint32_t *r = rec(j);
+                const int row = gi - (int)r[R::SEG] + (int)r[R::SLO];
+                const int32_t rp = (int32_t)r[R::RP], d = (int32_t)r[R::D];
+                const bool centre = row < d;
+                const int32_t y = centre ? row : row - d;
+                if (A.debug && (y < 0 || y >= d)) {
+                    atomicOr(A.err, FSM_ERR_BOUNDS);
+                } else {
+                    const int32_t anchor = __ldg(g.pcol + rp + y);
+                    bool in = false;
+                    int s = 0;
+#pragma unroll
+                    for (int t = 0; t < L; ++t) {
+                        const int32_t x = (int32_t)r[R::SS + t];
+                        in |= x == anchor;
+                        s += x < anchor;
+                    }
+                    uint32_t ok = in ? 0u : allowed(r, centre, s);
+                    if (centre) ok &= (1u << SL) - 1u;
+                    if (ok) {
+                        const int64_t lo = (int64_t)rec_u64(r, R::RLO), hi = (int64_t)rec_u64(r, R::RHI);
+                        const uint32_t slots = (ok | (ok >> SL)) & ((1u << SL) - 1u);
+                        const int s0 = __ffs(slots) - 1, s1 = 31 - __clz(slots);
+                        int32_t p0, p1;      // partner positions within its list
+                        int32_t lb0;         // that list's begin
+                        if (centre) {
+                            int32_t cpos = d;
+                            if (L == 2) cpos = (int32_t)r[R::BND + (((r[R::META] >> 3) & 7) ? 0 : 1)];
+                            const int64_t st = centre_row_start(y, cpos);
+                            p0 = (int32_t)max(lo - st, (int64_t)0);
+                            p1 = (int32_t)min(hi - st, (int64_t)min(y, cpos));
+                            if (s0 > 0) p0 = max(p0, (int32_t)r[R::BND + s0 - 1]);
+                            if (s1 < L) p1 = min(p1, (int32_t)r[R::BND + s1]);
+                            lb0 = rp;
+                        } else {
+                            const int64_t st = (int64_t)rec_u64(r, R::NC) + __ldg(g.pend + rp + y);
+                            lb0 = __ldg(g.prow + anchor);
+                            const int32_t da = __ldg(g.prow + anchor + 1) - lb0;
+                            p0 = (int32_t)max(lo - st, (int64_t)0);
+                            p1 = (int32_t)min(hi - st, (int64_t)da);
+                            // cut to the allowed slots (lists of a few entries are walked whole)
+                            if (p1 - p0 > 4) {
+                                if (s0 > 0) p0 = max(p0, below(g.pcol + lb0, da, (int32_t)r[R::SS + s0 - 1]));
+                                if (s1 < L) p1 = min(p1, below(g.pcol + lb0, da, (int32_t)r[R::SS + s1]));
+                            }
+                        }
+                        len = max(p1 - p0, 0);
+                        sm.sg_base[w][lane] = (uint32_t)(lb0 + p0);
+                        sm.sg_anchor[w][lane] = (uint32_t)anchor;
+                        sm.sg_info[w][lane] = ok | ((uint32_t)j << 16) | (centre ? 0u : 1u << 20);
+                    }
+                }
+            }
+            int inc = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int y = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += y;
+            }
+            const int total = __shfl_sync(0xffffffffu, inc, 31);
+            __syncwarp();
+            sm.sg_base[w][lane] -= (uint32_t)(inc - len);   // list index of candidate t is base + t
+            __syncwarp();
+            for (int t0 = 0; t0 < total; t0 += 32) {
+                const int t = t0 + lane;
+                int k = 0;
+#pragma unroll
+                for (int s = 16; s > 0; s >>= 1)
+                    if (__shfl_sync(0xffffffffu, inc, k + s - 1) <= t) k += s;
+                bool ok = t < total;
+                int32_t x = 0, anchor = 0;
+                uint32_t info = 0;
+                if (ok) {
+                    info = sm.sg_info[w][k];
+                    anchor = (int32_t)sm.sg_anchor[w][k];
+                    const int64_t at = (int64_t)(int32_t)(sm.sg_base[w][k] + (uint32_t)t);
+                    if (A.debug && (at < 0 || at >= __ldg(g.prow + g.n))) {
+                        atomicOr(A.err, FSM_ERR_BOUNDS);
+                        ok = false;
+                    } else {
+                        x = __ldg(g.pcol + at);
+                        const uint32_t *r = rec((info >> 16) & 15);
+                        int s = x > anchor ? SL : 0;
+#pragma unroll
+                        for (int t2 = 0; t2 < L; ++t2) {
+                            const int32_t y = (int32_t)r[R::SS + t2];
+                            ok &= y != x;
+                            s += y < x;
+                        }
+                        ok &= (info >> s) & 1u;
+                    }
+                }
+                const bool centre = !((info >> 20) & 1u);
+                push(ok, centre ? x : anchor, centre ? anchor : x, info >> 16);
+            }
+            __syncwarp();
+        }
+    }
+
+    // Quota variant: the drawn candidates of the loaded units, by their numbers.
+    __device__ __forceinline__ void walk_quota(int nu) {
+        const DevGraph &g = A.g;
+        for (int g0 = 0; g0 < total_seg; g0 += 32) {
+            const int gi = g0 + lane;
+            bool ok = gi < total_seg;
+            int32_t a = 0, b = 0;
+            uint32_t m = 0;
+            if (ok) {
+                const int j = unit_of(gi, nu);
+                const uint32_t *r = rec(j);
+                int64_t lq = (int64_t)rec_u64(r, R::RLO) + (gi - (int)r[R::SEG]);
+                const unsigned long long qc = rec_u64(r, R::QA + 4);
+                if (qc) lq = (int64_t)((rec_u64(r, R::QA) * (unsigned long long)lq + rec_u64(r, R::QA + 2)) % qc);
+                const int64_t nc = (int64_t)rec_u64(r, R::NC);
+                const int32_t rp = (int32_t)r[R::RP], d = (int32_t)r[R::D];
+                const bool centre = lq < nc;
+                int32_t anchor, x;
+                if (centre) {
+                    int32_t cpos = d;
+                    if (L == 2) cpos = (int32_t)r[R::BND + (((r[R::META] >> 3) & 7) ? 0 : 1)];
+                    const int32_t y = centre_row(lq, cpos, d);
+                    const int32_t p = (int32_t)(lq - centre_row_start(y, cpos));
+                    if (A.debug && (p < 0 || p >= y || y >= d)) { atomicOr(A.err, FSM_ERR_BOUNDS); ok = false; }
+                    anchor = ok ? __ldg(g.pcol + rp + y) : 0;
+                    x = ok ? __ldg(g.pcol + rp + p) : 0;
+                } else {
+                    const int32_t y = end_row(g.pend + rp, d, lq - nc);
+                    const int64_t p = lq - nc - __ldg(g.pend + rp + y);
+                    anchor = __ldg(g.pcol + rp + y);
+                    const int32_t lb0 = __ldg(g.prow + anchor);
+                    if (A.debug && (p < 0 || p >= __ldg(g.prow + anchor + 1) - lb0)) { atomicOr(A.err, FSM_ERR_BOUNDS); ok = false; }
+                    x = ok ? __ldg(g.pcol + lb0 + p) : 0;
+                }
+                int s = 0, sx = 0;
+#pragma unroll
+                for (int t = 0; t < L; ++t) {
+                    const int32_t y = (int32_t)r[R::SS + t];
+                    ok &= y != anchor && y != x;
+                    s += y < anchor;
+                    sx += y < x;
+                }
+                if (ok) ok = (allowed(r, centre, s) >> (sx + (x > anchor ? SL : 0))) & 1u;
+                a = centre ? x : anchor;
+                b = centre ? anchor : x;
+                m = (uint32_t)j | (centre ? 0u : 16u);
+            }
+            push(ok, a, b, m);
+        }
+    }
+
+    // Write the key table out and clear it (all threads of the block, between barriers).
+    __device__ __forceinline__ void flush_table() {
+        for (int x = threadIdx.x; x < SM::NS; x += blockDim.x) {
+            const unsigned long long key = sm.key[x];
+            if (key == FSM_EMPTY_KEY) continue;
+            if constexpr (SM::COUNTS) {
+                const int64_t slot = qp_insert(A.qp, key, A.err);
+                if (slot >= 0) atomicAdd(A.qp.count + slot, (unsigned long long)sm.cnt[x]);
+                sm.cnt[x] = 0u;
+            }
+            if constexpr (SM::OFFS) sm.off[0][x] = FSM_OFF_PENDING;
+            sm.key[x] = FSM_EMPTY_KEY;
+        }
+    }
+
+    // Every warp of the block meets here between its chunks when the key table is to be flushed,
+    // and from its last chunk on; true when all warps are out of work.
+    __device__ __forceinline__ bool meet() {
+        __syncthreads();
+        const bool done = ((volatile int *)&sm.done)[0] == 8;
+        if constexpr (SM::NS > 0)
+            if (done || ((volatile int *)&sm.flag)[0]) flush_table();
+        __syncthreads();
+        if (threadIdx.x == 0) { sm.flag = 0; sm.load = 0; }
+        __syncthreads();
+        return done;
+    }
+};
+
+template <int L, int PASS, bool QUOTA>
+__global__ void __launch_bounds__(256, 3) join_kernel(const __grid_constant__ ExtArgs A) {
+    extern __shared__ __align__(16) unsigned char join_smem[];
+    using J = Joiner<L, PASS, QUOTA>;
+    typename J::SM &sm = *reinterpret_cast<typename J::SM *>(join_smem);
+    for (int x = threadIdx.x; x < J::SM::NS; x += blockDim.x) {
+        sm.key[x] = FSM_EMPTY_KEY;
+        if (J::SM::COUNTS) sm.cnt[x] = 0u;
+        if (J::SM::OFFS) sm.off[0][x] = FSM_OFF_PENDING;
+    }
+    if (threadIdx.x == 0) { sm.load = 0; sm.flag = 0; sm.done = 0; }
+    __syncthreads();
+    J jn(A, sm);
+    const int lane = jn.lane;
+    const int64_t nunits = A.ne * L;
+    int64_t total = A.total, nchunks = A.nchunks, chunk = A.chunk;
+    if (total < 0) {
+        // device-resident size: no host round trip between the prefix sum and this launch
+        total = __ldg(A.unit_base + nunits);
+        if (chunk <= 0) chunk = join_chunk(total, nunits, (int64_t)gridDim.x * (blockDim.x >> 5));
+        nchunks = (total + chunk - 1) / chunk;
+    }
+    if (A.stats && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(A.stats + 2, (unsigned long long)total);
+    bool out = false;   // this warp has no more work
+    for (;;) {
+        const bool wait = out || __shfl_sync(0xffffffffu, ((volatile int *)&sm.flag)[0], 0) != 0;
+        if (wait) {
+            if (jn.meet()) break;
+            if (out) continue;
+        }
+        unsigned long long c = 0;
+        if (lane == 0) {
+            // stop early when the call ran out of time, when an overflowing count pass is to be
+            // repeated with a larger table, or when a one-pass level is to be redone in two passes
+            const int ew = *(volatile int *)A.err;
+            bool stop = (ew & FSM_ERR_TIMEOUT) || (PASS == PASS_COUNT && (ew & FSM_ERR_QP_OVERFLOW)) ||
+                        (PASS == PASS_FUSED && ew);
+            if (!stop && A.time_limit_ns && global_ns() - __ldcg(A.time_start) > A.time_limit_ns) {
+                atomicOr(A.err, FSM_ERR_TIMEOUT);
+                stop = true;
+            }
+            c = stop ? ~0ull : atomicAdd(A.chunk_ctr, 1ull);
+        }
+        c = __shfl_sync(0xffffffffu, c, 0);
+        if (c >= (unsigned long long)nchunks) {
+            out = true;
+            if (lane == 0) atomicAdd(&sm.done, 1);
+            __syncwarp();
+            continue;
+        }
+        const int64_t q0 = (int64_t)c * chunk;
+        const int64_t q1 = min(q0 + chunk, total);
+        const int64_t ulo = warp_last_le(A.unit_base, 0, nunits - 1, q0);
+        const int64_t uhi = warp_last_le(A.unit_base, ulo, nunits - 1, q1 - 1);
+        for (int64_t u = ulo; u <= uhi; u += J::R::U) {
+            const int nu = (int)min((int64_t)J::R::U, uhi - u + 1);
+            jn.load_units(u, nu, q0, q1);
+            if constexpr (QUOTA) jn.walk_quota(nu); else jn.walk(nu);
+            if (jn.qn > 0) jn.take(jn.qn);
+        }
+    }
+
+    // per-warp totals, one atomic per warp
+    unsigned long long t0 = jn.tested, t1 = jn.accepted;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        t0 += __shfl_xor_sync(0xffffffffu, t0, o);
+        t1 += __shfl_xor_sync(0xffffffffu, t1, o);
+    }
+    if (lane == 0 && A.stats) {
+        atomicAdd(A.stats + 0, t0);
+        atomicAdd(A.stats + 1, t1);
+    }
+}
+
+template <int L, int PASS, bool QUOTA>
+cudaError_t join_launch(const ExtArgs &A, int grid, cudaStream_t st) {
+    join_kernel<L, PASS, QUOTA><<<grid, 256, sizeof(JoinSmem<L, PASS, QUOTA>), st>>>(A);
+    return cudaGetLastError();
+}
+
+// resident blocks per SM; also opts the kernel into its shared memory on the current device
+template <int L, int PASS, bool QUOTA>
+cudaError_t join_occupancy(int *bps) {
+    const int bytes = (int)sizeof(JoinSmem<L, PASS, QUOTA>);
+    cudaError_t e = cudaFuncSetAttribute(join_kernel<L, PASS, QUOTA>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e != cudaSuccess) return e;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(bps, join_kernel<L, PASS, QUOTA>, 256, bytes);
+}
+
+// One pass's instantiations: launch (bps == NULL) or query occupancy.  Defined in one translation
+// unit per pass (join_<pass>), so they compile in parallel.
+template <int PASS, bool QUOTA>
+cudaError_t join_pass(int L, const ExtArgs *A, int grid, cudaStream_t st, int *bps) {
+    switch (L) {
+    case 1: return bps ? join_occupancy<1, PASS, QUOTA>(bps) : join_launch<1, PASS, QUOTA>(*A, grid, st);
+    case 2: return bps ? join_occupancy<2, PASS, QUOTA>(bps) : join_launch<2, PASS, QUOTA>(*A, grid, st);
+    case 3: return bps ? join_occupancy<3, PASS, QUOTA>(bps) : join_launch<3, PASS, QUOTA>(*A, grid, st);
+    case 4: return bps ? join_occupancy<4, PASS, QUOTA>(bps) : join_launch<4, PASS, QUOTA>(*A, grid, st);
+    case 5: return bps ? join_occupancy<5, PASS, QUOTA>(bps) : join_launch<5, PASS, QUOTA>(*A, grid, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+cudaError_t join_count(int L, const ExtArgs *A, int grid, cudaStream_t st, int *bps);
+cudaError_t join_domain(int L, const ExtArgs *A, int grid, cudaStream_t st, int *bps);
+cudaError_t join_emit(int L, const ExtArgs *A, int grid, cudaStream_t st, int *bps);
+cudaError_t join_fused(int L, const ExtArgs *A, int grid, cudaStream_t st, int *bps);
+cudaError_t join_quota_count(int L, const ExtArgs *A, int grid, cudaStream_t st, int *bps);
+cudaError_t join_quota_domain(int L, const ExtArgs *A, int grid, cudaStream_t st, int *bps);
+cudaError_t join_quota_emit(int L, const ExtArgs *A, int grid, cudaStream_t st, int *bps);
+
+} // namespace fsm

@@ -1,0 +1,10 @@
+// fsm_join_emit.cu -- instantiations of the join kernel (stored sizes 1..5) for PASS_EMIT.
+#include "fsm_join.cuh"
+
+namespace fsm {
+
+cudaError_t join_emit(int L, const ExtArgs *A, int grid, cudaStream_t st, int *bps) {
+    return join_pass<PASS_EMIT, false>(L, A, grid, st, bps);
+}
+
+} // namespace fsm

@@ -56,7 +56,7 @@ __global__ void validate_kernel(DevGraph g, int32_t num_labels, int *err) {
 }
 
 __global__ void prepare_kernel(DevGraph g, int64_t *piece_cnt, int32_t *end_off, int32_t *rank,
-                               int32_t *cls_size) {
+                               int32_t *cls_size, int4 *vinfo) {
     for (int64_t v = gtid(); v < g.n; v += gstride()) {
         const int32_t rb = g.row_ptr[v], re = g.row_ptr[v + 1];
         const int64_t d = re - rb;
@@ -67,7 +67,10 @@ __global__ void prepare_kernel(DevGraph g, int64_t *piece_cnt, int32_t *end_off,
             run += g.row_ptr[a + 1] - g.row_ptr[a];
         }
         piece_cnt[v] = d * (d - 1) / 2 + run;
-        rank[v] = atomicAdd(cls_size + g.labels[v], 1);
+        const int32_t lab = g.labels[v];
+        const int32_t rk = atomicAdd(cls_size + lab, 1);
+        rank[v] = rk;
+        vinfo[v] = make_int4(rb, re, lab, rk);
     }
 }
 
@@ -208,9 +211,9 @@ cudaError_t launch_validate(const DevGraph &g, int32_t num_labels, int *err, cud
 }
 
 cudaError_t launch_prepare(const DevGraph &g, int64_t *piece_cnt, int32_t *end_off, int32_t *rank,
-                           int32_t *cls_size, cudaStream_t st) {
+                           int32_t *cls_size, int4 *vinfo, cudaStream_t st) {
     LAUNCHED(1);
-    prepare_kernel<<<blocks_for(g.n), kThreads, 0, st>>>(g, piece_cnt, end_off, rank, cls_size);
+    prepare_kernel<<<blocks_for(g.n), kThreads, 0, st>>>(g, piece_cnt, end_off, rank, cls_size, vinfo);
     return cudaGetLastError();
 }
 
@@ -438,13 +441,13 @@ __global__ void pattern_counts_kernel(const int64_t *slots, int64_t nq, const in
 
 __global__ void domain_sizes_kernel(int K, const unsigned long long *pat_lab, const uint64_t *orbit,
                                     const int32_t *min_orbit, const unsigned long long *pat_count, int64_t np,
-                                    int64_t t, const int32_t *cls_size, uint8_t *live, int64_t *words) {
+                                    int64_t t, const int32_t *cls_size, int shift, uint8_t *live, int64_t *words) {
     for (int64_t P = gtid(); P < np; P += gstride()) {
         const bool lv = (unsigned long long)min_orbit[P] * pat_count[P] >= (unsigned long long)t;
         live[P] = lv ? 1 : 0;
         for (int c = 0; c < FSM_MAXK; ++c) {
             int64_t w = 0;
-            if (lv && c < K && nib_get(orbit[P], c) == c) w = ((int64_t)cls_size[clab_get(pat_lab[P], c)] + 31) / 32;
+            if (lv && c < K && nib_get(orbit[P], c) == c) w = bitmap_words(cls_size[clab_get(pat_lab[P], c)], shift);
             words[P * FSM_MAXK + c] = w;
         }
     }
@@ -577,12 +580,12 @@ cudaError_t launch_pattern_counts(const int64_t *slots, int64_t nq, const int32_
 
 cudaError_t launch_domain_sizes(int K, const unsigned long long *pat_lab, const uint64_t *orbit,
                                 const int32_t *min_orbit, const unsigned long long *pat_count,
-                                int64_t np, int64_t t, const int32_t *cls_size, uint8_t *live,
+                                int64_t np, int64_t t, const int32_t *cls_size, int shift, uint8_t *live,
                                 int64_t *words, cudaStream_t st) {
     if (np <= 0) return cudaSuccess;
     LAUNCHED(1);
     domain_sizes_kernel<<<blocks_for(np), kThreads, 0, st>>>(K, pat_lab, orbit, min_orbit, pat_count, np, t,
-                                                           cls_size, live, words);
+                                                           cls_size, shift, live, words);
     return cudaGetLastError();
 }
 
@@ -1236,7 +1239,7 @@ namespace {
 // position) hold ceil(|V_label| / 32) words each, in that order.  One warp per pattern.
 __global__ void fused_support_kernel(int K, const unsigned long long *plab, const uint64_t *padj, const uint64_t *orbit,
                                      int64_t np, const unsigned long long *ckeys, const unsigned long long *coff,
-                                     uint64_t cmask, const int32_t *cls_size, const uint32_t *pool,
+                                     uint64_t cmask, const int32_t *cls_size, int shift, const uint32_t *pool,
                                      unsigned long long *sigma) {
     const int lane = threadIdx.x & 31;
     for (int64_t P = gtid() >> 5; P < np; P += gstride() >> 5) {
@@ -1264,7 +1267,7 @@ __global__ void fused_support_kernel(int K, const unsigned long long *plab, cons
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
             if (cnt < mn) mn = cnt;
-            pre += nw;
+            pre += (uint64_t)bitmap_words(cls_size[clab_get(plab[P], c)], shift);
         }
         if (lane == 0) sigma[P] = mn;
     }
@@ -1274,26 +1277,27 @@ __global__ void fused_support_kernel(int K, const unsigned long long *plab, cons
 
 cudaError_t launch_fused_support(int K, const unsigned long long *plab, const uint64_t *padj, const uint64_t *orbit,
                                  int64_t np, const unsigned long long *ckeys, const unsigned long long *coff,
-                                 uint64_t cmask, const int32_t *cls_size, const uint32_t *pool, unsigned long long *sigma,
-                                 cudaStream_t st) {
+                                 uint64_t cmask, const int32_t *cls_size, int shift, const uint32_t *pool,
+                                 unsigned long long *sigma, cudaStream_t st) {
     if (np <= 0) return cudaSuccess;
     LAUNCHED(1);
     fused_support_kernel<<<blocks_for(np * 32), kThreads, 0, st>>>(K, plab, padj, orbit, np, ckeys, coff, cmask, cls_size,
-                                                                   pool, sigma);
+                                                                   shift, pool, sigma);
     return cudaGetLastError();
 }
 
 namespace {
 __global__ void slot_bases_kernel(int K, const int64_t *slots, int64_t nq, const int32_t *qp_pattern,
                                   const uint64_t *qp_perm, const uint8_t *live, const uint64_t *orbit,
-                                  const int64_t *dom_off, int64_t *slot_base) {
+                                  const int64_t *dom_off, int shift, int64_t *slot_base, uint32_t *slot_off) {
     for (int64_t q = gtid(); q < nq; q += gstride()) {
         const int64_t slot = slots[q];
         const int32_t P = qp_pattern[slot];
         for (int h = 0; h < FSM_MAXK; ++h) {
             int64_t b = -1;
             if (h < K && live[P]) b = dom_off[(int64_t)P * FSM_MAXK + nib_get(orbit[P], nib_get(qp_perm[slot], h))];
-            slot_base[slot * FSM_MAXK + h] = b;
+            if (slot_base) slot_base[slot * FSM_MAXK + h] = b;
+            else if (h < 8) slot_off[slot * 8 + h] = b < 0 ? 0xFFFFFFFFu : (uint32_t)(b >> shift);
         }
     }
 }
@@ -1301,11 +1305,33 @@ __global__ void slot_bases_kernel(int K, const int64_t *slots, int64_t nq, const
 
 cudaError_t launch_slot_bases(int K, const int64_t *slots, int64_t nq, const int32_t *qp_pattern,
                               const uint64_t *qp_perm, const uint8_t *live, const uint64_t *orbit,
-                              const int64_t *dom_off, int64_t *slot_base, cudaStream_t st) {
+                              const int64_t *dom_off, int shift, int64_t *slot_base, uint32_t *slot_off,
+                              cudaStream_t st) {
     if (nq <= 0) return cudaSuccess;
     LAUNCHED(1);
     slot_bases_kernel<<<blocks_for(nq), kThreads, 0, st>>>(K, slots, nq, qp_pattern, qp_perm, live, orbit, dom_off,
-                                                           slot_base);
+                                                           shift, slot_base, slot_off);
+    return cudaGetLastError();
+}
+
+namespace {
+// Size-3 frequencies as label masks (ExtArgs::lf): one word per thread.
+__global__ void label_masks_kernel(const uint8_t *pf, unsigned long long *lf) {
+    for (int64_t x = gtid(); x < 3 * 4096; x += gstride()) {
+        const int tab = (int)(x >> 12), p = (int)(x >> 6) & 63, q = (int)x & 63;
+        unsigned long long m = 0;
+        for (int z = 0; z < 64; ++z) {
+            const uint32_t idx = tab == 0 ? wedge_index(p, q, z) : tab == 1 ? wedge_index(z, p, q) : tri_index(p, q, z);
+            if (pf[idx]) m |= 1ull << z;
+        }
+        lf[x] = m;
+    }
+}
+} // namespace
+
+cudaError_t launch_label_masks(const uint8_t *piece_freq, unsigned long long *lf, cudaStream_t st) {
+    LAUNCHED(1);
+    label_masks_kernel<<<blocks_for(3 * 4096, 64), 64, 0, st>>>(piece_freq, lf);
     return cudaGetLastError();
 }
 

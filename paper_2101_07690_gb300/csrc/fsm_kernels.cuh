@@ -18,7 +18,7 @@ struct CodeRec {
 // ---- graph preparation
 cudaError_t launch_validate(const DevGraph &g, int32_t num_labels, int *err, cudaStream_t st);
 cudaError_t launch_prepare(const DevGraph &g, int64_t *piece_cnt, int32_t *end_off, int32_t *rank,
-                           int32_t *cls_size, cudaStream_t st);
+                           int32_t *cls_size, int4 *vinfo, cudaStream_t st);
 
 // ---- neighbour-adjacency matrices of vertices of degree >= dmin (DevGraph::tri_off):
 //      words[v] = d * ceil(d / 32) or 0; then, with off = exclusive prefix of words, the bits
@@ -78,7 +78,7 @@ cudaError_t launch_pattern_counts(const int64_t *slots, int64_t nq, const int32_
 // live patterns (count * smallest orbit >= t) and the words of each orbit bitmap
 cudaError_t launch_domain_sizes(int K, const unsigned long long *pat_lab, const uint64_t *orbit,
                                 const int32_t *min_orbit, const unsigned long long *pat_count,
-                                int64_t np, int64_t t, const int32_t *cls_size, uint8_t *live,
+                                int64_t np, int64_t t, const int32_t *cls_size, int shift, uint8_t *live,
                                 int64_t *words, cudaStream_t st);
 // offsets from the scanned sizes (-1 where no bitmap)
 cudaError_t launch_domain_offsets(const int64_t *words, const int64_t *scanned, int64_t n8, int64_t *off,
@@ -191,18 +191,21 @@ cudaError_t launch_stamp_time(unsigned long long *out, cudaStream_t st);
 // P's bitmap block, found through its entry in the code table (ckeys / coff, cmask + 1 slots)
 cudaError_t launch_fused_support(int K, const unsigned long long *plab, const uint64_t *padj, const uint64_t *orbit,
                                  int64_t np, const unsigned long long *ckeys, const unsigned long long *coff,
-                                 uint64_t cmask, const int32_t *cls_size, const uint32_t *pool, unsigned long long *sigma,
-                                 cudaStream_t st);
+                                 uint64_t cmask, const int32_t *cls_size, int shift, const uint32_t *pool,
+                                 unsigned long long *sigma, cudaStream_t st);
 
 // Domain pass helper: for every distinct key (slot) and local position h, the word offset of
 // the bitmap its vertex goes to (the orbit of canonical position perm[h] of its pattern), or -1
 // when the pattern has no domains.
 cudaError_t launch_slot_bases(int K, const int64_t *slots, int64_t nq, const int32_t *qp_pattern,
                               const uint64_t *qp_perm, const uint8_t *live, const uint64_t *orbit,
-                              const int64_t *dom_off, int64_t *slot_base, cudaStream_t st);
+                              const int64_t *dom_off, int shift, int64_t *slot_base, uint32_t *slot_off,
+                              cudaStream_t st);
 
 // ---- pieces: mark the frequent size-3 patterns by piece index
 cudaError_t launch_piece_table(const unsigned long long *lab, const uint64_t *adj, int64_t n,
                                uint8_t *piece_freq, cudaStream_t st);
+// ---- the same as label masks (ExtArgs::lf, 3 * 4096 words)
+cudaError_t launch_label_masks(const uint8_t *piece_freq, unsigned long long *lf, cudaStream_t st);
 
 } // namespace fsm
