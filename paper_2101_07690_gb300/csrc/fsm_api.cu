@@ -250,7 +250,7 @@ struct Miner {
     int V = FSM_EXPLORE_TV;   // exploration variant of this call (FSM_EXPLORE_*)
 
     // Stored sizes up to 5 of two-vertex exploration with index-based keys are joined by
-    // fsm_join.cuh (its header has the times of both kernels: 1.8 to 14 times less); the ablations'
+    // fsm_join.cuh (its header has the times of both kernels: 2.3 to 22 times less); the ablations'
     // key forms and sizes 6 and 7, whose acceptance tables would not fit, by fsm_extend.cuh.
     bool joins(int L) const { return L <= FSM_JOIN_MAXL && (V == FSM_EXPLORE_TV || V == FSM_EXPLORE_TV_QUOTA); }
 
@@ -530,6 +530,10 @@ struct Miner {
         if (joins(L)) {
             join_tables(L);
             A.acc = G->join_acc[L];
+            // label classes of fewer than 512 vertices on average (bitmaps of at most 16 words): size
+            // 6 on 1656 vertices, domain pass 14.7 ms with the read, 21.2 ms without; 100k vertices
+            // (108 words), one pass: 154 ms with, 146 ms without; 3.7M vertices, size 3: 9.4 and 7.8 ms
+            A.check_bits = (int64_t)G->n < (int64_t)512 * G->NL;
             A.any = G->join_any[L];
             if (piece_freq) {
                 lf = mem.get<unsigned long long>(3 * 4096);
@@ -575,8 +579,9 @@ struct Miner {
             while (cap < 4 * G->qp_hint[L] && cap < ((int64_t)1 << 30)) cap <<= 1;
         unsigned long long *keys = nullptr, *qcount = nullptr, *used = nullptr, *ptop = nullptr, *ckeys = nullptr,
                            *coff = nullptr;
-        uint32_t *soff = nullptr;
+        uint32_t *krec = nullptr;
         uint32_t *pool = nullptr;
+        const int rec_words = key_rec_words(K);
         int shift = 0;   // bitmap offsets are 32-bit, in units of 1 << shift words
         unsigned long long pool_words = 0;
         bool fused = final && G->fused && V == FSM_EXPLORE_TV && !sampled && K <= 7;
@@ -600,10 +605,10 @@ struct Miner {
             }
         }
         auto release_pass1 = [&]() {
-            for (void *q : {(void *)keys, (void *)qcount, (void *)used, (void *)ckeys, (void *)coff, (void *)soff})
+            for (void *q : {(void *)keys, (void *)qcount, (void *)used, (void *)ckeys, (void *)coff, (void *)krec})
                 if (q) mem.release(q);
             keys = qcount = used = ckeys = coff = nullptr;
-            soff = nullptr;
+            krec = nullptr;
         };
         auto clear_pass1 = [&]() {
             ck(launch_fill_u64(keys, FSM_EMPTY_KEY, cap, st), "fill");
@@ -614,7 +619,7 @@ struct Miner {
             if (fused) {
                 ck(launch_fill_u64(ckeys, FSM_EMPTY_KEY, cap, st), "fill");
                 ck(cudaMemsetAsync(coff, 0, sizeof(unsigned long long) * cap, st), "memset");
-                ck(cudaMemsetAsync(soff, 0xff, sizeof(uint32_t) * cap * 8, st), "memset");
+                ck(cudaMemsetAsync(krec, 0xff, sizeof(uint32_t) * cap * rec_words, st), "memset");
                 ck(cudaMemsetAsync(pool, 0, pool_words * 4, st), "memset");
                 ck(cudaMemsetAsync(ptop, 0, sizeof(unsigned long long), st), "memset");
             }
@@ -628,12 +633,12 @@ struct Miner {
                 // at most half full whenever that one is
                 ckeys = mem.get<unsigned long long>(cap);
                 coff = mem.get<unsigned long long>(cap);
-                soff = mem.get<uint32_t>(cap * 8);
+                krec = mem.get<uint32_t>(cap * rec_words);
                 A.pat_lab = in.lab8;
                 A.code_keys = ckeys;
                 A.code_off = coff;
                 A.code_mask = (uint64_t)cap - 1;
-                A.slot_off32 = soff;
+                A.key_rec = krec;
                 A.off_shift = shift;
                 A.pool = pool;
                 A.pool_top = ptop;
@@ -653,6 +658,20 @@ struct Miner {
                 // chunk size from trial count passes on a sample; their counts are then wiped
                 tune_chunk(in, A, PASS_COUNT);
                 clear_pass1();
+            }
+            if (fused) {
+                // Keys met for the first time are canonicalised by the lane that meets them, while
+                // the warps that meet them meanwhile do the same again.  Most are found by a sample
+                // of the pieces first and resolved with full warps (74k vertices, k = 5, 324k keys:
+                // 6.1M resolutions in the level and 59 ms without, 79k and 30.5 + 1.1 ms with it;
+                // 370 vertices, 451k keys: 5.2 ms without, 0.57 + 0.44 ms with it).
+                ExtArgs W = A;
+                W.warm = 1;
+                W.stats = nullptr;
+                run_pass(PASS_COUNT, in, W, pat_off);
+                ck(launch_resolve_keys(W, G->sms, st), "resolve keys");
+                rs.launches += 1;
+                ck(cudaMemsetAsync(qcount, 0, sizeof(unsigned long long) * cap, st), "memset");
             }
             run_pass(fused ? PASS_FUSED : PASS_COUNT, in, A, pat_off);
             const int ew = err_word();
@@ -761,10 +780,16 @@ struct Miner {
             A.orbit = orbit;
             A.dom_off = doff;
             A.dom = dom;
-            if (joins(L)) soff = mem.get<uint32_t>(cap * 8); else sbase = mem.get<int64_t>(cap * FSM_MAXK);
-            ck(launch_slot_bases(K, slots, nq, qpat, qperm, live, orbit, doff, shift, sbase, soff, st), "slot bases");
+            if (joins(L)) {
+                krec = mem.get<uint32_t>(cap * rec_words);
+                ck(cudaMemsetAsync(krec, 0xff, sizeof(uint32_t) * cap * rec_words, st), "memset");
+            } else {
+                sbase = mem.get<int64_t>(cap * FSM_MAXK);
+            }
+            ck(launch_slot_bases(K, slots, nq, qpat, qperm, live, orbit, doff, shift, sbase, keys, krec, rec_words, st),
+               "slot bases");
             A.slot_base = sbase;
-            A.slot_off32 = soff;
+            A.key_rec = krec;
             A.off_shift = shift;
             A.stats = nullptr;
             if (rs.live > 0) {

@@ -43,6 +43,13 @@ struct QPTab {
     unsigned long long max_used;   // overflow threshold (load factor 1/2)
 };
 
+// Key records (one-pass level and domain pass): per key slot, words 0-1 the key and words 2.. the
+// bitmap offset of each local position in units of 1 << off_shift words.  Every word starts as
+// all ones and is written once with its final value, so a reader that sees the key and no all-ones
+// offset has the whole record, whatever the order it saw the words in.
+FSM_HD constexpr int key_rec_words(int K) { return K <= 6 ? 8 : 16; }
+#define FSM_OFF_NONE 0xFFFFFFFFu     // word of a key record not yet published, or no bitmaps
+
 struct ExtArgs {
     DevGraph g;
     int mode;                      // 0 edge-induced, 1 vertex-induced
@@ -81,11 +88,10 @@ struct ExtArgs {
     unsigned long long *code_keys; // [code_mask + 1], FSM_EMPTY_KEY when free
     unsigned long long *code_off;  // [code_mask + 1]
     uint64_t code_mask;
-    // one bitmap offset per (key slot, local position), [cap * 8], in units of 1 << off_shift words:
-    // written by the one-pass level (FSM_OFF_NONE until published), read by the domain pass of
-    // fsm_join.cuh (FSM_OFF_NONE: pattern without bitmaps)
-    uint32_t *slot_off32;
+    uint32_t *key_rec;             // [cap] key records (fsm_join.cuh)
     int off_shift;
+    int check_bits;                // read a bitmap word before reducing into it
+    int warm;                      // count a sample of the chunks only (before a one-pass level)
     // tables of fsm_join.cuh for this level size, and the size-3 frequencies as label masks: W[c][x]
     // bit y (wedge of centre c, ends x, y), C[x][y] bit c (the same wedge by its centre) and
     // T[x][y] bit z (triangle), 64 x 64 words each; NULL at level 1
@@ -119,6 +125,16 @@ FSM_HD int64_t join_chunk(int64_t total, int64_t units, int64_t warps) {
     int64_t chunk = 256;
     while (chunk < 16384 && total / chunk > warps * 64 && chunk * 2 <= 16 * per_unit) chunk <<= 1;
     return chunk;
+}
+
+// Warm pass of a one-pass level: the keys of every warm_stride-th chunk of FSM_WARM_CHUNK pieces are
+// counted and resolved in bulk first, so that the level itself meets few keys for the first time.
+// All pieces up to 2^24 (small levels have most keys per piece), then 2^24 of them, from 2^31 on
+// one in 128 (a level of 7.5e9 pieces: 1 in 32 took 3.5 ms of 143, for the same few misses).
+#define FSM_WARM_CHUNK 1024
+FSM_HD int64_t warm_stride(int64_t total) {
+    const int64_t s = total >> 24;
+    return s < 1 ? 1 : s > 128 ? 128 : s;
 }
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -965,6 +981,7 @@ cudaError_t occupancy_extend_l7(int pass, int *blocks_per_sm);
 // one-pass level with FSM_EXPLORE_TV only)
 #define FSM_JOIN_MAXL 5
 cudaError_t launch_join(int pass, int L, int V, const ExtArgs &A, int grid, cudaStream_t st);
+cudaError_t launch_resolve_keys(const ExtArgs &A, int sms, cudaStream_t st);
 cudaError_t occupancy_join(int pass, int L, int V, int *blocks_per_sm);
 // its tables for stored size L: bytes of each, and the kernels that fill them (tmp: join_tmp_bytes)
 void join_table_bytes(int L, size_t *acc, size_t *any, size_t *tmp);

@@ -17,7 +17,8 @@
 //   segments   A unit's pieces are rows of sorted lists: centre row y (anchor b = y-th neighbour of
 //              v, partners a = the neighbours before it) and end list a (anchor a, partners b in
 //              N(a)).  One lane prepares one row: the slots its anchor allows its partner cut the
-//              row to a range (a row with none costs nothing more).
+//              row to a range (a row with none costs nothing more), and the anchor's label, cross
+//              edges and pruning bits are found once for the whole row.
 //   filter     Lanes then walk the surviving ranges side by side: one coalesced list read, the
 //              partner's slot by l comparisons, one bit test.  Survivors go to a per-warp queue.
 //   joins      Full warps take 32 survivors: labels and ranks (one 16-byte read per vertex), the
@@ -25,15 +26,18 @@
 //              list of s, misses are certain, hits are verified by binary search), joining-point
 //              pruning (Section 4.5) as cross bits that must or must not be set, then the subsets
 //              that are left and accepted by `acc`.
-//   accept     Keys go through one open-addressed table per block in shared memory that also holds
-//              each key's bitmap offsets; it is flushed between chunks when it fills.
+//   accept     One 32-byte record per key slot holds the key and its patterns' bitmap offsets, so
+//              a join finds both in one read; counts are single reductions that nothing waits for.
 //
-// One launch on a GB300, the extension kernel before and this one (same graph and output):
-//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms ->  77.7 ms
-//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms -> 283 ms
-//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms ->  18.5 ms
-//   5 -> 7, count, ST 8 quotas, 6.0e8 pieces, 1.2e8 joins:          248 ms ->  60.6 ms
-//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms ->  8.1 ms
+// One launch on a GB300 (same graph and output): the extension kernel before, this kernel with a
+// key table per block in shared memory (flushed between chunks) and both new vertices' tests made
+// per survivor, and as it is:
+//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms,  77.7 ms,  30.5 ms
+//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   140 ms
+//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,  11.8 ms
+//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   6.3 ms
+// The block tables missed 70 to 77 % of the lookups of levels 1 and 2, and their flushes made warps
+// wait for each other; a record read at the L2 costs each join one latency and no barrier.
 #pragma once
 #include "fsm_extend.cuh"
 
@@ -104,11 +108,17 @@ FSM_HD bool join_accepted(int cls, int form, int sa, int sb, int bgt, uint32_t s
 #define FSM_JOIN_QUEUE 64
 // shared words per warp for the Bloom filters of a batch of units
 #define FSM_JOIN_BLOOM 512
-// slots of a block's key table
-#define FSM_JOIN_SLOTS 512
-#define FSM_JOIN_PROBES 8
-#define FSM_OFF_NONE 0xFFFFFFFFu     // key whose pattern has no bitmaps
-#define FSM_OFF_PENDING 0xFFFFFFFEu  // offsets not yet known (never a valid offset)
+
+// A queued candidate, and a row's part of it, in one word: unit j (4 bits), end list (1), slot of the
+// anchor (3) and of the partner (3), and of the anchor its label (6), cross edges to the other
+// vertices of s (4), and the cross edges pruning asks of it (4) or forbids (4).
+#define FSM_M_END 4
+#define FSM_M_SA 5
+#define FSM_M_SP 8
+#define FSM_M_LAB 11
+#define FSM_M_CROSS 17
+#define FSM_M_MUST 21
+#define FSM_M_NO 25
 
 // A batch's units in shared memory: UW words each.
 template <int L, bool QUOTA> struct UnitRec {
@@ -116,25 +126,16 @@ template <int L, bool QUOTA> struct UnitRec {
     static constexpr int U = L <= 3 ? 16 : 8;        // units per batch
     static constexpr int RP = 0, D = 1, PID = 2, META = 3, CLS = 4, OLAB = 5, OPP = 6, SEG = 7, SLO = 8, RLO = 9,
                          RHI = 11, NC = 13, SS = 15, BND = SS + L, RK = BND + L, OB = RK + L, OE = OB + O, OK = OE + O,
-                         QA = OK + 6 * O, END = QA + (QUOTA ? 6 : 0);
+                         VB = OK + 6 * O, VE = VB + 1, QA = VE + 1, END = QA + (QUOTA ? 6 : 0);
     static constexpr int UW = END | 1;               // odd stride: lanes on different units hit different banks
 };
 
 template <int L, int PASS, bool QUOTA> struct JoinSmem {
     using R = UnitRec<L, QUOTA>;
-    static constexpr int K = L + 2;
-    static constexpr bool COUNTS = PASS == PASS_COUNT || PASS == PASS_FUSED;
-    static constexpr bool OFFS = PASS == PASS_DOMAIN || PASS == PASS_FUSED;
-    static constexpr int NS = PASS == PASS_EMIT ? 0 : FSM_JOIN_SLOTS;
-    unsigned long long key[NS ? NS : 1];
-    uint32_t cnt[COUNTS ? NS : 1];
-    uint32_t off[OFFS ? K : 1][OFFS ? NS : 1];
-    int load, flag, done;
     uint32_t unit[8][R::U * R::UW];
     uint32_t bloom[8][FSM_JOIN_BLOOM];
-    uint32_t qa[8][FSM_JOIN_QUEUE], qb[8][FSM_JOIN_QUEUE];
-    uint8_t qm[8][FSM_JOIN_QUEUE];
-    uint32_t sg_base[8][32], sg_anchor[8][32], sg_info[8][32];
+    uint32_t q_anchor[8][FSM_JOIN_QUEUE], q_partner[8][FSM_JOIN_QUEUE], q_meta[8][FSM_JOIN_QUEUE];
+    uint32_t sg_base[8][32], sg_anchor[8][32], sg_slots[8][32], sg_meta[8][32];
 };
 
 __device__ __forceinline__ int32_t sorted_has(const int32_t *col, int32_t lo, int32_t end, int32_t x) {
@@ -204,19 +205,10 @@ __device__ __forceinline__ int32_t end_row(const int32_t *pend, int32_t d, int64
     return lo;
 }
 
-// ---- one-pass last level: publication of a key slot's bitmap offsets (gpu-scope release/acquire)
-__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t *p) {
-    uint32_t v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
 __device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t *p) {
     uint32_t v;
     asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
-}
-__device__ __forceinline__ void st_release_u32(uint32_t *p, uint32_t v) {
-    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ void st_relaxed_u32(uint32_t *p, uint32_t v) {
     asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
@@ -225,17 +217,16 @@ __device__ __forceinline__ void st_relaxed_u32(uint32_t *p, uint32_t v) {
 // First sight of a quick pattern in the one-pass last level: canonicalise the graph its key
 // denotes, find or claim its pattern's entry in the code table, claim the pattern's orbit
 // bitmaps from the pool unless another lane already did (one CAS decides; a loser's pool words
-// stay unused), and publish the bitmap offset of each local position -- position 0 last, with
-// release semantics, so a reader that sees it set sees the others.  Lanes racing on one key
-// compute and write the same values.  On a full table or pool the error word says so and nothing
-// is published; the host then runs the last level as two passes.
+// stay unused), and publish the key's record.  Lanes racing on one key compute and write the same
+// values.  On a full table or pool the error word says so and nothing is published; the host then
+// runs the last level as two passes.
 struct ResolveArgs {
     const uint64_t *pat_lab, *pat_adj;
     const int32_t *cls_size;
     unsigned long long *code_keys, *code_off, *pool_top;
     uint64_t code_mask;
     unsigned long long pool_words;
-    uint32_t *slot_off;
+    uint32_t *key_rec;
     int shift;
     int *err;
     int explore, level;
@@ -273,36 +264,47 @@ static __device__ __noinline__ void resolve_slot(const ResolveArgs A, int64_t sl
         const unsigned long long old = atomicCAS(A.code_off + ci, 0ull, res + 1ull);
         off = old ? old : res + 1ull;
     }
-    uint32_t *so = A.slot_off + slot * 8;
-    for (int hh = K - 1; hh >= 0; --hh) {
-        const uint32_t v = (uint32_t)(((long long)(off - 1ull) + pre[rep[(inv >> (3 * hh)) & 7]]) >> A.shift);
-        if (hh) st_relaxed_u32(so + hh, v); else st_release_u32(so, v);
+    uint32_t *kr = A.key_rec + slot * key_rec_words(K);
+    for (int hh = 0; hh < K; ++hh)
+        st_relaxed_u32(kr + 2 + hh, (uint32_t)(((long long)(off - 1ull) + pre[rep[(inv >> (3 * hh)) & 7]]) >> A.shift));
+    st_relaxed_u32(kr, (uint32_t)key);
+    st_relaxed_u32(kr + 1, (uint32_t)(key >> 32));
+}
+
+// Four words of a key record: read-only in the domain pass, read at the L2 in the one-pass level
+// (an old empty copy in L1 would send its readers to the slow path until it is evicted).
+template <int PASS> __device__ __forceinline__ void ld_rec4(const uint32_t *p, uint32_t *x) {
+    if (PASS == PASS_DOMAIN) {
+        const uint4 v = __ldg((const uint4 *)p);
+        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
+    } else {
+        asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
+                     : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "l"(p) : "memory");
     }
 }
 
-// Offsets (in units of 1 << off_shift words) of a key's bitmaps from the global tables: the domain
-// pass's table, or in the one-pass level the published slot, resolved on first sight.
-template <int K, int PASS>
-__device__ __forceinline__ bool key_offsets(const ExtArgs &A, uint64_t key, int64_t slot, uint32_t (&off)[K]) {
-    if (PASS == PASS_DOMAIN) {
-        const uint32_t *sb = A.slot_off32 + slot * 8;
-#pragma unroll
-        for (int h = 0; h < K; ++h) off[h] = __ldg(sb + h);
-        return true;
+// First sight of a key (or a record this SM's L1 still holds empty): insert the key, publish its
+// record if nobody has, and read it at the L2.  False when a table or the pool is full (the error
+// word says so).
+template <int K>
+__device__ __noinline__ bool first_sight(const ExtArgs &A, uint64_t key, int64_t &slot, uint32_t *off) {
+    slot = qp_insert(A.qp, key, A.err);
+    if (slot < 0) return false;
+    const uint32_t *kr = A.key_rec + slot * key_rec_words(K);
+    for (int round = 0; round < 2; ++round) {
+        bool all = true;
+        for (int h = 0; h < K; ++h) {
+            off[h] = ld_relaxed_u32(kr + 2 + h);
+            all &= off[h] != FSM_OFF_NONE;
+        }
+        if (all) return true;
+        if (round == 0) {
+            const ResolveArgs R{A.pat_lab, A.pat_adj, A.cls_size, A.code_keys, A.code_off, A.pool_top,
+                                A.code_mask, A.pool_words, A.key_rec, A.off_shift, A.err, A.explore, A.level};
+            resolve_slot(R, slot, key);
+        }
     }
-    const uint32_t *so = A.slot_off32 + slot * 8;
-    uint32_t o0 = ld_acquire_u32(so);
-    if (o0 == FSM_OFF_NONE) {   // not yet published
-        const ResolveArgs R{A.pat_lab, A.pat_adj, A.cls_size, A.code_keys, A.code_off, A.pool_top,
-                            A.code_mask, A.pool_words, A.slot_off32, A.off_shift, A.err, A.explore, A.level};
-        resolve_slot(R, slot, key);
-        o0 = ld_acquire_u32(so);
-        if (o0 == FSM_OFF_NONE) return false;   // a table or the pool is full: the error word says so
-    }
-    off[0] = o0;
-#pragma unroll
-    for (int h = 1; h < K; ++h) off[h] = ld_relaxed_u32(so + h);
-    return true;
+    return false;
 }
 
 template <int L, int PASS, bool QUOTA>
@@ -336,25 +338,33 @@ struct Joiner {
         return (sm.bloom[w][((j * L + t) << (lb - 5)) + (h >> 5)] >> (h & 31)) & 1u;
     }
 
-    // ---- the block's key table
-    __device__ __forceinline__ int table_find(uint64_t key) {
-        uint32_t h = ((uint32_t)key * 0x9E3779B1u) ^ ((uint32_t)(key >> 32) * 0x85EBCA77u);
-        h = (h ^ (h >> 15)) & (FSM_JOIN_SLOTS - 1);
+    // Slot and bitmap offsets of a key from its record; false where the key has none (domain pass:
+    // an error), the record is not there yet, or a table is full.
+    __device__ __forceinline__ bool key_record(uint64_t key, int64_t &slot, uint32_t (&off)[K]) {
+        uint64_t h = mix64(key) & A.qp.mask;
+        constexpr int RW = key_rec_words(K);
 #pragma unroll 1
-        for (int p = 0; p < FSM_JOIN_PROBES; ++p) {
-            unsigned long long cur = ((volatile unsigned long long *)sm.key)[h];
-            if (cur == FSM_EMPTY_KEY) {
-                cur = atomicCAS(&sm.key[h], FSM_EMPTY_KEY, (unsigned long long)key);
-                if (cur == FSM_EMPTY_KEY) {
-                    if (atomicAdd(&sm.load, 1) >= FSM_JOIN_SLOTS * 3 / 4) sm.flag = 1;
-                    return (int)h;
+        for (int p = 0; p < FSM_MAX_PROBES; ++p) {
+            const uint32_t *kr = A.key_rec + h * RW;
+            uint32_t wd[12];
+            ld_rec4<PASS>(kr, wd);
+            ld_rec4<PASS>(kr + 4, wd + 4);
+            if (K > 6) ld_rec4<PASS>(kr + 8, wd + 8);
+            const uint64_t k = (uint64_t)wd[0] | ((uint64_t)wd[1] << 32);
+            if (k == key) {
+                bool all = true;
+#pragma unroll
+                for (int x = 0; x < K; ++x) {
+                    off[x] = wd[2 + x];
+                    all &= off[x] != FSM_OFF_NONE;
                 }
+                slot = (int64_t)h;
+                return all;
             }
-            if (cur == key) return (int)h;
-            h = (h + 1) & (FSM_JOIN_SLOTS - 1);
+            if (k == FSM_EMPTY_KEY) return false;
+            h = (h + 1) & A.qp.mask;
         }
-        sm.flag = 1;
-        return -1;
+        return false;
     }
 
     __device__ __forceinline__ void set_bits(const uint32_t (&off)[K], const uint32_t *r, uint32_t ra, uint32_t rb, bool swap) {
@@ -367,54 +377,36 @@ struct Joiner {
             wd[h] = base + ((uint64_t)off[h] << A.off_shift) + (rk >> 5);
             bit[h] = 1u << (rk & 31);
         }
-        // read first: most bits are set already, and the reads of one join overlap
+        // A reduction nothing waits for, except on small label classes (ExtArgs::check_bits), whose few
+        // words many joins would queue on: there most bits are set already and a read finds that.
+        if (A.check_bits) {
 #pragma unroll
-        for (int h = 0; h < K; ++h) old[h] = __ldcg(wd[h]);
+            for (int h = 0; h < K; ++h) old[h] = __ldcg(wd[h]);
 #pragma unroll
-        for (int h = 0; h < K; ++h)
-            if (!(old[h] & bit[h])) atomicOr(wd[h], bit[h]);
+            for (int h = 0; h < K; ++h)
+                if (!(old[h] & bit[h])) atomicOr(wd[h], bit[h]);
+        } else {
+#pragma unroll
+            for (int h = 0; h < K; ++h) atomicOr(wd[h], bit[h]);
+        }
     }
 
     // One accepted join of this lane (not warp-synchronous).
-    __device__ __forceinline__ void accept(const uint32_t *r, uint64_t key, int32_t a, int32_t b, uint32_t ra, uint32_t rb,
-                                           bool swap) {
+    __device__ __forceinline__ void accept(const uint32_t *r, uint64_t key, bool centre, int32_t anchor, int32_t x,
+                                           uint32_t rx, bool swap) {
         if constexpr (PASS == PASS_COUNT) {
-            const int e = table_find(key);
-            if (e >= 0) { atomicAdd(&sm.cnt[e], 1u); return; }
             const int64_t slot = qp_insert(A.qp, key, A.err);
             if (slot >= 0) atomicAdd(A.qp.count + slot, 1ull);
         } else if constexpr (PASS == PASS_FUSED || PASS == PASS_DOMAIN) {
-            const int e = table_find(key);
             uint32_t off[K];
-            off[0] = FSM_OFF_PENDING;
-            if (e >= 0) {
-                if (PASS == PASS_FUSED) atomicAdd(&sm.cnt[e], 1u);
-                off[0] = ((volatile uint32_t *)sm.off[0])[e];
-                if (off[0] != FSM_OFF_PENDING) {
-#pragma unroll
-                    for (int h = 1; h < K; ++h) off[h] = ((volatile uint32_t *)sm.off[h])[e];
-                }
+            int64_t slot;
+            if (!key_record(key, slot, off)) {
+                if (PASS == PASS_DOMAIN) return;   // pattern without bitmaps
+                if (!first_sight<K>(A, key, slot, off)) return;
             }
-            if (off[0] == FSM_OFF_PENDING) {
-                int64_t slot;
-                if (PASS == PASS_DOMAIN) {
-                    slot = qp_find(A.qp, key);
-                    if (slot < 0) { atomicOr(A.err, FSM_ERR_QP_MISSING); return; }
-                } else {
-                    slot = qp_insert(A.qp, key, A.err);
-                    if (slot < 0) return;
-                    if (e < 0) atomicAdd(A.qp.count + slot, 1ull);
-                }
-                if (!key_offsets<K, PASS>(A, key, slot, off)) return;
-                if (e >= 0) {   // lanes racing here write the same values; position 0 last
-#pragma unroll
-                    for (int h = 1; h < K; ++h) ((volatile uint32_t *)sm.off[h])[e] = off[h];
-                    __threadfence_block();
-                    ((volatile uint32_t *)sm.off[0])[e] = off[0];
-                }
-            }
-            if (off[0] == FSM_OFF_NONE) return;   // pattern without domains
-            set_bits(off, r, ra, rb, swap);
+            if (PASS == PASS_FUSED) atomicAdd(A.qp.count + slot, 1ull);
+            const uint32_t ranchor = (uint32_t)__ldg(A.g.vinfo + anchor).w;
+            set_bits(off, r, centre ? rx : ranchor, centre ? ranchor : rx, swap);
         } else {
             const int64_t slot = qp_find(A.qp, key);
             if (slot < 0) { atomicOr(A.err, FSM_ERR_QP_MISSING); return; }
@@ -429,6 +421,7 @@ struct Joiner {
             const int64_t pos = (int64_t)base + __popc(act & ((1u << lane) - 1u));
             if (pos >= A.out_N) { atomicOr(A.err, FSM_ERR_BOUNDS); return; }
             const uint32_t meta = r[R::META];
+            const int32_t a = centre ? x : anchor, b = centre ? anchor : x;
 #pragma unroll
             for (int t = 0; t < L; ++t) {
                 const int h = (int)(meta >> (12 + 3 * t)) & 7;   // canonical position of the t-th smallest
@@ -440,59 +433,128 @@ struct Joiner {
         }
     }
 
+    // Cross edges of a new vertex x to the other vertices of s (bit o: the o-th in id order), and with
+    // `key` to the key vertex (bit O).  What the Bloom filters leave is searched, each lane its own
+    // list per round, so a warp waits for its longest chain once and not once per list.
+    __device__ __forceinline__ uint32_t cross_of(const uint32_t *r, int j, int rv, int32_t x, bool key) const {
+        uint32_t c = key && maybe(j, rv, x) ? 1u << O : 0u;
+#pragma unroll
+        for (int o = 0; o < O; ++o) c |= (uint32_t)maybe(j, o + (o >= rv), x) << o;
+        for (uint32_t p = c; p; p &= p - 1) {
+            const int o = __ffs(p) - 1;
+            if (!sorted_has(A.g.col, (int32_t)r[o == O ? R::VB : R::OB + o], (int32_t)r[o == O ? R::VE : R::OE + o], x))
+                c &= ~(1u << o);
+        }
+        return c;
+    }
+
+    // bit o of the result: label lab is in the which-th mask of the o-th other vertex (see load_units)
+    __device__ __forceinline__ uint32_t labels_ok(const uint32_t *r, int which, int lab) const {
+        uint32_t m = 0;
+#pragma unroll
+        for (int o = 0; o < O; ++o) m |= ((r[R::OK + 6 * o + 2 * which + (lab >> 5)] >> (lab & 31)) & 1u) << o;
+        return m;
+    }
+    // is label z frequent in row (p, q) of the tab-th size-3 label table?
+    __device__ __forceinline__ bool frequent(int tab, int p, int q, int z) const {
+        return (__ldg((const uint32_t *)A.lf + 2 * (tab * 4096 + p * 64 + q) + (z >> 5)) >> (z & 31)) & 1u;
+    }
+
+    // The anchor's part of a candidate's word.
+    __device__ __forceinline__ uint32_t anchor_meta(const uint32_t *r, int j, int32_t anchor, int lab) const {
+        const int rv = (r[R::META] >> 3) & 7;
+        uint32_t must = 0, no = 0;
+        if (A.lf) {   // the anchor is next to the key vertex
+            constexpr uint32_t all = (1u << O) - 1u;
+            must = ~labels_ok(r, 0, lab) & all;
+            no = ~labels_ok(r, 1, lab) & all;
+        }
+        return ((uint32_t)lab << FSM_M_LAB) | (cross_of(r, j, rv, anchor, false) << FSM_M_CROSS) | (must << FSM_M_MUST) |
+               (no << FSM_M_NO);
+    }
+
     // The last n (<= 32) survivors of the queue, one per lane; warp-synchronous.
     __device__ __forceinline__ void take(int n) {
         __syncwarp();
         const bool on = lane < n;
         const int q = qn - n + (on ? lane : 0);
-        const uint32_t m = sm.qm[w][q];
-        const int32_t a = (int32_t)sm.qa[w][q], b = (int32_t)sm.qb[w][q];
+        uint32_t m = sm.q_meta[w][q];
+        const int32_t anchor = (int32_t)sm.q_anchor[w][q], x = (int32_t)sm.q_partner[w][q];
         const int j = m & 15;
-        const bool centre = (m & 16) == 0;
+        const bool centre = !((m >> FSM_M_END) & 1u);
         const uint32_t *r = rec(j);
         const uint32_t meta = r[R::META];
         const int ki = meta & 7, rv = (meta >> 3) & 7, lv = (meta >> 6) & 63;
         const int32_t v = (int32_t)r[R::SS + rv];
-        const int4 ia = __ldg(A.g.vinfo + a), ib = __ldg(A.g.vinfo + b);
-        const int la = ia.z, lb_ = ib.z;
+        const int4 ix = __ldg(A.g.vinfo + x);
+        const int lx = ix.z;
+        if (QUOTA) m |= anchor_meta(r, j, anchor, __ldg(A.g.vinfo + anchor).z);
+        const int la = (m >> FSM_M_LAB) & 63;
+        // bits of the anchor and of the partner in a cross subset: a's low, b's high
+        const int sh_a = centre ? O : 0, sh_x = centre ? 0 : O;
+        constexpr uint32_t all = (1u << O) - 1u;
         uint32_t forms = 0;
         if (on) {
+            // the piece's own size-3 pattern must be frequent
             if (centre) {
-                forms = 1u << FORM_CENTRE;
-                if (!tfe) {
-                    const bool shorter = ia.y - ia.x <= ib.y - ib.x;
-                    if (shorter ? sorted_has(A.g.col, ia.x, ia.y, b) : sorted_has(A.g.col, ib.x, ib.y, a))
-                        forms = A.mode == 1 ? 1u << FORM_TRI : forms | (1u << FORM_TRI);
-                }
+                if (!A.lf || frequent(0, lv, la, lx)) forms |= 1u << FORM_CENTRE;
+                if (!tfe && (!A.lf || frequent(2, lv, la, lx))) forms |= 1u << FORM_TRI;
             } else {
-                forms = 1u << FORM_END;
-                if (tfe) {
-                    if (a < b && maybe(j, rv, b) && sorted_has(A.g.col, (int32_t)r[R::RP], (int32_t)(r[R::RP] + r[R::D]), b))
-                        forms |= 1u << FORM_TRI;
-                } else if (A.mode == 1 && sorted_has(A.g.col, ib.x, ib.y, v)) {
-                    forms = 0;   // vertex-induced: only the triangle
-                }
+                if (!A.lf || frequent(0, la, lv, lx)) forms |= 1u << FORM_END;
+                if (tfe && x > anchor && (!A.lf || frequent(2, lv, la, lx))) forms |= 1u << FORM_TRI;
             }
         }
-        if (A.lf) {
-            // the piece's own size-3 pattern must be frequent
-            if ((forms & (1u << FORM_CENTRE)) && !((__ldg(A.lf + lv * 64 + la) >> lb_) & 1ull)) forms &= ~(1u << FORM_CENTRE);
-            if ((forms & (1u << FORM_END)) && !((__ldg(A.lf + la * 64 + lv) >> lb_) & 1ull)) forms &= ~(1u << FORM_END);
-            if ((forms & (1u << FORM_TRI)) && !((__ldg(A.lf + 8192 + lv * 64 + la) >> lb_) & 1ull)) forms &= ~(1u << FORM_TRI);
+        uint32_t avail = 0, must1 = 0, no1 = 0, no2 = 0;   // 1: partner next to v, 2: not
+        const uint32_t mustA = ((m >> FSM_M_MUST) & all) << sh_a, noA = ((m >> FSM_M_NO) & all) << sh_a;
+        if (forms) {
+            const bool key = tfe ? (forms >> FORM_TRI) & 1u : A.mode == 1 && !centre;
+            const uint32_t c = cross_of(r, j, rv, x, key);
+            avail = (((m >> FSM_M_CROSS) & all) << sh_a) | ((c & all) << sh_x);
+            if (key && !(c >> O)) forms &= tfe ? ~(1u << FORM_TRI) : ~0u;   // no triangle here
+            if (key && (c >> O) && !tfe) forms = 0;                         // vertex-induced: only the triangle
+            if (A.lf) {
+                must1 = (~labels_ok(r, 0, lx) & all) << sh_x;
+                no1 = (~labels_ok(r, 1, lx) & all) << sh_x;
+                no2 = (~labels_ok(r, 2, lx) & all) << sh_x;
+            }
         }
-        const bool ab = lab_id_less(la, a, lb_, b);
-        const bool va = lab_id_less(lv, v, la, a), vb = lab_id_less(lv, v, lb_, b);
+        const int sA = (m >> FSM_M_SA) & 7, sX = (m >> FSM_M_SP) & 7;
+        const bool later = x > anchor;   // partner after anchor; b > a for an end list, always for the others
+        const uint32_t *rows = A.acc + ((int64_t)r[R::CLS] * G::ROWS + ((centre ? sX : sA) * SL + (centre ? sA : sX)) * 2 +
+                                        (centre || later)) * G::W;
+        auto row_of = [&](int f) { return rows + (int64_t)f * (SL * SL * 2) * G::W; };
+        if (!tfe && centre && forms) {
+            // a ~ b decides between wedge and triangle: searched only where the answer matters
+            if (A.mode == 1) {
+#pragma unroll
+                for (int f = FORM_CENTRE; f <= FORM_TRI; f += 2)
+                    if ((forms >> f & 1u) && (((mustA | must1) & ~avail) || ((noA | no1) & avail) ||
+                                              !((__ldg(row_of(f) + (avail >> 5)) >> (avail & 31)) & 1u)))
+                        forms &= ~(1u << f);
+            }
+            if (A.mode == 1 ? forms != 0 : (forms >> FORM_TRI) & 1u) {
+                const int4 ia = __ldg(A.g.vinfo + anchor);
+                const bool shorter = ia.y - ia.x <= ix.y - ix.x;
+                const bool tri = shorter ? sorted_has(A.g.col, ia.x, ia.y, x) : sorted_has(A.g.col, ix.x, ix.y, anchor);
+                if (!tri) forms &= ~(1u << FORM_TRI);
+                else if (A.mode == 1) forms &= ~(1u << FORM_CENTRE);
+            }
+        }
+        const int32_t a = centre ? x : anchor, b = centre ? anchor : x;
+        const int la_ = centre ? lx : la, lb_ = centre ? la : lx;
+        const bool ab = lab_id_less(la_, a, lb_, b);
         auto piece = [&](int form, int &jpos) -> uint32_t {
+            const bool vb = lab_id_less(lv, v, lb_, b);
             if (form == FORM_CENTRE) {
                 jpos = 0;
-                return piece_index(PIECE_WEDGE, lv, ab ? la : lb_, ab ? lb_ : la);
+                return piece_index(PIECE_WEDGE, lv, ab ? la_ : lb_, ab ? lb_ : la_);
             }
             if (form == FORM_END) {
                 jpos = vb ? 1 : 2;
-                return piece_index(PIECE_WEDGE, la, vb ? lv : lb_, vb ? lb_ : lv);
+                return piece_index(PIECE_WEDGE, la_, vb ? lv : lb_, vb ? lb_ : lv);
             }
-            jpos = (va ? 0 : 1) + (vb ? 0 : 1);
-            return tri_index(lv, la, lb_);
+            jpos = (lab_id_less(lv, v, la_, a) ? 0 : 1) + (vb ? 0 : 1);
+            return tri_index(lv, la_, lb_);
         };
         if (A.piece_sel && forms) {
             int jp;
@@ -500,35 +562,6 @@ struct Joiner {
             for (int f = 0; f < 3; ++f)
                 if ((forms >> f & 1u) && !__ldg(A.piece_sel + piece(f, jp))) forms &= ~(1u << f);
         }
-        // cross edges, and the cross bits pruning forces off (no*) or on (must) -- a's for any
-        // form, b's for forms in which b is next to v (bv) or not (be)
-        uint32_t avail = 0, no_a = 0, must_a = 0, no_bv = 0, must_bv = 0, no_be = 0;
-        int sa = 0, sb = 0;
-        if (forms) {
-#pragma unroll
-            for (int t = 0; t < L; ++t) {
-                const int32_t x = (int32_t)r[R::SS + t];
-                sa += x < a;
-                sb += x < b;
-            }
-#pragma unroll
-            for (int o = 0; o < O; ++o) {
-                const int t = o + (o >= rv);
-                const int32_t ob = (int32_t)r[R::OB + o], oe = (int32_t)r[R::OE + o];
-                if (maybe(j, t, a) && sorted_has(A.g.col, ob, oe, a)) avail |= 1u << o;
-                if (maybe(j, t, b) && sorted_has(A.g.col, ob, oe, b)) avail |= 1u << (O + o);
-                if (A.lf) {
-                    const unsigned long long k0 = rec_u64(r, R::OK + 6 * o), k1 = rec_u64(r, R::OK + 6 * o + 2),
-                                             k2 = rec_u64(r, R::OK + 6 * o + 4);
-                    must_a |= (uint32_t)(~(k0 >> la) & 1ull) << o;
-                    no_a |= (uint32_t)(~(k1 >> la) & 1ull) << o;
-                    must_bv |= (uint32_t)(~(k0 >> lb_) & 1ull) << (O + o);
-                    no_bv |= (uint32_t)(~(k1 >> lb_) & 1ull) << (O + o);
-                    no_be |= (uint32_t)(~(k2 >> lb_) & 1ull) << (O + o);
-                }
-            }
-        }
-        const uint32_t *rows = A.acc + ((int64_t)r[R::CLS] * G::ROWS + (sa * SL + sb) * 2 + (b > a)) * G::W;
         int form = 0;
         uint32_t must = 0, free_ = 0, cur = 0, sub = 0;
         bool more = false;
@@ -541,8 +574,8 @@ struct Joiner {
                     if (!forms) break;
                     form = __ffs(forms) - 1;
                     forms &= forms - 1;
-                    const uint32_t no = no_a | (form == FORM_END ? no_be : no_bv);
-                    must = must_a | (form == FORM_END ? 0u : must_bv);
+                    const uint32_t no = noA | (form == FORM_END ? no2 : no1);
+                    must = mustA | (form == FORM_END ? 0u : must1);
                     if ((must & ~avail) || (must & no)) continue;
                     if (A.mode == 0) {
                         free_ = avail & ~no & ~must;
@@ -552,12 +585,12 @@ struct Joiner {
                         free_ = 0;
                     }
                     cur = free_;
-                    more = true;
-                    row = rows + (int64_t)form * (SL * SL * 2) * G::W;
+                    row = row_of(form);
                     if (G::W == 1) {
                         roww = __ldg(row);
-                        if (!roww) { more = false; continue; }
+                        if (!roww) continue;
                     }
+                    more = true;
                 }
                 sub = cur | must;
                 ++tested;
@@ -578,7 +611,7 @@ struct Joiner {
                     cross |= ((sub >> o) & 1u) << (2 * pp + (swap ? 1 : 0));
                     cross |= ((sub >> (O + o)) & 1u) << (2 * pp + (swap ? 0 : 1));
                 }
-                accept(r, make_key(r[R::PID], pidx, ki, jpos, cross, L), a, b, (uint32_t)ia.w, (uint32_t)ib.w, swap);
+                accept(r, make_key(r[R::PID], pidx, ki, jpos, cross, L), centre, anchor, x, (uint32_t)ix.w, swap);
             }
         }
         qn -= n;
@@ -586,13 +619,13 @@ struct Joiner {
     }
 
     // warp-synchronous: queue the survivors among the lanes' candidates, joining when 32 wait
-    __device__ __forceinline__ void push(bool ok, int32_t a, int32_t b, uint32_t m) {
+    __device__ __forceinline__ void push(bool ok, int32_t anchor, int32_t x, uint32_t m) {
         const unsigned bal = __ballot_sync(0xffffffffu, ok);
         if (ok) {
             const int p = qn + __popc(bal & ((1u << lane) - 1u));
-            sm.qa[w][p] = (uint32_t)a;
-            sm.qb[w][p] = (uint32_t)b;
-            sm.qm[w][p] = (uint8_t)m;
+            sm.q_anchor[w][p] = (uint32_t)anchor;
+            sm.q_partner[w][p] = (uint32_t)x;
+            sm.q_meta[w][p] = m;
         }
         qn += __popc(bal);
         if (qn >= 32) take(32);
@@ -629,7 +662,13 @@ struct Joiner {
 #pragma unroll
             for (int t = 0; t < L; ++t) {
                 nfo[t] = __ldg(g.vinfo + id[t]);
-                if (cp[t] == iu) { rv = t; v = id[t]; lv = nfo[t].z; }
+                if (cp[t] == iu) {
+                    rv = t;
+                    v = id[t];
+                    lv = nfo[t].z;
+                    r[R::VB] = (uint32_t)nfo[t].x;
+                    r[R::VE] = (uint32_t)nfo[t].y;
+                }
                 meta |= (uint32_t)cp[t] << (12 + 3 * t);
                 r[R::SS + t] = (uint32_t)id[t];
                 r[R::RK + cp[t]] = (uint32_t)nfo[t].w;
@@ -718,7 +757,8 @@ struct Joiner {
         }
         if (lane < nu) r[R::SEG] = (uint32_t)(inc - nseg);
         total_seg = __shfl_sync(0xffffffffu, inc, 31);
-        // Bloom filters of the lists of s (of the key vertex only where triangles need it)
+        // Bloom filters of the lists of s (of the key vertex only where end pieces are tested for
+        // closing a triangle)
         int bw = FSM_JOIN_BLOOM / (nu * L);
         lb = 5 + (31 - __clz(bw));
         __syncwarp();
@@ -731,9 +771,9 @@ struct Joiner {
             for (int t = 0; t < L; ++t) {
                 int32_t x0, x1;
                 if (t == rv) {
-                    if (!tfe) continue;
-                    x0 = (int32_t)rj[R::RP];
-                    x1 = x0 + (int32_t)rj[R::D];
+                    if (!tfe && A.mode == 0) continue;
+                    x0 = (int32_t)rj[R::VB];
+                    x1 = (int32_t)rj[R::VE];
                 } else {
                     const int o = t - (t > rv);
                     x0 = (int32_t)rj[R::OB + o];
@@ -790,6 +830,17 @@ struct Joiner {
                     }
                     uint32_t ok = in ? 0u : allowed(r, centre, s);
                     if (centre) ok &= (1u << SL) - 1u;
+                    uint32_t m = 0;
+                    int4 ia = make_int4(0, 0, 0, 0);
+                    if (ok) {
+                        ia = __ldg(g.vinfo + anchor);
+                        m = anchor_meta(r, j, anchor, ia.z) | (uint32_t)j | ((centre ? 0u : 1u) << FSM_M_END) |
+                            ((uint32_t)s << FSM_M_SA);
+                        const uint32_t all = (1u << O) - 1u;
+                        const uint32_t c = m >> FSM_M_CROSS, must = m >> FSM_M_MUST, no = m >> FSM_M_NO;
+                        // pruning rejects the anchor with any partner
+                        if (((must & (~c | no)) | (A.mode == 1 ? c & no : 0u)) & all) ok = 0;
+                    }
                     if (ok) {
                         const int64_t lo = (int64_t)rec_u64(r, R::RLO), hi = (int64_t)rec_u64(r, R::RHI);
                         const uint32_t slots = (ok | (ok >> SL)) & ((1u << SL) - 1u);
@@ -807,8 +858,8 @@ struct Joiner {
                             lb0 = rp;
                         } else {
                             const int64_t st = (int64_t)rec_u64(r, R::NC) + __ldg(g.pend + rp + y);
-                            lb0 = __ldg(g.prow + anchor);
-                            const int32_t da = __ldg(g.prow + anchor + 1) - lb0;
+                            lb0 = A.sampled ? __ldg(g.prow + anchor) : ia.x;
+                            const int32_t da = (A.sampled ? __ldg(g.prow + anchor + 1) : ia.y) - lb0;
                             p0 = (int32_t)max(lo - st, (int64_t)0);
                             p1 = (int32_t)min(hi - st, (int64_t)da);
                             // cut to the allowed slots (lists of a few entries are walked whole)
@@ -820,7 +871,8 @@ struct Joiner {
                         len = max(p1 - p0, 0);
                         sm.sg_base[w][lane] = (uint32_t)(lb0 + p0);
                         sm.sg_anchor[w][lane] = (uint32_t)anchor;
-                        sm.sg_info[w][lane] = ok | ((uint32_t)j << 16) | (centre ? 0u : 1u << 20);
+                        sm.sg_slots[w][lane] = ok;
+                        sm.sg_meta[w][lane] = m;
                     }
                 }
             }
@@ -842,9 +894,9 @@ struct Joiner {
                     if (__shfl_sync(0xffffffffu, inc, k + s - 1) <= t) k += s;
                 bool ok = t < total;
                 int32_t x = 0, anchor = 0;
-                uint32_t info = 0;
+                uint32_t m = 0;
                 if (ok) {
-                    info = sm.sg_info[w][k];
+                    m = sm.sg_meta[w][k];
                     anchor = (int32_t)sm.sg_anchor[w][k];
                     const int64_t at = (int64_t)(int32_t)(sm.sg_base[w][k] + (uint32_t)t);
                     if (A.debug && (at < 0 || at >= __ldg(g.prow + g.n))) {
@@ -852,19 +904,19 @@ struct Joiner {
                         ok = false;
                     } else {
                         x = __ldg(g.pcol + at);
-                        const uint32_t *r = rec((info >> 16) & 15);
-                        int s = x > anchor ? SL : 0;
+                        const uint32_t *r = rec(m & 15);
+                        int s = 0;
 #pragma unroll
                         for (int t2 = 0; t2 < L; ++t2) {
                             const int32_t y = (int32_t)r[R::SS + t2];
                             ok &= y != x;
                             s += y < x;
                         }
-                        ok &= (info >> s) & 1u;
+                        m |= (uint32_t)s << FSM_M_SP;
+                        ok &= (sm.sg_slots[w][k] >> (s + (x > anchor ? SL : 0))) & 1u;
                     }
                 }
-                const bool centre = !((info >> 20) & 1u);
-                push(ok, centre ? x : anchor, centre ? anchor : x, info >> 16);
+                push(ok, anchor, x, m);
             }
             __syncwarp();
         }
@@ -876,7 +928,7 @@ struct Joiner {
         for (int g0 = 0; g0 < total_seg; g0 += 32) {
             const int gi = g0 + lane;
             bool ok = gi < total_seg;
-            int32_t a = 0, b = 0;
+            int32_t anchor = 0, x = 0;
             uint32_t m = 0;
             if (ok) {
                 const int j = unit_of(gi, nu);
@@ -887,7 +939,6 @@ struct Joiner {
                 const int64_t nc = (int64_t)rec_u64(r, R::NC);
                 const int32_t rp = (int32_t)r[R::RP], d = (int32_t)r[R::D];
                 const bool centre = lq < nc;
-                int32_t anchor, x;
                 if (centre) {
                     int32_t cpos = d;
                     if (L == 2) cpos = (int32_t)r[R::BND + (((r[R::META] >> 3) & 7) ? 0 : 1)];
@@ -913,41 +964,12 @@ struct Joiner {
                     sx += y < x;
                 }
                 if (ok) ok = (allowed(r, centre, s) >> (sx + (x > anchor ? SL : 0))) & 1u;
-                a = centre ? x : anchor;
-                b = centre ? anchor : x;
-                m = (uint32_t)j | (centre ? 0u : 16u);
+                m = (uint32_t)j | ((centre ? 0u : 1u) << FSM_M_END) | ((uint32_t)s << FSM_M_SA) | ((uint32_t)sx << FSM_M_SP);
             }
-            push(ok, a, b, m);
+            push(ok, anchor, x, m);
         }
     }
 
-    // Write the key table out and clear it (all threads of the block, between barriers).
-    __device__ __forceinline__ void flush_table() {
-        for (int x = threadIdx.x; x < SM::NS; x += blockDim.x) {
-            const unsigned long long key = sm.key[x];
-            if (key == FSM_EMPTY_KEY) continue;
-            if constexpr (SM::COUNTS) {
-                const int64_t slot = qp_insert(A.qp, key, A.err);
-                if (slot >= 0) atomicAdd(A.qp.count + slot, (unsigned long long)sm.cnt[x]);
-                sm.cnt[x] = 0u;
-            }
-            if constexpr (SM::OFFS) sm.off[0][x] = FSM_OFF_PENDING;
-            sm.key[x] = FSM_EMPTY_KEY;
-        }
-    }
-
-    // Every warp of the block meets here between its chunks when the key table is to be flushed,
-    // and from its last chunk on; true when all warps are out of work.
-    __device__ __forceinline__ bool meet() {
-        __syncthreads();
-        const bool done = ((volatile int *)&sm.done)[0] == 8;
-        if constexpr (SM::NS > 0)
-            if (done || ((volatile int *)&sm.flag)[0]) flush_table();
-        __syncthreads();
-        if (threadIdx.x == 0) { sm.flag = 0; sm.load = 0; }
-        __syncthreads();
-        return done;
-    }
 };
 
 template <int L, int PASS, bool QUOTA>
@@ -955,13 +977,6 @@ __global__ void __launch_bounds__(256, 3) join_kernel(const __grid_constant__ Ex
     extern __shared__ __align__(16) unsigned char join_smem[];
     using J = Joiner<L, PASS, QUOTA>;
     typename J::SM &sm = *reinterpret_cast<typename J::SM *>(join_smem);
-    for (int x = threadIdx.x; x < J::SM::NS; x += blockDim.x) {
-        sm.key[x] = FSM_EMPTY_KEY;
-        if (J::SM::COUNTS) sm.cnt[x] = 0u;
-        if (J::SM::OFFS) sm.off[0][x] = FSM_OFF_PENDING;
-    }
-    if (threadIdx.x == 0) { sm.load = 0; sm.flag = 0; sm.done = 0; }
-    __syncthreads();
     J jn(A, sm);
     const int lane = jn.lane;
     const int64_t nunits = A.ne * L;
@@ -972,14 +987,14 @@ __global__ void __launch_bounds__(256, 3) join_kernel(const __grid_constant__ Ex
         if (chunk <= 0) chunk = join_chunk(total, nunits, (int64_t)gridDim.x * (blockDim.x >> 5));
         nchunks = (total + chunk - 1) / chunk;
     }
+    int64_t stride = 1;
+    if (A.warm) {   // a sample: every stride-th chunk
+        stride = warm_stride(total);
+        chunk = min(chunk, (int64_t)FSM_WARM_CHUNK);
+        nchunks = ((total + chunk - 1) / chunk + stride - 1) / stride;
+    }
     if (A.stats && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(A.stats + 2, (unsigned long long)total);
-    bool out = false;   // this warp has no more work
     for (;;) {
-        const bool wait = out || __shfl_sync(0xffffffffu, ((volatile int *)&sm.flag)[0], 0) != 0;
-        if (wait) {
-            if (jn.meet()) break;
-            if (out) continue;
-        }
         unsigned long long c = 0;
         if (lane == 0) {
             // stop early when the call ran out of time, when an overflowing count pass is to be
@@ -994,13 +1009,8 @@ __global__ void __launch_bounds__(256, 3) join_kernel(const __grid_constant__ Ex
             c = stop ? ~0ull : atomicAdd(A.chunk_ctr, 1ull);
         }
         c = __shfl_sync(0xffffffffu, c, 0);
-        if (c >= (unsigned long long)nchunks) {
-            out = true;
-            if (lane == 0) atomicAdd(&sm.done, 1);
-            __syncwarp();
-            continue;
-        }
-        const int64_t q0 = (int64_t)c * chunk;
+        if (c >= (unsigned long long)nchunks) break;
+        const int64_t q0 = (int64_t)c * stride * chunk;
         const int64_t q1 = min(q0 + chunk, total);
         const int64_t ulo = warp_last_le(A.unit_base, 0, nunits - 1, q0);
         const int64_t uhi = warp_last_le(A.unit_base, ulo, nunits - 1, q1 - 1);
@@ -1022,6 +1032,17 @@ __global__ void __launch_bounds__(256, 3) join_kernel(const __grid_constant__ Ex
     if (lane == 0 && A.stats) {
         atomicAdd(A.stats + 0, t0);
         atomicAdd(A.stats + 1, t1);
+    }
+}
+
+// Publish the record of every key in the table (after a warm pass): one thread per slot, so that
+// canonicalising runs with full warps.
+static __global__ void resolve_keys_kernel(const ExtArgs A) {
+    const ResolveArgs R{A.pat_lab, A.pat_adj, A.cls_size, A.code_keys, A.code_off, A.pool_top,
+                        A.code_mask, A.pool_words, A.key_rec, A.off_shift, A.err, A.explore, A.level};
+    for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s <= A.qp.mask; s += (uint64_t)gridDim.x * blockDim.x) {
+        const unsigned long long key = A.qp.keys[s];
+        if (key != FSM_EMPTY_KEY) resolve_slot(R, (int64_t)s, key);
     }
 }
 

@@ -1289,15 +1289,20 @@ cudaError_t launch_fused_support(int K, const unsigned long long *plab, const ui
 namespace {
 __global__ void slot_bases_kernel(int K, const int64_t *slots, int64_t nq, const int32_t *qp_pattern,
                                   const uint64_t *qp_perm, const uint8_t *live, const uint64_t *orbit,
-                                  const int64_t *dom_off, int shift, int64_t *slot_base, uint32_t *slot_off) {
+                                  const int64_t *dom_off, int shift, int64_t *slot_base, const unsigned long long *keys,
+                                  uint32_t *key_rec, int rec_words) {
     for (int64_t q = gtid(); q < nq; q += gstride()) {
         const int64_t slot = slots[q];
+        if (!slot_base) {
+            key_rec[slot * rec_words] = (uint32_t)keys[slot];
+            key_rec[slot * rec_words + 1] = (uint32_t)(keys[slot] >> 32);
+        }
         const int32_t P = qp_pattern[slot];
         for (int h = 0; h < FSM_MAXK; ++h) {
             int64_t b = -1;
             if (h < K && live[P]) b = dom_off[(int64_t)P * FSM_MAXK + nib_get(orbit[P], nib_get(qp_perm[slot], h))];
             if (slot_base) slot_base[slot * FSM_MAXK + h] = b;
-            else if (h < 8) slot_off[slot * 8 + h] = b < 0 ? 0xFFFFFFFFu : (uint32_t)(b >> shift);
+            else if (h < K) key_rec[slot * rec_words + 2 + h] = b < 0 ? 0xFFFFFFFFu : (uint32_t)(b >> shift);
         }
     }
 }
@@ -1305,12 +1310,12 @@ __global__ void slot_bases_kernel(int K, const int64_t *slots, int64_t nq, const
 
 cudaError_t launch_slot_bases(int K, const int64_t *slots, int64_t nq, const int32_t *qp_pattern,
                               const uint64_t *qp_perm, const uint8_t *live, const uint64_t *orbit,
-                              const int64_t *dom_off, int shift, int64_t *slot_base, uint32_t *slot_off,
-                              cudaStream_t st) {
+                              const int64_t *dom_off, int shift, int64_t *slot_base, const unsigned long long *keys,
+                              uint32_t *key_rec, int rec_words, cudaStream_t st) {
     if (nq <= 0) return cudaSuccess;
     LAUNCHED(1);
     slot_bases_kernel<<<blocks_for(nq), kThreads, 0, st>>>(K, slots, nq, qp_pattern, qp_perm, live, orbit, dom_off,
-                                                           shift, slot_base, slot_off);
+                                                           shift, slot_base, keys, key_rec, rec_words);
     return cudaGetLastError();
 }
 

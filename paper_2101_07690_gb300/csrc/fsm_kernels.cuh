@@ -199,8 +199,8 @@ cudaError_t launch_fused_support(int K, const unsigned long long *plab, const ui
 // when the pattern has no domains.
 cudaError_t launch_slot_bases(int K, const int64_t *slots, int64_t nq, const int32_t *qp_pattern,
                               const uint64_t *qp_perm, const uint8_t *live, const uint64_t *orbit,
-                              const int64_t *dom_off, int shift, int64_t *slot_base, uint32_t *slot_off,
-                              cudaStream_t st);
+                              const int64_t *dom_off, int shift, int64_t *slot_base, const unsigned long long *keys,
+                              uint32_t *key_rec, int rec_words, cudaStream_t st);
 
 // ---- pieces: mark the frequent size-3 patterns by piece index
 cudaError_t launch_piece_table(const unsigned long long *lab, const uint64_t *adj, int64_t n,
