@@ -718,19 +718,18 @@ struct Miner {
         G->qp_hint[L] = std::max(G->qp_hint[L], nq);
         int32_t *qpat = mem.get<int32_t>(cap);
         uint64_t *qperm = mem.get<uint64_t>(cap);
-        int64_t M = 1;
-        while (M < nq) M <<= 1;
-        CodeRec *recs = mem.get<CodeRec>(M);
+        CodeRec *recs = mem.get<CodeRec>(nq), *recs2 = mem.get<CodeRec>(nq), *sorted = nullptr;
+        void *sort_tmp = mem.get<char>((int64_t)sort_temp_bytes(nq));
         ck(launch_qp_canon(L, V, keys, slots, nq, in.lab8, in.adj8, recs, qperm, st), "canonicalise");
-        ck(launch_sort_codes(recs, nq, st), "sort codes");
+        ck(launch_sort_codes(K, recs, recs2, nq, sort_tmp, &sorted, st), "sort codes");
         int64_t *flag = mem.get<int64_t>(nq + 1);
         int64_t *ids = mem.get<int64_t>(nq + 1);
         void *stmp = mem.get<char>((int64_t)scan_temp_bytes(nq) + 16);
         unsigned long long *plab = mem.get<unsigned long long>(nq);
         uint64_t *padj = mem.get<uint64_t>(nq);
-        ck(launch_assign_patterns(recs, nq, slots, flag, ids, stmp, qpat, plab, padj, st), "assign patterns");
+        ck(launch_assign_patterns(sorted, nq, slots, flag, ids, stmp, qpat, plab, padj, st), "assign patterns");
         const int64_t np = nq > 0 ? d2h(ids + nq, st) : 0;
-        mem.release(recs);
+        for (void *q : {(void *)recs, (void *)recs2, sort_tmp}) mem.release(q);
         // ---- orbits, counts, live patterns, domain bitmaps
         uint64_t *orbit = mem.get<uint64_t>(np);
         int32_t *minorb = mem.get<int32_t>(np);

@@ -1,53 +1,28 @@
 // fsm_canon7.cuh -- canonical codes for the one-pass last level (K <= 7 vertices).
 //
-// The same canonical form as fsm_canon.cuh (the smallest (label sequence, adjacency sequence)
-// over all vertex orders, found by enumerating the label-preserving orders of the label-sorted
-// positions), in the compact words this level has always used: label bytes (byte 7 - c holds
-// canonical position c), a 32-bit adjacency word (at most 21 pair bits, first pair most
+// The same canonical form as fsm_canon.cuh (canon7, orbits7) in compact words: label bytes (byte
+// 7 - c holds canonical position c), a 32-bit adjacency word (at most 21 pair bits, first pair most
 // significant) and 3-bit vertex orders, with 8-entry scratch arrays.  The one-pass kernel calls
-// only these on first sight of a quick pattern, so its code stays what it was before patterns of
-// 8 and 9 vertices needed the wider words and the cell search of fsm_canon.cuh.  The host build
-// of tests/device_helpers_check.cu checks them against fsm_canon.cuh.
+// only these on first sight of a quick pattern.  The host build of tests/device_helpers_check.cu
+// checks them against fsm_canon.cuh.
 #pragma once
 #include "fsm_canon.cuh"
 
 namespace fsm {
 
-FSM_HD uint32_t adj_code7(int K, const uint32_t *adj, const int *perm) {
-    uint32_t code = 0;
-    for (int c1 = 0; c1 < K; ++c1) {
-        const uint32_t row = adj[perm[c1]];
-        for (int c2 = c1 + 1; c2 < K; ++c2) code = (code << 1) | ((row >> perm[c2]) & 1u);
-    }
-    return code;
-}
-
 // clab7: label of canonical position c in byte 7 - c; cadj7: adjacency word; inv7: vertex h ->
 // canonical position in bits 3h..3h+2 (first optimal order).
 static __host__ __device__ __noinline__ void canonicalise7(int K, const int *lab, const uint32_t *adj,
                                                            unsigned long long &clab7, uint32_t &cadj7, uint32_t &inv7) {
-    int perm[8], seg[8], best[8];
-    for (int h = 0; h < K; ++h) perm[h] = h;
-    for (int a = 1; a < K; ++a)          // insertion sort by label (stable)
-        for (int b = a; b > 0 && lab[perm[b - 1]] > lab[perm[b]]; --b) { int t = perm[b]; perm[b] = perm[b - 1]; perm[b - 1] = t; }
-    for (int c = 0; c < K; ++c) seg[c] = (c > 0 && lab[perm[c]] == lab[perm[c - 1]]) ? seg[c - 1] : c;
-    // within each segment start from ascending vertex index (next_perm enumerates from there)
-    for (int c = 0; c < K; ++c)
-        for (int b = c; b > seg[c] && perm[b - 1] > perm[b]; --b) { int t = perm[b]; perm[b] = perm[b - 1]; perm[b - 1] = t; }
-    uint32_t bc = 0xffffffffu;
-    do {
-        const uint32_t code = adj_code7(K, adj, perm);
-        if (code < bc) {
-            bc = code;
-            for (int c = 0; c < K; ++c) best[c] = perm[c];
-        }
-    } while (next_label_perm(K, seg, perm));
+    uint32_t order;
+    cadj7 = canon7(K, lab, adj, order);
+    int best[8];
+    for (int c = 0; c < K; ++c) best[c] = nib_get(order, c);
     unsigned long long l = 0;
     for (int c = 0; c < K; ++c) l |= (unsigned long long)(lab[best[c]] & 0xff) << (8 * (7 - c));
     uint32_t iv = 0;
     for (int c = 0; c < K; ++c) iv |= (uint32_t)c << (3 * best[c]);
     clab7 = l;
-    cadj7 = bc;
     inv7 = iv;
 }
 
@@ -105,20 +80,12 @@ FSM_HD void decode_code7(int K, unsigned long long clab7, uint32_t cadj7, int *l
             if ((cadj7 >> (np - 1 - q)) & 1u) { adj[c1] |= 1u << c2; adj[c2] |= 1u << c1; }
 }
 
-// Orbit representatives (as orbit_reps of fsm_canon.cuh), by enumeration.
+// Orbit representatives (as orbit_reps of fsm_canon.cuh), 
 static __host__ __device__ __noinline__ void orbit_reps7(int K, unsigned long long clab7, uint32_t cadj7, int *rep) {
-    int lab[8], perm[8], seg[8];
+    int lab[8];
     uint32_t adj[8];
     decode_code7(K, clab7, cadj7, lab, adj);
-    for (int c = 0; c < K; ++c) {
-        perm[c] = c;
-        rep[c] = c;
-        seg[c] = (c > 0 && lab[c] == lab[c - 1]) ? seg[c - 1] : c;
-    }
-    do {
-        if (adj_code7(K, adj, perm) == cadj7)
-            for (int c = 0; c < K; ++c) if (perm[c] < rep[c]) rep[c] = perm[c];
-    } while (next_label_perm(K, seg, perm));
+    orbits7(K, lab, adj, rep);
 }
 
 // pack_code of fsm_canon.cuh from the compact words: the same 63-bit value.

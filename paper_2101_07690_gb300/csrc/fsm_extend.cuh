@@ -129,12 +129,13 @@ FSM_HD int64_t join_chunk(int64_t total, int64_t units, int64_t warps) {
 
 // Warm pass of a one-pass level: the keys of every warm_stride-th chunk of FSM_WARM_CHUNK pieces are
 // counted and resolved in bulk first, so that the level itself meets few keys for the first time.
-// All pieces up to 2^24 (small levels have most keys per piece), then 2^24 of them, from 2^31 on
-// one in 128 (a level of 7.5e9 pieces: 1 in 32 took 3.5 ms of 143, for the same few misses).
+// All pieces up to 2^24 (small levels have most keys per piece), then 2^24 of them, from 2^29 on
+// one in 32: with one in 102, the level of 1.7e9 pieces met enough new keys to take 36.8 ms
+// instead of 30.5 ms, far more than the 0.7 ms that the smaller sample saved.
 #define FSM_WARM_CHUNK 1024
 FSM_HD int64_t warm_stride(int64_t total) {
     const int64_t s = total >> 24;
-    return s < 1 ? 1 : s > 128 ? 128 : s;
+    return s < 1 ? 1 : s > 32 ? 32 : s;
 }
 
 __device__ __forceinline__ unsigned long long global_ns() {

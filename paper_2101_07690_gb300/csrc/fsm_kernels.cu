@@ -380,19 +380,91 @@ __device__ __forceinline__ bool rec_less(const CodeRec &a, const CodeRec &b) {
     return a.idx < b.idx;
 }
 
-__global__ void bitonic_step_kernel(CodeRec *r, int64_t M, int64_t j, int64_t k) {
-    for (int64_t t = gtid(); t < M; t += gstride()) {
-        const int64_t p = t ^ j;
-        if (p <= t) continue;
-        const bool up = (t & k) == 0;
-        CodeRec a = r[t], b = r[p];
-        if (up ? rec_less(b, a) : rec_less(a, b)) { r[t] = b; r[p] = a; }
+// ---- sort by (lab, adj, idx)
+//
+// Up to FSM_SORT_BLOCK records (small graphs and levels, where a launch costs more than the work):
+// one block sorts them in shared memory.  Above: least-significant-digit radix sort of the code as
+// one integer of 6 K + K (K - 1) / 2 bits (labels above pairs), eight bits a pass, stable, so equal
+// codes keep their order.  A pass reads the records twice and writes them once.  Before, a bitonic
+// network over global memory took one launch and one reading and writing of all records per step:
+// 300 launches and 25.7 ms for 11.8M codes of 7 vertices, 190 launches and 0.9 ms for 330k of 5;
+// now 2.3 ms and 0.12 ms, and one launch of 21 us instead of 66 launches for 2000 codes.
+constexpr int kSortBlock = 2048;
+constexpr int kRadixItems = 8;
+constexpr int kRadixTile = kThreads * kRadixItems;
+
+__global__ void __launch_bounds__(1024) sort_block_kernel(CodeRec *r, int n, int M) {
+    __shared__ CodeRec s[kSortBlock];
+    for (int t = threadIdx.x; t < M; t += blockDim.x) {
+        if (t < n) s[t] = r[t];
+        else { s[t].lab = ~0ull; s[t].adj = ~0ull; s[t].idx = ~0u; }
     }
+    __syncthreads();
+    for (int k = 2; k <= M; k <<= 1)
+        for (int j = k >> 1; j > 0; j >>= 1) {
+            for (int t = threadIdx.x; t < M; t += blockDim.x) {
+                const int p = t ^ j;
+                if (p <= t) continue;
+                const CodeRec a = s[t], b = s[p];
+                if ((t & k) == 0 ? rec_less(b, a) : rec_less(a, b)) { s[t] = b; s[p] = a; }
+            }
+            __syncthreads();
+        }
+    for (int t = threadIdx.x; t < n; t += blockDim.x) r[t] = s[t];
 }
 
-__global__ void pad_recs_kernel(CodeRec *r, int64_t n, int64_t M) {
-    for (int64_t t = n + gtid(); t < M; t += gstride()) {
-        r[t].lab = ~0ull; r[t].adj = ~0ull; r[t].idx = ~0u;
+// digit number `pass` of a code of K vertices
+__device__ __forceinline__ uint32_t code_digit(const CodeRec &x, int K, int pass) {
+    const int np = K * (K - 1) / 2, sh = 8 * pass;
+    const uint64_t lab = x.lab >> (6 * (FSM_MAXK - K));
+    const uint64_t lo = x.adj | (lab << np), hi = np ? lab >> (64 - np) : 0ull;
+    const uint64_t v = sh < 64 ? (lo >> sh) | (sh ? hi << (64 - sh) : 0ull) : hi >> (sh - 64);
+    return (uint32_t)v & 255u;
+}
+
+__global__ void radix_hist_kernel(const CodeRec *r, int64_t n, int K, int pass, int64_t tiles, int64_t *hist) {
+    __shared__ uint32_t h[256];
+    h[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t t0 = (int64_t)blockIdx.x * kRadixTile;
+    for (int i = threadIdx.x; i < kRadixTile && t0 + i < n; i += kThreads) atomicAdd(&h[code_digit(r[t0 + i], K, pass)], 1u);
+    __syncthreads();
+    hist[(int64_t)threadIdx.x * tiles + blockIdx.x] = h[threadIdx.x];
+}
+
+__global__ void radix_scatter_kernel(const CodeRec *r, CodeRec *out, int64_t n, int K, int pass, int64_t tiles,
+                                     const int64_t *base) {
+    __shared__ uint32_t wh[kThreads / 32][256];   // per warp: records of each digit, then where they go
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int d = lane; d < 256; d += 32) wh[w][d] = 0;
+    __syncwarp();
+    // a warp's records are consecutive: rank within the warp in input order
+    const int64_t t0 = (int64_t)blockIdx.x * kRadixTile + w * (32 * kRadixItems);
+    uint32_t dg[kRadixItems], rk[kRadixItems];
+#pragma unroll
+    for (int i = 0; i < kRadixItems; ++i) {
+        const int64_t t = t0 + i * 32 + lane;
+        const bool on = t < n;
+        dg[i] = on ? code_digit(r[t], K, pass) : 256u;
+        const unsigned same = __match_any_sync(0xffffffffu, dg[i]);
+        rk[i] = on ? wh[w][dg[i]] + __popc(same & ((1u << lane) - 1u)) : 0u;
+        __syncwarp();
+        if (on && lane == __ffs(same) - 1) wh[w][dg[i]] += __popc(same);
+        __syncwarp();
+    }
+    __syncthreads();
+    uint32_t run = (uint32_t)base[(int64_t)threadIdx.x * tiles + blockIdx.x];
+#pragma unroll
+    for (int x = 0; x < kThreads / 32; ++x) {
+        const uint32_t c = wh[x][threadIdx.x];
+        wh[x][threadIdx.x] = run;
+        run += c;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < kRadixItems; ++i) {
+        const int64_t t = t0 + i * 32 + lane;
+        if (t < n) out[wh[w][dg[i]] + rk[i]] = r[t];
     }
 }
 
@@ -534,17 +606,38 @@ cudaError_t launch_qp_canon(int L, int V, const unsigned long long *keys, const 
     return cudaGetLastError();
 }
 
-cudaError_t launch_sort_codes(CodeRec *recs, int64_t n, cudaStream_t st) {
+size_t sort_temp_bytes(int64_t n) {
+    if (n <= kSortBlock) return 16;
+    const int64_t tiles = (n + kRadixTile - 1) / kRadixTile;
+    return (size_t)(2 * 256 * tiles + 1) * sizeof(int64_t) + scan_temp_bytes(256 * tiles) + 16;
+}
+
+cudaError_t launch_sort_codes(int K, CodeRec *recs, CodeRec *other, int64_t n, void *tmp, CodeRec **sorted,
+                              cudaStream_t st) {
+    *sorted = recs;
     if (n <= 1) return cudaSuccess;
-    int64_t M = 1;
-    while (M < n) M <<= 1;
-    LAUNCHED(1);
-    pad_recs_kernel<<<blocks_for(M - n + 1), kThreads, 0, st>>>(recs, n, M);
-    for (int64_t k = 2; k <= M; k <<= 1)
-        for (int64_t j = k >> 1; j > 0; j >>= 1) {
-            LAUNCHED(1);
-            bitonic_step_kernel<<<blocks_for(M), kThreads, 0, st>>>(recs, M, j, k);
-        }
+    if (n <= kSortBlock) {
+        int M = 32;
+        while (M < n) M <<= 1;
+        LAUNCHED(1);
+        sort_block_kernel<<<1, M < 1024 ? M : 1024, 0, st>>>(recs, (int)n, M);
+        return cudaGetLastError();
+    }
+    const int64_t tiles = (n + kRadixTile - 1) / kRadixTile;
+    int64_t *hist = (int64_t *)tmp, *base = hist + 256 * tiles;
+    void *stmp = base + 256 * tiles + 1;
+    CodeRec *a = recs, *b = other;
+    for (int pass = 0; pass * 8 < 6 * K + K * (K - 1) / 2; ++pass) {
+        LAUNCHED(2);
+        radix_hist_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(a, n, K, pass, tiles, hist);
+        cudaError_t e = launch_scan_i64(hist, base, 256 * tiles, stmp, st);
+        if (e != cudaSuccess) return e;
+        radix_scatter_kernel<<<(unsigned)tiles, kThreads, 0, st>>>(a, b, n, K, pass, tiles, base);
+        CodeRec *t = a;
+        a = b;
+        b = t;
+    }
+    *sorted = a;
     return cudaGetLastError();
 }
 

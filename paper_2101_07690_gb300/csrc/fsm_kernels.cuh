@@ -61,8 +61,11 @@ cudaError_t launch_qp_compact(const unsigned long long *keys, int64_t cap, int64
 cudaError_t launch_qp_canon(int L, int V, const unsigned long long *keys, const int64_t *slots, int64_t nq,
                             const uint64_t *pat_lab8, const uint64_t *pat_adj8, CodeRec *recs,
                             uint64_t *perm, cudaStream_t st);
-// sort recs[0..n) ascending by (lab, adj, idx); recs must have room for next_pow2(n) entries
-cudaError_t launch_sort_codes(CodeRec *recs, int64_t n, cudaStream_t st);
+// sort recs[0..n), codes of K vertices, ascending by (lab, adj), equal codes in input order or by
+// idx; other: n more records; tmp: sort_temp_bytes(n).  *sorted = recs or other
+size_t sort_temp_bytes(int64_t n);
+cudaError_t launch_sort_codes(int K, CodeRec *recs, CodeRec *other, int64_t n, void *tmp, CodeRec **sorted,
+                              cudaStream_t st);
 // after sorting: pattern ids.  flags/ids scratch of n+1 entries.  Writes qp_pattern[slot],
 // pattern codes pat_lab/pat_adj, and *n_pat.
 cudaError_t launch_assign_patterns(const CodeRec *recs, int64_t n, const int64_t *slots, int64_t *flag,
