@@ -398,7 +398,8 @@ struct Miner {
                 if (total == 0) continue;
                 bytes(r);
                 int64_t chunk = chunk_for(L);
-                if (chunk <= 0) chunk = join_chunk(total, r.ne * L, warps);   // as the kernel does when the total stays on the device
+                // as the kernel does when the total stays on the device
+                if (chunk <= 0) chunk = joins(L) ? join_chunk(total, warps) : extend_chunk(total, r.ne * L, warps);
                 A.e0 = r.e0;
                 A.ne = r.ne;
                 A.total = total;

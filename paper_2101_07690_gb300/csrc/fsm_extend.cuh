@@ -117,13 +117,22 @@ struct ExtArgs {
     int *err;
 };
 
-// Pieces per work-stealing chunk of a pass of `total` pieces over `units` units on `warps` warps:
-// at least 64 chunks per warp, and at most about 16 units' pieces per chunk (a chunk over a few
-// units prepares them together).
-FSM_HD int64_t join_chunk(int64_t total, int64_t units, int64_t warps) {
+// Pieces per work-stealing chunk of a pass of `total` pieces over `units` units on `warps` warps.
+// Extension kernel: at least 64 chunks per warp, and at most about 16 units' pieces per chunk (a chunk
+// over a few units prepares them together).
+FSM_HD int64_t extend_chunk(int64_t total, int64_t units, int64_t warps) {
     const int64_t per_unit = total / (units > 0 ? units : 1);
     int64_t chunk = 256;
     while (chunk < 16384 && total / chunk > warps * 64 && chunk * 2 <= 16 * per_unit) chunk <<= 1;
+    return chunk;
+}
+// Join kernel, which prepares units in batches of its own: a chunk costs two searches of the prefix
+// and a part-filled last batch, so it is as large as leaves 8 chunks per warp, from 64 to 8192 (3 -> 5
+// count, 1.7e8 pieces: 1.83 ms at 1024, 1.63 at 4096, 1.74 at 8192; 5 -> 7 count, 6.0e8: 35 ms at
+// 512, 27 at 8192, 30 at 65536; 1 -> 3, 6.3e8: 7.9 ms at 512, 5.7 at 8192).
+FSM_HD int64_t join_chunk(int64_t total, int64_t warps) {
+    int64_t chunk = 64;
+    while (chunk < 8192 && total >= chunk * 2 * 8 * warps) chunk <<= 1;
     return chunk;
 }
 
@@ -783,7 +792,7 @@ __global__ void __launch_bounds__(256, ExtMinBlocks<PASS>::value) extend_kernel(
     if (total < 0) {
         // device-resident size: no host round trip between the prefix sum and this launch
         total = __ldg(A.unit_base + nunits);
-        if (chunk <= 0) chunk = join_chunk(total, nunits, (int64_t)gridDim.x * (blockDim.x >> 5));
+        if (chunk <= 0) chunk = extend_chunk(total, nunits, (int64_t)gridDim.x * (blockDim.x >> 5));
         nchunks = (total + chunk - 1) / chunk;
     }
     if (A.stats && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(A.stats + 2, (unsigned long long)total);

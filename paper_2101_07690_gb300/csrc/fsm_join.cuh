@@ -32,12 +32,16 @@
 // One launch on a GB300 (same graph and output): the extension kernel before, this kernel with a
 // key table per block in shared memory (flushed between chunks) and both new vertices' tests made
 // per survivor, and as it is:
-//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms,  77.7 ms,  30.5 ms
-//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   140 ms
-//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,  11.8 ms
-//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   6.3 ms
+//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms,  77.7 ms,  24.2 ms
+//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   126 ms
+//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,   9.7 ms
+//   5 -> 7, count, ST 8 quotas, 6.0e8 pieces, 1.2e8 joins:          248 ms,  60.6 ms,  24.9 ms
+//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   4.9 ms
 // The block tables missed 70 to 77 % of the lookups of levels 1 and 2, and their flushes made warps
-// wait for each other; a record read at the L2 costs each join one latency and no barrier.
+// wait for each other; a record read at the L2 costs each join one latency and no barrier.  What is
+// left is bound by scattered requests (2 -> 4: load-store unit 66 %, L2 58 % busy) and, where the body
+// is large, by instruction fetch: one copy of the joins (take) instead of two took 5 -> 7 from 55 to
+// 35 ms.
 #pragma once
 #include "fsm_extend.cuh"
 
@@ -106,8 +110,8 @@ FSM_HD bool join_accepted(int cls, int form, int sa, int sb, int bgt, uint32_t s
 
 // survivors of the filter wait here until 32 are there
 #define FSM_JOIN_QUEUE 64
-// shared words per warp for the Bloom filters of a batch of units
-#define FSM_JOIN_BLOOM 512
+// per warp: key slots whose bits of s the batch's units have set (see accept)
+#define FSM_JOIN_SEEN 128
 
 // A queued candidate, and a row's part of it, in one word: unit j (4 bits), end list (1), slot of the
 // anchor (3) and of the partner (3), and of the anchor its label (6), cross edges to the other
@@ -123,7 +127,12 @@ FSM_HD bool join_accepted(int cls, int form, int sa, int sb, int bgt, uint32_t s
 // A batch's units in shared memory: UW words each.
 template <int L, bool QUOTA> struct UnitRec {
     static constexpr int O = L - 1;
-    static constexpr int U = L <= 3 ? 16 : 8;        // units per batch
+    // Units per batch and shared words per warp for their Bloom filters (L lists each).  8 units against
+    // 16: 3 -> 5 one pass 25.5 and 26.8 ms, 2 -> 4 one pass 127 and 131 ms, 1 -> 3 count 6.3 and 6.1
+    // ms; 4 units against 8: 5 -> 7 count 38.8 and 35.2 ms.  Twice the words cost more L1 than the
+    // searches they save (3 -> 5 one pass 28.2 ms).
+    static constexpr int U = L == 1 ? 16 : 8;
+    static constexpr int BLOOM = L <= 3 ? 256 : 512;
     static constexpr int RP = 0, D = 1, PID = 2, META = 3, CLS = 4, OLAB = 5, OPP = 6, SEG = 7, SLO = 8, RLO = 9,
                          RHI = 11, NC = 13, SS = 15, BND = SS + L, RK = BND + L, OB = RK + L, OE = OB + O, OK = OE + O,
                          VB = OK + 6 * O, VE = VB + 1, QA = VE + 1, END = QA + (QUOTA ? 6 : 0);
@@ -133,9 +142,11 @@ template <int L, bool QUOTA> struct UnitRec {
 template <int L, int PASS, bool QUOTA> struct JoinSmem {
     using R = UnitRec<L, QUOTA>;
     uint32_t unit[8][R::U * R::UW];
-    uint32_t bloom[8][FSM_JOIN_BLOOM];
+    uint32_t bloom[8][R::BLOOM];
     uint32_t q_anchor[8][FSM_JOIN_QUEUE], q_partner[8][FSM_JOIN_QUEUE], q_meta[8][FSM_JOIN_QUEUE];
-    uint32_t sg_base[8][32], sg_anchor[8][32], sg_slots[8][32], sg_meta[8][32];
+    uint32_t q_rank[8][FSM_JOIN_QUEUE];              // the anchor's rank
+    uint32_t sg_base[8][32], sg_anchor[8][32], sg_slots[8][32], sg_meta[8][32], sg_rank[8][32];
+    uint32_t seen[8][PASS == PASS_FUSED || PASS == PASS_DOMAIN ? FSM_JOIN_SEEN : 1];
 };
 
 __device__ __forceinline__ int32_t sorted_has(const int32_t *col, int32_t lo, int32_t end, int32_t x) {
@@ -271,40 +282,37 @@ static __device__ __noinline__ void resolve_slot(const ResolveArgs A, int64_t sl
     st_relaxed_u32(kr + 1, (uint32_t)(key >> 32));
 }
 
-// Four words of a key record: read-only in the domain pass, read at the L2 in the one-pass level
-// (an old empty copy in L1 would send its readers to the slow path until it is evicted).
-template <int PASS> __device__ __forceinline__ void ld_rec4(const uint32_t *p, uint32_t *x) {
-    if (PASS == PASS_DOMAIN) {
-        const uint4 v = __ldg((const uint4 *)p);
-        x[0] = v.x; x[1] = v.y; x[2] = v.z; x[3] = v.w;
-    } else {
-        asm volatile("ld.global.cg.v4.u32 {%0, %1, %2, %3}, [%4];"
-                     : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "l"(p) : "memory");
-    }
+// Eight words of a key record in one request: read-only in the domain pass, read at the L2 in the
+// one-pass level (an old empty copy in L1 would send its readers to the slow path until it is
+// evicted).  A join's scattered requests are what the load-store unit is busy with.
+template <int PASS> __device__ __forceinline__ void ld_rec8(const uint32_t *p, uint32_t *x) {
+    if (PASS == PASS_DOMAIN)
+        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]) : "l"(p));
+    else
+        asm volatile("ld.relaxed.gpu.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                     : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7])
+                     : "l"(p) : "memory");
 }
 
-// First sight of a key (or a record this SM's L1 still holds empty): insert the key, publish its
-// record if nobody has, and read it at the L2.  False when a table or the pool is full (the error
-// word says so).
+// First sight of a key: insert it and publish its record if nobody has.  Its slot, or -1 when a
+// table or the pool is full (the error word says so).
 template <int K>
-__device__ __noinline__ bool first_sight(const ExtArgs &A, uint64_t key, int64_t &slot, uint32_t *off) {
-    slot = qp_insert(A.qp, key, A.err);
-    if (slot < 0) return false;
+__device__ __noinline__ int64_t first_sight(const ExtArgs &A, uint64_t key) {
+    const int64_t slot = qp_insert(A.qp, key, A.err);
+    if (slot < 0) return -1;
     const uint32_t *kr = A.key_rec + slot * key_rec_words(K);
     for (int round = 0; round < 2; ++round) {
         bool all = true;
-        for (int h = 0; h < K; ++h) {
-            off[h] = ld_relaxed_u32(kr + 2 + h);
-            all &= off[h] != FSM_OFF_NONE;
-        }
-        if (all) return true;
+        for (int h = 0; h < K; ++h) all &= ld_relaxed_u32(kr + 2 + h) != FSM_OFF_NONE;
+        if (all) return slot;
         if (round == 0) {
             const ResolveArgs R{A.pat_lab, A.pat_adj, A.cls_size, A.code_keys, A.code_off, A.pool_top,
                                 A.code_mask, A.pool_words, A.key_rec, A.off_shift, A.err, A.explore, A.level};
             resolve_slot(R, slot, key);
         }
     }
-    return false;
+    return -1;
 }
 
 template <int L, int PASS, bool QUOTA>
@@ -338,18 +346,17 @@ struct Joiner {
         return (sm.bloom[w][((j * L + t) << (lb - 5)) + (h >> 5)] >> (h & 31)) & 1u;
     }
 
-    // Slot and bitmap offsets of a key from its record; false where the key has none (domain pass:
-    // an error), the record is not there yet, or a table is full.
+    // Slot and bitmap offsets of a key from its record, looked for from `slot` (from its hash if that
+    // is negative) on; false where the key has no bitmaps or the record is not there yet.
     __device__ __forceinline__ bool key_record(uint64_t key, int64_t &slot, uint32_t (&off)[K]) {
-        uint64_t h = mix64(key) & A.qp.mask;
+        uint64_t h = slot >= 0 ? (uint64_t)slot : mix64(key) & A.qp.mask;
         constexpr int RW = key_rec_words(K);
 #pragma unroll 1
         for (int p = 0; p < FSM_MAX_PROBES; ++p) {
             const uint32_t *kr = A.key_rec + h * RW;
-            uint32_t wd[12];
-            ld_rec4<PASS>(kr, wd);
-            ld_rec4<PASS>(kr + 4, wd + 4);
-            if (K > 6) ld_rec4<PASS>(kr + 8, wd + 8);
+            uint32_t wd[K > 6 ? 16 : 8];
+            ld_rec8<PASS>(kr, wd);
+            if (K > 6) ld_rec8<PASS>(kr + 8, wd + (K > 6 ? 8 : 0));
             const uint64_t k = (uint64_t)wd[0] | ((uint64_t)wd[1] << 32);
             if (k == key) {
                 bool all = true;
@@ -367,7 +374,9 @@ struct Joiner {
         return false;
     }
 
-    __device__ __forceinline__ void set_bits(const uint32_t (&off)[K], const uint32_t *r, uint32_t ra, uint32_t rb, bool swap) {
+    // Bits of the join's vertices; those of s (the first L positions) only when `own` is set.
+    __device__ __forceinline__ void set_bits(const uint32_t (&off)[K], const uint32_t *r, uint32_t ra, uint32_t rb, bool swap,
+                                             bool own) {
         uint32_t *base = PASS == PASS_DOMAIN ? A.dom : A.pool;
         uint32_t *wd[K];
         uint32_t bit[K], old[K];
@@ -376,37 +385,46 @@ struct Joiner {
             const uint32_t rk = h < L ? r[R::RK + (h < L ? h : 0)] : ((h == L) != swap ? ra : rb);
             wd[h] = base + ((uint64_t)off[h] << A.off_shift) + (rk >> 5);
             bit[h] = 1u << (rk & 31);
+            old[h] = 0u;
         }
         // A reduction nothing waits for, except on small label classes (ExtArgs::check_bits), whose few
         // words many joins would queue on: there most bits are set already and a read finds that.
         if (A.check_bits) {
 #pragma unroll
-            for (int h = 0; h < K; ++h) old[h] = __ldcg(wd[h]);
-#pragma unroll
             for (int h = 0; h < K; ++h)
-                if (!(old[h] & bit[h])) atomicOr(wd[h], bit[h]);
-        } else {
-#pragma unroll
-            for (int h = 0; h < K; ++h) atomicOr(wd[h], bit[h]);
+                if (h >= L || own) old[h] = __ldcg(wd[h]);
         }
+#pragma unroll
+        for (int h = 0; h < K; ++h)
+            if ((h >= L || own) && !(old[h] & bit[h])) atomicOr(wd[h], bit[h]);
     }
 
     // One accepted join of this lane (not warp-synchronous).
-    __device__ __forceinline__ void accept(const uint32_t *r, uint64_t key, bool centre, int32_t anchor, int32_t x,
-                                           uint32_t rx, bool swap) {
+    __device__ __forceinline__ void accept(const uint32_t *r, int j, uint64_t key, bool centre, int32_t anchor, int32_t x,
+                                           uint32_t ranchor, uint32_t rx, bool swap) {
         if constexpr (PASS == PASS_COUNT) {
             const int64_t slot = qp_insert(A.qp, key, A.err);
             if (slot >= 0) atomicAdd(A.qp.count + slot, 1ull);
         } else if constexpr (PASS == PASS_FUSED || PASS == PASS_DOMAIN) {
             uint32_t off[K];
-            int64_t slot;
-            if (!key_record(key, slot, off)) {
+            int64_t slot = -1;
+            while (!key_record(key, slot, off)) {
                 if (PASS == PASS_DOMAIN) return;   // pattern without bitmaps
-                if (!first_sight<K>(A, key, slot, off)) return;
+                slot = first_sight<K>(A, key);     // published now, so the next look finds it
+                if (slot < 0) return;
             }
             if (PASS == PASS_FUSED) atomicAdd(A.qp.count + slot, 1ull);
-            const uint32_t ranchor = (uint32_t)__ldg(A.g.vinfo + anchor).w;
-            set_bits(off, r, centre ? rx : ranchor, centre ? ranchor : rx, swap);
+            // A unit's joins of one key set the same bits of s: a small table of (unit, slot) pairs
+            // already seen in this batch keeps most of those reductions away.  A lost entry or a race
+            // only repeats them.
+            const uint32_t tag = (uint32_t)slot * 16u + (uint32_t)j;
+            bool own = slot >= (1 << 28) - 1;      // such slots do not fit the tag
+            if (!own) {
+                uint32_t *sn = &sm.seen[w][(tag ^ (tag >> 7)) & (FSM_JOIN_SEEN - 1)];
+                own = *(volatile uint32_t *)sn != tag;
+                if (own) *(volatile uint32_t *)sn = tag;
+            }
+            set_bits(off, r, centre ? rx : ranchor, centre ? ranchor : rx, swap, own);
         } else {
             const int64_t slot = qp_find(A.qp, key);
             if (slot < 0) { atomicOr(A.err, FSM_ERR_QP_MISSING); return; }
@@ -488,7 +506,12 @@ struct Joiner {
         const int32_t v = (int32_t)r[R::SS + rv];
         const int4 ix = __ldg(A.g.vinfo + x);
         const int lx = ix.z;
-        if (QUOTA) m |= anchor_meta(r, j, anchor, __ldg(A.g.vinfo + anchor).z);
+        uint32_t ranchor = QUOTA ? 0u : sm.q_rank[w][q];
+        if (QUOTA) {
+            const int4 ia = __ldg(A.g.vinfo + anchor);
+            ranchor = (uint32_t)ia.w;
+            m |= anchor_meta(r, j, anchor, ia.z);
+        }
         const int la = (m >> FSM_M_LAB) & 63;
         // bits of the anchor and of the partner in a cross subset: a's low, b's high
         const int sh_a = centre ? O : 0, sh_x = centre ? 0 : O;
@@ -611,24 +634,26 @@ struct Joiner {
                     cross |= ((sub >> o) & 1u) << (2 * pp + (swap ? 1 : 0));
                     cross |= ((sub >> (O + o)) & 1u) << (2 * pp + (swap ? 0 : 1));
                 }
-                accept(r, make_key(r[R::PID], pidx, ki, jpos, cross, L), centre, anchor, x, (uint32_t)ix.w, swap);
+                accept(r, j, make_key(r[R::PID], pidx, ki, jpos, cross, L), centre, anchor, x, ranchor, (uint32_t)ix.w, swap);
             }
         }
         qn -= n;
         __syncwarp();
     }
 
-    // warp-synchronous: queue the survivors among the lanes' candidates, joining when 32 wait
-    __device__ __forceinline__ void push(bool ok, int32_t anchor, int32_t x, uint32_t m) {
+    // warp-synchronous: queue the survivors among the lanes' candidates; join when 32 wait, or what
+    // there is when nothing more comes (`drain`)
+    __device__ __forceinline__ void push(bool ok, int32_t anchor, int32_t x, uint32_t m, uint32_t ranchor, bool drain) {
         const unsigned bal = __ballot_sync(0xffffffffu, ok);
         if (ok) {
             const int p = qn + __popc(bal & ((1u << lane) - 1u));
             sm.q_anchor[w][p] = (uint32_t)anchor;
             sm.q_partner[w][p] = (uint32_t)x;
             sm.q_meta[w][p] = m;
+            if (!QUOTA) sm.q_rank[w][p] = ranchor;
         }
         qn += __popc(bal);
-        if (qn >= 32) take(32);
+        if (qn >= 32 || (drain && qn > 0)) take(min(qn, 32));
     }
 
     // Load units u0 .. u0 + nu - 1 (raw candidate range [q0, q1) of the chunk) into shared memory.
@@ -710,9 +735,9 @@ struct Joiner {
             }
             r[R::OPP] = opp;
             int32_t cpos = d;
-#pragma unroll
+#pragma unroll 1
             for (int t = 0; t < L; ++t) {
-                const int32_t bd = below(g.pcol + rp, d, id[t]);
+                const int32_t bd = below(g.pcol + rp, d, (int32_t)r[R::SS + t]);
                 r[R::BND + t] = (uint32_t)bd;
                 if (L == 2 && t != rv) cpos = bd;
             }
@@ -759,15 +784,17 @@ struct Joiner {
         total_seg = __shfl_sync(0xffffffffu, inc, 31);
         // Bloom filters of the lists of s (of the key vertex only where end pieces are tested for
         // closing a triangle)
-        int bw = FSM_JOIN_BLOOM / (nu * L);
+        int bw = R::BLOOM / (nu * L);
         lb = 5 + (31 - __clz(bw));
         __syncwarp();
-        for (int x = lane; x < FSM_JOIN_BLOOM; x += 32) sm.bloom[w][x] = 0u;
+        for (int x = lane; x < R::BLOOM; x += 32) sm.bloom[w][x] = 0u;
+        if (PASS == PASS_FUSED || PASS == PASS_DOMAIN)
+            for (int x = lane; x < FSM_JOIN_SEEN; x += 32) sm.seen[w][x] = 0xFFFFFFFFu;
         __syncwarp();
         for (int j = 0; j < nu; ++j) {
             const uint32_t *rj = rec(j);
             const int rv = (rj[R::META] >> 3) & 7;
-#pragma unroll
+#pragma unroll 1
             for (int t = 0; t < L; ++t) {
                 int32_t x0, x1;
                 if (t == rv) {
@@ -806,7 +833,8 @@ struct Joiner {
     // The candidates of the loaded units, row by row.
     __device__ __forceinline__ void walk(int nu) {
         const DevGraph &g = A.g;
-        for (int g0 = 0; g0 < total_seg; g0 += 32) {
+        for (int g0 = 0;; g0 += 32) {
+            const bool drain = g0 >= total_seg;   // one round more joins what is left in the queue
             int len = 0;
             const int gi = g0 + lane;
             if (gi < total_seg) {
@@ -873,6 +901,7 @@ struct Joiner {
                         sm.sg_anchor[w][lane] = (uint32_t)anchor;
                         sm.sg_slots[w][lane] = ok;
                         sm.sg_meta[w][lane] = m;
+                        sm.sg_rank[w][lane] = (uint32_t)ia.w;
                     }
                 }
             }
@@ -886,7 +915,7 @@ struct Joiner {
             __syncwarp();
             sm.sg_base[w][lane] -= (uint32_t)(inc - len);   // list index of candidate t is base + t
             __syncwarp();
-            for (int t0 = 0; t0 < total; t0 += 32) {
+            for (int t0 = 0; t0 < total || (drain && t0 == 0); t0 += 32) {
                 const int t = t0 + lane;
                 int k = 0;
 #pragma unroll
@@ -894,8 +923,9 @@ struct Joiner {
                     if (__shfl_sync(0xffffffffu, inc, k + s - 1) <= t) k += s;
                 bool ok = t < total;
                 int32_t x = 0, anchor = 0;
-                uint32_t m = 0;
+                uint32_t m = 0, ranchor = 0;
                 if (ok) {
+                    ranchor = sm.sg_rank[w][k];
                     m = sm.sg_meta[w][k];
                     anchor = (int32_t)sm.sg_anchor[w][k];
                     const int64_t at = (int64_t)(int32_t)(sm.sg_base[w][k] + (uint32_t)t);
@@ -916,16 +946,18 @@ struct Joiner {
                         ok &= (sm.sg_slots[w][k] >> (s + (x > anchor ? SL : 0))) & 1u;
                     }
                 }
-                push(ok, anchor, x, m);
+                push(ok, anchor, x, m, ranchor, drain);
             }
             __syncwarp();
+            if (drain) break;
         }
     }
 
     // Quota variant: the drawn candidates of the loaded units, by their numbers.
     __device__ __forceinline__ void walk_quota(int nu) {
         const DevGraph &g = A.g;
-        for (int g0 = 0; g0 < total_seg; g0 += 32) {
+        for (int g0 = 0;; g0 += 32) {
+            const bool drain = g0 >= total_seg;
             const int gi = g0 + lane;
             bool ok = gi < total_seg;
             int32_t anchor = 0, x = 0;
@@ -966,14 +998,23 @@ struct Joiner {
                 if (ok) ok = (allowed(r, centre, s) >> (sx + (x > anchor ? SL : 0))) & 1u;
                 m = (uint32_t)j | ((centre ? 0u : 1u) << FSM_M_END) | ((uint32_t)s << FSM_M_SA) | ((uint32_t)sx << FSM_M_SP);
             }
-            push(ok, anchor, x, m);
+            push(ok, anchor, x, m, 0u, drain);
+            if (drain) break;
         }
     }
 
 };
 
+// Resident blocks per SM: four (64 registers) hide more latency in the count and emission passes
+// (3.7M vertices, 1 -> 3: 5.2 ms against 6.1 ms with three) and in the domain pass up to l = 4 (13.3
+// and 13.9 ms); the one-pass level and the domain pass of l = 5 spill too much at 64 registers (2 -> 4
+// one pass: 157 and 131 ms).
+template <int L, int PASS> struct JoinBlocks {
+    static constexpr int value = PASS == PASS_FUSED || (PASS == PASS_DOMAIN && L == 5) ? 3 : 4;
+};
+
 template <int L, int PASS, bool QUOTA>
-__global__ void __launch_bounds__(256, 3) join_kernel(const __grid_constant__ ExtArgs A) {
+__global__ void __launch_bounds__(256, JoinBlocks<L, PASS>::value) join_kernel(const __grid_constant__ ExtArgs A) {
     extern __shared__ __align__(16) unsigned char join_smem[];
     using J = Joiner<L, PASS, QUOTA>;
     typename J::SM &sm = *reinterpret_cast<typename J::SM *>(join_smem);
@@ -984,7 +1025,7 @@ __global__ void __launch_bounds__(256, 3) join_kernel(const __grid_constant__ Ex
     if (total < 0) {
         // device-resident size: no host round trip between the prefix sum and this launch
         total = __ldg(A.unit_base + nunits);
-        if (chunk <= 0) chunk = join_chunk(total, nunits, (int64_t)gridDim.x * (blockDim.x >> 5));
+        if (chunk <= 0) chunk = join_chunk(total, (int64_t)gridDim.x * (blockDim.x >> 5));
         nchunks = (total + chunk - 1) / chunk;
     }
     int64_t stride = 1;
@@ -1018,7 +1059,6 @@ __global__ void __launch_bounds__(256, 3) join_kernel(const __grid_constant__ Ex
             const int nu = (int)min((int64_t)J::R::U, uhi - u + 1);
             jn.load_units(u, nu, q0, q1);
             if constexpr (QUOTA) jn.walk_quota(nu); else jn.walk(nu);
-            if (jn.qn > 0) jn.take(jn.qn);
         }
     }
 
@@ -1032,17 +1072,6 @@ __global__ void __launch_bounds__(256, 3) join_kernel(const __grid_constant__ Ex
     if (lane == 0 && A.stats) {
         atomicAdd(A.stats + 0, t0);
         atomicAdd(A.stats + 1, t1);
-    }
-}
-
-// Publish the record of every key in the table (after a warm pass): one thread per slot, so that
-// canonicalising runs with full warps.
-static __global__ void resolve_keys_kernel(const ExtArgs A) {
-    const ResolveArgs R{A.pat_lab, A.pat_adj, A.cls_size, A.code_keys, A.code_off, A.pool_top,
-                        A.code_mask, A.pool_words, A.key_rec, A.off_shift, A.err, A.explore, A.level};
-    for (uint64_t s = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; s <= A.qp.mask; s += (uint64_t)gridDim.x * blockDim.x) {
-        const unsigned long long key = A.qp.keys[s];
-        if (key != FSM_EMPTY_KEY) resolve_slot(R, (int64_t)s, key);
     }
 }
 
