@@ -727,6 +727,36 @@ cudaError_t launch_gather_frequent(int K, const int32_t *newid, int64_t np, cons
     return cudaGetLastError();
 }
 
+namespace {
+// one pattern per thread: canonical labels and the two adjacency encodings of the result
+__global__ void decode_patterns_kernel(int K, const unsigned long long *lab, const uint64_t *code, int64_t n,
+                                       int32_t *labels, uint64_t *adj, uint64_t *pairs) {
+    const int np = K * (K - 1) / 2;
+    for (int64_t p = gtid(); p < n; p += gstride()) {
+        for (int c = 0; c < K; ++c) labels[p * K + c] = clab_get(lab[p], c);
+        const uint64_t w = code[p];
+        uint64_t bits = 0, pr = 0;
+        int q = 0;
+        for (int i = 0; i < K; ++i)
+            for (int j = i + 1; j < K; ++j, ++q)
+                if ((w >> (np - 1 - q)) & 1ull) {
+                    if (K <= 8) bits |= 1ull << (i * K + j);
+                    pr |= 1ull << q;
+                }
+        adj[p] = bits;
+        pairs[p] = pr;
+    }
+}
+} // namespace
+
+cudaError_t launch_decode_patterns(int K, const unsigned long long *lab, const uint64_t *code, int64_t n,
+                                   int32_t *labels, uint64_t *adj, uint64_t *pairs, cudaStream_t st) {
+    if (n <= 0) return cudaSuccess;
+    LAUNCHED(1);
+    decode_patterns_kernel<<<blocks_for(n), kThreads, 0, st>>>(K, lab, code, n, labels, adj, pairs);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_sum_frequent(const int32_t *newid, const unsigned long long *pat_count, int64_t np,
                                 unsigned long long *sum, cudaStream_t st) {
     if (np <= 0) return cudaSuccess;

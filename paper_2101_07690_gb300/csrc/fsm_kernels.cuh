@@ -205,6 +205,10 @@ cudaError_t launch_slot_bases(int K, const int64_t *slots, int64_t nq, const int
                               const int64_t *dom_off, int shift, int64_t *slot_base, const unsigned long long *keys,
                               uint32_t *key_rec, int rec_words, cudaStream_t st);
 
+// ---- results: canonical labels [n * K], bit (i * K + j) words (0 for K = 9) and pair-bit words
+cudaError_t launch_decode_patterns(int K, const unsigned long long *lab, const uint64_t *code, int64_t n,
+                                   int32_t *labels, uint64_t *adj, uint64_t *pairs, cudaStream_t st);
+
 // ---- pieces: mark the frequent size-3 patterns by piece index
 cudaError_t launch_piece_table(const unsigned long long *lab, const uint64_t *adj, int64_t n,
                                uint8_t *piece_freq, cudaStream_t st);
