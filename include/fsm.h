@@ -128,8 +128,9 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
  *                still reach t (default).  Identical results; when the bitmap pool or the pattern
  *                table runs out, the level is counted again and finished in two passes (stat
  *                "fused_fallbacks").
- *   "fused_pool" size in 32-bit words of the one-pass level's bitmap pool (0 = twice what the
- *                previous call used, else 40% of the free device memory).
+ *   "fused_pool" size in 32-bit words of the one-pass level's bitmap pool (0 = twice what a sample of
+ *                the level or the previous call needed, grown on demand up to 40% of the free device
+ *                memory).
  *   "seed"       64-bit seed of the piece sampling of fsm_mine with sample_rate < 1 (default 0).
  *   "candidates" 1 = sampled mining returns every candidate pattern of the sampled level with
  *                its estimated support (smallest orbit popcount / p) and its 32 features

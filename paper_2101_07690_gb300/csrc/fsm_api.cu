@@ -597,24 +597,17 @@ struct Miner {
         int shift = 0;   // bitmap offsets are 32-bit, in units of 1 << shift words
         unsigned long long pool_words = 0;
         bool fused = final && G->fused && V == FSM_EXPLORE_TV && !sampled && K <= 7;
+        // Bitmap pool of the one-pass level.  Offsets are given out up to pool_words; the memory is
+        // allocated once the warm pass has shown what most keys need, twice that (the first call on a
+        // graph used to take and clear 40% of the free memory: 12 ms).  Up to 2^32 words offsets count
+        // single words; a level that needs more starts again with a larger shift.
+        unsigned long long pool_limit = 0, pool_min = 0;
         if (fused) {
             size_t fr = 0, tot = 0;
             ck(cudaMemGetInfo(&fr, &tot), "memory info");
-            // twice what the last call needed, else 40% of the free memory
-            const unsigned long long cap_words = (unsigned long long)(fr / 4 * 2 / 5);
-            pool_words = G->pool_hint[L] ? std::min(cap_words, 2 * G->pool_hint[L] + (1ull << 22)) : cap_words;
-            pool_words = std::max<unsigned long long>(pool_words, 1ull << 20);
-            if (G->pool_force) pool_words = G->pool_force;
-            void *pp = nullptr;
-            if (cudaMallocAsync(&pp, pool_words * 4, st) != cudaSuccess) {
-                cudaGetLastError();
-                fused = false;   // no room for the pool: separate count and domain passes
-            } else {
-                pool = (uint32_t *)pp;
-                mem.ptrs.push_back(pp);
-                ptop = mem.get<unsigned long long>(1);
-                while ((pool_words >> shift) >= 0xFFFFFFFEull) ++shift;
-            }
+            pool_limit = std::max<unsigned long long>(1ull << 20, (unsigned long long)(fr / 4 * 2 / 5));   // 40% of it
+            pool_min = std::min(pool_limit, 2 * G->pool_hint[L] + (1ull << 22));
+            ptop = mem.get<unsigned long long>(1);
         }
         auto release_pass1 = [&]() {
             for (void *q : {(void *)keys, (void *)qcount, (void *)used, (void *)ckeys, (void *)coff, (void *)krec})
@@ -632,7 +625,6 @@ struct Miner {
                 ck(launch_fill_u64(ckeys, FSM_EMPTY_KEY, cap, st), "fill");
                 ck(cudaMemsetAsync(coff, 0, sizeof(unsigned long long) * cap, st), "memset");
                 ck(cudaMemsetAsync(krec, 0xff, sizeof(uint32_t) * cap * rec_words, st), "memset");
-                ck(cudaMemsetAsync(pool, 0, pool_words * 4, st), "memset");
                 ck(cudaMemsetAsync(ptop, 0, sizeof(unsigned long long), st), "memset");
             }
         };
@@ -646,13 +638,15 @@ struct Miner {
                 ckeys = mem.get<unsigned long long>(cap);
                 coff = mem.get<unsigned long long>(cap);
                 krec = mem.get<uint32_t>(cap * rec_words);
+                pool_words = G->pool_force ? G->pool_force
+                                           : std::min(pool_limit, std::max<unsigned long long>(pool_min, 0xFFFFFFFDull));
+                for (shift = 0; (pool_words >> shift) >= 0xFFFFFFFEull;) ++shift;
                 A.pat_lab = in.lab8;
                 A.code_keys = ckeys;
                 A.code_off = coff;
                 A.code_mask = (uint64_t)cap - 1;
                 A.key_rec = krec;
                 A.off_shift = shift;
-                A.pool = pool;
                 A.pool_top = ptop;
                 A.pool_words = pool_words;
                 A.cls_size = G->cls_size;
@@ -684,10 +678,34 @@ struct Miner {
                 ck(launch_resolve_keys(W, G->sms, st), "resolve keys");
                 rs.launches += 1;
                 ck(cudaMemsetAsync(qcount, 0, sizeof(unsigned long long) * cap, st), "memset");
+                const unsigned long long want = 2 * d2h(ptop, st) + (1ull << 22);
+                if (!G->pool_force && want > pool_words && pool_words < pool_limit) {
+                    pool_min = want;
+                    release_pass1();
+                    continue;
+                }
+                if (!G->pool_force) pool_words = std::min(pool_words, std::max(want, pool_min));
+                A.pool_words = pool_words;
+                void *pp = nullptr;
+                if (cudaMallocAsync(&pp, pool_words * 4, st) != cudaSuccess) {
+                    cudaGetLastError();
+                    fused = false;   // no room for the pool: separate count and domain passes
+                    shift = 0;
+                    release_pass1();
+                    continue;
+                }
+                pool = (uint32_t *)pp;
+                mem.ptrs.push_back(pp);
+                A.pool = pool;
+                ck(cudaMemsetAsync(pool, 0, pool_words * 4, st), "memset");
             }
             run_pass(fused ? PASS_FUSED : PASS_COUNT, in, A, pat_off);
             const int ew = err_word();
             if (ew & (FSM_ERR_TIMEOUT | FSM_ERR_BOUNDS)) fail_word(ew);
+            if (ew && pool) {
+                mem.release(pool);
+                pool = nullptr;
+            }
             if (ew & FSM_ERR_QP_OVERFLOW) {
                 release_pass1();
                 if (cap >= ((int64_t)1 << 31)) fail(FSM_EUNSUPPORTED, "more than 2^30 distinct quick patterns in one level");
@@ -697,8 +715,14 @@ struct Miner {
             }
             if (ew & ~(FSM_ERR_POOL | FSM_ERR_CODE_FULL)) fail_word(ew);
             if (ew) {
-                // pool or pattern table too small: the one-pass level stopped early; count again
-                // in a clean count pass and fill the domains in a domain pass
+                // pool or pattern table too small: the one-pass level stopped early.  A pool that was
+                // not the largest allowed grows; else count again in a clean count pass and fill the
+                // domains in a domain pass
+                if (!(ew & FSM_ERR_CODE_FULL) && !G->pool_force && pool_words < pool_limit) {
+                    pool_min = 4 * pool_words;
+                    release_pass1();
+                    continue;
+                }
                 fused = false;
                 shift = 0;
                 G->pool_hint[L] = 0;
