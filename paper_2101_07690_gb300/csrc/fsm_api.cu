@@ -176,6 +176,7 @@ struct fsm_graph {
     uint32_t *join_acc[FSM_JOIN_MAXL + 1] = {};
     uint16_t *join_any[FSM_JOIN_MAXL + 1] = {};
     int4 *vinfo = nullptr;
+    uint32_t *linfo = nullptr;
     int32_t *row_ptr = nullptr, *col = nullptr, *labels = nullptr, *rank = nullptr, *cls_size = nullptr,
             *end_off = nullptr;
     int64_t *piece_cnt = nullptr;
@@ -198,6 +199,8 @@ struct fsm_graph {
         g.pend = end_off;
         g.ppc = piece_cnt;
         g.vinfo = vinfo;
+        g.pinfo = linfo;
+        g.packed = n < (1 << 26);
         g.tri_off = tri_off;
         g.tri_bits = tri_bits;
         return g;
@@ -573,11 +576,13 @@ struct Miner {
             int32_t *prow = mem.get<int32_t>(G->n + 1);
             int32_t *pcol = mem.get<int32_t>(std::max<int64_t>(kept, 1));
             int32_t *pend = mem.get<int32_t>(std::max<int64_t>(kept, 1));
+            uint32_t *pinfo = mem.get<uint32_t>(std::max<int64_t>(kept, 1));
             int64_t *ppc = mem.get<int64_t>(G->n);
-            ck(launch_sample_lists(A.g, G->seed, thr, prow64, prow, pcol, pend, ppc, st), "sample lists");
+            ck(launch_sample_lists(A.g, G->seed, thr, prow64, prow, pcol, pinfo, pend, ppc, st), "sample lists");
             A.g.prow = prow;
             A.g.pcol = pcol;
             A.g.pend = pend;
+            A.g.pinfo = pinfo;
             A.g.ppc = ppc;
             A.g.tri_off = nullptr;   // the matrices index the full lists
             A.g.tri_bits = nullptr;
@@ -1212,6 +1217,7 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
         dalloc((void **)&g->labels, sizeof(int32_t) * n);
         dalloc((void **)&g->rank, sizeof(int32_t) * n);
         dalloc((void **)&g->vinfo, sizeof(int4) * n);
+        dalloc((void **)&g->linfo, sizeof(uint32_t) * nnz);
         dalloc((void **)&g->cls_size, sizeof(int32_t) * 64);
         dalloc((void **)&g->end_off, sizeof(int32_t) * nnz);
         dalloc((void **)&g->piece_cnt, sizeof(int64_t) * n);
@@ -1226,6 +1232,7 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
         const int ew = d2h(g->err, st);
         if (ew) fail(FSM_EINVAL, "malformed CSR: rows must be sorted, symmetric, without self-loops or duplicates, labels in range");
         ck(launch_prepare(g->dg(), g->piece_cnt, g->end_off, g->rank, g->cls_size, g->vinfo, st), "prepare");
+        ck(launch_list_info(g->dg(), g->linfo, st), "list labels");
         {
             // Neighbour-adjacency matrices for the triangle test of centre pairs, for vertices
             // of degree >= dmin; dmin doubles until they fit the budget.
@@ -1577,7 +1584,7 @@ void fsm_free_graph(fsm_graph *g) {
     if (!g) return;
     cudaStream_t st = g->stream ? g->stream : g->own_stream;
     void *ps[] = {g->row_ptr, g->col, g->labels, g->rank, g->cls_size, g->end_off, g->piece_cnt, g->tri_off, g->tri_bits, g->err, g->stats,
-                  g->by_rank, g->cls_off, g->vinfo};
+                  g->by_rank, g->cls_off, g->vinfo, g->linfo};
     for (void *p : ps)
         if (p) cudaFreeAsync(p, st);
     for (int L = 0; L <= FSM_JOIN_MAXL; ++L) {

@@ -53,6 +53,9 @@ struct DevGraph {
     // adjacency tests always use row_ptr / col.
     const int32_t *prow, *pcol, *pend;
     const int64_t *ppc;
+    // per entry of pcol: label in the low 6 bits and, when `packed` (fewer than 2^26 vertices), rank above
+    const uint32_t *pinfo;
+    int packed;
     // per vertex {row_ptr[v], row_ptr[v+1], label, rank}: one 16-byte read where a join needs them all
     const int4 *vinfo;
     // Neighbour adjacency of high-degree vertices: for v with tri_off[v] >= 0, bit y of row x

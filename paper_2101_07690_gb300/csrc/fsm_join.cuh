@@ -19,9 +19,10 @@
 //              N(a)).  One lane prepares one row: the slots its anchor allows its partner cut the
 //              row to a range (a row with none costs nothing more), and the anchor's label, cross
 //              edges and pruning bits are found once for the whole row.
-//   filter     Lanes then walk the surviving ranges side by side: one coalesced list read, the
+//   filter     Lanes then walk the surviving ranges side by side: one coalesced list read (with the
+//              labels and ranks, which lie in an array beside the lists), the
 //              partner's slot by l comparisons, one bit test.  Survivors go to a per-warp queue.
-//   joins      Full warps take 32 survivors: labels and ranks (one 16-byte read per vertex), the
+//   joins      Full warps take 32 survivors: the
 //              size-3 frequency of the piece, cross edges (a shared-memory Bloom filter of each
 //              list of s, misses are certain, hits are verified by binary search), joining-point
 //              pruning (Section 4.5) as cross bits that must or must not be set, then the subsets
@@ -32,11 +33,11 @@
 // One launch on a GB300 (same graph and output): the extension kernel before, this kernel with a
 // key table per block in shared memory (flushed between chunks) and both new vertices' tests made
 // per survivor, and as it is:
-//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms,  77.7 ms,  24.2 ms
-//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   126 ms
-//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,   9.7 ms
-//   5 -> 7, count, ST 8 quotas, 6.0e8 pieces, 1.2e8 joins:          248 ms,  60.6 ms,  24.9 ms
-//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   4.9 ms
+//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms,  77.7 ms,  22.4 ms
+//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   123 ms
+//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,   9.6 ms
+//   5 -> 7, count, ST 8 quotas, 6.0e8 pieces, 1.2e8 joins:          248 ms,  60.6 ms,  25.3 ms
+//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   4.6 ms
 // The block tables missed 70 to 77 % of the lookups of levels 1 and 2, and their flushes made warps
 // wait for each other; a record read at the L2 costs each join one latency and no barrier.  What is
 // left is bound by scattered requests (2 -> 4: load-store unit 66 %, L2 58 % busy) and, where the body
@@ -114,15 +115,14 @@ FSM_HD bool join_accepted(int cls, int form, int sa, int sb, int bgt, uint32_t s
 #define FSM_JOIN_SEEN 128
 
 // A queued candidate, and a row's part of it, in one word: unit j (4 bits), end list (1), slot of the
-// anchor (3) and of the partner (3), and of the anchor its label (6), cross edges to the other
-// vertices of s (4), and the cross edges pruning asks of it (4) or forbids (4).
+// anchor (3) and of the partner (3), and of the anchor its cross edges to the other vertices of s
+// (4), and the cross edges pruning asks of it (4) or forbids (4).
 #define FSM_M_END 4
 #define FSM_M_SA 5
 #define FSM_M_SP 8
-#define FSM_M_LAB 11
-#define FSM_M_CROSS 17
-#define FSM_M_MUST 21
-#define FSM_M_NO 25
+#define FSM_M_CROSS 11
+#define FSM_M_MUST 15
+#define FSM_M_NO 19
 
 // A batch's units in shared memory: UW words each.
 template <int L, bool QUOTA> struct UnitRec {
@@ -144,8 +144,8 @@ template <int L, int PASS, bool QUOTA> struct JoinSmem {
     uint32_t unit[8][R::U * R::UW];
     uint32_t bloom[8][R::BLOOM];
     uint32_t q_anchor[8][FSM_JOIN_QUEUE], q_partner[8][FSM_JOIN_QUEUE], q_meta[8][FSM_JOIN_QUEUE];
-    uint32_t q_rank[8][FSM_JOIN_QUEUE];              // the anchor's rank
-    uint32_t sg_base[8][32], sg_anchor[8][32], sg_slots[8][32], sg_meta[8][32], sg_rank[8][32];
+    uint32_t q_ainfo[8][FSM_JOIN_QUEUE], q_xinfo[8][FSM_JOIN_QUEUE];   // DevGraph::pinfo of anchor, partner
+    uint32_t sg_base[8][32], sg_anchor[8][32], sg_slots[8][32], sg_meta[8][32], sg_info[8][32];
     uint32_t seen[8][PASS == PASS_FUSED || PASS == PASS_DOMAIN ? FSM_JOIN_SEEN : 1];
 };
 
@@ -326,7 +326,7 @@ struct Joiner {
     SM &sm;
     const int w, lane;
     int qn = 0;                       // survivors waiting
-    int lb = 5;                       // log2 bits of one Bloom filter of this batch
+    int lb = 0;                       // log2 words of one Bloom filter of this batch
     bool tfe;                         // triangles are made from end lists (see take)
     unsigned long long tested = 0, accepted = 0;
 
@@ -340,10 +340,13 @@ struct Joiner {
 
     __device__ __forceinline__ uint32_t *rec(int j) { return sm.unit[w] + j * R::UW; }
 
-    // x in the list of the t-th smallest vertex of unit j's s?  A clear Bloom bit is a certain no.
+    // Two bits of one word stand for a vertex in a Bloom filter: one read tests both (3
+    // -> 5 one pass: 23.3 ms with one bit, 22.4 with two).
+    __device__ __forceinline__ static uint32_t bloom_mask(uint32_t h) { return (1u << (h & 31)) | (1u << ((h >> 5) & 31)); }
+    // x in the list of the t-th smallest vertex of unit j's s?  A clear bit is a certain no.
     __device__ __forceinline__ bool maybe(int j, int t, int32_t x) const {
-        const uint32_t h = ((uint32_t)x * 0x9E3779B1u) >> (32 - lb);
-        return (sm.bloom[w][((j * L + t) << (lb - 5)) + (h >> 5)] >> (h & 31)) & 1u;
+        const uint32_t h = (uint32_t)x * 0x9E3779B1u, k = bloom_mask(h >> 7);
+        return (sm.bloom[w][((j * L + t) << lb) + (lb ? h >> (32 - lb) : 0u)] & k) == k;
     }
 
     // Slot and bitmap offsets of a key from its record, looked for from `slot` (from its hash if that
@@ -401,7 +404,7 @@ struct Joiner {
 
     // One accepted join of this lane (not warp-synchronous).
     __device__ __forceinline__ void accept(const uint32_t *r, int j, uint64_t key, bool centre, int32_t anchor, int32_t x,
-                                           uint32_t ranchor, uint32_t rx, bool swap) {
+                                           uint32_t ainfo, uint32_t xinfo, bool swap) {
         if constexpr (PASS == PASS_COUNT) {
             const int64_t slot = qp_insert(A.qp, key, A.err);
             if (slot >= 0) atomicAdd(A.qp.count + slot, 1ull);
@@ -424,6 +427,8 @@ struct Joiner {
                 own = *(volatile uint32_t *)sn != tag;
                 if (own) *(volatile uint32_t *)sn = tag;
             }
+            const uint32_t ranchor = A.g.packed ? ainfo >> 6 : (uint32_t)__ldg(A.g.rank + anchor);
+            const uint32_t rx = A.g.packed ? xinfo >> 6 : (uint32_t)__ldg(A.g.rank + x);
             set_bits(off, r, centre ? rx : ranchor, centre ? ranchor : rx, swap, own);
         } else {
             const int64_t slot = qp_find(A.qp, key);
@@ -487,8 +492,7 @@ struct Joiner {
             must = ~labels_ok(r, 0, lab) & all;
             no = ~labels_ok(r, 1, lab) & all;
         }
-        return ((uint32_t)lab << FSM_M_LAB) | (cross_of(r, j, rv, anchor, false) << FSM_M_CROSS) | (must << FSM_M_MUST) |
-               (no << FSM_M_NO);
+        return (cross_of(r, j, rv, anchor, false) << FSM_M_CROSS) | (must << FSM_M_MUST) | (no << FSM_M_NO);
     }
 
     // The last n (<= 32) survivors of the queue, one per lane; warp-synchronous.
@@ -504,15 +508,9 @@ struct Joiner {
         const uint32_t meta = r[R::META];
         const int ki = meta & 7, rv = (meta >> 3) & 7, lv = (meta >> 6) & 63;
         const int32_t v = (int32_t)r[R::SS + rv];
-        const int4 ix = __ldg(A.g.vinfo + x);
-        const int lx = ix.z;
-        uint32_t ranchor = QUOTA ? 0u : sm.q_rank[w][q];
-        if (QUOTA) {
-            const int4 ia = __ldg(A.g.vinfo + anchor);
-            ranchor = (uint32_t)ia.w;
-            m |= anchor_meta(r, j, anchor, ia.z);
-        }
-        const int la = (m >> FSM_M_LAB) & 63;
+        const uint32_t ainfo = sm.q_ainfo[w][q], xinfo = sm.q_xinfo[w][q];
+        const int la = ainfo & 63, lx = xinfo & 63;
+        if (QUOTA) m |= anchor_meta(r, j, anchor, la);
         // bits of the anchor and of the partner in a cross subset: a's low, b's high
         const int sh_a = centre ? O : 0, sh_x = centre ? 0 : O;
         constexpr uint32_t all = (1u << O) - 1u;
@@ -556,7 +554,7 @@ struct Joiner {
                         forms &= ~(1u << f);
             }
             if (A.mode == 1 ? forms != 0 : (forms >> FORM_TRI) & 1u) {
-                const int4 ia = __ldg(A.g.vinfo + anchor);
+                const int4 ia = __ldg(A.g.vinfo + anchor), ix = __ldg(A.g.vinfo + x);
                 const bool shorter = ia.y - ia.x <= ix.y - ix.x;
                 const bool tri = shorter ? sorted_has(A.g.col, ia.x, ia.y, x) : sorted_has(A.g.col, ix.x, ix.y, anchor);
                 if (!tri) forms &= ~(1u << FORM_TRI);
@@ -634,7 +632,7 @@ struct Joiner {
                     cross |= ((sub >> o) & 1u) << (2 * pp + (swap ? 1 : 0));
                     cross |= ((sub >> (O + o)) & 1u) << (2 * pp + (swap ? 0 : 1));
                 }
-                accept(r, j, make_key(r[R::PID], pidx, ki, jpos, cross, L), centre, anchor, x, ranchor, (uint32_t)ix.w, swap);
+                accept(r, j, make_key(r[R::PID], pidx, ki, jpos, cross, L), centre, anchor, x, ainfo, xinfo, swap);
             }
         }
         qn -= n;
@@ -643,14 +641,16 @@ struct Joiner {
 
     // warp-synchronous: queue the survivors among the lanes' candidates; join when 32 wait, or what
     // there is when nothing more comes (`drain`)
-    __device__ __forceinline__ void push(bool ok, int32_t anchor, int32_t x, uint32_t m, uint32_t ranchor, bool drain) {
+    __device__ __forceinline__ void push(bool ok, int32_t anchor, int32_t x, uint32_t m, uint32_t ainfo, uint32_t xinfo,
+                                         bool drain) {
         const unsigned bal = __ballot_sync(0xffffffffu, ok);
         if (ok) {
             const int p = qn + __popc(bal & ((1u << lane) - 1u));
             sm.q_anchor[w][p] = (uint32_t)anchor;
             sm.q_partner[w][p] = (uint32_t)x;
             sm.q_meta[w][p] = m;
-            if (!QUOTA) sm.q_rank[w][p] = ranchor;
+            sm.q_ainfo[w][p] = ainfo;
+            sm.q_xinfo[w][p] = xinfo;
         }
         qn += __popc(bal);
         if (qn >= 32 || (drain && qn > 0)) take(min(qn, 32));
@@ -785,7 +785,7 @@ struct Joiner {
         // Bloom filters of the lists of s (of the key vertex only where end pieces are tested for
         // closing a triangle)
         int bw = R::BLOOM / (nu * L);
-        lb = 5 + (31 - __clz(bw));
+        lb = 31 - __clz(bw);
         __syncwarp();
         for (int x = lane; x < R::BLOOM; x += 32) sm.bloom[w][x] = 0u;
         if (PASS == PASS_FUSED || PASS == PASS_DOMAIN)
@@ -807,8 +807,8 @@ struct Joiner {
                     x1 = (int32_t)rj[R::OE + o];
                 }
                 for (int32_t x = x0 + lane; x < x1; x += 32) {
-                    const uint32_t h = ((uint32_t)__ldg(g.col + x) * 0x9E3779B1u) >> (32 - lb);
-                    atomicOr(&sm.bloom[w][((j * L + t) << (lb - 5)) + (h >> 5)], 1u << (h & 31));
+                    const uint32_t h = (uint32_t)__ldg(g.col + x) * 0x9E3779B1u;
+                    atomicOr(&sm.bloom[w][((j * L + t) << lb) + (lb ? h >> (32 - lb) : 0u)], bloom_mask(h >> 7));
                 }
             }
         }
@@ -848,6 +848,7 @@ struct Joiner {
                     atomicOr(A.err, FSM_ERR_BOUNDS);
                 } else {
                     const int32_t anchor = __ldg(g.pcol + rp + y);
+                    const uint32_t ainfo = __ldg(g.pinfo + rp + y);
                     bool in = false;
                     int s = 0;
 #pragma unroll
@@ -859,10 +860,8 @@ struct Joiner {
                     uint32_t ok = in ? 0u : allowed(r, centre, s);
                     if (centre) ok &= (1u << SL) - 1u;
                     uint32_t m = 0;
-                    int4 ia = make_int4(0, 0, 0, 0);
                     if (ok) {
-                        ia = __ldg(g.vinfo + anchor);
-                        m = anchor_meta(r, j, anchor, ia.z) | (uint32_t)j | ((centre ? 0u : 1u) << FSM_M_END) |
+                        m = anchor_meta(r, j, anchor, ainfo & 63) | (uint32_t)j | ((centre ? 0u : 1u) << FSM_M_END) |
                             ((uint32_t)s << FSM_M_SA);
                         const uint32_t all = (1u << O) - 1u;
                         const uint32_t c = m >> FSM_M_CROSS, must = m >> FSM_M_MUST, no = m >> FSM_M_NO;
@@ -886,8 +885,8 @@ struct Joiner {
                             lb0 = rp;
                         } else {
                             const int64_t st = (int64_t)rec_u64(r, R::NC) + __ldg(g.pend + rp + y);
-                            lb0 = A.sampled ? __ldg(g.prow + anchor) : ia.x;
-                            const int32_t da = (A.sampled ? __ldg(g.prow + anchor + 1) : ia.y) - lb0;
+                            lb0 = __ldg(g.prow + anchor);
+                            const int32_t da = __ldg(g.prow + anchor + 1) - lb0;
                             p0 = (int32_t)max(lo - st, (int64_t)0);
                             p1 = (int32_t)min(hi - st, (int64_t)da);
                             // cut to the allowed slots (lists of a few entries are walked whole)
@@ -901,7 +900,7 @@ struct Joiner {
                         sm.sg_anchor[w][lane] = (uint32_t)anchor;
                         sm.sg_slots[w][lane] = ok;
                         sm.sg_meta[w][lane] = m;
-                        sm.sg_rank[w][lane] = (uint32_t)ia.w;
+                        sm.sg_info[w][lane] = ainfo;
                     }
                 }
             }
@@ -923,9 +922,9 @@ struct Joiner {
                     if (__shfl_sync(0xffffffffu, inc, k + s - 1) <= t) k += s;
                 bool ok = t < total;
                 int32_t x = 0, anchor = 0;
-                uint32_t m = 0, ranchor = 0;
+                uint32_t m = 0, ainfo = 0, xinfo = 0;
                 if (ok) {
-                    ranchor = sm.sg_rank[w][k];
+                    ainfo = sm.sg_info[w][k];
                     m = sm.sg_meta[w][k];
                     anchor = (int32_t)sm.sg_anchor[w][k];
                     const int64_t at = (int64_t)(int32_t)(sm.sg_base[w][k] + (uint32_t)t);
@@ -934,6 +933,7 @@ struct Joiner {
                         ok = false;
                     } else {
                         x = __ldg(g.pcol + at);
+                        xinfo = __ldg(g.pinfo + at);
                         const uint32_t *r = rec(m & 15);
                         int s = 0;
 #pragma unroll
@@ -946,7 +946,7 @@ struct Joiner {
                         ok &= (sm.sg_slots[w][k] >> (s + (x > anchor ? SL : 0))) & 1u;
                     }
                 }
-                push(ok, anchor, x, m, ranchor, drain);
+                push(ok, anchor, x, m, ainfo, xinfo, drain);
             }
             __syncwarp();
             if (drain) break;
@@ -961,7 +961,7 @@ struct Joiner {
             const int gi = g0 + lane;
             bool ok = gi < total_seg;
             int32_t anchor = 0, x = 0;
-            uint32_t m = 0;
+            uint32_t m = 0, ainfo = 0, xinfo = 0;
             if (ok) {
                 const int j = unit_of(gi, nu);
                 const uint32_t *r = rec(j);
@@ -977,15 +977,23 @@ struct Joiner {
                     const int32_t y = centre_row(lq, cpos, d);
                     const int32_t p = (int32_t)(lq - centre_row_start(y, cpos));
                     if (A.debug && (p < 0 || p >= y || y >= d)) { atomicOr(A.err, FSM_ERR_BOUNDS); ok = false; }
-                    anchor = ok ? __ldg(g.pcol + rp + y) : 0;
-                    x = ok ? __ldg(g.pcol + rp + p) : 0;
+                    if (ok) {
+                        anchor = __ldg(g.pcol + rp + y);
+                        ainfo = __ldg(g.pinfo + rp + y);
+                        x = __ldg(g.pcol + rp + p);
+                        xinfo = __ldg(g.pinfo + rp + p);
+                    }
                 } else {
                     const int32_t y = end_row(g.pend + rp, d, lq - nc);
                     const int64_t p = lq - nc - __ldg(g.pend + rp + y);
                     anchor = __ldg(g.pcol + rp + y);
+                    ainfo = __ldg(g.pinfo + rp + y);
                     const int32_t lb0 = __ldg(g.prow + anchor);
                     if (A.debug && (p < 0 || p >= __ldg(g.prow + anchor + 1) - lb0)) { atomicOr(A.err, FSM_ERR_BOUNDS); ok = false; }
-                    x = ok ? __ldg(g.pcol + lb0 + p) : 0;
+                    if (ok) {
+                        x = __ldg(g.pcol + lb0 + p);
+                        xinfo = __ldg(g.pinfo + lb0 + p);
+                    }
                 }
                 int s = 0, sx = 0;
 #pragma unroll
@@ -998,7 +1006,7 @@ struct Joiner {
                 if (ok) ok = (allowed(r, centre, s) >> (sx + (x > anchor ? SL : 0))) & 1u;
                 m = (uint32_t)j | ((centre ? 0u : 1u) << FSM_M_END) | ((uint32_t)s << FSM_M_SA) | ((uint32_t)sx << FSM_M_SP);
             }
-            push(ok, anchor, x, m, 0u, drain);
+            push(ok, anchor, x, m, ainfo, xinfo, drain);
             if (drain) break;
         }
     }
@@ -1006,11 +1014,11 @@ struct Joiner {
 };
 
 // Resident blocks per SM: four (64 registers) hide more latency in the count and emission passes
-// (3.7M vertices, 1 -> 3: 5.2 ms against 6.1 ms with three) and in the domain pass up to l = 4 (13.3
-// and 13.9 ms); the one-pass level and the domain pass of l = 5 spill too much at 64 registers (2 -> 4
-// one pass: 157 and 131 ms).
+// (3.7M vertices, 1 -> 3: 5.2 ms against 6.1 ms with three) and in the domain pass up to l = 3 (11.4
+// and 12.6 ms); the one-pass level and the domain passes of l = 4 and 5 spill too much at 64
+// registers (4 -> 6: 14.5 and 13.7 ms; 2 -> 4 one pass: 157 and 131 ms).
 template <int L, int PASS> struct JoinBlocks {
-    static constexpr int value = PASS == PASS_FUSED || (PASS == PASS_DOMAIN && L == 5) ? 3 : 4;
+    static constexpr int value = PASS == PASS_FUSED || (PASS == PASS_DOMAIN && L >= 4) ? 3 : 4;
 };
 
 template <int L, int PASS, bool QUOTA>

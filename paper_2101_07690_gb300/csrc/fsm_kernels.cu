@@ -210,6 +210,22 @@ cudaError_t launch_validate(const DevGraph &g, int32_t num_labels, int *err, cud
     return cudaGetLastError();
 }
 
+namespace {
+__global__ void list_info_kernel(const DevGraph g, uint32_t *info) {
+    for (int64_t j = gtid(); j < g.nnz; j += gstride()) {
+        const int4 x = __ldg(g.vinfo + g.col[j]);
+        info[j] = (uint32_t)x.z | (g.packed ? (uint32_t)x.w << 6 : 0u);
+    }
+}
+} // namespace
+
+cudaError_t launch_list_info(const DevGraph &g, uint32_t *info, cudaStream_t st) {
+    if (g.nnz <= 0) return cudaSuccess;
+    LAUNCHED(1);
+    list_info_kernel<<<blocks_for(g.nnz), kThreads, 0, st>>>(g, info);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_prepare(const DevGraph &g, int64_t *piece_cnt, int32_t *end_off, int32_t *rank,
                            int32_t *cls_size, int4 *vinfo, cudaStream_t st) {
     LAUNCHED(1);
@@ -1143,13 +1159,16 @@ __global__ void sample_count_kernel(const DevGraph g, uint64_t seed, uint64_t th
     }
 }
 __global__ void sample_fill_kernel(const DevGraph g, uint64_t seed, uint64_t thr, const int64_t *prow64, int32_t *prow,
-                                   int32_t *pcol) {
+                                   int32_t *pcol, uint32_t *pinfo) {
     for (int64_t v = gtid(); v < g.n; v += gstride()) {
         int64_t o = prow64[v];
         prow[v] = (int32_t)o;
         if (v == g.n - 1) prow[g.n] = (int32_t)prow64[g.n];
         for (int32_t j = g.row_ptr[v]; j < g.row_ptr[v + 1]; ++j)
-            if (keep_edge(seed, thr, (int32_t)v, g.col[j])) pcol[o++] = g.col[j];
+            if (keep_edge(seed, thr, (int32_t)v, g.col[j])) {
+                pinfo[o] = g.pinfo[j];
+                pcol[o++] = g.col[j];
+            }
     }
 }
 __global__ void sample_pieces_kernel(int32_t n, const int32_t *prow, const int32_t *pcol, int32_t *pend, int64_t *ppc) {
@@ -1173,9 +1192,9 @@ cudaError_t launch_sample_count(const DevGraph &g, uint64_t seed, uint64_t thr, 
 }
 
 cudaError_t launch_sample_lists(const DevGraph &g, uint64_t seed, uint64_t thr, const int64_t *prow64, int32_t *prow,
-                                int32_t *pcol, int32_t *pend, int64_t *ppc, cudaStream_t st) {
+                                int32_t *pcol, uint32_t *pinfo, int32_t *pend, int64_t *ppc, cudaStream_t st) {
     LAUNCHED(2);
-    sample_fill_kernel<<<blocks_for(g.n), kThreads, 0, st>>>(g, seed, thr, prow64, prow, pcol);
+    sample_fill_kernel<<<blocks_for(g.n), kThreads, 0, st>>>(g, seed, thr, prow64, prow, pcol, pinfo);
     sample_pieces_kernel<<<blocks_for(g.n), kThreads, 0, st>>>(g.n, prow, pcol, pend, ppc);
     return cudaGetLastError();
 }

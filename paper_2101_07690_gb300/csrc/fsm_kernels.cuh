@@ -20,6 +20,9 @@ cudaError_t launch_validate(const DevGraph &g, int32_t num_labels, int *err, cud
 cudaError_t launch_prepare(const DevGraph &g, int64_t *piece_cnt, int32_t *end_off, int32_t *rank,
                            int32_t *cls_size, int4 *vinfo, cudaStream_t st);
 
+// ---- label and rank of every list entry (DevGraph::pinfo), after launch_prepare
+cudaError_t launch_list_info(const DevGraph &g, uint32_t *info, cudaStream_t st);
+
 // ---- neighbour-adjacency matrices of vertices of degree >= dmin (DevGraph::tri_off):
 //      words[v] = d * ceil(d / 32) or 0; then, with off = exclusive prefix of words, the bits
 //      and tri_off (-1 for vertices without a matrix); bits must be zeroed first
@@ -144,7 +147,7 @@ void note_launches(int64_t n);
 // (after an exclusive scan into prow64) the lists, the end-piece prefixes and piece counts.
 cudaError_t launch_sample_count(const DevGraph &g, uint64_t seed, uint64_t thr, int64_t *cnt, cudaStream_t st);
 cudaError_t launch_sample_lists(const DevGraph &g, uint64_t seed, uint64_t thr, const int64_t *prow64, int32_t *prow,
-                                int32_t *pcol, int32_t *pend, int64_t *ppc, cudaStream_t st);
+                                int32_t *pcol, uint32_t *pinfo, int32_t *pend, int64_t *ppc, cudaStream_t st);
 // by_rank[cls_off[l] + rank[v]] = v for every vertex v of label l (cls_off: exclusive prefix of
 // class sizes, computed by the kernel itself)
 cudaError_t launch_by_rank(const DevGraph &g, int32_t NL, const int32_t *cls_size, int64_t *cls_off,
