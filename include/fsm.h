@@ -75,11 +75,10 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
  *                0 restores the library's own stream.  The caller keeps ownership.
  *   "launch"     0 = one launch per frontier batch of at most "batch" embeddings, sized on
  *                the host (default); 1 = one persistent work-stealing launch per pass over the
- *                whole frontier, all sizes kept on the device, captured with its prefix kernels
- *                in a CUDA graph (its per-unit piece prefix takes 8 bytes per embedding and key
- *                position; a frontier whose prefix would exceed a quarter of the free device
- *                memory is split into the fewest equal ranges that fit, one launch each, in the
- *                same graph); 2 = one launch per frontier
+ *                whole frontier (its per-unit piece prefix takes 8 bytes per embedding and key position;
+ *                a frontier whose prefix would exceed a quarter of the free device memory is split into
+ *                the fewest equal ranges that fit, one launch each, sizes kept on the device, captured
+ *                with their prefix kernels in a CUDA graph); 2 = one launch per frontier
  *                pattern (the frontier grouped by pattern id), captured in one CUDA graph.  All
  *                modes give identical results.
  *   "group"      with launch 1: 1 = group the frontier by pattern id before each level (as

@@ -67,26 +67,44 @@ void keep_pool(int dev) {
     });
 }
 
-// Stream-ordered device allocations released together.
+// Stream-ordered device allocations released together.  Small ones (most of the hundred or so of a
+// call) are cut from blocks that live until the end, so they cost no call of the allocator.
 struct Arena {
+    static constexpr size_t kSmall = 16 << 10, kBlock = 1 << 20;
     cudaStream_t st;
     std::vector<void *> ptrs;
+    std::vector<void *> blocks;      // the blocks among ptrs: release() leaves their first piece alone
+    char *block = nullptr;
+    size_t left = 0;                 // bytes of the current block not given out
     int64_t made = 0, fail_at = 0;   // fail_at > 0: the fail_at-th allocation reports failure (test hook)
     explicit Arena(cudaStream_t s) : st(s) {}
+    void *raw(size_t bytes) {
+        void *p = nullptr;
+        ck(cudaMallocAsync(&p, bytes, st), "device allocation");
+        ptrs.push_back(p);
+        return p;
+    }
     template <class T>
     T *get(int64_t n) {
-        void *p = nullptr;
         size_t bytes = (size_t)std::max<int64_t>(n, 1) * sizeof(T);
         bytes = (bytes + 255) & ~(size_t)255;
         if (fail_at > 0 && ++made == fail_at)
             fail(FSM_ENOMEM, "device allocation: injected failure (option fail_alloc_after)");
-        ck(cudaMallocAsync(&p, bytes, st), "device allocation");
-        ptrs.push_back(p);
+        if (bytes > kSmall) return (T *)raw(bytes);
+        if (left < bytes) {
+            block = (char *)raw(kBlock);
+            blocks.push_back(block);
+            left = kBlock;
+        }
+        void *p = block;
+        block += bytes;
+        left -= bytes;
         return (T *)p;
     }
+    // give a large allocation back now (small ones stay in their block)
     void release(void *p) {
         auto it = std::find(ptrs.begin(), ptrs.end(), p);
-        if (it != ptrs.end()) {
+        if (it != ptrs.end() && std::find(blocks.begin(), blocks.end(), p) == blocks.end()) {
             cudaFreeAsync(p, st);
             ptrs.erase(it);
         }
@@ -182,8 +200,10 @@ struct fsm_graph {
     int64_t *piece_cnt = nullptr;
     int64_t *tri_off = nullptr;   // neighbour-adjacency matrices of high-degree vertices
     uint32_t *tri_bits = nullptr;
-    int *err = nullptr;
-    unsigned long long *stats = nullptr;   // [0] tested, [1] accepted, [2..] scratch counters
+    // The call's scalars in one array, so that what the host needs at one point is one copy (Scalar)
+    unsigned long long *stats = nullptr;
+    int *err = nullptr;            // = &stats[S_ERR]
+    int32_t cls_host[64] = {};     // vertices per label
     DevGraph dg() const {
         DevGraph g;
         g.n = n;
@@ -216,6 +236,8 @@ template <class T> struct Unset : std::allocator<T> {
     }
 };
 template <class T> using HostArray = std::vector<T, Unset<T>>;
+
+enum { S_TESTED, S_ACCEPTED, S_PIECES, S_KEYS, S_ERR, S_POOL, S_LIVE, S_WORDS, S_FREQ, S_SUM, S_WROTE, S_START, S_COUNT };
 
 struct fsm_result {
     int k = 0;
@@ -331,10 +353,62 @@ struct Miner {
     //             ranges that fit, each one launch of the same graph;
     //   launch 2: one launch per frontier pattern (the frontier grouped by pattern id), all
     //             captured into one CUDA graph.
-    void run_pass(int pass, const LevelSet &in, ExtArgs A, const std::vector<int64_t> &pat_off) {
+    // A frontier of one range keeps its prefix for every pass of the level (`pre`), and its later passes
+    // are single launches; only a pass of several ranges, or per-pattern launches, is a graph.
+    struct Prefix {
+        int64_t *base = nullptr;
+        int64_t total = -1;   // pieces, when the host knows them
+    };
+    // One range for the whole frontier: compute its prefix once, and read the total back.
+    void make_prefix(const LevelSet &in, const ExtArgs &A, Prefix &pre) {
+        const int L = in.L;
+        if (in.N == 0 || pre.base || !one_range(in)) return;
+        pre.base = mem.get<int64_t>(in.N * L + 1);
+        void *tmp = mem.get<char>((int64_t)scan_temp_bytes(in.N * L) + 16);
+        ck(launch_unit_counts(A.g, in.fv, in.N, 0, in.N, L, V, A.quota, A.edge_quota, A.qseed, pre.base, st), "unit counts");
+        ck(launch_scan_i64(pre.base, pre.base, in.N * L, tmp, st), "unit scan");
+        pre.total = d2h(pre.base + in.N * L, st);
+        mem.release(tmp);
+    }
+    int64_t batch_size(int L) const { return G->batch > 0 ? G->batch : std::max<int64_t>(1024, ((int64_t)1 << 24) / L); }
+    int64_t prefix_fit(int L) const {   // embeddings whose prefix a quarter of the free memory holds
+        size_t fr = 0, tot = 0;
+        ck(cudaMemGetInfo(&fr, &tot), "memory info");
+        return std::max<int64_t>(1 << 20, (int64_t)(fr / 4 / sizeof(int64_t)) / L);
+    }
+    bool one_range(const LevelSet &in) const {
+        if (G->launch == 2 || G->profile) return false;   // profiled passes time their own prefix
+        if (G->launch == 1) return in.N <= 1 << 20 || in.N <= prefix_fit(in.L);
+        return in.N <= batch_size(in.L);
+    }
+
+    void run_pass(int pass, const LevelSet &in, ExtArgs A, const std::vector<int64_t> &pat_off, const Prefix &pre) {
         const int L = in.L;
         if (in.N == 0) return;
-        int64_t B = G->batch > 0 ? G->batch : std::max<int64_t>(1024, ((int64_t)1 << 24) / L);
+        if (pre.base) {
+            if (pre.total == 0) return;
+            unsigned long long *ctr = mem.get<unsigned long long>(1);
+            const int grid = grid_for(L, pass);
+            int64_t chunk = chunk_for(L);
+            const int64_t warps = (int64_t)grid * 8;
+            if (chunk <= 0) chunk = joins(L) ? join_chunk(pre.total, warps) : extend_chunk(pre.total, in.N * L, warps);
+            A.fv = in.fv;
+            A.fpid = in.fpid;
+            A.fN = in.N;
+            A.e0 = 0;
+            A.ne = in.N;
+            A.unit_base = pre.base;
+            A.chunk_ctr = ctr;
+            A.total = pre.total;
+            A.chunk = (int32_t)chunk;
+            A.nchunks = (pre.total + chunk - 1) / chunk;
+            ck(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), st), "memset");
+            ck(launch_pass(pass, L, A, grid), "extension kernel");
+            rs.launches += 1;
+            rs.pass_launches[L][pass] += 1;
+            return;
+        }
+        const int64_t B = batch_size(L);
         std::vector<Range> ranges;
         bool device_total = false;
         if (G->launch == 2 && (int64_t)pat_off.size() == in.P + 1) {  // frontier grouped by pattern
@@ -343,9 +417,7 @@ struct Miner {
                     ranges.push_back({e0, std::min(B, pat_off[p + 1] - e0)});
             device_total = true;
         } else if (G->launch == 1) {
-            size_t fr = 0, tot = 0;
-            ck(cudaMemGetInfo(&fr, &tot), "memory info");
-            const int64_t fit = std::max<int64_t>(1 << 20, (int64_t)(fr / 4 / sizeof(int64_t)) / L);   // embeddings
+            const int64_t fit = prefix_fit(L);
             const int64_t parts = (in.N + fit - 1) / fit;
             const int64_t per = (in.N + parts - 1) / parts;
             for (int64_t e0 = 0; e0 < in.N; e0 += per) ranges.push_back({e0, std::min(per, in.N - e0)});
@@ -509,7 +581,16 @@ struct Miner {
         for (void *p : {(void *)cnt, (void *)base, tmp, (void *)ctr}) mem.release(p);
     }
 
-    int err_word() { return d2h(G->err, st); }
+    // the call's scalars as they are on the device
+    struct Scalars {
+        unsigned long long v[S_COUNT];
+        int err() const { return (int)v[S_ERR]; }
+        unsigned long long operator[](int i) const { return v[i]; }
+    };
+    Scalars scalars() { return d2h((const Scalars *)G->stats, st); }
+    void put_scalar(int i, const void *src) {
+        ck(cudaMemcpyAsync(G->stats + i, src, sizeof(unsigned long long), cudaMemcpyDeviceToDevice, st), "copy");
+    }
 
     // Fail with the code a kernel's error word stands for (after the recoverable bits are handled)
     [[noreturn]] void fail_word(int ew) {
@@ -540,7 +621,7 @@ struct Miner {
         A.sampled = sampled ? 1 : 0;
         A.debug = G->debug;
         A.time_limit_ns = (uint64_t)G->time_limit_ms * 1000000ull;
-        A.time_start = G->stats + 4;
+        A.time_start = G->stats + S_START;
         unsigned long long *lf = nullptr;
         if (joins(L)) {
             join_tables(L);
@@ -591,7 +672,13 @@ struct Miner {
         const int64_t t_live = sampled ? 1 : t;   // sampled counts say nothing about reaching t
         // ---- pass 1: quick patterns and their embedding counts; at the last level (k <= 7, exact
         // mining) also the MNI domains, in the same enumeration, when option "fused" is set
+        Prefix pre;
+        make_prefix(in, A, pre);
         int64_t cap = G->qp_initial > 0 ? G->qp_initial : (int64_t)1 << 20;
+        // few pieces have few keys: small levels clear and scan tables of four slots per piece (1000
+        // vertices, 60k pieces: 2^18 slots instead of 2^20)
+        if (G->qp_initial == 0 && pre.total >= 0)
+            while (cap > 4096 && cap / 2 >= 4 * pre.total) cap >>= 1;
         if (G->qp_initial == 0)
             while (cap < 4 * G->qp_hint[L] && cap < ((int64_t)1 << 30)) cap <<= 1;
         unsigned long long *keys = nullptr, *qcount = nullptr, *used = nullptr, *ptop = nullptr, *ckeys = nullptr,
@@ -612,36 +699,36 @@ struct Miner {
             ck(cudaMemGetInfo(&fr, &tot), "memory info");
             pool_limit = std::max<unsigned long long>(1ull << 20, (unsigned long long)(fr / 4 * 2 / 5));   // 40% of it
             pool_min = std::min(pool_limit, 2 * G->pool_hint[L] + (1ull << 22));
-            ptop = mem.get<unsigned long long>(1);
+            ptop = G->stats + S_POOL;
         }
+        int64_t *slots = nullptr;
+        unsigned long long *zeros = nullptr;
         auto release_pass1 = [&]() {
-            for (void *q : {(void *)keys, (void *)qcount, (void *)used, (void *)ckeys, (void *)coff, (void *)krec})
+            for (void *q : {(void *)keys, (void *)zeros, (void *)krec, (void *)slots})
                 if (q) mem.release(q);
-            keys = qcount = used = ckeys = coff = nullptr;
+            keys = zeros = qcount = ckeys = coff = nullptr;
             krec = nullptr;
+            slots = nullptr;
         };
         auto clear_pass1 = [&]() {
-            ck(launch_fill_u64(keys, FSM_EMPTY_KEY, cap, st), "fill");
-            ck(cudaMemsetAsync(qcount, 0, sizeof(unsigned long long) * cap, st), "memset");
-            ck(cudaMemsetAsync(used, 0, sizeof(unsigned long long), st), "memset");
-            ck(cudaMemsetAsync(G->err, 0, sizeof(int), st), "memset");
-            ck(cudaMemsetAsync(G->stats, 0, 3 * sizeof(unsigned long long), st), "memset");
-            if (fused) {
-                ck(launch_fill_u64(ckeys, FSM_EMPTY_KEY, cap, st), "fill");
-                ck(cudaMemsetAsync(coff, 0, sizeof(unsigned long long) * cap, st), "memset");
-                ck(cudaMemsetAsync(krec, 0xff, sizeof(uint32_t) * cap * rec_words, st), "memset");
-                ck(cudaMemsetAsync(ptop, 0, sizeof(unsigned long long), st), "memset");
-            }
+            // all-ones: empty keys, empty codes; zero: counts, code offsets; scalars up to the pool top
+            ck(cudaMemsetAsync(keys, 0xff, sizeof(unsigned long long) * cap * (fused ? 2 : 1), st), "memset");
+            ck(cudaMemsetAsync(zeros, 0, sizeof(unsigned long long) * (cap * (fused ? 2 : 1) + 1), st), "memset");
+            ck(cudaMemsetAsync(G->stats, 0, sizeof(unsigned long long) * (S_POOL + 1), st), "memset");
+            if (fused) ck(cudaMemsetAsync(krec, 0xff, sizeof(uint32_t) * cap * rec_words, st), "memset");
         };
+        Scalars sc;
         for (;;) {
-            keys = mem.get<unsigned long long>(cap);
-            qcount = mem.get<unsigned long long>(cap);
-            used = mem.get<unsigned long long>(1);
+            // the pattern (code) table has as many slots as the quick-pattern table, so it is at most
+            // half full whenever that one is
+            keys = mem.get<unsigned long long>(cap * (fused ? 2 : 1));
+            zeros = mem.get<unsigned long long>(cap * (fused ? 2 : 1) + 1);
+            used = zeros;
+            qcount = zeros + 1;
+            slots = mem.get<int64_t>(cap);
             if (fused) {
-                // the pattern (code) table has as many slots as the quick-pattern table, so it is
-                // at most half full whenever that one is
-                ckeys = mem.get<unsigned long long>(cap);
-                coff = mem.get<unsigned long long>(cap);
+                ckeys = keys + cap;
+                coff = qcount + cap;
                 krec = mem.get<uint32_t>(cap * rec_words);
                 pool_words = G->pool_force ? G->pool_force
                                            : std::min(pool_limit, std::max<unsigned long long>(pool_min, 0xFFFFFFFDull));
@@ -679,7 +766,7 @@ struct Miner {
                 ExtArgs W = A;
                 W.warm = 1;
                 W.stats = nullptr;
-                run_pass(PASS_COUNT, in, W, pat_off);
+                run_pass(PASS_COUNT, in, W, pat_off, pre);
                 ck(launch_resolve_keys(W, G->sms, st), "resolve keys");
                 rs.launches += 1;
                 ck(cudaMemsetAsync(qcount, 0, sizeof(unsigned long long) * cap, st), "memset");
@@ -704,8 +791,10 @@ struct Miner {
                 A.pool = pool;
                 ck(cudaMemsetAsync(pool, 0, pool_words * 4, st), "memset");
             }
-            run_pass(fused ? PASS_FUSED : PASS_COUNT, in, A, pat_off);
-            const int ew = err_word();
+            run_pass(fused ? PASS_FUSED : PASS_COUNT, in, A, pat_off, pre);
+            ck(launch_qp_compact(keys, cap, slots, G->stats + S_KEYS, st), "compact");
+            sc = scalars();
+            const int ew = sc.err();
             if (ew & (FSM_ERR_TIMEOUT | FSM_ERR_BOUNDS)) fail_word(ew);
             if (ew && pool) {
                 mem.release(pool);
@@ -736,25 +825,18 @@ struct Miner {
                 continue;
             }
             if (fused) {
-                G->pool_hint[L] = d2h(ptop, st);
+                G->pool_hint[L] = sc[S_POOL];
                 rs.fused_pool_words = (int64_t)G->pool_hint[L];
             }
             break;
         }
-        unsigned long long st2[3];
-        ck(cudaMemcpyAsync(st2, G->stats, sizeof(st2), cudaMemcpyDeviceToHost, st), "copy");
-        ck(cudaStreamSynchronize(st), "sync");
-        rs.tested += (int64_t)st2[0];
-        rs.accepted += (int64_t)st2[1];
-        rs.pieces += (int64_t)st2[2];
-        rs.pieces_l[L] += (int64_t)st2[2];
-        if (final) rs.final_accepted = (int64_t)st2[1];
+        rs.tested += (int64_t)sc[S_TESTED];
+        rs.accepted += (int64_t)sc[S_ACCEPTED];
+        rs.pieces += (int64_t)sc[S_PIECES];
+        rs.pieces_l[L] += (int64_t)sc[S_PIECES];
+        if (final) rs.final_accepted = (int64_t)sc[S_ACCEPTED];
         // ---- distinct quick patterns -> canonical codes -> pattern ids
-        int64_t *slots = mem.get<int64_t>(cap);
-        unsigned long long *nq_d = mem.get<unsigned long long>(1);
-        ck(cudaMemsetAsync(nq_d, 0, sizeof(unsigned long long), st), "memset");
-        ck(launch_qp_compact(keys, cap, slots, nq_d, st), "compact");
-        const int64_t nq = (int64_t)d2h(nq_d, st);
+        const int64_t nq = (int64_t)sc[S_KEYS];
         rs.qps += nq;
         G->qp_hint[L] = std::max(G->qp_hint[L], nq);
         int32_t *qpat = mem.get<int32_t>(cap);
@@ -784,7 +866,7 @@ struct Miner {
         int64_t *doff = mem.get<int64_t>(np * FSM_MAXK);
         void *stmp2 = mem.get<char>((int64_t)scan_temp_bytes(np * FSM_MAXK) + 16);
         unsigned long long *sigma = mem.get<unsigned long long>(np);
-        ck(launch_fill_u64(sigma, ~0ull, np, st), "fill");
+        ck(cudaMemsetAsync(sigma, 0xff, sizeof(unsigned long long) * std::max<int64_t>(np, 1), st), "memset");
         uint32_t *dom = nullptr;
         int64_t *sbase = nullptr;
         rs.patterns = np;
@@ -797,22 +879,19 @@ struct Miner {
         } else {
             int64_t nwords = 0;
             for (shift = 0;; ++shift) {   // past 2^32 words, bitmaps start on multiples of 2, 4, ... words
-                ck(launch_domain_sizes(K, plab, orbit, minorb, pcount, np, t_live, G->cls_size, shift, live, words, st),
-                   "domain sizes");
+                ck(cudaMemsetAsync(G->stats + S_LIVE, 0, sizeof(unsigned long long), st), "memset");
+                ck(launch_domain_sizes(K, plab, orbit, minorb, pcount, np, t_live, G->cls_size, shift, live, words,
+                                       G->stats + S_LIVE, st), "domain sizes");
                 ck(launch_scan_i64(words, woff, np * FSM_MAXK, stmp2, st), "domain scan");
-                nwords = d2h(woff + np * FSM_MAXK, st);
+                put_scalar(S_WORDS, woff + np * FSM_MAXK);
+                sc = scalars();
+                nwords = (int64_t)sc[S_WORDS];
+                rs.live = (int64_t)sc[S_LIVE];
                 if (!joins(L) || (nwords >> shift) < 0xFFFFFFFEll) break;
             }
             ck(launch_domain_offsets(words, woff, np * FSM_MAXK, doff, st), "domain offsets");
             dom = mem.get<uint32_t>(nwords);
             ck(cudaMemsetAsync(dom, 0, sizeof(uint32_t) * std::max<int64_t>(nwords, 1), st), "memset");
-            // live pattern count (for statistics)
-            std::vector<uint8_t> hl((size_t)np);
-            if (np) {
-                ck(cudaMemcpyAsync(hl.data(), live, (size_t)np, cudaMemcpyDeviceToHost, st), "copy");
-                ck(cudaStreamSynchronize(st), "sync");
-            }
-            rs.live = std::count(hl.begin(), hl.end(), (uint8_t)1);
             // ---- pass 2: MNI domains (Definition 2)
             A.qp.pattern = qpat;
             A.qp.perm = qperm;
@@ -834,11 +913,13 @@ struct Miner {
             A.stats = nullptr;
             if (rs.live > 0) {
                 tune_chunk(in, A);
-                run_pass(PASS_DOMAIN, in, A, pat_off);
+                run_pass(PASS_DOMAIN, in, A, pat_off, pre);
                 if (G->profile) {
                     // algorithmic bytes of the domain updates: one 4-byte bitmap word per position
                     // of every accepted join of a live pattern (the list reads are in run_pass)
+                    std::vector<uint8_t> hl((size_t)np);
                     std::vector<unsigned long long> hc((size_t)np);
+                    ck(cudaMemcpyAsync(hl.data(), live, (size_t)np, cudaMemcpyDeviceToHost, st), "copy");
                     ck(cudaMemcpyAsync(hc.data(), pcount, sizeof(unsigned long long) * np, cudaMemcpyDeviceToHost, st),
                        "copy");
                     ck(cudaStreamSynchronize(st), "sync");
@@ -869,7 +950,13 @@ struct Miner {
         ck(launch_freq_flags(sigma, np, sampled ? 1 : t, fflag, st), "frequent flags");
         ck(launch_scan_i64(fflag, fscan, np, stmp2, st), "frequent scan");
         ck(launch_new_ids(fflag, fscan, np, newid, st), "new ids");
-        const int64_t nf = d2h(fscan + np, st);
+        put_scalar(S_FREQ, fscan + np);
+        if (!final) {   // embeddings of the frequent patterns, for the emission pass
+            ck(cudaMemsetAsync(G->stats + S_SUM, 0, 2 * sizeof(unsigned long long), st), "memset");   // and S_WROTE
+            ck(launch_sum_frequent(newid, pcount, np, G->stats + S_SUM, st), "sum");
+        }
+        sc = scalars();
+        const int64_t nf = (int64_t)sc[S_FREQ];
         if (dom) mem.release(dom);
         // ---- frequent patterns of size K
         out.P = nf;
@@ -888,34 +975,28 @@ struct Miner {
         }
         if (!final && nf > 0) {
             // ---- pass 3: store the frequent size-K embeddings in canonical order
-            unsigned long long *sum = mem.get<unsigned long long>(1);
-            ck(cudaMemsetAsync(sum, 0, sizeof(unsigned long long), st), "memset");
-            ck(launch_sum_frequent(newid, pcount, np, sum, st), "sum");
-            const int64_t N2 = (int64_t)d2h(sum, st);
+            const int64_t N2 = (int64_t)sc[S_SUM];
             out.N = N2;
             out.fv = mem.get<int32_t>(N2 * K);
             out.fpid = mem.get<int32_t>(N2);
-            unsigned long long *cursor = mem.get<unsigned long long>(1);
-            ck(cudaMemsetAsync(cursor, 0, sizeof(unsigned long long), st), "memset");
             A.newid = newid;
             A.out_v = out.fv;
             A.out_pid = out.fpid;
             A.out_N = N2;
-            A.out_cursor = cursor;
-            run_pass(PASS_EMIT, in, A, pat_off);
-            const int64_t wrote = (int64_t)d2h(cursor, st);
+            A.out_cursor = G->stats + S_WROTE;
+            run_pass(PASS_EMIT, in, A, pat_off, pre);
+            sc = scalars();
+            const int64_t wrote = (int64_t)sc[S_WROTE];
             if (wrote != N2) fail(FSM_ECUDA, "frontier emission wrote " + std::to_string(wrote) + " of " + std::to_string(N2));
             if (G->profile) rs.pass_bytes[L][PASS_EMIT] += N2 * 4 * (K + 1);   // output written
             rs.frontier_max = std::max(rs.frontier_max, N2);
-            mem.release(sum);
-            mem.release(cursor);
         }
-        const int ew = err_word();
-        if (ew) fail_word(ew);
+        if (sc.err()) fail_word(sc.err());
+        if (pre.base) mem.release(pre.base);
         if (sbase) mem.release(sbase);
         if (lf) mem.release(lf);
         release_pass1();
-        for (void *p : std::initializer_list<void *>{slots, nq_d, qpat, qperm, flag, ids, stmp, plab,
+        for (void *p : std::initializer_list<void *>{qpat, qperm, flag, ids, stmp, plab,
                                                      padj, orbit, minorb, pcount, live, words, woff, doff, stmp2, sigma,
                                                      fflag, fscan, newid})
             mem.release(p);
@@ -937,17 +1018,20 @@ struct Miner {
         unsigned long long *nf = mem.get<unsigned long long>(1);
         ck(launch_level1_tables(NL, G->cls_size, t, lnew, s.lab8, s.adj8, s.clab, s.cadj, s.sigma, s.count, nf, st),
            "level 1");
-        s.P = (int64_t)d2h(nf, st);
-                if (with_frontier) {
+        for (int l = 0; l < NL; ++l)
+            if (G->cls_host[l] >= t && G->cls_host[l] > 0) {
+                s.P += 1;
+                s.N += G->cls_host[l];   // vertices with a frequent label
+            }
+        if (!with_frontier) s.N = 0;
+        if (with_frontier) {
             int64_t *flag = mem.get<int64_t>(G->n);
             int64_t *scanned = mem.get<int64_t>(G->n + 1);
             void *tmp = mem.get<char>((int64_t)scan_temp_bytes(G->n) + 16);
-            // size: number of vertices with a frequent label
             s.fv = mem.get<int32_t>(G->n);
             s.fpid = mem.get<int32_t>(G->n);
             ck(launch_level1_frontier(G->dg(), lnew, flag, scanned, tmp, s.fv, s.fpid, st), "level 1 frontier");
-            s.N = d2h(scanned + G->n, st);
-                        mem.release(flag);
+            mem.release(flag);
             mem.release(scanned);
             mem.release(tmp);
         }
@@ -963,7 +1047,10 @@ struct Miner {
         int64_t *poff = mem.get<int64_t>(NP * 2);
         int64_t *tw = mem.get<int64_t>(1);
         ck(launch_level2_offsets(NL, G->cls_size, poff, tw, st), "level 2 offsets");
-        const int64_t words = d2h(tw, st);
+        int64_t words = 0;   // as level2_offsets_kernel lays them out
+        for (int lo = 0; lo < NL; ++lo)
+            for (int hi = lo; hi < NL; ++hi)
+                words += bitmap_words(G->cls_host[lo], 0) + (hi > lo ? bitmap_words(G->cls_host[hi], 0) : 0);
         uint32_t *dom = mem.get<uint32_t>(words);
         unsigned long long *pc = mem.get<unsigned long long>(NP);
         unsigned long long *ps = mem.get<unsigned long long>(NP);
@@ -978,26 +1065,23 @@ struct Miner {
         s.cadj = mem.get<uint64_t>(NP);
         s.sigma = mem.get<unsigned long long>(NP);
         s.count = mem.get<unsigned long long>(NP);
-        unsigned long long *nf = mem.get<unsigned long long>(1);
-        ck(launch_level2_tables(NL, ps, pc, t, pnew, s.lab8, s.adj8, s.clab, s.cadj, s.sigma, s.count, nf, st),
-           "level 2 tables");
-        s.P = (int64_t)d2h(nf, st);
-                if (with_frontier && s.P > 0) {
+        ck(launch_level2_tables(NL, ps, pc, t, pnew, s.lab8, s.adj8, s.clab, s.cadj, s.sigma, s.count,
+                                G->stats + S_FREQ, st), "level 2 tables");
+        ck(cudaMemsetAsync(G->stats + S_SUM, 0, sizeof(unsigned long long), st), "memset");
+        if (with_frontier) ck(launch_sum_frequent(pnew, pc, NP, G->stats + S_SUM, st), "sum");
+        const Scalars sc = scalars();
+        s.P = (int64_t)sc[S_FREQ];
+        if (with_frontier && s.P > 0) {
             int64_t *flag = mem.get<int64_t>(G->n);
             int64_t *scanned = mem.get<int64_t>(G->n + 1);
             void *tmp = mem.get<char>((int64_t)scan_temp_bytes(G->n) + 16);
-            // stored edges = embeddings of the frequent pairs
-            unsigned long long *sum = mem.get<unsigned long long>(1);
-            ck(cudaMemsetAsync(sum, 0, sizeof(unsigned long long), st), "memset");
-            ck(launch_sum_frequent(pnew, pc, NP, sum, st), "sum");
-            s.N = (int64_t)d2h(sum, st);
-            mem.release(sum);
+            s.N = (int64_t)sc[S_SUM];   // stored edges = embeddings of the frequent pairs
             s.fv = mem.get<int32_t>(s.N * 2);
             s.fpid = mem.get<int32_t>(s.N);
             ck(launch_level2_frontier(G->dg(), NL, pnew, flag, scanned, tmp, s.fv, s.N, s.fpid, st), "level 2 frontier");
             const int64_t wrote = d2h(scanned + G->n, st);
             if (wrote != s.N) fail(FSM_ECUDA, "level 2 frontier size mismatch");
-                        mem.release(flag);
+            mem.release(flag);
             mem.release(scanned);
             mem.release(tmp);
         }
@@ -1221,12 +1305,12 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
         dalloc((void **)&g->cls_size, sizeof(int32_t) * 64);
         dalloc((void **)&g->end_off, sizeof(int32_t) * nnz);
         dalloc((void **)&g->piece_cnt, sizeof(int64_t) * n);
-        dalloc((void **)&g->err, sizeof(int) * 4);
-        dalloc((void **)&g->stats, sizeof(unsigned long long) * 8);
+        dalloc((void **)&g->stats, sizeof(unsigned long long) * S_COUNT);
+        g->err = (int *)(g->stats + S_ERR);
         ck(cudaMemcpyAsync(g->row_ptr, row_ptr, sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, st), "copy");
         if (nnz) ck(cudaMemcpyAsync(g->col, col, sizeof(int32_t) * nnz, cudaMemcpyHostToDevice, st), "copy");
         ck(cudaMemcpyAsync(g->labels, labels, sizeof(int32_t) * n, cudaMemcpyHostToDevice, st), "copy");
-        ck(cudaMemsetAsync(g->err, 0, sizeof(int) * 4, st), "memset");
+        ck(cudaMemsetAsync(g->stats, 0, sizeof(unsigned long long) * S_COUNT, st), "memset");
         ck(cudaMemsetAsync(g->cls_size, 0, sizeof(int32_t) * 64, st), "memset");
         ck(launch_validate(g->dg(), num_labels, g->err, st), "validate");
         const int ew = d2h(g->err, st);
@@ -1262,6 +1346,7 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
         dalloc((void **)&g->by_rank, sizeof(int32_t) * n);
         dalloc((void **)&g->cls_off, sizeof(int64_t) * 65);
         ck(launch_by_rank(g->dg(), num_labels, g->cls_size, g->cls_off, g->by_rank, st), "rank table");
+        ck(cudaMemcpyAsync(g->cls_host, g->cls_size, sizeof(g->cls_host), cudaMemcpyDeviceToHost, st), "copy");
         ck(cudaStreamSynchronize(st), "sync");
         *out = g;
         return FSM_OK;
@@ -1385,7 +1470,7 @@ int fsm_mine(fsm_graph *g, int32_t k, int64_t min_support, double sample_rate, f
         {
             Arena mem(st);
             mem.fail_at = g->fail_alloc_after;
-            ck(launch_stamp_time(g->stats + 4, st), "time stamp");
+            ck(launch_stamp_time(g->stats + S_START, st), "time stamp");
             Miner m{g, st, mem, min_support, rs};
             m.V = V;
             if (g->profile) {
@@ -1583,7 +1668,7 @@ void fsm_free_result(fsm_result *r) { delete r; }
 void fsm_free_graph(fsm_graph *g) {
     if (!g) return;
     cudaStream_t st = g->stream ? g->stream : g->own_stream;
-    void *ps[] = {g->row_ptr, g->col, g->labels, g->rank, g->cls_size, g->end_off, g->piece_cnt, g->tri_off, g->tri_bits, g->err, g->stats,
+    void *ps[] = {g->row_ptr, g->col, g->labels, g->rank, g->cls_size, g->end_off, g->piece_cnt, g->tri_off, g->tri_bits, g->stats,
                   g->by_rank, g->cls_off, g->vinfo, g->linfo};
     for (void *p : ps)
         if (p) cudaFreeAsync(p, st);

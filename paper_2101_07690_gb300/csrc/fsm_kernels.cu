@@ -529,16 +529,22 @@ __global__ void pattern_counts_kernel(const int64_t *slots, int64_t nq, const in
 
 __global__ void domain_sizes_kernel(int K, const unsigned long long *pat_lab, const uint64_t *orbit,
                                     const int32_t *min_orbit, const unsigned long long *pat_count, int64_t np,
-                                    int64_t t, const int32_t *cls_size, int shift, uint8_t *live, int64_t *words) {
+                                    int64_t t, const int32_t *cls_size, int shift, uint8_t *live, int64_t *words,
+                                    unsigned long long *n_live) {
+    unsigned alive = 0;
     for (int64_t P = gtid(); P < np; P += gstride()) {
         const bool lv = (unsigned long long)min_orbit[P] * pat_count[P] >= (unsigned long long)t;
         live[P] = lv ? 1 : 0;
+        alive += lv;
         for (int c = 0; c < FSM_MAXK; ++c) {
             int64_t w = 0;
             if (lv && c < K && nib_get(orbit[P], c) == c) w = bitmap_words(cls_size[clab_get(pat_lab[P], c)], shift);
             words[P * FSM_MAXK + c] = w;
         }
     }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) alive += __shfl_xor_sync(0xffffffffu, alive, o);
+    if ((threadIdx.x & 31) == 0 && alive) atomicAdd(n_live, (unsigned long long)alive);
 }
 
 __global__ void domain_offsets_kernel(const int64_t *words, const int64_t *scanned, int64_t n8, int64_t *off) {
@@ -690,11 +696,11 @@ cudaError_t launch_pattern_counts(const int64_t *slots, int64_t nq, const int32_
 cudaError_t launch_domain_sizes(int K, const unsigned long long *pat_lab, const uint64_t *orbit,
                                 const int32_t *min_orbit, const unsigned long long *pat_count,
                                 int64_t np, int64_t t, const int32_t *cls_size, int shift, uint8_t *live,
-                                int64_t *words, cudaStream_t st) {
+                                int64_t *words, unsigned long long *n_live, cudaStream_t st) {
     if (np <= 0) return cudaSuccess;
     LAUNCHED(1);
     domain_sizes_kernel<<<blocks_for(np), kThreads, 0, st>>>(K, pat_lab, orbit, min_orbit, pat_count, np, t,
-                                                           cls_size, shift, live, words);
+                                                           cls_size, shift, live, words, n_live);
     return cudaGetLastError();
 }
 

@@ -85,7 +85,7 @@ cudaError_t launch_pattern_counts(const int64_t *slots, int64_t nq, const int32_
 cudaError_t launch_domain_sizes(int K, const unsigned long long *pat_lab, const uint64_t *orbit,
                                 const int32_t *min_orbit, const unsigned long long *pat_count,
                                 int64_t np, int64_t t, const int32_t *cls_size, int shift, uint8_t *live,
-                                int64_t *words, cudaStream_t st);
+                                int64_t *words, unsigned long long *n_live, cudaStream_t st);
 // offsets from the scanned sizes (-1 where no bitmap)
 cudaError_t launch_domain_offsets(const int64_t *words, const int64_t *scanned, int64_t n8, int64_t *off,
                                   cudaStream_t st);
