@@ -17,7 +17,8 @@
 //   segments   A unit's pieces are rows of sorted lists: centre row y (anchor b = y-th neighbour of
 //              v, partners a = the neighbours before it) and end list a (anchor a, partners b in
 //              N(a)).  One lane prepares one row: the slots its anchor allows its partner cut the
-//              row to a range (a row with none costs nothing more), and the anchor's label, cross
+//              row to a range, rows of anchors that allow none are not in the unit's row ranges at
+//              all, and the anchor's label, cross
 //              edges and pruning bits are found once for the whole row.
 //   filter     Lanes then walk the surviving ranges side by side: one coalesced list read (with the
 //              labels and ranks, which lie in an array beside the lists), the
@@ -37,7 +38,7 @@
 //   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   123 ms
 //   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,   9.6 ms
 //   5 -> 7, count, ST 8 quotas, 6.0e8 pieces, 1.2e8 joins:          248 ms,  60.6 ms,  25.3 ms
-//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   4.6 ms
+//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   4.2 ms
 // The block tables missed 70 to 77 % of the lookups of levels 1 and 2, and their flushes made warps
 // wait for each other; a record read at the L2 costs each join one latency and no barrier.  What is
 // left is bound by scattered requests (2 -> 4: load-store unit 66 %, L2 58 % busy) and, where the body
@@ -134,7 +135,7 @@ template <int L, bool QUOTA> struct UnitRec {
     static constexpr int U = L == 1 ? 16 : 8;
     static constexpr int BLOOM = L <= 3 ? 256 : 512;
     static constexpr int RP = 0, D = 1, PID = 2, META = 3, CLS = 4, OLAB = 5, OPP = 6, SEG = 7, SLO = 8, RLO = 9,
-                         RHI = 11, NC = 13, SS = 15, BND = SS + L, RK = BND + L, OB = RK + L, OE = OB + O, OK = OE + O,
+                         RHI = 11, NC = 13, SCN = 15, SEO = 16, SS = 17, BND = SS + L, RK = BND + L, OB = RK + L, OE = OB + O, OK = OE + O,
                          VB = OK + 6 * O, VE = VB + 1, QA = VE + 1, END = QA + (QUOTA ? 6 : 0);
     static constexpr int UW = END | 1;               // odd stride: lanes on different units hit different banks
 };
@@ -764,14 +765,40 @@ struct Joiner {
                 nseg = (int)(hi > lo ? hi - lo : 0);   // candidates of this unit in the chunk
                 r[R::SLO] = 0;
             } else {
-                int s0 = 0, s1 = 0;
+                // rows of the chunk: centre rows [c0, c1), end lists [e0, e1)
+                int32_t c0 = 0, c1 = 0, e0 = 0, e1 = 0;
                 if (hi > lo) {
-                    s0 = lo <= 0 ? 0 : lo < nc ? centre_row(lo, cpos, d) : d + end_row(g.pend + rp, d, lo - nc);
-                    s1 = hi >= ue - ub ? 2 * d : hi - 1 < nc ? centre_row(hi - 1, cpos, d) + 1
-                                                             : d + end_row(g.pend + rp, d, hi - 1 - nc) + 1;
+                    if (lo < nc) {
+                        c0 = lo <= 0 ? 0 : centre_row(lo, cpos, d);
+                        c1 = hi >= nc ? d : centre_row(hi - 1, cpos, d) + 1;
+                    }
+                    if (hi > nc) {
+                        e0 = lo <= nc ? 0 : end_row(g.pend + rp, d, lo - nc);
+                        e1 = hi >= ue - ub ? d : end_row(g.pend + rp, d, hi - 1 - nc) + 1;
+                    }
+                    // and of those only the anchors in slots that allow some partner (1 -> 3: every row
+                    // whose anchor is below the key vertex goes; 3.7M vertices, count 4.56 -> 4.18 ms)
+#pragma unroll 1
+                    for (int k = 0; k < 2; ++k) {
+                        int a0 = SL, a1 = -1;
+#pragma unroll 1
+                        for (int t = 0; t < SL; ++t) {
+                            uint32_t ok = allowed(r, k == 0, t);
+                            if (k == 0) ok &= (1u << SL) - 1u;
+                            if (ok) { a0 = min(a0, t); a1 = t; }
+                        }
+                        const int32_t p0 = a1 < 0 ? d : a0 > 0 ? (int32_t)r[R::BND + a0 - 1] : 0;
+                        const int32_t p1 = a1 < L ? (a1 < 0 ? 0 : (int32_t)r[R::BND + a1]) : d;
+                        if (k == 0) { c0 = max(c0, p0); c1 = min(c1, p1); }
+                        else { e0 = max(e0, p0); e1 = min(e1, p1); }
+                    }
                 }
-                r[R::SLO] = (uint32_t)s0;
-                nseg = s1 - s0;
+                c1 = max(c1, c0);
+                e1 = max(e1, e0);
+                r[R::SLO] = (uint32_t)c0;
+                r[R::SCN] = (uint32_t)(c1 - c0);
+                r[R::SEO] = (uint32_t)e0;
+                nseg = (c1 - c0) + (e1 - e0);
             }
         }
         int inc = nseg;
@@ -840,10 +867,10 @@ struct Joiner {
             if (gi < total_seg) {
                 const int j = unit_of(gi, nu);
                 const uint32_t *r = rec(j);
-                const int row = gi - (int)r[R::SEG] + (int)r[R::SLO];
+                const int row = gi - (int)r[R::SEG], ncr = (int)r[R::SCN];
                 const int32_t rp = (int32_t)r[R::RP], d = (int32_t)r[R::D];
-                const bool centre = row < d;
-                const int32_t y = centre ? row : row - d;
+                const bool centre = row < ncr;
+                const int32_t y = centre ? (int32_t)r[R::SLO] + row : (int32_t)r[R::SEO] + row - ncr;
                 if (A.debug && (y < 0 || y >= d)) {
                     atomicOr(A.err, FSM_ERR_BOUNDS);
                 } else {
