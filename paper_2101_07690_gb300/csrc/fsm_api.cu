@@ -874,7 +874,7 @@ struct Miner {
             // every pattern has its orbit bitmaps in the pool already: MNI from there
             rs.live = np;
             ck(launch_fused_support(K, plab, padj, orbit, np, ckeys, coff, (uint64_t)cap - 1, G->cls_size, shift, pool,
-                                    sigma, st), "fused support");
+                                    G->n, G->NL, sigma, st), "fused support");
             if (G->profile) rs.pass_bytes[L][PASS_FUSED] += rs.final_accepted * 4 * K;   // one bitmap word per position
         } else {
             int64_t nwords = 0;
@@ -929,7 +929,7 @@ struct Miner {
                     rs.pass_bytes[L][PASS_DOMAIN] += joins * 4 * K;
                 }
             }
-            ck(launch_support(K, orbit, live, doff, words, dom, np, sigma, st), "support");
+            ck(launch_support(K, orbit, live, doff, words, dom, np, G->n, G->NL, sigma, st), "support");
         }
         if (pool) {
             mem.release(pool);

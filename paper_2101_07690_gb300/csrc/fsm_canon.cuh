@@ -323,10 +323,10 @@ static __host__ __device__ __noinline__ uint32_t canon7(int K, const int *lab, c
     return best;
 }
 
-// Is there an automorphism taking vertex a to vertex b?  cand: byte h = the vertices h may go to
-// (same label and degree).  Vertices are placed one by one; every placement cuts the others'
-// candidates to those with the right adjacency to it.
-FSM_HD bool aut7(int K, uint64_t R, uint64_t cand, int a, int b) {
+// Automorphisms of a graph of K <= 7 vertices, those taking vertex a to vertex b only when a >= 0; stops
+// at `most`.  cand: byte h = the vertices h may go to (same label and degree).  Vertices are placed one
+// by one; every placement cuts the others' candidates to those with the right adjacency to it.
+FSM_HD int64_t place7(int K, uint64_t R, uint64_t cand, int a, int b, int64_t most) {
     auto put = [&](uint64_t cd, int u, int x) -> uint64_t {
         const uint64_t ones = 0x0101010101010101ull;
         const uint64_t next = (((uint64_t)byte_of(R, u) * 0x0002040810204081ull) & ones) * 0xffull;   // bytes of u's neighbours
@@ -335,25 +335,31 @@ FSM_HD bool aut7(int K, uint64_t R, uint64_t cand, int a, int b) {
     };
     uint64_t cd[7];
     uint32_t op[7];
-    uint32_t todo = ((1u << K) - 1u) & ~(1u << a);
-    cd[0] = put(cand, a, b);
+    uint32_t todo = (1u << K) - 1u;
+    cd[0] = cand;
+    if (a >= 0) {
+        todo &= ~(1u << a);
+        cd[0] = put(cand, a, b);
+    }
+    if (!todo) return 1;
     int d = 0;
-    uint32_t seq = 0;                                    // vertex placed at depth d in bits 4d..4d+3
-    if (!todo) return true;
-    int u = low_bit(todo);
-    seq = (uint32_t)u;
-    op[0] = byte_of(cd[0], u);
+    int64_t found = 0;
+    uint32_t seq = (uint32_t)low_bit(todo);              // vertex placed at depth d in bits 4d..4d+3
+    op[0] = byte_of(cd[0], low_bit(todo));
     for (;;) {
         if (!op[d]) {
-            if (--d < 0) return false;
+            if (--d < 0) return found;
             todo |= 1u << ((seq >> (4 * d)) & 15u);
             continue;
         }
         const int x = low_bit(op[d]);
         op[d] &= op[d] - 1;
-        u = (int)((seq >> (4 * d)) & 15u);
+        const int u = (int)((seq >> (4 * d)) & 15u);
         const uint32_t rest = todo & ~(1u << u);
-        if (!rest) return true;
+        if (!rest) {
+            if (++found >= most) return found;
+            continue;
+        }
         const uint64_t nx = put(cd[d], u, x);
         todo = rest;
         ++d;
@@ -364,20 +370,30 @@ FSM_HD bool aut7(int K, uint64_t R, uint64_t cand, int a, int b) {
     }
 }
 
-// Orbit representatives of a labeled graph of K <= 7 vertices (see orbit_reps).
-static __host__ __device__ __noinline__ void orbits7(int K, const int *lab, const uint32_t *adj, int *rep) {
-    const uint64_t R = rows_word(K, adj);
+FSM_HD uint64_t candidates7(int K, const int *lab, const uint32_t *adj) {
     uint64_t cand = 0;
     for (int c = 0; c < K; ++c)
         for (int x = 0; x < K; ++x)
             if (lab[c] == lab[x] && popc32(adj[c]) == popc32(adj[x])) cand |= 1ull << (8 * c + x);
+    return cand;
+}
+
+// Number of automorphisms of a labeled graph of K <= 7 vertices.
+FSM_HD int64_t automorphisms7(int K, const int *lab, const uint32_t *adj) {
+    return place7(K, rows_word(K, adj), candidates7(K, lab, adj), -1, -1, 1 << 30);
+}
+
+// Orbit representatives of a labeled graph of K <= 7 vertices (see orbit_reps).
+static __host__ __device__ __noinline__ void orbits7(int K, const int *lab, const uint32_t *adj, int *rep) {
+    const uint64_t R = rows_word(K, adj);
+    const uint64_t cand = candidates7(K, lab, adj);
     for (int c = 0; c < K; ++c) {
         rep[c] = c;
         for (uint32_t t = byte_of(cand, c) & ((1u << c) - 1u); t; t &= t - 1) {
             const int x = low_bit(t);
             if (rep[x] != x) continue;
             const bool twin = (adj[c] & ~(1u << x)) == (adj[x] & ~(1u << c));
-            if (twin || aut7(K, R, cand, c, x)) { rep[c] = x; break; }
+            if (twin || place7(K, R, cand, c, x, 1)) { rep[c] = x; break; }
         }
     }
 }

@@ -271,7 +271,18 @@ static __device__ __noinline__ void resolve_slot(const ResolveArgs A, int64_t sl
     if (ci < 0) { atomicOr(A.err, FSM_ERR_CODE_FULL); return; }
     unsigned long long off = __ldcg(A.code_off + ci);
     if (off == 0ull) {
-        const unsigned long long res = atomicAdd(A.pool_top, (unsigned long long)words);
+        // one reservation for the lanes here together: the bulk resolution makes hundreds of thousands
+        const unsigned am = __activemask();
+        const int lane = threadIdx.x & 31, leader = __ffs(am) - 1;
+        unsigned long long before = 0, sum = 0;
+        for (unsigned m = am; m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            const unsigned long long x = __shfl_sync(am, (unsigned long long)words, src);
+            if (src < lane) before += x;
+            sum += x;
+        }
+        unsigned long long res = lane == leader ? atomicAdd(A.pool_top, sum) : 0ull;
+        res = __shfl_sync(am, res, leader) + before;
         if (res + (unsigned long long)words > A.pool_words) { atomicOr(A.err, FSM_ERR_POOL); return; }
         const unsigned long long old = atomicCAS(A.code_off + ci, 0ull, res + 1ull);
         off = old ? old : res + 1ull;

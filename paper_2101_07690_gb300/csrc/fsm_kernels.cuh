@@ -91,7 +91,7 @@ cudaError_t launch_domain_offsets(const int64_t *words, const int64_t *scanned, 
                                   cudaStream_t st);
 // MNI support: sigma[P] = min over orbit bitmaps of popcount (0 for non-live patterns)
 cudaError_t launch_support(int K, const uint64_t *orbit, const uint8_t *live, const int64_t *dom_off,
-                           const int64_t *words, const uint32_t *dom, int64_t np,
+                           const int64_t *words, const uint32_t *dom, int64_t np, int64_t n, int labels,
                            unsigned long long *sigma, cudaStream_t st);
 // frequent flags (sigma >= t) as int64 0/1 for scanning, and the new ids afterwards
 cudaError_t launch_freq_flags(const unsigned long long *sigma, int64_t np, int64_t t, int64_t *flag,
@@ -197,8 +197,8 @@ cudaError_t launch_stamp_time(unsigned long long *out, cudaStream_t st);
 // P's bitmap block, found through its entry in the code table (ckeys / coff, cmask + 1 slots)
 cudaError_t launch_fused_support(int K, const unsigned long long *plab, const uint64_t *padj, const uint64_t *orbit,
                                  int64_t np, const unsigned long long *ckeys, const unsigned long long *coff,
-                                 uint64_t cmask, const int32_t *cls_size, int shift, const uint32_t *pool,
-                                 unsigned long long *sigma, cudaStream_t st);
+                                 uint64_t cmask, const int32_t *cls_size, int shift, const uint32_t *pool, int64_t n,
+                                 int labels, unsigned long long *sigma, cudaStream_t st);
 
 // Domain pass helper: for every distinct key (slot) and local position h, the word offset of
 // the bitmap its vertex goes to (the orbit of canonical position perm[h] of its pattern), or -1
