@@ -120,13 +120,14 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
  *                past half is grown x4 and its pass repeated (stat "qp_grows"); results are
  *                identical.
  *   "fused"      1 = the last level of exact mining (k <= 7) is enumerated once: each accepted
- *                join is counted under its quick pattern and sets its MNI domain bits at once;
- *                the first lane to meet a quick pattern canonicalises it and claims its
- *                pattern's orbit bitmaps (every pattern gets bitmaps, frequent or not); 0 = a
- *                count pass, canonicalisation, then a domain pass for the patterns that can
- *                still reach t (default).  Identical results; when the bitmap pool or the pattern
- *                table runs out, the level is counted again and finished in two passes (stat
- *                "fused_fallbacks").
+ *                join is counted under its quick pattern and sets its MNI domain bits at once.  A
+ *                sample of the level finds most quick patterns first; they are canonicalised and given
+ *                their patterns' orbit bitmaps (every pattern gets bitmaps, frequent or not); joins of
+ *                the others are put aside and entered after the level.  0 = a count pass,
+ *                canonicalisation, then a domain pass for the patterns that can still reach t
+ *                (default).  Identical results; when the bitmap pool, the pattern table or the space
+ *                for joins put aside runs out, the level is counted again and finished in two passes
+ *                (stat "fused_fallbacks").
  *   "fused_pool" size in 32-bit words of the one-pass level's bitmap pool (0 = twice what a sample of
  *                the level or the previous call needed, grown on demand up to 40% of the free device
  *                memory).
@@ -233,7 +234,8 @@ int fsm_result_features(const fsm_result *r, float *features);
  *   tested), "embeddings" (accepted joins, all levels),
  *   "final_embeddings" (accepted joins of the last level), "qp_grows" (quick-pattern table
  *   overflows, each a grown table and a repeated pass), "fused_fallbacks" (one-pass last levels
- *   redone in two passes), "fused_pool_words" (bitmap pool words the one-pass level used),
+ *   redone in two passes), "fused_pool_words" (bitmap pool words the one-pass level used), "fused_deferred" (its joins
+ *   whose quick patterns its sample had not met, entered after the level),
  *   "quick_patterns" (distinct index
  *   based quick patterns, i.e. canonicalisations, all levels), "patterns" (distinct patterns
  *   of the last level), "live_patterns" (last-level patterns given a domain),

@@ -237,7 +237,7 @@ template <class T> struct Unset : std::allocator<T> {
 };
 template <class T> using HostArray = std::vector<T, Unset<T>>;
 
-enum { S_TESTED, S_ACCEPTED, S_PIECES, S_KEYS, S_ERR, S_POOL, S_LIVE, S_WORDS, S_FREQ, S_SUM, S_WROTE, S_START, S_COUNT };
+enum { S_TESTED, S_ACCEPTED, S_PIECES, S_KEYS, S_ERR, S_POOL, S_DEFER, S_LIVE, S_WORDS, S_FREQ, S_SUM, S_WROTE, S_START, S_COUNT };
 
 struct fsm_result {
     int k = 0;
@@ -271,6 +271,7 @@ struct RunStats {
     int64_t recount_patterns = 0, recount_frontier = 0, candidates_sampled = 0, sampled_edges = 0;
     int64_t qp_grows = 0;                  // quick-pattern table overflows (table grown x4, pass repeated)
     int64_t fused_fallbacks = 0;           // one-pass last levels redone as two passes (pool or table full)
+    int64_t fused_deferred = 0;            // joins of the one-pass level whose keys its sample missed
     int64_t fused_pool_words = 0;          // bitmap pool words the one-pass last level used
     int64_t pieces_l[FSM_MAXL + 1] = {};   // pieces enumerated by the count pass, per extended level size
     double pass_ns[FSM_MAXL + 1][4] = {};
@@ -711,13 +712,15 @@ struct Miner {
             slots = nullptr;
         };
         auto clear_pass1 = [&]() {
-            // all-ones: empty keys, empty codes; zero: counts, code offsets; scalars up to the pool top
+            // all-ones: empty keys, empty codes; zero: counts, code offsets; scalars up to the deferred joins
             ck(cudaMemsetAsync(keys, 0xff, sizeof(unsigned long long) * cap * (fused ? 2 : 1), st), "memset");
             ck(cudaMemsetAsync(zeros, 0, sizeof(unsigned long long) * (cap * (fused ? 2 : 1) + 1), st), "memset");
-            ck(cudaMemsetAsync(G->stats, 0, sizeof(unsigned long long) * (S_POOL + 1), st), "memset");
+            ck(cudaMemsetAsync(G->stats, 0, sizeof(unsigned long long) * (S_DEFER + 1), st), "memset");
             if (fused) ck(cudaMemsetAsync(krec, 0xff, sizeof(uint32_t) * cap * rec_words, st), "memset");
         };
         Scalars sc;
+        // pieces of the level, an upper bound where the host does not know them
+        const unsigned long long pieces = pre.total >= 0 ? (unsigned long long)pre.total : 1ull << 32;
         for (;;) {
             // the pattern (code) table has as many slots as the quick-pattern table, so it is at most
             // half full whenever that one is
@@ -758,11 +761,12 @@ struct Miner {
                 clear_pass1();
             }
             if (fused) {
-                // Keys met for the first time are canonicalised by the lane that meets them, while
-                // the warps that meet them meanwhile do the same again.  Most are found by a sample
-                // of the pieces first and resolved with full warps (74k vertices, k = 5, 324k keys:
-                // 6.1M resolutions in the level and 59 ms without, 79k and 30.5 + 1.1 ms with it;
-                // 370 vertices, 451k keys: 5.2 ms without, 0.57 + 0.44 ms with it).
+                // A sample of the pieces finds most keys; they are resolved (canonicalised, given
+                // bitmaps) with full warps before the level.  Joins of the others are put aside and
+                // their keys resolved after it.  Resolving them in the level, by the lane that met one
+                // first, made the warps that met it meanwhile do the same again (74k vertices, 324k
+                // keys: 6.1M resolutions and 59 ms without a sample) and cost every join the
+                // registers of that path (2 -> 4 one pass: 121 ms with it, 113 ms without; 3 -> 5: 22.0 and 19.1).
                 ExtArgs W = A;
                 W.warm = 1;
                 W.stats = nullptr;
@@ -789,11 +793,24 @@ struct Miner {
                 pool = (uint32_t *)pp;
                 mem.ptrs.push_back(pp);
                 A.pool = pool;
+                A.defer_top = G->stats + S_DEFER;
+                // 32 bytes each; past 2^24 the level is redone in two passes
+                A.defer_cap = std::min<unsigned long long>(1ull << 24, std::max<unsigned long long>(1ull << 18, pieces / 8));
+                A.defer = mem.get<uint32_t>((int64_t)A.defer_cap * FSM_DEFER_WORDS);
                 ck(cudaMemsetAsync(pool, 0, pool_words * 4, st), "memset");
             }
             run_pass(fused ? PASS_FUSED : PASS_COUNT, in, A, pat_off, pre);
             ck(launch_qp_compact(keys, cap, slots, G->stats + S_KEYS, st), "compact");
             sc = scalars();
+            if (fused && sc[S_DEFER] > 0 && !sc.err()) {
+                ck(launch_resolve_keys(A, G->sms, st), "resolve keys");
+                ck(launch_deferred_bits(A, G->sms, st), "deferred joins");
+                rs.launches += 2;
+                sc = scalars();
+            }
+            if (fused) rs.fused_deferred = (int64_t)sc[S_DEFER];
+            if (A.defer) mem.release(A.defer);
+            A.defer = nullptr;
             const int ew = sc.err();
             if (ew & (FSM_ERR_TIMEOUT | FSM_ERR_BOUNDS)) fail_word(ew);
             if (ew && pool) {
@@ -1575,6 +1592,7 @@ int fsm_mine(fsm_graph *g, int32_t k, int64_t min_support, double sample_rate, f
         r->stats["qp_grows"] = rs.qp_grows;
         r->stats["fused_fallbacks"] = rs.fused_fallbacks;
         r->stats["fused_pool_words"] = rs.fused_pool_words;
+        r->stats["fused_deferred"] = rs.fused_deferred;
         for (int L = 1; L <= FSM_MAXL; ++L) r->stats["chunk_l" + std::to_string(L)] = g->tuned_chunk[L];
         for (int L = 1; L <= FSM_MAXL; ++L) r->stats["pieces_l" + std::to_string(L)] = rs.pieces_l[L];
         const char *pn[4] = {"count", "domain", "emit", "fused"};

@@ -2,8 +2,8 @@
 //
 // The same canonical form as fsm_canon.cuh (canon7, orbits7) in compact words: label bytes (byte
 // 7 - c holds canonical position c), a 32-bit adjacency word (at most 21 pair bits, first pair most
-// significant) and 3-bit vertex orders, with 8-entry scratch arrays.  The one-pass kernel calls
-// only these on first sight of a quick pattern.  The host build of tests/device_helpers_check.cu
+// significant) and 3-bit vertex orders, with 8-entry scratch arrays.  The one-pass level's bulk
+// resolution (fsm_join_fused.cu) calls these.  The host build of tests/device_helpers_check.cu
 // checks them against fsm_canon.cuh.
 #pragma once
 #include "fsm_canon.cuh"

@@ -17,11 +17,9 @@
 //   PASS_COUNT   insert the key into the quick-pattern table and count it;
 //   PASS_DOMAIN  set the MNI domain bits of its pattern's orbits (Definition 2);
 //   PASS_EMIT    write it, permuted into canonical order, to the next frontier;
-//   PASS_FUSED   (last level, k <= 7) count it and set the MNI domain bits of its pattern's
-//                orbits in the same enumeration: the lane that first meets a quick pattern
-//                canonicalises it, claims its pattern's orbit bitmaps (one CAS on the pattern's
-//                entry in a table of canonical codes) and publishes the bitmap word offset of
-//                every local position; nothing waits on another lane.
+//   PASS_FUSED   (last level, k <= 7; fsm_join.cuh only) count it and set the MNI domain bits of its
+//                pattern's orbits in the same enumeration, for keys that a sample has resolved; joins
+//                of other keys are put aside and entered after the level.
 //
 // Scheduling: the pieces of a batch of units form one index space [0, total) (exclusive prefix
 // `unit_base`); warps take fixed-size chunks of it from an atomic counter, so hub vertices
@@ -48,6 +46,7 @@ struct QPTab {
 // all ones and is written once with its final value, so a reader that sees the key and no all-ones
 // offset has the whole record, whatever the order it saw the words in.
 FSM_HD constexpr int key_rec_words(int K) { return K <= 6 ? 8 : 16; }
+#define FSM_DEFER_WORDS 8
 #define FSM_OFF_NONE 0xFFFFFFFFu     // word of a key record not yet published, or no bitmaps
 
 struct ExtArgs {
@@ -90,6 +89,11 @@ struct ExtArgs {
     uint64_t code_mask;
     uint32_t *key_rec;             // [cap] key records (fsm_join.cuh)
     int off_shift;
+    // one-pass level: joins whose key had no record yet, FSM_DEFER_WORDS words each (key slot, rank of
+    // every local position)
+    uint32_t *defer;
+    unsigned long long *defer_top;
+    unsigned long long defer_cap;
     int check_bits;                // read a bitmap word before reducing into it
     int warm;                      // count a sample of the chunks only (before a one-pass level)
     // tables of fsm_join.cuh for this level size, and the size-3 frequencies as label masks: W[c][x]
@@ -138,12 +142,13 @@ FSM_HD int64_t join_chunk(int64_t total, int64_t warps) {
 
 // Warm pass of a one-pass level: the keys of every warm_stride-th chunk of FSM_WARM_CHUNK pieces are
 // counted and resolved in bulk first, so that the level itself meets few keys for the first time.
-// All pieces up to 2^24 (small levels have most keys per piece), then 2^24 of them, from 2^29 on
-// one in 32: with one in 102, the level of 1.7e9 pieces met enough new keys to take 36.8 ms
-// instead of 30.5 ms, far more than the 0.7 ms that the smaller sample saved.
+// All pieces up to 2^25 (small levels have most keys per piece), then 2^25 of them, from 2^30 on
+// one in 32.  What the sample misses costs a join about ten times the others: with 36 joins a key
+// (7400 vertices, size 5, 1.8M keys), one in 15 pieces left 14 % of the joins to be entered after the
+// level; with 1000 joins a key, one in 32 leaves under 1 %.
 #define FSM_WARM_CHUNK 1024
 FSM_HD int64_t warm_stride(int64_t total) {
-    const int64_t s = total >> 24;
+    const int64_t s = total >> 25;
     return s < 1 ? 1 : s > 32 ? 32 : s;
 }
 
@@ -992,6 +997,7 @@ cudaError_t occupancy_extend_l7(int pass, int *blocks_per_sm);
 #define FSM_JOIN_MAXL 5
 cudaError_t launch_join(int pass, int L, int V, const ExtArgs &A, int grid, cudaStream_t st);
 cudaError_t launch_resolve_keys(const ExtArgs &A, int sms, cudaStream_t st);
+cudaError_t launch_deferred_bits(const ExtArgs &A, int sms, cudaStream_t st);
 cudaError_t occupancy_join(int pass, int L, int V, int *blocks_per_sm);
 // its tables for stored size L: bytes of each, and the kernels that fill them (tmp: join_tmp_bytes)
 void join_table_bytes(int L, size_t *acc, size_t *any, size_t *tmp);

@@ -34,9 +34,9 @@
 // One launch on a GB300 (same graph and output): the extension kernel before, this kernel with a
 // key table per block in shared memory (flushed between chunks) and both new vertices' tests made
 // per survivor, and as it is:
-//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms,  77.7 ms,  22.4 ms
-//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   123 ms
-//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,   9.6 ms
+//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms,  77.7 ms,  19.1 ms
+//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   113 ms
+//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,   9.4 ms
 //   5 -> 7, count, ST 8 quotas, 6.0e8 pieces, 1.2e8 joins:          248 ms,  60.6 ms,  25.3 ms
 //   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   4.2 ms
 // The block tables missed 70 to 77 % of the lookups of levels 1 and 2, and their flushes made warps
@@ -217,114 +217,11 @@ __device__ __forceinline__ int32_t end_row(const int32_t *pend, int32_t d, int64
     return lo;
 }
 
-__device__ __forceinline__ uint32_t ld_relaxed_u32(const uint32_t *p) {
-    uint32_t v;
-    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-__device__ __forceinline__ void st_relaxed_u32(uint32_t *p, uint32_t v) {
-    asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// First sight of a quick pattern in the one-pass last level: canonicalise the graph its key
-// denotes, find or claim its pattern's entry in the code table, claim the pattern's orbit
-// bitmaps from the pool unless another lane already did (one CAS decides; a loser's pool words
-// stay unused), and publish the key's record.  Lanes racing on one key compute and write the same
-// values.  On a full table or pool the error word says so and nothing is published; the host then
-// runs the last level as two passes.
-struct ResolveArgs {
-    const uint64_t *pat_lab, *pat_adj;
-    const int32_t *cls_size;
-    unsigned long long *code_keys, *code_off, *pool_top;
-    uint64_t code_mask;
-    unsigned long long pool_words;
-    uint32_t *key_rec;
-    int shift;
-    int *err;
-    int explore, level;
-};
-
-static __device__ __noinline__ void resolve_slot(const ResolveArgs A, int64_t slot, uint64_t key) {
-    // K <= 7 here: the compact words of fsm_canon7.cuh
-    int K, lab[8], rep[8];
-    uint32_t adj[8];
-    key_graph7(A.explore, A.level, key, A.pat_lab, A.pat_adj, K, lab, adj);
-    unsigned long long clab;
-    uint32_t cadj, inv;
-    canonicalise7(K, lab, adj, clab, cadj, inv);
-    orbit_reps7(K, clab, cadj, rep);
-    int64_t pre[8], words = 0;
-    for (int c = 0; c < K; ++c) {
-        pre[c] = words;
-        if (rep[c] == c)
-            words += bitmap_words(__ldg(A.cls_size + ((clab >> (8 * (7 - c))) & 0xff)), A.shift);
-    }
-    const uint64_t pk = pack_code7(K, clab, cadj);
-    uint64_t h = mix64(pk) & A.code_mask;
-    int64_t ci = -1;
-    for (int probe = 0; probe < FSM_MAX_PROBES; ++probe) {
-        unsigned long long cur = __ldcg(A.code_keys + h);
-        if (cur == FSM_EMPTY_KEY) cur = atomicCAS(A.code_keys + h, FSM_EMPTY_KEY, pk);
-        if (cur == FSM_EMPTY_KEY || cur == pk) { ci = (int64_t)h; break; }
-        h = (h + 1) & A.code_mask;
-    }
-    if (ci < 0) { atomicOr(A.err, FSM_ERR_CODE_FULL); return; }
-    unsigned long long off = __ldcg(A.code_off + ci);
-    if (off == 0ull) {
-        // one reservation for the lanes here together: the bulk resolution makes hundreds of thousands
-        const unsigned am = __activemask();
-        const int lane = threadIdx.x & 31, leader = __ffs(am) - 1;
-        unsigned long long before = 0, sum = 0;
-        for (unsigned m = am; m; m &= m - 1) {
-            const int src = __ffs(m) - 1;
-            const unsigned long long x = __shfl_sync(am, (unsigned long long)words, src);
-            if (src < lane) before += x;
-            sum += x;
-        }
-        unsigned long long res = lane == leader ? atomicAdd(A.pool_top, sum) : 0ull;
-        res = __shfl_sync(am, res, leader) + before;
-        if (res + (unsigned long long)words > A.pool_words) { atomicOr(A.err, FSM_ERR_POOL); return; }
-        const unsigned long long old = atomicCAS(A.code_off + ci, 0ull, res + 1ull);
-        off = old ? old : res + 1ull;
-    }
-    uint32_t *kr = A.key_rec + slot * key_rec_words(K);
-    for (int hh = 0; hh < K; ++hh)
-        st_relaxed_u32(kr + 2 + hh, (uint32_t)(((long long)(off - 1ull) + pre[rep[(inv >> (3 * hh)) & 7]]) >> A.shift));
-    st_relaxed_u32(kr, (uint32_t)key);
-    st_relaxed_u32(kr + 1, (uint32_t)(key >> 32));
-}
-
-// Eight words of a key record in one request: read-only in the domain pass, read at the L2 in the
-// one-pass level (an old empty copy in L1 would send its readers to the slow path until it is
-// evicted).  A join's scattered requests are what the load-store unit is busy with.
-template <int PASS> __device__ __forceinline__ void ld_rec8(const uint32_t *p, uint32_t *x) {
-    if (PASS == PASS_DOMAIN)
-        asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-            : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]) : "l"(p));
-    else
-        asm volatile("ld.relaxed.gpu.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                     : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7])
-                     : "l"(p) : "memory");
-}
-
-// First sight of a key: insert it and publish its record if nobody has.  Its slot, or -1 when a
-// table or the pool is full (the error word says so).
-template <int K>
-__device__ __noinline__ int64_t first_sight(const ExtArgs &A, uint64_t key) {
-    const int64_t slot = qp_insert(A.qp, key, A.err);
-    if (slot < 0) return -1;
-    const uint32_t *kr = A.key_rec + slot * key_rec_words(K);
-    for (int round = 0; round < 2; ++round) {
-        bool all = true;
-        for (int h = 0; h < K; ++h) all &= ld_relaxed_u32(kr + 2 + h) != FSM_OFF_NONE;
-        if (all) return slot;
-        if (round == 0) {
-            const ResolveArgs R{A.pat_lab, A.pat_adj, A.cls_size, A.code_keys, A.code_off, A.pool_top,
-                                A.code_mask, A.pool_words, A.key_rec, A.off_shift, A.err, A.explore, A.level};
-            resolve_slot(R, slot, key);
-        }
-    }
-    return -1;
+// Eight words of a key record in one request (a join's scattered requests are what the load-store unit
+// is busy with).  Records do not change during a pass.
+__device__ __forceinline__ void ld_rec8(const uint32_t *p, uint32_t *x) {
+    asm("ld.global.nc.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]) : "l"(p));
 }
 
 template <int L, int PASS, bool QUOTA>
@@ -361,17 +258,16 @@ struct Joiner {
         return (sm.bloom[w][((j * L + t) << lb) + (lb ? h >> (32 - lb) : 0u)] & k) == k;
     }
 
-    // Slot and bitmap offsets of a key from its record, looked for from `slot` (from its hash if that
-    // is negative) on; false where the key has no bitmaps or the record is not there yet.
+    // Slot and bitmap offsets of a key from its record; false where the key has no bitmaps or no record.
     __device__ __forceinline__ bool key_record(uint64_t key, int64_t &slot, uint32_t (&off)[K]) {
-        uint64_t h = slot >= 0 ? (uint64_t)slot : mix64(key) & A.qp.mask;
+        uint64_t h = mix64(key) & A.qp.mask;
         constexpr int RW = key_rec_words(K);
 #pragma unroll 1
         for (int p = 0; p < FSM_MAX_PROBES; ++p) {
             const uint32_t *kr = A.key_rec + h * RW;
             uint32_t wd[K > 6 ? 16 : 8];
-            ld_rec8<PASS>(kr, wd);
-            if (K > 6) ld_rec8<PASS>(kr + 8, wd + (K > 6 ? 8 : 0));
+            ld_rec8(kr, wd);
+            if (K > 6) ld_rec8(kr + 8, wd + (K > 6 ? 8 : 0));
             const uint64_t k = (uint64_t)wd[0] | ((uint64_t)wd[1] << 32);
             if (k == key) {
                 bool all = true;
@@ -414,6 +310,22 @@ struct Joiner {
             if ((h >= L || own) && !(old[h] & bit[h])) atomicOr(wd[h], bit[h]);
     }
 
+    // One-pass level, a key the warm pass did not meet: count the join and leave its bits for after the
+    // level, when such keys are resolved in bulk (deferred_bits_kernel).
+    __device__ __forceinline__ void defer(const uint32_t *r, uint64_t key, uint32_t r0, uint32_t r1) {
+        const int64_t slot = qp_insert(A.qp, key, A.err);
+        if (slot < 0) return;
+        atomicAdd(A.qp.count + slot, 1ull);
+        const unsigned long long at = atomicAdd(A.defer_top, 1ull);
+        if (at >= A.defer_cap) { atomicOr(A.err, FSM_ERR_CODE_FULL); return; }
+        uint32_t *d = A.defer + at * FSM_DEFER_WORDS;
+        d[0] = (uint32_t)slot;
+#pragma unroll
+        for (int h = 0; h < L; ++h) d[1 + h] = r[R::RK + h];
+        d[1 + L] = r0;
+        d[2 + L] = r1;
+    }
+
     // One accepted join of this lane (not warp-synchronous).
     __device__ __forceinline__ void accept(const uint32_t *r, int j, uint64_t key, bool centre, int32_t anchor, int32_t x,
                                            uint32_t ainfo, uint32_t xinfo, bool swap) {
@@ -423,10 +335,12 @@ struct Joiner {
         } else if constexpr (PASS == PASS_FUSED || PASS == PASS_DOMAIN) {
             uint32_t off[K];
             int64_t slot = -1;
-            while (!key_record(key, slot, off)) {
-                if (PASS == PASS_DOMAIN) return;   // pattern without bitmaps
-                slot = first_sight<K>(A, key);     // published now, so the next look finds it
-                if (slot < 0) return;
+            const uint32_t ranchor = A.g.packed ? ainfo >> 6 : (uint32_t)__ldg(A.g.rank + anchor);
+            const uint32_t rx = A.g.packed ? xinfo >> 6 : (uint32_t)__ldg(A.g.rank + x);
+            const uint32_t ra = centre ? rx : ranchor, rb = centre ? ranchor : rx;
+            if (!key_record(key, slot, off)) {
+                if (PASS == PASS_FUSED) defer(r, key, swap ? rb : ra, swap ? ra : rb);
+                return;   // domain pass: pattern without bitmaps
             }
             if (PASS == PASS_FUSED) atomicAdd(A.qp.count + slot, 1ull);
             // A unit's joins of one key set the same bits of s: a small table of (unit, slot) pairs
@@ -439,9 +353,7 @@ struct Joiner {
                 own = *(volatile uint32_t *)sn != tag;
                 if (own) *(volatile uint32_t *)sn = tag;
             }
-            const uint32_t ranchor = A.g.packed ? ainfo >> 6 : (uint32_t)__ldg(A.g.rank + anchor);
-            const uint32_t rx = A.g.packed ? xinfo >> 6 : (uint32_t)__ldg(A.g.rank + x);
-            set_bits(off, r, centre ? rx : ranchor, centre ? ranchor : rx, swap, own);
+            set_bits(off, r, ra, rb, swap, own);
         } else {
             const int64_t slot = qp_find(A.qp, key);
             if (slot < 0) { atomicOr(A.err, FSM_ERR_QP_MISSING); return; }
@@ -1052,11 +964,11 @@ struct Joiner {
 };
 
 // Resident blocks per SM: four (64 registers) hide more latency in the count and emission passes
-// (3.7M vertices, 1 -> 3: 5.2 ms against 6.1 ms with three) and in the domain pass up to l = 3 (11.4
-// and 12.6 ms); the one-pass level and the domain passes of l = 4 and 5 spill too much at 64
-// registers (4 -> 6: 14.5 and 13.7 ms; 2 -> 4 one pass: 157 and 131 ms).
+// (3.7M vertices, 1 -> 3: 5.2 ms against 6.1 ms with three) and in the domain pass and the one-pass
+// level up to l = 3 (domain 11.4 and 12.6 ms); those of l = 4 and 5 spill too much at 64 registers
+// (4 -> 6 domain pass: 14.5 and 13.7 ms).
 template <int L, int PASS> struct JoinBlocks {
-    static constexpr int value = PASS == PASS_FUSED || (PASS == PASS_DOMAIN && L >= 4) ? 3 : 4;
+    static constexpr int value = (PASS == PASS_FUSED || PASS == PASS_DOMAIN) && L >= 4 ? 3 : 4;
 };
 
 template <int L, int PASS, bool QUOTA>

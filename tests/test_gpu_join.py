@@ -59,3 +59,25 @@ def test_join_kernel_matches_oracle(fsm, case, mode):
             G.close()
             for key in ("labels", "adj", "support", "count"):
                 assert np.array_equal(got[key], exp[key]), (k, opts, key)
+
+
+@pytest.mark.parametrize("mode", ["edge", "vertex"])
+@pytest.mark.parametrize("k,scale", [(5, 0.002), (4, 0.1), (3, 0.3)])
+def test_one_pass_level_with_keys_its_sample_missed(fsm, k, scale, mode):
+    """Levels large enough that the one-pass form samples their pieces first (more than 2^26): joins
+    whose keys the sample missed are put aside and entered after the level.  Same result as the count
+    and domain passes, also when the bitmap pool runs out on the way."""
+    g = gg.workload("cl3700k", scale=scale, cap=20)
+    t = max(2, g.n // 400)
+    out = []
+    for opts in ({"fused": 0}, {"fused": 1}, {"fused": 1, "launch": 1}, {"fused": 1, "fused_pool": 1 << 20}):
+        G = fsm.Graph.from_graphgen(g, mode)
+        for key, val in opts.items():
+            G.set_option(key, val)
+        out.append(G.mine(k, t, stats=True))
+        G.close()
+    assert out[0]["stats"]["pieces"] >> 26 and len(out[0]["support"]) > 0
+    assert out[1]["stats"]["fused_fallbacks"] == 0 and out[1]["stats"]["fused_deferred"] > 0
+    for got in out[1:]:
+        for key in ("labels", "adj", "support", "count"):
+            assert np.array_equal(got[key], out[0][key]), key
