@@ -1,4 +1,5 @@
-// fsm_join_fused.cu -- instantiations of the join kernel (stored sizes 1..5) for PASS_FUSED.
+// fsm_join_fused.cu -- the one-pass last level: instantiations of the join kernel (stored sizes 1..5) for
+// PASS_FUSED, the bulk resolution of its keys, and the bits of the joins it put aside.
 #include "fsm_join.cuh"
 
 namespace fsm {
@@ -9,10 +10,10 @@ cudaError_t join_fused(int L, const ExtArgs *A, int grid, cudaStream_t st, int *
 
 namespace {
 
-// Resolve a key of the one-pass last level: canonicalise the graph its key denotes, find or claim its pattern's entry in the code table, claim the pattern's orbit
-// bitmaps from the pool unless another lane already did (one CAS decides; a loser's pool words
-// stay unused), and publish the key's record.  On a full table or pool the error word says so and nothing is published; the host then
-// runs the last level as two passes.
+// Resolve a key of the one-pass last level: canonicalise the graph its key denotes, find or claim its
+// pattern's entry in the code table, claim the pattern's orbit bitmaps from the pool unless another
+// lane already did (one CAS decides; a loser's pool words stay unused), and publish the key's record.
+// On a full table or pool the error word says so and nothing is published.
 struct ResolveArgs {
     const uint64_t *pat_lab, *pat_adj;
     const int32_t *cls_size;
