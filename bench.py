@@ -204,17 +204,17 @@ def read_peaks():
 
 
 def kernel_source_sha() -> str:
-    """sha256 prefix of the extension kernel's source: fsm_extend.cuh and the two headers it
-    compiles in (the canonicaliser and the device helpers)."""
+    """sha256 prefix of the join kernel's source: fsm_join.cuh and the headers it compiles in (the
+    extension kernel's, the canonicaliser and the device helpers)."""
     h = hashlib.sha256()
-    for f in ("fsm_extend.cuh", "fsm_canon.cuh", "fsm_device.cuh"):
+    for f in ("fsm_join.cuh", "fsm_extend.cuh", "fsm_canon7.cuh", "fsm_canon.cuh", "fsm_device.cuh"):
         h.update(open(os.path.join(ROOT, "paper_2101_07690_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
 
 def traffic_for(kernel_pass: str):
     """DRAM bytes per launch from the committed ncu summary, if it was taken on the current
-    source of the extension kernel (else None)."""
+    source of the join kernel (else None)."""
     path = os.path.join(ROOT, "profiles", "extend_traffic.json")
     if not os.path.exists(path):
         return None
@@ -407,7 +407,7 @@ def run_ours(args, rank, world, local_rank):
     ns, byts, nl = passes[dom]
     peak, peak_kind = read_peaks()
     achieved = (byts / nl) / (ns / nl) if ns > 0 and nl > 0 else 0.0   # bytes per ns == GB/s
-    roofline = {"bound": "hbm", "kernel": f"extend_kernel<{dom[1]}, PASS_{dom[0].upper()}>",
+    roofline = {"bound": "hbm", "kernel": f"join_kernel<{dom[1]}, PASS_{dom[0].upper()}>",
                 "achieved": round(achieved, 2), "peak": peak, "unit": "GB/s",
                 "frac": round(achieved / peak, 5), "peak_source": f"{peak_kind} hbm_gbs",
                 "traffic": traffic_for(f"{dom[0]}_l{dom[1]}"), "launches": nl, "avg_launch_ms": round(ns / nl / 1e6, 3) if nl else None,

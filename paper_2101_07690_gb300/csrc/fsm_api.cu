@@ -345,13 +345,13 @@ struct Miner {
         return 0;
     }
 
-    // Run one pass of the extension kernel over the frontier.
+    // Run one pass of the join (or extension) kernel over the frontier.
     //   launch 0: batches of at most `batch` embeddings, each sized on the host;
-    //   launch 1: one persistent work-stealing launch over the whole frontier (sizes stay on the
-    //             device), captured with its prefix kernels into a CUDA graph.  The per-unit piece
+    //   launch 1: one persistent work-stealing launch over the whole frontier.  The per-unit piece
     //             prefix takes 8 bytes per (embedding, key position); only when a quarter of the
     //             free device memory cannot hold it is the frontier split into the fewest equal
-    //             ranges that fit, each one launch of the same graph;
+    //             ranges that fit, each one launch, captured with its prefix kernels into one CUDA
+    //             graph (sizes stay on the device);
     //   launch 2: one launch per frontier pattern (the frontier grouped by pattern id), all
     //             captured into one CUDA graph.
     // A frontier of one range keeps its prefix for every pass of the level (`pre`), and its later passes
@@ -508,9 +508,10 @@ struct Miner {
     std::vector<int64_t> group_by_pattern(LevelSet &in) {
         std::vector<int64_t> off;
         // Per-pattern launches need the frontier grouped.  The persistent launch groups it from
-        // size 3 on (option "group" = 2): consecutive units then share the pattern, so the count
-        // pass's warp tables hit (k = 5 on the 3.7M-vertex graph: count pass -12 %).  Edges keep
-        // emission order, whose consecutive units share key vertices (measured faster there).
+        // size 3 on (option "group" = 2): consecutive units then share the pattern, and
+        // its key records and bitmaps stay in the caches (one-pass level 3 of the 3.7M-vertex graph,
+        // k = 5: at 1/10 scale 165 -> 110 ms, at 3/10 533 -> 439 ms).  Edges keep emission order,
+        // whose consecutive units share key vertices (measured faster there).
         const bool grouped = G->launch == 2 || (G->launch == 1 && (G->group == 1 || (G->group == 2 && in.L >= 3)));
         if (!grouped || in.N == 0 || in.P == 0) return off;
         int64_t *cnt = mem.get<int64_t>(in.P);
@@ -912,9 +913,6 @@ struct Miner {
             // ---- pass 2: MNI domains (Definition 2)
             A.qp.pattern = qpat;
             A.qp.perm = qperm;
-            A.live = live;
-            A.orbit = orbit;
-            A.dom_off = doff;
             A.dom = dom;
             if (joins(L)) {
                 krec = mem.get<uint32_t>(cap * rec_words);

@@ -69,9 +69,6 @@ struct ExtArgs {
     const uint8_t *piece_sel;
     QPTab qp;
     // domains (PASS_DOMAIN)
-    const uint8_t *live;           // [P'] pattern has domains
-    const uint64_t *orbit;         // [P'] orbit word: representative per canonical position
-    const int64_t *dom_off;        // [P'*FSM_MAXK] word offset per orbit representative
     uint32_t *dom;
     const int64_t *slot_base;      // [cap*FSM_MAXK] bitmap word offset per (key slot, local position), -1 none
     // emission (PASS_EMIT)

@@ -18,16 +18,14 @@
 //              v, partners a = the neighbours before it) and end list a (anchor a, partners b in
 //              N(a)).  One lane prepares one row: the slots its anchor allows its partner cut the
 //              row to a range, rows of anchors that allow none are not in the unit's row ranges at
-//              all, and the anchor's label, cross
-//              edges and pruning bits are found once for the whole row.
+//              all, and the anchor's label, cross edges and pruning bits are found once for the row.
 //   filter     Lanes then walk the surviving ranges side by side: one coalesced list read (with the
 //              labels and ranks, which lie in an array beside the lists), the
 //              partner's slot by l comparisons, one bit test.  Survivors go to a per-warp queue.
-//   joins      Full warps take 32 survivors: the
-//              size-3 frequency of the piece, cross edges (a shared-memory Bloom filter of each
-//              list of s, misses are certain, hits are verified by binary search), joining-point
-//              pruning (Section 4.5) as cross bits that must or must not be set, then the subsets
-//              that are left and accepted by `acc`.
+//   joins      Full warps take 32 survivors: the size-3 frequency of the piece, cross edges (a
+//              shared-memory Bloom filter of each list of s, misses are certain, hits are verified
+//              by binary search), joining-point pruning (Section 4.5) as cross bits that must or
+//              must not be set, then the subsets that are left and accepted by `acc`.
 //   accept     One 32-byte record per key slot holds the key and its patterns' bitmap offsets, so
 //              a join finds both in one read; counts are single reductions that nothing waits for.
 //
@@ -35,15 +33,16 @@
 // key table per block in shared memory (flushed between chunks) and both new vertices' tests made
 // per survivor, and as it is:
 //   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms,  77.7 ms,  19.1 ms
-//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   113 ms
+//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   110 ms
 //   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,   9.4 ms
 //   5 -> 7, count, ST 8 quotas, 6.0e8 pieces, 1.2e8 joins:          248 ms,  60.6 ms,  25.3 ms
 //   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   4.2 ms
 // The block tables missed 70 to 77 % of the lookups of levels 1 and 2, and their flushes made warps
 // wait for each other; a record read at the L2 costs each join one latency and no barrier.  What is
-// left is bound by scattered requests (2 -> 4: load-store unit 66 %, L2 58 % busy) and, where the body
-// is large, by instruction fetch: one copy of the joins (take) instead of two took 5 -> 7 from 55 to
-// 35 ms.
+// left is bound by issue and dependent loads (3 -> 5, one pass, 370k vertices: 9.3 warp instructions a
+// piece where the extension kernel took 80, 60 % of the issue slots, 21.7 of 32 lanes, DRAM at 3 %), by
+// scattered requests (2 -> 4: load-store unit 66 %, L2 58 % busy) and, where the body is large, by
+// instruction fetch: one copy of the joins (take) instead of two took 5 -> 7 from 55 to 35 ms.
 #pragma once
 #include "fsm_extend.cuh"
 

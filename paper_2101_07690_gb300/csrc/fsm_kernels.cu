@@ -277,10 +277,6 @@ __global__ void unit_counts_kernel(const DevGraph g, const int32_t *fv, int64_t 
     }
 }
 
-__global__ void fill_u64_kernel(unsigned long long *p, unsigned long long v, int64_t n) {
-    for (int64_t i = gtid(); i < n; i += gstride()) p[i] = v;
-}
-
 // One reservation per warp and 256 entries (the slots of the occupied ones, in any order): one per
 // key made every warp queue on the counter (11.8M keys: 1.4 ms, by 32 entries 0.8 ms).
 __global__ void qp_compact_kernel(const unsigned long long *keys, int64_t cap, int64_t *slots,
@@ -384,12 +380,6 @@ cudaError_t launch_u64_to_i64(const unsigned long long *in, int64_t *out, int64_
     if (n <= 0) return cudaSuccess;
     LAUNCHED(1);
     u64_to_i64_kernel<<<blocks_for(n), kThreads, 0, st>>>(in, out, n);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_fill_u64(unsigned long long *p, unsigned long long v, int64_t n, cudaStream_t st) {
-    LAUNCHED(1);
-    fill_u64_kernel<<<blocks_for(n), kThreads, 0, st>>>(p, v, n);
     return cudaGetLastError();
 }
 

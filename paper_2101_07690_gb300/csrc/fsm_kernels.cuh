@@ -57,7 +57,6 @@ cudaError_t launch_group_by_pattern(const int32_t *fv, const int32_t *fpid, int6
 cudaError_t launch_u64_to_i64(const unsigned long long *in, int64_t *out, int64_t n, cudaStream_t st);
 
 // ---- quick-pattern table
-cudaError_t launch_fill_u64(unsigned long long *p, unsigned long long v, int64_t n, cudaStream_t st);
 cudaError_t launch_qp_compact(const unsigned long long *keys, int64_t cap, int64_t *slots,
                               unsigned long long *n_out, cudaStream_t st);
 // canonical code of each distinct key; writes recs[q] (idx = q) and perm[slot]
