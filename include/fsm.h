@@ -235,7 +235,9 @@ int fsm_result_features(const fsm_result *r, float *features);
  *   "final_embeddings" (accepted joins of the last level), "qp_grows" (quick-pattern table
  *   overflows, each a grown table and a repeated pass), "fused_fallbacks" (one-pass last levels
  *   redone in two passes), "fused_pool_words" (bitmap pool words the one-pass level used), "fused_deferred" (its joins
- *   whose quick patterns its sample had not met, entered after the level),
+ *   whose quick patterns its sample had not met, entered after the level), "kept_levels" (levels
+ *   whose domain bits came from joins that the count pass kept instead of a second enumeration;
+ *   with option "profile", launch mode 2 and levels of several ranges none do),
  *   "quick_patterns" (distinct index
  *   based quick patterns, i.e. canonicalisations, all levels), "patterns" (distinct patterns
  *   of the last level), "live_patterns" (last-level patterns given a domain),

@@ -76,11 +76,19 @@ struct Arena {
     std::vector<void *> blocks;      // the blocks among ptrs: release() leaves their first piece alone
     char *block = nullptr;
     size_t left = 0;                 // bytes of the current block not given out
+    void *spare = nullptr;           // an allocation the call can do without: given back when one fails
     int64_t made = 0, fail_at = 0;   // fail_at > 0: the fail_at-th allocation reports failure (test hook)
     explicit Arena(cudaStream_t s) : st(s) {}
     void *raw(size_t bytes) {
         void *p = nullptr;
-        ck(cudaMallocAsync(&p, bytes, st), "device allocation");
+        cudaError_t e = cudaMallocAsync(&p, bytes, st);
+        if (e != cudaSuccess && spare) {
+            cudaGetLastError();
+            drop_spare();
+            cudaStreamSynchronize(st);
+            e = cudaMallocAsync(&p, bytes, st);
+        }
+        ck(e, "device allocation");
         ptrs.push_back(p);
         return p;
     }
@@ -109,7 +117,12 @@ struct Arena {
             ptrs.erase(it);
         }
     }
+    void drop_spare() {
+        if (spare) cudaFreeAsync(spare, st);
+        spare = nullptr;
+    }
     ~Arena() {
+        drop_spare();
         for (void *p : ptrs) cudaFreeAsync(p, st);
     }
 };
@@ -237,7 +250,7 @@ template <class T> struct Unset : std::allocator<T> {
 };
 template <class T> using HostArray = std::vector<T, Unset<T>>;
 
-enum { S_TESTED, S_ACCEPTED, S_PIECES, S_KEYS, S_ERR, S_POOL, S_DEFER, S_LIVE, S_WORDS, S_FREQ, S_SUM, S_WROTE, S_START, S_COUNT };
+enum { S_TESTED, S_ACCEPTED, S_PIECES, S_KEYS, S_ERR, S_POOL, S_KEEP, S_DEFER, S_LIVE, S_WORDS, S_FREQ, S_SUM, S_WROTE, S_START, S_COUNT };
 
 struct fsm_result {
     int k = 0;
@@ -271,6 +284,7 @@ struct RunStats {
     int64_t recount_patterns = 0, recount_frontier = 0, candidates_sampled = 0, sampled_edges = 0;
     int64_t qp_grows = 0;                  // quick-pattern table overflows (table grown x4, pass repeated)
     int64_t fused_fallbacks = 0;           // one-pass last levels redone as two passes (pool or table full)
+    int64_t kept_levels = 0;               // levels whose domain bits came from joins the count pass kept
     int64_t fused_deferred = 0;            // joins of the one-pass level whose keys its sample missed
     int64_t fused_pool_words = 0;          // bitmap pool words the one-pass last level used
     int64_t pieces_l[FSM_MAXL + 1] = {};   // pieces enumerated by the count pass, per extended level size
@@ -345,6 +359,8 @@ struct Miner {
         return 0;
     }
 
+    // Pieces from which a level keeps its joins; below, both ways take a few launches of some 20 us.
+    static constexpr int64_t kKeepPieces = 1 << 14;
     // Run one pass of the join (or extension) kernel over the frontier.
     //   launch 0: batches of at most `batch` embeddings, each sized on the host;
     //   launch 1: one persistent work-stealing launch over the whole frontier.  The per-unit piece
@@ -403,6 +419,7 @@ struct Miner {
             A.total = pre.total;
             A.chunk = (int32_t)chunk;
             A.nchunks = (pre.total + chunk - 1) / chunk;
+            if (!mem.spare) A.keep = nullptr;
             ck(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), st), "memset");
             ck(launch_pass(pass, L, A, grid), "extension kernel");
             rs.launches += 1;
@@ -676,6 +693,7 @@ struct Miner {
         // mining) also the MNI domains, in the same enumeration, when option "fused" is set
         Prefix pre;
         make_prefix(in, A, pre);
+        int keep_shards = 0;
         int64_t cap = G->qp_initial > 0 ? G->qp_initial : (int64_t)1 << 20;
         // few pieces have few keys: small levels clear and scan tables of four slots per piece (1000
         // vertices, 60k pieces: 2^18 slots instead of 2^20)
@@ -800,6 +818,27 @@ struct Miner {
                 A.defer = mem.get<uint32_t>((int64_t)A.defer_cap * FSM_DEFER_WORDS);
                 ck(cudaMemsetAsync(pool, 0, pool_words * 4, st), "memset");
             }
+            // Keep the accepted joins where the domain pass would enumerate again and there is room: 16
+            // bytes each for three in eight pieces (levels accept 0.14 to 0.32 of them; one that accepts
+            // more drops the records and enumerates), at most an eighth of the free memory, given back to
+            // any allocation that needs it.  Whole calls by two passes and by records: size 6 on 1656
+            // vertices 23.7 and 16.0 ms, size 7 under ST 8 72 and 54, size 5 on 37k, vertex-induced, 21.5 and
+            // 17.1.  Not at l = 1, where enumerating costs no more than the records do (size 3 on 3.7M
+            // vertices 10.3 and 9.9, but three small mines of a 1.1M-vertex graph 3.1 and 3.4).
+            if (!fused && !mem.spare && L >= 2 && joins(L) && pre.base && pre.total >= kKeepPieces && in.N < (1ll << 32)) {
+                keep_shards = grid_for(L, PASS_COUNT);
+                A.keep_cap = (uint32_t)std::min<int64_t>((pre.total / 8 * 3) / keep_shards + 1024, 0x7FFFFFFF);
+                const size_t bytes = (size_t)A.keep_cap * keep_shards * sizeof(uint4);
+                size_t fr = 0, tot = 0;
+                if (bytes > (1ull << 30)) ck(cudaMemGetInfo(&fr, &tot), "memory info");
+                A.keep_n = mem.get<uint32_t>(keep_shards);
+                A.keep_over = G->stats + S_KEEP;
+                if ((bytes > (1ull << 30) && bytes > fr / 8) || cudaMallocAsync(&mem.spare, bytes, st) != cudaSuccess) {
+                    cudaGetLastError();
+                    mem.spare = nullptr;
+                }
+                A.keep = (uint4 *)mem.spare;
+            }
             run_pass(fused ? PASS_FUSED : PASS_COUNT, in, A, pat_off, pre);
             ck(launch_qp_compact(keys, cap, slots, G->stats + S_KEYS, st), "compact");
             sc = scalars();
@@ -853,6 +892,7 @@ struct Miner {
         rs.pieces += (int64_t)sc[S_PIECES];
         rs.pieces_l[L] += (int64_t)sc[S_PIECES];
         if (final) rs.final_accepted = (int64_t)sc[S_ACCEPTED];
+        if (sc[S_KEEP] > 0) mem.drop_spare();   // more joins than fit
         // ---- distinct quick patterns -> canonical codes -> pattern ids
         const int64_t nq = (int64_t)sc[S_KEYS];
         rs.qps += nq;
@@ -928,7 +968,16 @@ struct Miner {
             A.stats = nullptr;
             if (rs.live > 0) {
                 tune_chunk(in, A);
-                run_pass(PASS_DOMAIN, in, A, pat_off, pre);
+                if (mem.spare) {
+                    A.fv = in.fv;
+                    A.fN = in.N;
+                    ck(launch_kept_bits(L, A, keep_shards, st), "kept joins");
+                    rs.launches += 1;
+                    rs.pass_launches[L][PASS_DOMAIN] += 1;
+                    rs.kept_levels += 1;
+                } else {
+                    run_pass(PASS_DOMAIN, in, A, pat_off, pre);
+                }
                 if (G->profile) {
                     // algorithmic bytes of the domain updates: one 4-byte bitmap word per position
                     // of every accepted join of a live pattern (the list reads are in run_pass)
@@ -944,6 +993,8 @@ struct Miner {
                     rs.pass_bytes[L][PASS_DOMAIN] += joins * 4 * K;
                 }
             }
+            mem.drop_spare();
+            A.keep = nullptr;
             ck(launch_support(K, orbit, live, doff, words, dom, np, G->n, G->NL, sigma, st), "support");
         }
         if (pool) {
@@ -1590,6 +1641,7 @@ int fsm_mine(fsm_graph *g, int32_t k, int64_t min_support, double sample_rate, f
         r->stats["qp_grows"] = rs.qp_grows;
         r->stats["fused_fallbacks"] = rs.fused_fallbacks;
         r->stats["fused_pool_words"] = rs.fused_pool_words;
+        r->stats["kept_levels"] = rs.kept_levels;
         r->stats["fused_deferred"] = rs.fused_deferred;
         for (int L = 1; L <= FSM_MAXL; ++L) r->stats["chunk_l" + std::to_string(L)] = g->tuned_chunk[L];
         for (int L = 1; L <= FSM_MAXL; ++L) r->stats["pieces_l" + std::to_string(L)] = rs.pieces_l[L];

@@ -91,6 +91,13 @@ struct ExtArgs {
     uint32_t *defer;
     unsigned long long *defer_top;
     unsigned long long defer_cap;
+    // count pass whose accepted joins are kept for the domain bits (kept_bits_kernel): one region of
+    // keep_cap records {key slot, embedding, rank of the first and of the second new vertex} a block,
+    // the number each block met, and how many blocks met more than fit; NULL: none are kept
+    uint4 *keep;
+    uint32_t *keep_n;
+    uint32_t keep_cap;
+    unsigned long long *keep_over;
     int check_bits;                // read a bitmap word before reducing into it
     int warm;                      // count a sample of the chunks only (before a one-pass level)
     // tables of fsm_join.cuh for this level size, and the size-3 frequencies as label masks: W[c][x]
@@ -994,6 +1001,8 @@ cudaError_t occupancy_extend_l7(int pass, int *blocks_per_sm);
 #define FSM_JOIN_MAXL 5
 cudaError_t launch_join(int pass, int L, int V, const ExtArgs &A, int grid, cudaStream_t st);
 cudaError_t launch_resolve_keys(const ExtArgs &A, int sms, cudaStream_t st);
+// Domain bits of the joins a count pass of `shards` blocks kept.
+cudaError_t launch_kept_bits(int L, const ExtArgs &A, int shards, cudaStream_t st);
 cudaError_t launch_deferred_bits(const ExtArgs &A, int sms, cudaStream_t st);
 cudaError_t occupancy_join(int pass, int L, int V, int *blocks_per_sm);
 // its tables for stored size L: bytes of each, and the kernels that fill them (tmp: join_tmp_bytes)

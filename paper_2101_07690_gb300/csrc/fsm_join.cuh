@@ -135,7 +135,7 @@ template <int L, bool QUOTA> struct UnitRec {
     static constexpr int BLOOM = L <= 3 ? 256 : 512;
     static constexpr int RP = 0, D = 1, PID = 2, META = 3, CLS = 4, OLAB = 5, OPP = 6, SEG = 7, SLO = 8, RLO = 9,
                          RHI = 11, NC = 13, SCN = 15, SEO = 16, SS = 17, BND = SS + L, RK = BND + L, OB = RK + L, OE = OB + O, OK = OE + O,
-                         VB = OK + 6 * O, VE = VB + 1, QA = VE + 1, END = QA + (QUOTA ? 6 : 0);
+                         VB = OK + 6 * O, VE = VB + 1, EI = VE + 1, QA = EI + 1, END = QA + (QUOTA ? 6 : 0);
     static constexpr int UW = END | 1;               // odd stride: lanes on different units hit different banks
 };
 
@@ -147,6 +147,7 @@ template <int L, int PASS, bool QUOTA> struct JoinSmem {
     uint32_t q_ainfo[8][FSM_JOIN_QUEUE], q_xinfo[8][FSM_JOIN_QUEUE];   // DevGraph::pinfo of anchor, partner
     uint32_t sg_base[8][32], sg_anchor[8][32], sg_slots[8][32], sg_meta[8][32], sg_info[8][32];
     uint32_t seen[8][PASS == PASS_FUSED || PASS == PASS_DOMAIN ? FSM_JOIN_SEEN : 1];
+    uint32_t kept;                 // joins the block met (ExtArgs::keep)
 };
 
 __device__ __forceinline__ int32_t sorted_has(const int32_t *col, int32_t lo, int32_t end, int32_t x) {
@@ -330,7 +331,25 @@ struct Joiner {
                                            uint32_t ainfo, uint32_t xinfo, bool swap) {
         if constexpr (PASS == PASS_COUNT) {
             const int64_t slot = qp_insert(A.qp, key, A.err);
-            if (slot >= 0) atomicAdd(A.qp.count + slot, 1ull);
+            if (slot < 0) return;
+            atomicAdd(A.qp.count + slot, 1ull);
+            if (A.keep) {
+                const unsigned act = __activemask();
+                const int leader = __ffs(act) - 1;
+                uint32_t at = 0;
+                if (lane == leader) {
+                    at = atomicAdd(&sm.kept, (uint32_t)__popc(act));
+                    if (at >> 31) atomicExch(&sm.kept, 1u << 31);   // never wraps round
+                }
+                at = __shfl_sync(act, at, leader) + __popc(act & ((1u << lane) - 1u));
+                if (at < A.keep_cap) {
+                    const uint32_t ranchor = A.g.packed ? ainfo >> 6 : (uint32_t)__ldg(A.g.rank + anchor);
+                    const uint32_t rx = A.g.packed ? xinfo >> 6 : (uint32_t)__ldg(A.g.rank + x);
+                    const bool flip = centre != swap;   // the first new vertex is x
+                    __stcs(A.keep + (uint64_t)blockIdx.x * A.keep_cap + at,
+                           make_uint4((uint32_t)slot, r[R::EI], flip ? rx : ranchor, flip ? ranchor : rx));
+                }
+            }
         } else if constexpr (PASS == PASS_FUSED || PASS == PASS_DOMAIN) {
             uint32_t off[K];
             int64_t slot = -1;
@@ -588,6 +607,7 @@ struct Joiner {
             const int64_t u = u0 + lane;
             const int64_t e = A.e0 + u / L;
             const int iu = (int)(u % L);
+            r[R::EI] = (uint32_t)e;
             const int32_t pid = __ldg(A.fpid + e);
             const uint64_t srows = L >= 2 ? __ldg(A.pat_adj + pid) : 0ull;
             int32_t id[L];
@@ -991,6 +1011,10 @@ __global__ void __launch_bounds__(256, JoinBlocks<L, PASS>::value) join_kernel(c
         chunk = min(chunk, (int64_t)FSM_WARM_CHUNK);
         nchunks = ((total + chunk - 1) / chunk + stride - 1) / stride;
     }
+    if (PASS == PASS_COUNT && A.keep) {
+        if (threadIdx.x == 0) sm.kept = 0;
+        __syncthreads();
+    }
     if (A.stats && blockIdx.x == 0 && threadIdx.x == 0) atomicAdd(A.stats + 2, (unsigned long long)total);
     for (;;) {
         unsigned long long c = 0;
@@ -1019,6 +1043,13 @@ __global__ void __launch_bounds__(256, JoinBlocks<L, PASS>::value) join_kernel(c
         }
     }
 
+    if (PASS == PASS_COUNT && A.keep) {
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            A.keep_n[blockIdx.x] = min(sm.kept, A.keep_cap);
+            if (sm.kept > A.keep_cap) atomicAdd(A.keep_over, 1ull);
+        }
+    }
     // per-warp totals, one atomic per warp
     unsigned long long t0 = jn.tested, t1 = jn.accepted;
 #pragma unroll

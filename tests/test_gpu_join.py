@@ -61,6 +61,29 @@ def test_join_kernel_matches_oracle(fsm, case, mode):
                 assert np.array_equal(got[key], exp[key]), (k, opts, key)
 
 
+@pytest.mark.parametrize("opts", [{}, {"launch": 1}, {"join_quota": 3}], ids=["default", "persistent", "quota"])
+@pytest.mark.parametrize("n,deg,k", [(700, 6.0, 4), (300, 5.0, 5), (200, 4.0, 7), (150, 4.0, 6), (40, 20.0, 4)])
+@pytest.mark.parametrize("mode", ["edge", "vertex"])
+def test_domain_bits_from_kept_joins(fsm, mode, n, deg, k, opts):
+    """Levels of enough pieces keep their accepted joins in the count pass and set the domain bits from
+    them.  Launches per pattern never do: the same result.  The dense graphs accept more joins a piece
+    than there is room for, so their levels enumerate again."""
+    g = gg.erdos_renyi(n, deg, seed=5, num_labels=3)
+    out = []
+    for o in (opts, {**opts, "launch": 2}):
+        G = fsm.Graph.from_graphgen(g, mode)
+        for key, val in o.items():
+            G.set_option(key, val)
+        out.append(G.mine(k, max(2, n // 40), stats=True))
+        G.close()
+    assert out[1]["stats"]["kept_levels"] == 0
+    if n >= 300 and not opts.get("join_quota"):
+        assert out[0]["stats"]["kept_levels"] > 0
+    assert len(out[0]["support"]) > 0
+    for key in ("labels", "adj", "support", "count"):
+        assert np.array_equal(out[0][key], out[1][key]), key
+
+
 @pytest.mark.parametrize("mode", ["edge", "vertex"])
 @pytest.mark.parametrize("k,scale", [(5, 0.002), (4, 0.1), (3, 0.3)])
 def test_one_pass_level_with_keys_its_sample_missed(fsm, k, scale, mode):
