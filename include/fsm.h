@@ -276,7 +276,8 @@ const char *fsm_last_error(void);
  *   fsm_mlp_gradients    mean squared error over X[n][32], Y[n] and its gradient (6337 floats).
  *   fsm_mlp_train        epochs of shuffled minibatches (order from a splitmix64 stream of seed),
  *                        Adam (beta 0.9, 0.999, eps 1e-8) at rate lr; final_loss = last epoch's
- *                        mean squared error.
+ *                        mean squared error.  The same arguments give the same
+ *                        parameters, bit for bit, as they do gradients.
  *   fsm_mlp_predict      outputs (predicted log support) for X[n][32].
  *   fsm_mlp_predict_device the same on device arrays, on stream.
  */

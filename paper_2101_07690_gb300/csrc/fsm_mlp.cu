@@ -24,6 +24,8 @@ void set_last_error_message(const std::string &m);
 #define MLP_H 64
 #define MLP_NPARAM (MLP_IN * MLP_H + MLP_H + MLP_H * MLP_H + MLP_H + MLP_H + 1)
 #define MLP_TILE 32   // samples per block
+#define MLP_SLOT (MLP_NPARAM + 1)   // floats of a block's sums: the gradients, then the squared error
+#define MLP_MAXGRID 1024            // blocks of a minibatch, each with a slot (26 MB at most)
 
 namespace {
 
@@ -107,11 +109,14 @@ __global__ void __launch_bounds__(MLP_H) infer_kernel(const float *X, int64_t n,
     }
 }
 
-// forward + backward of one minibatch (rows[base .. base+nb)); gradients of the mean squared
-// error are added into grad (FP32); loss_sum gets the summed squared error
+// forward + backward of one minibatch (rows[base .. base+nb)): each block leaves the gradients of the
+// mean squared error (FP32) and the summed squared error of its tiles in its own slot of `parts`.
+// Adding them into one array by atomics let the order in which the blocks arrived into the sums, and
+// a last bit that differs can round a BF16 weight the other way: two fits of 20000 rows (158 Adam steps)
+// then ended up to 1.4e-3 apart (relative, over all parameters).
 __global__ void __launch_bounds__(MLP_H) grad_kernel(const float *X, const float *Y, const int64_t *rows, int64_t base0,
                                                      int64_t nb, const __nv_bfloat16 *wbf, const float *master,
-                                                     const float *mu, const float *sd, float *grad, float *loss_sum) {
+                                                     const float *mu, const float *sd, float *parts) {
     extern __shared__ float smem_raw[];
     Smem &s = *reinterpret_cast<Smem *>(smem_raw);
     stage_weights(s, wbf, master);
@@ -119,19 +124,24 @@ __global__ void __launch_bounds__(MLP_H) grad_kernel(const float *X, const float
     const float b3 = master[OFF_B3];
     const int j = threadIdx.x;
     const float inv = 1.f / (float)nb;
+    float *slot = parts + (int64_t)blockIdx.x * MLP_SLOT;
+    bool first = true;   // a word of the slot is always the same thread's
+    auto add = [&](int x, float g) { slot[x] = first ? g : slot[x] + g; };
     for (int64_t t0 = (int64_t)blockIdx.x * MLP_TILE; t0 < nb; t0 += (int64_t)gridDim.x * MLP_TILE) {
         const int nrows = (int)(nb - t0 < MLP_TILE ? nb - t0 : MLP_TILE);
         forward_tile(s, X, rows, base0 + t0, nrows, mu, sd, b3);
         // dL/dy for the mean squared error, zero for padding rows
         if (j < MLP_TILE) {
-            float d = 0.f;
+            float d = 0.f, sq = 0.f;
             if (j < nrows) {
                 const int64_t row = rows ? rows[base0 + t0 + j] : base0 + t0 + j;
                 const float e = s.y[j] - Y[row];
-                atomicAdd(loss_sum, e * e);
+                sq = e * e;
                 d = 2.f * e * inv;
             }
             s.y[j] = d;
+            for (int o = 16; o > 0; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+            if (j == 0) add(MLP_NPARAM, sq);
         }
         __syncthreads();
         // layer 3
@@ -141,17 +151,17 @@ __global__ void __launch_bounds__(MLP_H) grad_kernel(const float *X, const float
             gb3 += s.y[r];
             s.dz[r][j] = s.h2[r][j] > 0.f ? s.y[r] * s.w3[j] : 0.f;   // dz2
         }
-        atomicAdd(grad + OFF_W3 + j, gw3);
-        if (j == 0) atomicAdd(grad + OFF_B3, gb3);
+        add(OFF_W3 + j, gw3);
+        if (j == 0) add(OFF_B3, gb3);
         __syncthreads();
         // layer 2: thread j is output unit j of W2
         float gb2 = 0.f;
         for (int r = 0; r < MLP_TILE; ++r) gb2 += s.dz[r][j];
-        atomicAdd(grad + OFF_B2 + j, gb2);
+        add(OFF_B2 + j, gb2);
         for (int i = 0; i < MLP_H; ++i) {
             float g = 0.f;
             for (int r = 0; r < MLP_TILE; ++r) g = fmaf(fmaxf(s.h1[r][i], 0.f), s.dz[r][j], g);
-            atomicAdd(grad + OFF_W2 + i * MLP_H + j, g);
+            add(OFF_W2 + i * MLP_H + j, g);
         }
         // dz1 (thread j now is hidden unit j of layer 1): dh1 = W2 dz2, masked by z1 > 0
         float dz1[MLP_TILE];
@@ -165,20 +175,39 @@ __global__ void __launch_bounds__(MLP_H) grad_kernel(const float *X, const float
         __syncthreads();
         float gb1 = 0.f;
         for (int r = 0; r < MLP_TILE; ++r) gb1 += s.dz[r][j];
-        atomicAdd(grad + OFF_B1 + j, gb1);
+        add(OFF_B1 + j, gb1);
         for (int i = 0; i < MLP_IN; ++i) {
             float g = 0.f;
             for (int r = 0; r < MLP_TILE; ++r) g = fmaf(s.x[r][i], s.dz[r][j], g);
-            atomicAdd(grad + OFF_W1 + i * MLP_H + j, g);
+            add(OFF_W1 + i * MLP_H + j, g);
         }
         __syncthreads();
+        first = false;
     }
 }
 
-__global__ void adam_kernel(float *w, float *m, float *v, const float *g, __nv_bfloat16 *wbf, int n, float lr,
-                            float b1, float b2, float eps, float c1, float c2) {
-    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x) {
-        const float gx = g[x];
+// Word x of `blocks` slots, added in FP64 and rounded once: whatever order FP32 additions could have
+// taken, their sum lies around this one.
+__device__ __forceinline__ float slot_sum(const float *parts, int blocks, int x) {
+    double s = 0.0;
+    for (int b = 0; b < blocks; ++b) s += (double)parts[(int64_t)b * MLP_SLOT + x];
+    return (float)s;
+}
+
+__global__ void sum_kernel(const float *parts, int blocks, float *out) {
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < MLP_SLOT; x += gridDim.x * blockDim.x)
+        out[x] = slot_sum(parts, blocks, x);
+}
+
+// the minibatch's squared error is added to *loss (one launch after another on one stream)
+__global__ void adam_kernel(float *w, float *m, float *v, const float *parts, int blocks, __nv_bfloat16 *wbf, float lr,
+                            float b1, float b2, float eps, float c1, float c2, float *loss) {
+    for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < MLP_SLOT; x += gridDim.x * blockDim.x) {
+        const float gx = slot_sum(parts, blocks, x);
+        if (x == MLP_NPARAM) {
+            *loss += gx;
+            continue;
+        }
         const float mx = b1 * m[x] + (1.f - b1) * gx;
         const float vx = b2 * v[x] + (1.f - b2) * gx * gx;
         m[x] = mx;
@@ -223,6 +252,8 @@ int mlp_fail(int code, const std::string &m) {
 
 struct fsm_mlp {
     float *w = nullptr, *m = nullptr, *v = nullptr, *g = nullptr, *mu = nullptr, *sd = nullptr, *loss = nullptr;
+    float *parts = nullptr;   // slots of the largest minibatch so far
+    int slots = 0;
     __nv_bfloat16 *wbf = nullptr;
     int64_t steps = 0;
 };
@@ -231,9 +262,25 @@ namespace {
 bool mlp_alloc(fsm_mlp *M) {
     const size_t P = MLP_NPARAM;
     return cudaMalloc(&M->w, P * 4) == cudaSuccess && cudaMalloc(&M->m, P * 4) == cudaSuccess &&
-           cudaMalloc(&M->v, P * 4) == cudaSuccess && cudaMalloc(&M->g, P * 4) == cudaSuccess &&
+           cudaMalloc(&M->v, P * 4) == cudaSuccess && cudaMalloc(&M->g, MLP_SLOT * 4) == cudaSuccess &&
            cudaMalloc(&M->mu, MLP_IN * 4) == cudaSuccess && cudaMalloc(&M->sd, MLP_IN * 4) == cudaSuccess &&
            cudaMalloc(&M->loss, 4) == cudaSuccess && cudaMalloc(&M->wbf, P * 2) == cudaSuccess;
+}
+
+// blocks of a minibatch of nb rows, or -1 when their slots do not fit the device
+int mlp_blocks(fsm_mlp *M, int64_t nb) {
+    const int blocks = (int)std::min<int64_t>((nb + MLP_TILE - 1) / MLP_TILE, MLP_MAXGRID);
+    if (blocks > M->slots) {
+        cudaFree(M->parts);
+        M->parts = nullptr;
+        M->slots = 0;
+        if (cudaMalloc(&M->parts, (size_t)blocks * MLP_SLOT * 4) != cudaSuccess) {
+            cudaGetLastError();
+            return -1;
+        }
+        M->slots = blocks;
+    }
+    return blocks;
 }
 } // namespace
 
@@ -355,16 +402,16 @@ int fsm_mlp_gradients(fsm_mlp *M, const float *X, const float *Y, int64_t n, flo
     if (!M || !X || !Y || !grads || n < 1) return mlp_fail(FSM_EINVAL, "NULL argument or n < 1");
     float *dX = nullptr, *dY = nullptr;
     int rc = mlp_upload(X, Y, n, &dX, &dY);
+    const int grid = rc == FSM_OK ? mlp_blocks(M, n) : 0;
+    if (grid < 0) rc = FSM_ENOMEM;
     if (rc == FSM_OK) {
-        cudaMemset(M->g, 0, (size_t)MLP_NPARAM * 4);
-        cudaMemset(M->loss, 0, 4);
-        const int grid = (int)std::min<int64_t>((n + MLP_TILE - 1) / MLP_TILE, 4096);
-        grad_kernel<<<grid, MLP_H, sizeof(Smem)>>>(dX, dY, nullptr, 0, n, M->wbf, M->w, M->mu, M->sd, M->g, M->loss);
-        fsm::note_launches(1);
+        grad_kernel<<<grid, MLP_H, sizeof(Smem)>>>(dX, dY, nullptr, 0, n, M->wbf, M->w, M->mu, M->sd, M->parts);
+        sum_kernel<<<(MLP_SLOT + 255) / 256, 256>>>(M->parts, grid, M->g);
+        fsm::note_launches(2);
         float ls = 0.f;
         cudaError_t e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaMemcpy(grads, M->g, (size_t)MLP_NPARAM * 4, cudaMemcpyDeviceToHost);
-        if (e == cudaSuccess) e = cudaMemcpy(&ls, M->loss, 4, cudaMemcpyDeviceToHost);
+        if (e == cudaSuccess) e = cudaMemcpy(&ls, M->g + MLP_NPARAM, 4, cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) rc = mlp_fail(FSM_ECUDA, cudaGetErrorString(e));
         else if (loss) *loss = ls / (float)n;
     } else {
@@ -384,6 +431,7 @@ int fsm_mlp_train(fsm_mlp *M, const float *X, const float *Y, int64_t n, int32_t
     int64_t *drows = nullptr;
     int rc = mlp_upload(X, Y, n, &dX, &dY);
     if (rc == FSM_OK && cudaMalloc(&drows, (size_t)n * 8) != cudaSuccess) rc = FSM_ENOMEM;
+    if (rc == FSM_OK && mlp_blocks(M, std::min<int64_t>(batch, n)) < 0) rc = FSM_ENOMEM;
     if (rc != FSM_OK) {
         cudaFree(dX); cudaFree(dY); cudaFree(drows);
         return mlp_fail(rc, "could not stage the training data on the device");
@@ -400,12 +448,11 @@ int fsm_mlp_train(fsm_mlp *M, const float *X, const float *Y, int64_t n, int32_t
         cudaMemset(M->loss, 0, 4);
         for (int64_t b0 = 0; b0 < n && e == cudaSuccess; b0 += batch) {
             const int64_t nb = std::min<int64_t>(batch, n - b0);
-            cudaMemset(M->g, 0, (size_t)MLP_NPARAM * 4);
-            const int grid = (int)std::min<int64_t>((nb + MLP_TILE - 1) / MLP_TILE, 1024);
-            grad_kernel<<<grid, MLP_H, sizeof(Smem)>>>(dX, dY, drows, b0, nb, M->wbf, M->w, M->mu, M->sd, M->g, M->loss);
+            const int grid = mlp_blocks(M, nb);
+            grad_kernel<<<grid, MLP_H, sizeof(Smem)>>>(dX, dY, drows, b0, nb, M->wbf, M->w, M->mu, M->sd, M->parts);
             M->steps += 1;
             const float c1 = 1.f - std::pow(b1, (float)M->steps), c2 = 1.f - std::pow(b2, (float)M->steps);
-            adam_kernel<<<(MLP_NPARAM + 255) / 256, 256>>>(M->w, M->m, M->v, M->g, M->wbf, MLP_NPARAM, lr, b1, b2, eps, c1, c2);
+            adam_kernel<<<(MLP_SLOT + 255) / 256, 256>>>(M->w, M->m, M->v, M->parts, grid, M->wbf, lr, b1, b2, eps, c1, c2, M->loss);
             fsm::note_launches(2);
             e = cudaGetLastError();
         }
@@ -446,7 +493,7 @@ int fsm_mlp_predict_device(const fsm_mlp *M, const float *d_X, int64_t n, float 
 void fsm_mlp_free(fsm_mlp *M) {
     if (!M) return;
     cudaFree(M->w); cudaFree(M->m); cudaFree(M->v); cudaFree(M->g);
-    cudaFree(M->mu); cudaFree(M->sd); cudaFree(M->loss); cudaFree(M->wbf);
+    cudaFree(M->mu); cudaFree(M->sd); cudaFree(M->loss); cudaFree(M->wbf); cudaFree(M->parts);
     delete M;
 }
 
