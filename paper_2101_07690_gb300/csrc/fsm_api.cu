@@ -1022,6 +1022,7 @@ struct Miner {
             ck(launch_sum_frequent(newid, pcount, np, G->stats + S_SUM, st), "sum");
         }
         sc = scalars();
+        if (sc.err()) fail_word(sc.err());   // a pass that stopped early leaves supports too small
         const int64_t nf = (int64_t)sc[S_FREQ];
         if (dom) mem.release(dom);
         // ---- frequent patterns of size K
@@ -1052,12 +1053,12 @@ struct Miner {
             A.out_cursor = G->stats + S_WROTE;
             run_pass(PASS_EMIT, in, A, pat_off, pre);
             sc = scalars();
+            if (sc.err()) fail_word(sc.err());
             const int64_t wrote = (int64_t)sc[S_WROTE];
             if (wrote != N2) fail(FSM_ECUDA, "frontier emission wrote " + std::to_string(wrote) + " of " + std::to_string(N2));
             if (G->profile) rs.pass_bytes[L][PASS_EMIT] += N2 * 4 * (K + 1);   // output written
             rs.frontier_max = std::max(rs.frontier_max, N2);
         }
-        if (sc.err()) fail_word(sc.err());
         if (pre.base) mem.release(pre.base);
         if (sbase) mem.release(sbase);
         if (lf) mem.release(lf);
