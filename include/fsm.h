@@ -149,6 +149,10 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
  *                FSM_ETIMEOUT with no result; the handle stays usable; 0 = no limit (default).
  *   "fail_alloc_after" test hook: > 0 makes the call's n-th device allocation report failure, so
  *                the call returns FSM_ENOMEM (everything it allocated is released); 0 = off.
+ *   "refuse_alloc" test hook: > 0 makes the device refuse the call's n-th request for memory once, as
+ *                when it is short: the call does without that memory where it can (the one-pass level
+ *                then runs as two passes, kept joins are enumerated again), with the same result, and
+ *                returns FSM_ENOMEM where it cannot; 0 = off.
  *   "profile"    1 = time every extension-kernel launch with CUDA events and sum its algorithmic
  *                bytes (reported by fsm_result_stat); adds one synchronisation per launch.
  * Unknown keys or out-of-range values give FSM_EINVAL.

@@ -78,10 +78,22 @@ struct Arena {
     size_t left = 0;                 // bytes of the current block not given out
     void *spare = nullptr;           // an allocation the call can do without: given back when one fails
     int64_t made = 0, fail_at = 0;   // fail_at > 0: the fail_at-th allocation reports failure (test hook)
+    int64_t asked = 0, refuse_at = 0;   // refuse_at > 0: the device refuses the refuse_at-th request (test hook)
     explicit Arena(cudaStream_t s) : st(s) {}
+    cudaError_t ask(void **p, size_t bytes) {
+        if (refuse_at > 0 && ++asked == refuse_at) return cudaErrorMemoryAllocation;
+        return cudaMallocAsync(p, bytes, st);
+    }
+    // memory the call can do without: nullptr where there is none
+    void *optional(size_t bytes) {
+        void *p = nullptr;
+        if (ask(&p, bytes) == cudaSuccess) return p;
+        cudaGetLastError();
+        return nullptr;
+    }
     void *raw(size_t bytes) {
         void *p = nullptr;
-        cudaError_t e = cudaMallocAsync(&p, bytes, st);
+        cudaError_t e = ask(&p, bytes);
         if (e != cudaSuccess && spare) {
             cudaGetLastError();
             drop_spare();
@@ -188,6 +200,7 @@ struct fsm_graph {
     int debug = 0;                        // option "debug": device bounds checks on decoded indices
     int64_t time_limit_ms = 0;            // option "time_limit_ms": FSM_ETIMEOUT past it (0 = none)
     int64_t fail_alloc_after = 0;         // option "fail_alloc_after": injected allocation failure
+    int64_t refuse_alloc = 0;             // option "refuse_alloc": one request of the device refused
     int64_t join_quota = 0;               // option "join_quota": ST x of Section 5 (0 = off)
     int64_t match_quota = 0;              // option "match_quota": M.ST of Section 5 (0 = off)
     int autotune = 0;
@@ -708,7 +721,8 @@ struct Miner {
         const int rec_words = key_rec_words(K);
         int shift = 0;   // bitmap offsets are 32-bit, in units of 1 << shift words
         unsigned long long pool_words = 0;
-        bool fused = final && G->fused && V == FSM_EXPLORE_TV && !sampled && K <= 7;
+        // a level without pieces has nothing to enumerate once
+        bool fused = final && G->fused && V == FSM_EXPLORE_TV && !sampled && K <= 7 && in.N > 0 && pre.total != 0;
         // Bitmap pool of the one-pass level.  Offsets are given out up to pool_words; the memory is
         // allocated once the warm pass has shown what most keys need, twice that (the first call on a
         // graph used to take and clear 40% of the free memory: 12 ms).  Up to 2^32 words offsets count
@@ -738,8 +752,6 @@ struct Miner {
             if (fused) ck(cudaMemsetAsync(krec, 0xff, sizeof(uint32_t) * cap * rec_words, st), "memset");
         };
         Scalars sc;
-        // pieces of the level, an upper bound where the host does not know them
-        const unsigned long long pieces = pre.total >= 0 ? (unsigned long long)pre.total : 1ull << 32;
         for (;;) {
             // the pattern (code) table has as many slots as the quick-pattern table, so it is at most
             // half full whenever that one is
@@ -787,13 +799,15 @@ struct Miner {
                 // keys: 6.1M resolutions and 59 ms without a sample) and cost every join the
                 // registers of that path (2 -> 4 one pass: 121 ms with it, 113 ms without; 3 -> 5: 22.0 and 19.1).
                 ExtArgs W = A;
-                W.warm = 1;
-                W.stats = nullptr;
+                W.warm = 1;   // its statistics say how many pieces the level has
                 run_pass(PASS_COUNT, in, W, pat_off, pre);
                 ck(launch_resolve_keys(W, G->sms, st), "resolve keys");
                 rs.launches += 1;
                 ck(cudaMemsetAsync(qcount, 0, sizeof(unsigned long long) * cap, st), "memset");
-                const unsigned long long want = 2 * d2h(ptop, st) + (1ull << 22);
+                sc = scalars();
+                ck(cudaMemsetAsync(G->stats, 0, sizeof(unsigned long long) * (S_PIECES + 1), st), "memset");
+                const int64_t pieces = (int64_t)sc[S_PIECES];
+                const unsigned long long want = 2 * sc[S_POOL] + (1ull << 22);
                 if (!G->pool_force && want > pool_words && pool_words < pool_limit) {
                     pool_min = want;
                     release_pass1();
@@ -801,21 +815,24 @@ struct Miner {
                 }
                 if (!G->pool_force) pool_words = std::min(pool_words, std::max(want, pool_min));
                 A.pool_words = pool_words;
-                void *pp = nullptr;
-                if (cudaMallocAsync(&pp, pool_words * 4, st) != cudaSuccess) {
-                    cudaGetLastError();
-                    fused = false;   // no room for the pool: separate count and domain passes
+                // Joins put aside: 32 bytes each, room for one in eight pieces; past 2^24 the level is redone
+                // in two passes.  A sample of every piece has met every key.
+                A.defer_cap = warm_stride(pieces) == 1 ? 256 : std::min<unsigned long long>(1ull << 24, pieces / 8);
+                pool = (uint32_t *)mem.optional(pool_words * 4);
+                if (pool) mem.ptrs.push_back(pool);
+                A.defer = pool ? (uint32_t *)mem.optional(A.defer_cap * FSM_DEFER_WORDS * 4) : nullptr;
+                if (A.defer) mem.ptrs.push_back(A.defer);
+                if (!A.defer) {   // no room for one of them: separate count and domain passes
+                    if (pool) mem.release(pool);
+                    pool = nullptr;
+                    fused = false;
                     shift = 0;
+                    rs.fused_fallbacks += 1;
                     release_pass1();
                     continue;
                 }
-                pool = (uint32_t *)pp;
-                mem.ptrs.push_back(pp);
                 A.pool = pool;
                 A.defer_top = G->stats + S_DEFER;
-                // 32 bytes each; past 2^24 the level is redone in two passes
-                A.defer_cap = std::min<unsigned long long>(1ull << 24, std::max<unsigned long long>(1ull << 18, pieces / 8));
-                A.defer = mem.get<uint32_t>((int64_t)A.defer_cap * FSM_DEFER_WORDS);
                 ck(cudaMemsetAsync(pool, 0, pool_words * 4, st), "memset");
             }
             // Keep the accepted joins where the domain pass would enumerate again and there is room: 16
@@ -833,10 +850,7 @@ struct Miner {
                 if (bytes > (1ull << 30)) ck(cudaMemGetInfo(&fr, &tot), "memory info");
                 A.keep_n = mem.get<uint32_t>(keep_shards);
                 A.keep_over = G->stats + S_KEEP;
-                if ((bytes > (1ull << 30) && bytes > fr / 8) || cudaMallocAsync(&mem.spare, bytes, st) != cudaSuccess) {
-                    cudaGetLastError();
-                    mem.spare = nullptr;
-                }
+                if (bytes <= (1ull << 30) || bytes <= fr / 8) mem.spare = mem.optional(bytes);
                 A.keep = (uint4 *)mem.spare;
             }
             run_pass(fused ? PASS_FUSED : PASS_COUNT, in, A, pat_off, pre);
@@ -1474,6 +1488,9 @@ int fsm_set_option(fsm_graph *g, const char *key, int64_t value) {
         } else if (k == "fail_alloc_after") {
             if (value < 0) fail(FSM_EINVAL, "fail_alloc_after must be >= 0");
             g->fail_alloc_after = value;
+        } else if (k == "refuse_alloc") {
+            if (value < 0) fail(FSM_EINVAL, "refuse_alloc must be >= 0");
+            g->refuse_alloc = value;
         } else if (k == "join_quota") {
             if (value < 0 || value > 65536) fail(FSM_EINVAL, "join_quota must be in [0, 65536]");
             g->join_quota = value;
@@ -1537,6 +1554,7 @@ int fsm_mine(fsm_graph *g, int32_t k, int64_t min_support, double sample_rate, f
         {
             Arena mem(st);
             mem.fail_at = g->fail_alloc_after;
+            mem.refuse_at = g->refuse_alloc;
             ck(launch_stamp_time(g->stats + S_START, st), "time stamp");
             Miner m{g, st, mem, min_support, rs};
             m.V = V;

@@ -39,3 +39,60 @@ def test_a_time_limit_that_runs_out_in_any_pass_is_reported_as_one(fsm, k, scale
     finally:
         G.close()
     assert stopped > 0
+
+
+def _refused_one_by_one(fsm, g, k, t, opts, most=60):
+    """Results (or None for FSM_ENOMEM) of a mine whose n-th request for device memory is refused."""
+    G = fsm.Graph.from_graphgen(g)
+    for key, val in opts.items():
+        G.set_option(key, val)
+    try:
+        whole = G.mine(k, t, stats=True)
+        out = []
+        for n in range(1, most):
+            G.set_option("refuse_alloc", n)
+            try:
+                out.append(G.mine(k, t, stats=True))
+            except fsm.FsmError as e:
+                assert e.code == fsm.FSM_ENOMEM, (n, e)
+                out.append(None)
+    finally:
+        G.close()
+    for got in out:
+        if got:
+            for key in ("labels", "adj", "support", "count"):
+                assert np.array_equal(got[key], whole[key]), key
+    return whole, out
+
+
+@pytest.mark.parametrize("opts", [{}, {"launch": 1}, {"launch": 2}, {"profile": 1}],
+                         ids=["batches", "persistent", "per pattern", "profiled"])
+def test_the_one_pass_level_does_without_its_pool_and_its_buffer(fsm, opts):
+    """Refused one or the other, the level is finished in two passes."""
+    g = gg.workload("cl3700k", scale=0.001, cap=20)
+    whole, out = _refused_one_by_one(fsm, g, 5, 20, {**opts, "fused": 1})
+    assert whole["stats"]["fused_fallbacks"] == 0 and len(whole["support"]) > 0
+    assert sum(1 for r in out if r and r["stats"]["fused_fallbacks"] == 1) == 2
+
+
+def _device_memory_taken(body):
+    """Bytes of device memory a fresh process holds after `body`, beyond those it held after loading."""
+    import os
+    import subprocess
+    import sys
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    code = ("import torch, numpy as np, graphgen as gg\nfrom paper_2101_07690_gb300 import fsm\n"
+            "def free():\n    torch.cuda.synchronize()\n    return torch.cuda.mem_get_info()[0]\n" + body)
+    r = subprocess.run([sys.executable, "-c", code], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0, r.stderr
+    return int(r.stdout.split()[-1])
+
+
+@pytest.mark.parametrize("launch,t,mib", [(0, 10 ** 6, 8), (1, 10 ** 6, 8), (2, 10 ** 6, 8), (0, 30, 64), (2, 30, 64)])
+def test_a_small_one_pass_level_takes_little_memory(fsm, launch, t, mib):
+    """Nothing frequent, hence no stored embeddings (two-pass mining of it first, so that only what the
+    one-pass form adds is seen), and a thousand vertices: no buffer for joins that cannot be put aside."""
+    body = ("G = fsm.Graph.from_graphgen(gg.workload('er1000'))\n"
+            f"G.set_option('launch', {launch})\nG.mine(5, {t})\nf = free()\n"
+            f"G.set_option('fused', 1)\nG.mine(5, {t})\nprint(f - free())\n")
+    assert _device_memory_taken(body) <= mib << 20
