@@ -76,7 +76,10 @@ struct Arena {
     std::vector<void *> blocks;      // the blocks among ptrs: release() leaves their first piece alone
     char *block = nullptr;
     size_t left = 0;                 // bytes of the current block not given out
-    void *spare = nullptr;           // an allocation the call can do without: given back when one fails
+    // allocations the call can do without, given back when another fails: a level's kept joins, then its
+    // unit prefix (*prefix, which is nulled: the passes that are left make theirs in ranges that fit)
+    void *spare = nullptr;
+    int64_t **prefix = nullptr;
     int64_t made = 0, fail_at = 0;   // fail_at > 0: the fail_at-th allocation reports failure (test hook)
     int64_t asked = 0, refuse_at = 0;   // refuse_at > 0: the device refuses the refuse_at-th request (test hook)
     explicit Arena(cudaStream_t s) : st(s) {}
@@ -94,9 +97,8 @@ struct Arena {
     void *raw(size_t bytes) {
         void *p = nullptr;
         cudaError_t e = ask(&p, bytes);
-        if (e != cudaSuccess && spare) {
+        while (e != cudaSuccess && give_back()) {
             cudaGetLastError();
-            drop_spare();
             cudaStreamSynchronize(st);
             e = cudaMallocAsync(&p, bytes, st);
         }
@@ -132,6 +134,19 @@ struct Arena {
     void drop_spare() {
         if (spare) cudaFreeAsync(spare, st);
         spare = nullptr;
+    }
+    void drop_prefix() {
+        if (prefix && *prefix) {
+            release(*prefix);
+            *prefix = nullptr;
+        }
+        prefix = nullptr;
+    }
+    bool give_back() {
+        if (!spare && !prefix) return false;
+        if (spare) drop_spare();
+        else drop_prefix();
+        return true;
     }
     ~Arena() {
         drop_spare();
@@ -399,6 +414,7 @@ struct Miner {
         ck(launch_scan_i64(pre.base, pre.base, in.N * L, tmp, st), "unit scan");
         pre.total = d2h(pre.base + in.N * L, st);
         mem.release(tmp);
+        mem.prefix = &pre.base;
     }
     int64_t batch_size(int L) const { return G->batch > 0 ? G->batch : std::max<int64_t>(1024, ((int64_t)1 << 24) / L); }
     int64_t prefix_fit(int L) const {   // embeddings whose prefix a quarter of the free memory holds
@@ -415,9 +431,10 @@ struct Miner {
     void run_pass(int pass, const LevelSet &in, ExtArgs A, const std::vector<int64_t> &pat_off, const Prefix &pre) {
         const int L = in.L;
         if (in.N == 0) return;
+        unsigned long long *ctr = mem.get<unsigned long long>(1);   // before the prefix is looked at: it may give it back
+        if (!mem.spare) A.keep = nullptr;
         if (pre.base) {
             if (pre.total == 0) return;
-            unsigned long long *ctr = mem.get<unsigned long long>(1);
             const int grid = grid_for(L, pass);
             int64_t chunk = chunk_for(L);
             const int64_t warps = (int64_t)grid * 8;
@@ -432,7 +449,6 @@ struct Miner {
             A.total = pre.total;
             A.chunk = (int32_t)chunk;
             A.nchunks = (pre.total + chunk - 1) / chunk;
-            if (!mem.spare) A.keep = nullptr;
             ck(cudaMemsetAsync(ctr, 0, sizeof(unsigned long long), st), "memset");
             ck(launch_pass(pass, L, A, grid), "extension kernel");
             rs.launches += 1;
@@ -462,7 +478,7 @@ struct Miner {
         // per-unit piece counts, then their exclusive prefix in place (one extra entry: the total)
         int64_t *base = mem.get<int64_t>(maxu + 1);
         void *tmp = mem.get<char>((int64_t)scan_temp_bytes(maxu) + 16);
-        unsigned long long *ctr = mem.get<unsigned long long>(1);
+        if (!mem.spare) A.keep = nullptr;
         const int grid = grid_for(L, pass);
         const int64_t warps = (int64_t)grid * 8;
         const bool prof = G->profile != 0;
@@ -1073,7 +1089,7 @@ struct Miner {
             if (G->profile) rs.pass_bytes[L][PASS_EMIT] += N2 * 4 * (K + 1);   // output written
             rs.frontier_max = std::max(rs.frontier_max, N2);
         }
-        if (pre.base) mem.release(pre.base);
+        mem.drop_prefix();
         if (sbase) mem.release(sbase);
         if (lf) mem.release(lf);
         release_pass1();

@@ -47,6 +47,7 @@ def _refused_one_by_one(fsm, g, k, t, opts, most=60):
     for key, val in opts.items():
         G.set_option(key, val)
     try:
+        G.mine(k, t)   # the handle's tables are made
         whole = G.mine(k, t, stats=True)
         out = []
         for n in range(1, most):
@@ -96,3 +97,19 @@ def test_a_small_one_pass_level_takes_little_memory(fsm, launch, t, mib):
             f"G.set_option('launch', {launch})\nG.mine(5, {t})\nf = free()\n"
             f"G.set_option('fused', 1)\nG.mine(5, {t})\nprint(f - free())\n")
     assert _device_memory_taken(body) <= mib << 20
+
+
+@pytest.mark.parametrize("launch", [0, 1])
+def test_a_level_gives_its_prefix_back(fsm, launch):
+    """Size 3, which keeps no joins: the prefix of the level's units is the one allocation to give back, and
+    every pass left makes its own."""
+    whole, out = _refused_one_by_one(fsm, gg.workload("cl3700k", scale=0.001, cap=20), 3, 5, {"launch": launch})
+    assert len(whole["support"]) > 0
+    assert sum(r is not None and r["stats"]["kernel_launches"] > whole["stats"]["kernel_launches"] for r in out) >= 5
+
+
+@pytest.mark.parametrize("launch", [0, 1])
+def test_a_level_gives_its_kept_joins_back(fsm, launch):
+    whole, out = _refused_one_by_one(fsm, gg.workload("cl3700k", scale=0.001, cap=20), 5, 20, {"launch": launch})
+    assert whole["stats"]["kept_levels"] == 1
+    assert sum(r is not None and r["stats"]["kept_levels"] == 0 for r in out) >= 2
