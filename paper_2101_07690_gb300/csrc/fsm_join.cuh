@@ -168,6 +168,12 @@ __device__ __forceinline__ int32_t below(const int32_t *a, int32_t n, int32_t x)
     return lo;
 }
 
+// Option "debug": does index `at` of the piece lists lie in the list a row's partners come from, that of
+// the key vertex [rp, rp + d) for a centre row, that of the anchor [al, al + ad) for an end list?
+FSM_HD bool partner_in_list(bool centre, int64_t at, int64_t rp, int64_t d, int64_t al, int64_t ad) {
+    return centre ? at >= rp && at < rp + d : at >= al && at < al + ad;
+}
+
 // Largest u in [lo, hi] with base[u] <= x (base[lo] <= x), by the whole warp: 32 probes per step,
 // so a prefix of millions of units takes five dependent reads instead of over twenty.
 __device__ __forceinline__ int64_t warp_last_le(const int64_t *base, int64_t lo, int64_t hi, int64_t x) {
@@ -818,7 +824,8 @@ struct Joiner {
                 } else {
                     const int32_t anchor = __ldg(g.pcol + rp + y);
                     const uint32_t ainfo = __ldg(g.pinfo + rp + y);
-                    bool in = false;
+                    bool in = A.debug && (anchor < 0 || anchor >= g.n);   // it indexes the lists
+                    if (in) atomicOr(A.err, FSM_ERR_BOUNDS);
                     int s = 0;
 #pragma unroll
                     for (int t = 0; t < L; ++t) {
@@ -897,13 +904,19 @@ struct Joiner {
                     m = sm.sg_meta[w][k];
                     anchor = (int32_t)sm.sg_anchor[w][k];
                     const int64_t at = (int64_t)(int32_t)(sm.sg_base[w][k] + (uint32_t)t);
-                    if (A.debug && (at < 0 || at >= __ldg(g.prow + g.n))) {
+                    const uint32_t *r = rec(m & 15);
+                    bool in = true;
+                    if (A.debug) {
+                        const int32_t al = __ldg(g.prow + anchor);
+                        in = partner_in_list(!((m >> FSM_M_END) & 1u), at, (int32_t)r[R::RP], (int32_t)r[R::D], al,
+                                             __ldg(g.prow + anchor + 1) - al);
+                    }
+                    if (!in) {
                         atomicOr(A.err, FSM_ERR_BOUNDS);
                         ok = false;
                     } else {
                         x = __ldg(g.pcol + at);
                         xinfo = __ldg(g.pinfo + at);
-                        const uint32_t *r = rec(m & 15);
                         int s = 0;
 #pragma unroll
                         for (int t2 = 0; t2 < L; ++t2) {
@@ -957,6 +970,7 @@ struct Joiner {
                     const int64_t p = lq - nc - __ldg(g.pend + rp + y);
                     anchor = __ldg(g.pcol + rp + y);
                     ainfo = __ldg(g.pinfo + rp + y);
+                    if (A.debug && (anchor < 0 || anchor >= g.n)) { atomicOr(A.err, FSM_ERR_BOUNDS); anchor = 0; ok = false; }
                     const int32_t lb0 = __ldg(g.prow + anchor);
                     if (A.debug && (p < 0 || p >= __ldg(g.prow + anchor + 1) - lb0)) { atomicOr(A.err, FSM_ERR_BOUNDS); ok = false; }
                     if (ok) {
