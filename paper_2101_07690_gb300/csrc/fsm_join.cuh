@@ -824,8 +824,7 @@ struct Joiner {
                 } else {
                     const int32_t anchor = __ldg(g.pcol + rp + y);
                     const uint32_t ainfo = __ldg(g.pinfo + rp + y);
-                    bool in = A.debug && (anchor < 0 || anchor >= g.n);   // it indexes the lists
-                    if (in) atomicOr(A.err, FSM_ERR_BOUNDS);
+                    bool in = false;
                     int s = 0;
 #pragma unroll
                     for (int t = 0; t < L; ++t) {
@@ -970,7 +969,6 @@ struct Joiner {
                     const int64_t p = lq - nc - __ldg(g.pend + rp + y);
                     anchor = __ldg(g.pcol + rp + y);
                     ainfo = __ldg(g.pinfo + rp + y);
-                    if (A.debug && (anchor < 0 || anchor >= g.n)) { atomicOr(A.err, FSM_ERR_BOUNDS); anchor = 0; ok = false; }
                     const int32_t lb0 = __ldg(g.prow + anchor);
                     if (A.debug && (p < 0 || p >= __ldg(g.prow + anchor + 1) - lb0)) { atomicOr(A.err, FSM_ERR_BOUNDS); ok = false; }
                     if (ok) {
