@@ -679,6 +679,9 @@ struct Miner {
             // (108 words), one pass: 154 ms with, 146 ms without; 3.7M vertices, size 3: 9.4 and 7.8 ms
             A.check_bits = (int64_t)G->n < (int64_t)512 * G->NL;
             A.any = G->join_any[L];
+            // few stored patterns and labels: few keys (37 labels, l = 1: 1369; 4 labels: 16; the counts of
+            // both are at count_join)
+            A.merge = in.P * G->NL < 1024;
             if (piece_freq) {
                 lf = mem.get<unsigned long long>(3 * 4096);
                 ck(launch_label_masks(piece_freq, lf, st), "label masks");

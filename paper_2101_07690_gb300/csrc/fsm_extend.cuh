@@ -98,6 +98,7 @@ struct ExtArgs {
     uint32_t *keep_n;
     uint32_t keep_cap;
     unsigned long long *keep_over;
+    int merge;                     // join kernel's count pass: lanes of one key add to its count once
     int check_bits;                // read a bitmap word before reducing into it
     int warm;                      // count a sample of the chunks only (before a one-pass level)
     // tables of fsm_join.cuh for this level size, and the size-3 frequencies as label masks: W[c][x]

@@ -347,13 +347,27 @@ struct Joiner {
         d[2 + L] = r1;
     }
 
+    // One more join of key slot `slot`, for the lanes here together: lanes of one key add once.  A few keys
+    // that take all of a level's joins (few labels, hubs) queue on their counters otherwise: 30k vertices, 4
+    // labels, two hubs of degree 20000, 4e8 joins of 138 keys, 1 -> 3 count 24.6 ms, 6.2 this way; 2 -> 4 one
+    // pass, 3.2e9 joins, whole call 114 and 95 ms.  Where a count pass meets many keys the match only costs
+    // (4 -> 6, 2.9e8 joins, whole call 18.5 and 18.9 ms; 1 -> 3, 37 labels, 10.5 and 10.8): ExtArgs::merge.
+    __device__ __forceinline__ void count_join(int64_t slot) {
+        if (PASS == PASS_FUSED || A.merge) {
+            const unsigned same = __match_any_sync(__activemask(), (uint32_t)slot);
+            if (lane == __ffs(same) - 1) atomicAdd(A.qp.count + slot, (unsigned long long)__popc(same));
+        } else {
+            atomicAdd(A.qp.count + slot, 1ull);
+        }
+    }
+
     // One accepted join of this lane (not warp-synchronous).
     __device__ __forceinline__ void accept(const uint32_t *r, int j, uint64_t key, bool centre, int32_t anchor, int32_t x,
                                            uint32_t ainfo, uint32_t xinfo, bool swap) {
         if constexpr (PASS == PASS_COUNT) {
             const int64_t slot = qp_insert(A.qp, key, A.err);
             if (slot < 0) return;
-            atomicAdd(A.qp.count + slot, 1ull);
+            count_join(slot);
             if (A.keep) {
                 const unsigned act = __activemask();
                 const int leader = __ffs(act) - 1;
@@ -381,7 +395,7 @@ struct Joiner {
                 if (PASS == PASS_FUSED) defer(r, key, swap ? rb : ra, swap ? ra : rb);
                 return;   // domain pass: pattern without bitmaps
             }
-            if (PASS == PASS_FUSED) atomicAdd(A.qp.count + slot, 1ull);
+            if (PASS == PASS_FUSED) count_join(slot);
             // A unit's joins of one key set the same bits of s: a small table of (unit, slot) pairs
             // already seen in this batch keeps most of those reductions away.  A lost entry or a race
             // only repeats them.

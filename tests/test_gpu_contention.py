@@ -1,0 +1,45 @@
+"""What a level costs does not hang on how its joins fall: few keys, hubs, rare pieces.  Times of a pass are
+those of option profile, best of three, compared with the same enumeration in another dress."""
+import numpy as np
+import pytest
+
+import graphgen as gg
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def fsm():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_2101_07690_gb300 import build, fsm as f
+    build.build()
+    f.load()
+    return f
+
+
+def _two_hubs(labels, degree=20000, n=30000):
+    """Two vertices of that degree over a sparse rest."""
+    rng = np.random.default_rng(1)
+    pairs = np.concatenate([np.stack([np.full(degree, h), rng.choice(np.arange(2, n), degree, replace=False)], 1)
+                            for h in (0, 1)] + [rng.integers(2, n, (n - 10000, 2))])
+    pairs = np.unique(np.sort(pairs[pairs[:, 0] != pairs[:, 1]], 1), axis=0)
+    ids = rng.permutation(n)
+    return gg.from_edges(n, ids[pairs], rng.integers(0, labels, n).astype(np.int32), labels)
+
+
+def _pass_ms(fsm, g, k, t, name, options=None):
+    G = fsm.Graph.from_graphgen(g)
+    for key, val in {**(options or {}), "profile": 1}.items():
+        G.set_option(key, val)
+    try:
+        return min(G.mine(k, t, stats=True)["stats"][name] for _ in range(4)) / 1e6
+    finally:
+        G.close()
+
+
+def test_few_keys_cost_no_more_than_many(fsm):
+    """Size 3 on two hubs: 4e8 joins of some 100 quick patterns (4 labels) or of 100000 (64 labels)."""
+    few, many = (_pass_ms(fsm, _two_hubs(labels), 3, 100, "count_ns_l1") for labels in (4, 64))
+    assert few <= 1.5 * many, (few, many)
