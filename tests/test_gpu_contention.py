@@ -43,3 +43,25 @@ def test_few_keys_cost_no_more_than_many(fsm):
     """Size 3 on two hubs: 4e8 joins of some 100 quick patterns (4 labels) or of 100000 (64 labels)."""
     few, many = (_pass_ms(fsm, _two_hubs(labels), 3, 100, "count_ns_l1") for labels in (4, 64))
     assert few <= 1.5 * many, (few, many)
+
+
+@pytest.mark.parametrize("name", ["count_ns_l1", "domain_ns_l1"])
+def test_a_level_that_draws_nothing_costs_what_an_exact_one_does(fsm, name):
+    """Join quotas draw nothing at size 3."""
+    g = gg.workload("cl3700k", scale=0.1, cap=300)
+    exact, quota = (_pass_ms(fsm, g, 3, 2000, name, o) for o in ({}, {"join_quota": 2}))
+    assert quota <= 1.25 * exact, (exact, quota)
+
+
+def test_matching_quota_alone_leaves_the_joins_exact(fsm):
+    """With match_quota large enough to cut nothing and no join_quota: exact mining, in all three sizes."""
+    g = gg.workload("cl3700k", scale=0.002, cap=40)
+    G = fsm.Graph.from_graphgen(g)
+    exact = [G.mine(k, 30) for k in (3, 4, 5)]
+    G.set_option("match_quota", 1 << 32)
+    for k, want in zip((3, 4, 5), exact):
+        got = G.mine(k, 30)
+        assert len(want["support"]) > 0
+        for key in ("labels", "adj", "support", "count"):
+            assert np.array_equal(got[key], want[key]), (k, key)
+    G.close()
