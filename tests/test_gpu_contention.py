@@ -65,3 +65,8 @@ def test_matching_quota_alone_leaves_the_joins_exact(fsm):
         for key in ("labels", "adj", "support", "count"):
             assert np.array_equal(got[key], want[key]), (k, key)
     G.close()
+
+
+def test_a_hub_in_an_embedding_does_not_cost_its_list_per_batch(fsm):
+    """Quota 2 joins the edges of two hubs of degree 20000: some 2e5 pieces, at most 5 ns each."""
+    assert _pass_ms(fsm, _two_hubs(4), 4, 100, "count_ns_l2", {"join_quota": 2}) <= 1.0
