@@ -445,7 +445,7 @@ struct Miner {
             const int grid = grid_for(L, pass);
             int64_t chunk = chunk_for(L);
             const int64_t warps = (int64_t)grid * 8;
-            if (chunk <= 0) chunk = joins(L) ? join_chunk(pre.total, warps) : extend_chunk(pre.total, in.N * L, warps);
+            if (chunk <= 0) chunk = joins(L) ? join_chunk(pre.total, in.N * L, warps) : extend_chunk(pre.total, in.N * L, warps);
             A.fv = in.fv;
             A.fpid = in.fpid;
             A.fN = in.N;
@@ -539,7 +539,7 @@ struct Miner {
                 bytes(r);
                 int64_t chunk = chunk_for(L);
                 // as the kernel does when the total stays on the device
-                if (chunk <= 0) chunk = joins(L) ? join_chunk(total, warps) : extend_chunk(total, r.ne * L, warps);
+                if (chunk <= 0) chunk = joins(L) ? join_chunk(total, r.ne * L, warps) : extend_chunk(total, r.ne * L, warps);
                 A.e0 = r.e0;
                 A.ne = r.ne;
                 A.total = total;

@@ -1052,7 +1052,7 @@ __global__ void __launch_bounds__(256, JoinBlocks<L, PASS>::value) join_kernel(c
     if (total < 0) {
         // device-resident size: no host round trip between the prefix sum and this launch
         total = __ldg(A.unit_base + nunits);
-        if (chunk <= 0) chunk = join_chunk(total, (int64_t)gridDim.x * (blockDim.x >> 5));
+        if (chunk <= 0) chunk = join_chunk(total, nunits, (int64_t)gridDim.x * (blockDim.x >> 5));
         nchunks = (total + chunk - 1) / chunk;
     }
     int64_t stride = 1;

@@ -70,3 +70,38 @@ def test_matching_quota_alone_leaves_the_joins_exact(fsm):
 def test_a_hub_in_an_embedding_does_not_cost_its_list_per_batch(fsm):
     """Quota 2 joins the edges of two hubs of degree 20000: some 2e5 pieces, at most 5 ns each."""
     assert _pass_ms(fsm, _two_hubs(4), 4, 100, "count_ns_l2", {"join_quota": 2}) <= 1.0
+
+
+def _sampled_ms(fsm, g, rate):
+    G = fsm.Graph.from_graphgen(g)
+    G.set_option("profile", 1)
+    try:
+        return min(G.mine(3, 2, sample_rate=rate, stats=True)["stats"]["count_ns_l1"] for _ in range(4)) / 1e6
+    finally:
+        G.close()
+
+
+@pytest.mark.parametrize("rate", [1e-2, 1e-3, 1e-4])
+def test_rare_pieces_cost_no_more_than_frequent_ones(fsm, rate):
+    """A path of 200k vertices: 10000, 1000, 100 pieces among as many units take no more than twice the
+    time of 100000."""
+    n = 200000
+    g = gg.from_edges(n, [(i, i + 1) for i in range(n - 1)], (np.arange(n) % 5).astype(np.int32), 5)
+    assert _sampled_ms(fsm, g, rate) <= 2 * _sampled_ms(fsm, g, 0.1)
+
+
+def test_sampled_results_do_not_depend_on_the_chunk(fsm):
+    """The chunks of a sparse level (8 pieces) and given ones find the same joins."""
+    g = gg.workload("cl3700k", scale=0.002, cap=20)
+    out = []
+    for opts in ({}, {"launch": 1}, {"chunk": 32}, {"chunk": 4096, "launch": 1}):
+        G = fsm.Graph.from_graphgen(g)
+        for key, val in {**opts, "candidates": 1}.items():
+            G.set_option(key, val)
+        out.append([G.mine(k, 20, sample_rate=p) for k, p in ((5, 0.001), (4, 0.01), (3, 0.01))])
+        G.close()
+    assert all(len(r["support"]) > 0 for r in out[0])
+    for got in out[1:]:
+        for a, b in zip(got, out[0]):
+            for key in ("labels", "adj", "support", "count"):
+                assert np.array_equal(a[key], b[key]), key
