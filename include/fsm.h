@@ -131,6 +131,8 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
  *   "fused_pool" size in 32-bit words of the one-pass level's bitmap pool (0 = twice what a sample of
  *                the level or the previous call needed, grown on demand up to 40% of the free device
  *                memory).
+ *   "fused_defer" joins that the one-pass level puts aside at most, 32 bytes each (0 = one in eight of its
+ *                pieces, at most 2^24; none where the sample is the whole level).
  *   "seed"       64-bit seed of the piece sampling of fsm_mine with sample_rate < 1 (default 0).
  *   "candidates" 1 = sampled mining returns every candidate pattern of the sampled level with
  *                its estimated support (smallest orbit popcount / p) and its 32 features

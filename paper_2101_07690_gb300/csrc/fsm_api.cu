@@ -223,6 +223,7 @@ struct fsm_graph {
     int fused = 0;
     unsigned long long pool_hint[FSM_MAXL + 1] = {};   // pool words the fused pass used last time
     unsigned long long pool_force = 0;                 // option "fused_pool": fixed pool size
+    unsigned long long defer_force = 0;                // option "fused_defer": fixed room for joins put aside
     int32_t tuned_chunk[FSM_MAXL + 1] = {};   // chunk size chosen by the autotuner per level
     // sampled mining
     uint64_t seed = 0;
@@ -843,7 +844,8 @@ struct Miner {
                 A.pool_words = pool_words;
                 // Joins put aside: 32 bytes each, room for one in eight pieces; past 2^24 the level is redone
                 // in two passes.  A sample of every piece has met every key.
-                A.defer_cap = warm_stride(pieces) == 1 ? 256 : std::min<unsigned long long>(1ull << 24, pieces / 8);
+                A.defer_cap = G->defer_force ? G->defer_force
+                            : warm_stride(pieces) == 1 ? 256 : std::min<unsigned long long>(1ull << 24, pieces / 8);
                 pool = (uint32_t *)mem.optional(pool_words * 4);
                 if (pool) mem.ptrs.push_back(pool);
                 A.defer = pool ? (uint32_t *)mem.optional(A.defer_cap * FSM_DEFER_WORDS * 4) : nullptr;
@@ -888,7 +890,6 @@ struct Miner {
                 rs.launches += 2;
                 sc = scalars();
             }
-            if (fused) rs.fused_deferred = (int64_t)sc[S_DEFER];
             if (A.defer) mem.release(A.defer);
             A.defer = nullptr;
             const int ew = sc.err();
@@ -924,6 +925,7 @@ struct Miner {
             if (fused) {
                 G->pool_hint[L] = sc[S_POOL];
                 rs.fused_pool_words = (int64_t)G->pool_hint[L];
+                rs.fused_deferred = (int64_t)sc[S_DEFER];
             }
             break;
         }
@@ -1478,6 +1480,9 @@ int fsm_set_option(fsm_graph *g, const char *key, int64_t value) {
         } else if (k == "fused_pool") {
             if (value < 0) fail(FSM_EINVAL, "fused_pool must be >= 0");
             g->pool_force = (unsigned long long)value;
+        } else if (k == "fused_defer") {
+            if (value < 0 || value > (1 << 24)) fail(FSM_EINVAL, "fused_defer must be in [0, 2^24]");
+            g->defer_force = (unsigned long long)value;
         } else if (k == "seed") {
             g->seed = (uint64_t)value;
         } else if (k == "candidates") {

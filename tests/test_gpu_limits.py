@@ -113,3 +113,41 @@ def test_a_level_gives_its_kept_joins_back(fsm, launch):
     whole, out = _refused_one_by_one(fsm, gg.workload("cl3700k", scale=0.001, cap=20), 5, 20, {"launch": launch})
     assert whole["stats"]["kept_levels"] == 1
     assert sum(r is not None and r["stats"]["kept_levels"] == 0 for r in out) >= 2
+
+
+def test_the_one_pass_level_falls_back_when_joins_put_aside_run_out(fsm):
+    """A level larger than its sample (2^26 pieces) meets keys the sample missed; with room for 16 of their
+    joins it is redone in two passes, and has put none aside."""
+    g = gg.workload("cl3700k", scale=0.002, cap=20)
+    out = []
+    for defer in (0, 16):
+        G = fsm.Graph.from_graphgen(g)
+        G.set_option("fused", 1)
+        G.set_option("fused_defer", defer)
+        out.append(G.mine(5, g.n // 400, stats=True))
+        G.close()
+    assert out[0]["stats"]["fused_deferred"] > 16 and out[0]["stats"]["fused_fallbacks"] == 0
+    assert out[1]["stats"]["fused_deferred"] == 0 and out[1]["stats"]["fused_fallbacks"] == 1
+    for key in ("labels", "adj", "support", "count"):
+        assert np.array_equal(out[0][key], out[1][key]), key
+
+
+def test_a_pool_too_small_puts_nothing_aside(fsm):
+    """Pools with room for the sample's patterns but not for those met later, too: joins were put aside, then
+    the level was redone in two passes, and the statistics are those of the passes that count.  (How many
+    words a call uses varies by what lanes that resolve one pattern together reserve twice.)"""
+    g = gg.workload("cl3700k", scale=0.002, cap=20)
+    G = fsm.Graph.from_graphgen(g)
+    G.set_option("fused", 1)
+    whole = G.mine(5, g.n // 400, stats=True)
+    fell_back = 0
+    for percent in (50, 90, 94, 96, 97, 98, 99):
+        G.set_option("fused_pool", whole["stats"]["fused_pool_words"] * percent // 100)
+        got = G.mine(5, g.n // 400, stats=True)
+        if got["stats"]["fused_fallbacks"]:
+            fell_back += 1
+            assert got["stats"]["fused_deferred"] == 0, percent
+        for key in ("labels", "adj", "support", "count"):
+            assert np.array_equal(got[key], whole[key]), key
+    G.close()
+    assert fell_back > 0
