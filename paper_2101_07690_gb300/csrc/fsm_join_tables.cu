@@ -1,133 +1,28 @@
 // fsm_join_tables.cu -- the acceptance tables of the join kernel (JoinGeo, fsm_join.cuh) and the
 // dispatch of its passes.
-#include "fsm_join.cuh"
+#include "fsm_join_tables.cuh"
 #include "fsm_kernels.cuh"
 
 namespace fsm {
 namespace {
 
-// one 32-subset word of one row per thread
+// one entry per thread
 template <int L>
 __global__ void acc_kernel(uint32_t *acc) {
-    using G = JoinGeo<L>;
-    const int64_t n = (int64_t)G::CLS * G::ROWS * G::W;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < n; x += (int64_t)gridDim.x * blockDim.x) {
-        const int wd = (int)(x % G::W);
-        int64_t y = x / G::W;
-        const int bgt = (int)(y & 1);
-        y >>= 1;
-        const int sb = (int)(y % G::SL);
-        y /= G::SL;
-        const int sa = (int)(y % G::SL);
-        y /= G::SL;
-        const int form = (int)(y % 3), cls = (int)(y / 3);
-        uint32_t m = 0;
-        const int subs = G::SUBS < 32 ? G::SUBS : 32;
-        for (int s = 0; s < subs; ++s)
-            if (join_accepted<L>(cls, form, sa, sb, bgt, (uint32_t)(wd * 32 + s))) m |= 1u << s;
-        acc[x] = m;
-    }
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < JoinGeo<L>::ACC_WORDS; x += (int64_t)gridDim.x * blockDim.x)
+        acc[x] = acc_word<L>(x);
 }
-
-// Seven vertices (l = 5) have 283M combinations but only 2^21 graphs on ordered ids: dissect each
-// graph once (part mask | join vertex << 7, 0 if disconnected), then look them up.  Bit of pair
-// (x, y), x < y: y (y - 1) / 2 + x.
 __global__ void dissect7_kernel(uint16_t *code) {
-    const int32_t gid[7] = {0, 1, 2, 3, 4, 5, 6};
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < (1 << 21); c += gridDim.x * blockDim.x) {
-        uint32_t adj[7] = {0, 0, 0, 0, 0, 0, 0};
-        for (int y = 1; y < 7; ++y)
-            for (int x = 0; x < y; ++x)
-                if ((c >> (y * (y - 1) / 2 + x)) & 1) { adj[x] |= 1u << y; adj[y] |= 1u << x; }
-        uint16_t r = 0;
-        if (mask_connected(127u, adj, 7)) {
-            uint32_t lm = 0;
-            int jn = -1;
-            dissect3(7, gid, adj, lm, jn);
-            r = (uint16_t)(lm | ((uint32_t)jn << 7));
-        }
-        code[c] = r;
-    }
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < (1 << 21); c += gridDim.x * blockDim.x) code[c] = dissect7_code(c);
 }
-__device__ __forceinline__ uint32_t pair_bit(int x, int y) {
-    const int a = x < y ? x : y, b = x < y ? y : x;
-    return 1u << (b * (b - 1) / 2 + a);
+__global__ void acc5_kernel(const uint16_t *__restrict__ code, uint32_t *acc) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < JoinGeo<5>::ACC_WORDS; i += (int64_t)gridDim.x * blockDim.x)
+        acc[i] = acc5_word(code, i);
 }
-__global__ void acc5_kernel(const uint16_t *code, uint32_t *acc) {
-    constexpr int L = 5;
-    using G = JoinGeo<L>;
-    const int64_t n = (int64_t)G::CLS * G::ROWS * G::W;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int wd = (int)(i % G::W);
-        int64_t y = i / G::W;
-        const int bgt = (int)(y & 1);
-        y >>= 1;
-        const int sb = (int)(y % G::SL);
-        y /= G::SL;
-        const int sa = (int)(y % G::SL);
-        y /= G::SL;
-        const int form = (int)(y % 3), cls = (int)(y / 3), rv = cls >> G::EB;
-        uint32_t m = 0;
-        const bool order = (sa == sb || (sb > sa) == (bgt != 0)) && (form == FORM_END || bgt);
-        uint32_t sadj[5] = {0, 0, 0, 0, 0};
-        int bit = 0;
-        for (int t = 0; t < L; ++t)
-            for (int u = t + 1; u < L; ++u, ++bit)
-                if ((cls >> bit) & 1) { sadj[t] |= 1u << u; sadj[u] |= 1u << t; }
-        if (order && mask_connected(31u, sadj, L)) {
-            int pos[L];
-            for (int t = 0; t < L; ++t) pos[t] = t + (sa <= t) + (sb <= t);
-            const int pa = sa + (bgt ? 0 : 1), pb = sb + (bgt ? 1 : 0), pv = pos[rv];
-            uint32_t base = pair_bit(pv, pa);
-            if (form != FORM_END) base |= pair_bit(pv, pb);
-            if (form != FORM_CENTRE) base |= pair_bit(pa, pb);
-            for (int t = 0; t < L; ++t)
-                for (int u = t + 1; u < L; ++u)
-                    if ((sadj[t] >> u) & 1u) base |= pair_bit(pos[t], pos[u]);
-            uint32_t cb[8];
-            for (int r = 0; r < 4; ++r) {
-                const int t = r + (r >= rv);
-                cb[r] = pair_bit(pos[t], pa);
-                cb[4 + r] = pair_bit(pos[t], pb);
-            }
-            const uint32_t want = (1u << pv) | (1u << pa) | (1u << pb) | ((uint32_t)pv << 7);
-            for (int q = 5; q < 8; ++q)
-                if ((wd >> (q - 5)) & 1) base |= cb[q];
-            for (int s = 0; s < 32; ++s) {
-                uint32_t c = base;
-                for (int q = 0; q < 5; ++q)
-                    if ((s >> q) & 1) c |= cb[q];
-                if (__ldg(code + c) == want) m |= 1u << s;
-            }
-        }
-        acc[i] = m;
-    }
-}
-
-// entry (class, ANY_*, anchor slot): partner slots that some subset and form accept
 template <int L>
 __global__ void any_kernel(const uint32_t *acc, uint16_t *any) {
-    using G = JoinGeo<L>;
-    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < G::ANY_ENTRIES; x += (int64_t)gridDim.x * blockDim.x) {
-        const int s = (int)(x % G::SL), kind = (int)(x / G::SL) & 3;
-        const int64_t cls = x / (4 * G::SL);
-        auto some = [&](int form, int sa, int sb, int bgt) {
-            const uint32_t *r = acc + (cls * G::ROWS + ((int64_t)(form * G::SL + sa) * G::SL + sb) * 2 + bgt) * G::W;
-            uint32_t m = 0;
-            for (int i = 0; i < G::W; ++i) m |= r[i];
-            return m != 0;
-        };
-        uint32_t m = 0;
-        for (int p = 0; p < G::SL; ++p) {
-            if (kind == ANY_C || kind == ANY_CT) {   // anchor b, partner a < b
-                if (some(FORM_CENTRE, p, s, 1) || (kind == ANY_CT && some(FORM_TRI, p, s, 1))) m |= 1u << p;
-            } else {                                 // anchor a, partner b
-                if (some(FORM_END, s, p, 0)) m |= 1u << p;
-                if (some(FORM_END, s, p, 1) || (kind == ANY_ET && some(FORM_TRI, s, p, 1))) m |= 1u << (p + G::SL);
-            }
-        }
-        any[x] = (uint16_t)m;
-    }
+    for (int64_t x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; x < JoinGeo<L>::ANY_ENTRIES; x += (int64_t)gridDim.x * blockDim.x)
+        any[x] = any_entry<L>(acc, x);
 }
 
 template <int L>

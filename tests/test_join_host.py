@@ -23,3 +23,9 @@ def report(tmp_path_factory):
 
 def test_debug_checks_an_index_against_its_own_list(report):
     assert report["bounds"] == "0"
+
+
+def test_tables_as_the_device_fills_them_match_the_rule(report):
+    """Both tables of every stored size, that of size 5 by its own way over the 2^21 graphs of 7 vertices."""
+    assert int(report["kept"]) > 1000
+    assert report["acc"] == "0" and report["any"] == "0"
