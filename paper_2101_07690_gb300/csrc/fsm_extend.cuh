@@ -178,24 +178,51 @@ __device__ __forceinline__ int64_t last_le(const int64_t *base, int64_t lo, int6
 // table is too small, so the pass is flagged, abandoned and repeated with a larger table.
 #define FSM_MAX_PROBES 256
 
-__device__ __forceinline__ int64_t qp_insert(const QPTab &t, uint64_t key, int *err) {
-    uint64_t h = mix64(key) & t.mask;
-    for (uint64_t probe = 0; probe <= t.mask && probe < FSM_MAX_PROBES; ++probe) {
-        unsigned long long cur = __ldcg(t.keys + h);
-        if (cur == key) return (int64_t)h;
-        if (cur == FSM_EMPTY_KEY) {
-            unsigned long long old = atomicCAS(t.keys + h, FSM_EMPTY_KEY, key);
-            if (old == FSM_EMPTY_KEY) {
-                unsigned long long u = atomicAdd(t.used, 1ull);
-                if (u >= t.max_used) atomicOr(err, FSM_ERR_QP_OVERFLOW);
-                return (int64_t)h;
-            }
-            if (old == key) return (int64_t)h;
+// one slot of the probe sequence: true when it is the key's (claimed where it was empty)
+__device__ __forceinline__ bool qp_try(const QPTab &t, uint64_t key, uint64_t h, int *err) {
+    unsigned long long cur = __ldcg(t.keys + h);
+    if (cur == key) return true;
+    if (cur == FSM_EMPTY_KEY) {
+        unsigned long long old = atomicCAS(t.keys + h, FSM_EMPTY_KEY, key);
+        if (old == FSM_EMPTY_KEY) {
+            unsigned long long u = atomicAdd(t.used, 1ull);
+            if (u >= t.max_used) atomicOr(err, FSM_ERR_QP_OVERFLOW);
+            return true;
         }
+        if (old == key) return true;
+    }
+    return false;
+}
+
+// The rest of a long probe sequence, out of line: a key of a half-full table rarely gets here.  A table that
+// overflows is full before its pass stops, and every key would be looked for in FSM_MAX_PROBES slots until
+// then: 30k vertices, size 3, from 64 slots up to 2^18, 98.6 ms, 11.9 this way; 37k, size 5, count 3 -> 5, 109 and
+// 19.7 ms.  Near probes 8 or 16: 4 -> 6 whole call 18.7 and 18.0 ms, 3 -> 5 one pass 23.4 and 22.3 (18.7 and 22.9
+// with all of them inline).
+#define FSM_NEAR_PROBES 16   // the smallest table has 64 slots
+static __device__ __noinline__ int64_t qp_insert_far(unsigned long long *keys, unsigned long long *used, uint64_t mask,
+                                                     unsigned long long max_used, uint64_t key, uint64_t h, int *err) {
+    QPTab t;
+    t.keys = keys;
+    t.used = used;
+    t.mask = mask;
+    t.max_used = max_used;
+    for (uint64_t probe = FSM_NEAR_PROBES; probe <= t.mask && probe < FSM_MAX_PROBES; ++probe) {
+        if ((probe & 15) == 0 && (*(volatile int *)err & FSM_ERR_QP_OVERFLOW)) return -1;
+        if (qp_try(t, key, h, err)) return (int64_t)h;
         h = (h + 1) & t.mask;
     }
     atomicOr(err, FSM_ERR_QP_OVERFLOW);
     return -1;
+}
+
+__device__ __forceinline__ int64_t qp_insert(const QPTab &t, uint64_t key, int *err) {
+    uint64_t h = mix64(key) & t.mask;
+    for (int probe = 0; probe < FSM_NEAR_PROBES; ++probe) {
+        if (qp_try(t, key, h, err)) return (int64_t)h;
+        h = (h + 1) & t.mask;
+    }
+    return qp_insert_far(t.keys, t.used, t.mask, t.max_used, key, h, err);
 }
 
 __device__ __forceinline__ int64_t qp_find(const QPTab &t, uint64_t key) {

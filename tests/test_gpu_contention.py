@@ -105,3 +105,18 @@ def test_sampled_results_do_not_depend_on_the_chunk(fsm):
         for a, b in zip(got, out[0]):
             for key in ("labels", "adj", "support", "count"):
                 assert np.array_equal(a[key], b[key]), key
+
+
+def test_a_table_that_overflows_is_left_at_once(fsm):
+    """Size 3 of 45000 quick patterns from a table of 64 slots, grown to 2^18 in six steps: at most ten times
+    the call that has its table from the start."""
+    g = gg.workload("cl100k", scale=0.3, cap=300)
+    took = []
+    for cap in (1 << 20, 64):
+        G = fsm.Graph.from_graphgen(g)
+        G.set_option("qp_capacity", cap)
+        r = [G.mine(3, 150, stats=True)["stats"] for _ in range(3)]
+        G.close()
+        assert r[0]["qp_grows"] == (0 if cap > 64 else 6)
+        took.append(min(x["time_ns"] for x in r) / 1e6)
+    assert took[1] <= 10 * took[0], took
