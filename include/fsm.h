@@ -88,8 +88,8 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
  *                frontier for chunk sizes 256, 1024, 4096, 16384 and keep the fastest for later
  *                passes and calls (reported as stat "chunk_l<l>"); 0 = forget tuned values.
  *   "chunk"      pieces per work-stealing chunk (power of two, 32..65536; 0 = default: the largest
- *                power of two from 64 to 8192 that leaves at least 8 chunks per warp; where the
- *                extension kernel runs -- the ablations, and levels extended from size 6 and 7 -- the
+ *                power of two from 64 to 8192 that leaves at least 8 chunks per warp, or 2 below
+ *                256, and from 8 where units outnumber pieces four to one; where the extension kernel runs -- the ablations, and levels extended from size 6 and 7 -- the
  *                largest from 256 to 16384 that leaves at least 64 chunks per warp and spans at most
  *                about 16 units' pieces).
  *   "batch"      frontier embeddings per batch (>= 1024; 0 = default).

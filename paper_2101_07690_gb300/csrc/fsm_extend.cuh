@@ -136,14 +136,15 @@ FSM_HD int64_t extend_chunk(int64_t total, int64_t units, int64_t warps) {
     return chunk;
 }
 // Join kernel, which prepares units in batches of its own: a chunk costs two searches of the prefix
-// and a part-filled last batch, so it is as large as leaves 8 chunks per warp, from 64 to 8192 (3 -> 5
-// count, 1.7e8 pieces: 1.83 ms at 1024, 1.63 at 4096, 1.74 at 8192; 5 -> 7 count, 6.0e8: 35 ms at
+// and a part-filled last batch, so it is as large as leaves 8 chunks per warp, or 2 below 256, from 64 to
+// 8192 (100k vertices with hubs, size 3 in batches of 1024 vertices, 3.3e6 pieces each, whole call: 8.3 ms at
+// 64, 6.4 at 128, 5.4 at 256; 3 -> 5 count, 1.7e8 pieces: 1.83 ms at 1024, 1.63 at 4096, 1.74 at 8192; 5 -> 7 count, 6.0e8: 35 ms at
 // 512, 27 at 8192, 30 at 65536; 1 -> 3, 6.3e8: 7.9 ms at 512, 5.7 at 8192).  Where at most one unit in four
 // has a piece (sampling), every piece of a chunk costs a search for its unit, one after another: from 8
 // pieces on (path of 200k vertices, rate 1e-3, 965 pieces: count 0.05 ms, 0.24 at 64).
 FSM_HD int64_t join_chunk(int64_t total, int64_t units, int64_t warps) {
     int64_t chunk = units >= 4 * total ? 8 : 64;
-    while (chunk < 8192 && total >= chunk * 2 * 8 * warps) chunk <<= 1;
+    while (chunk < 8192 && total >= chunk * 2 * (chunk < 256 ? 2 : 8) * warps) chunk <<= 1;
     return chunk;
 }
 

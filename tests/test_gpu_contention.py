@@ -120,3 +120,18 @@ def test_a_table_that_overflows_is_left_at_once(fsm):
         assert r[0]["qp_grows"] == (0 if cap > 64 else 6)
         took.append(min(x["time_ns"] for x in r) / 1e6)
     assert took[1] <= 10 * took[0], took
+
+
+def test_small_launches_take_chunks_that_pay(fsm):
+    """Size 3 around hubs in batches of 1024 vertices, and per label: no more than 1.25 times what chunks of
+    256 pieces take."""
+    g = gg.workload("cl100k", scale=0.3, cap=300)
+    for opts in ({"batch": 1024}, {"launch": 2}):
+        took = []
+        for chunk in (256, 0):
+            G = fsm.Graph.from_graphgen(g)
+            for key, val in {**opts, "chunk": chunk}.items():
+                G.set_option(key, val)
+            took.append(min(G.mine(3, 150, stats=True)["stats"]["time_ns"] for _ in range(4)) / 1e6)
+            G.close()
+        assert took[1] <= 1.25 * took[0], (opts, took)
