@@ -195,35 +195,15 @@ __device__ __forceinline__ bool qp_try(const QPTab &t, uint64_t key, uint64_t h,
     return false;
 }
 
-// The rest of a long probe sequence, out of line: a key of a half-full table rarely gets here.  A table that
-// overflows is full before its pass stops, and every key would be looked for in FSM_MAX_PROBES slots until
-// then: 30k vertices, size 3, from 64 slots up to 2^18, 98.6 ms, 11.9 this way; 37k, size 5, count 3 -> 5, 109 and
-// 19.7 ms.  Near probes 8 or 16: 4 -> 6 whole call 18.7 and 18.0 ms, 3 -> 5 one pass 23.4 and 22.3 (18.7 and 22.9
-// with all of them inline).
-#define FSM_NEAR_PROBES 16   // the smallest table has 64 slots
-static __device__ __noinline__ int64_t qp_insert_far(unsigned long long *keys, unsigned long long *used, uint64_t mask,
-                                                     unsigned long long max_used, uint64_t key, uint64_t h, int *err) {
-    QPTab t;
-    t.keys = keys;
-    t.used = used;
-    t.mask = mask;
-    t.max_used = max_used;
-    for (uint64_t probe = FSM_NEAR_PROBES; probe <= t.mask && probe < FSM_MAX_PROBES; ++probe) {
-        if ((probe & 15) == 0 && (*(volatile int *)err & FSM_ERR_QP_OVERFLOW)) return -1;
+// The extension kernel's form; fsm_join.cuh has another (qp_insert_near).
+__device__ __forceinline__ int64_t qp_insert(const QPTab &t, uint64_t key, int *err) {
+    uint64_t h = mix64(key) & t.mask;
+    for (uint64_t probe = 0; probe <= t.mask && probe < FSM_MAX_PROBES; ++probe) {
         if (qp_try(t, key, h, err)) return (int64_t)h;
         h = (h + 1) & t.mask;
     }
     atomicOr(err, FSM_ERR_QP_OVERFLOW);
     return -1;
-}
-
-__device__ __forceinline__ int64_t qp_insert(const QPTab &t, uint64_t key, int *err) {
-    uint64_t h = mix64(key) & t.mask;
-    for (int probe = 0; probe < FSM_NEAR_PROBES; ++probe) {
-        if (qp_try(t, key, h, err)) return (int64_t)h;
-        h = (h + 1) & t.mask;
-    }
-    return qp_insert_far(t.keys, t.used, t.mask, t.max_used, key, h, err);
 }
 
 __device__ __forceinline__ int64_t qp_find(const QPTab &t, uint64_t key) {

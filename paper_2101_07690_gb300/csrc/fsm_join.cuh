@@ -245,6 +245,38 @@ __device__ __forceinline__ void ld_rec8(const uint32_t *p, uint32_t *x) {
         : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]), "=r"(x[4]), "=r"(x[5]), "=r"(x[6]), "=r"(x[7]) : "l"(p));
 }
 
+// The rest of a long probe sequence, out of line: a key of a half-full table rarely gets here.  A table that
+// overflows is full before its pass stops, and every key would be looked for in FSM_MAX_PROBES slots until
+// then: 30k vertices, size 3, from 64 slots up to 2^18, 98.6 ms, 11.9 this way; 37k, size 5, count 3 -> 5, 109 and
+// 19.7 ms.  Near probes 8 or 16: 4 -> 6 whole call 18.7 and 18.0 ms, 3 -> 5 one pass 23.4 and 22.3 (18.7 and 22.9
+// with all of them inline).  The extension kernel, whose chunks are small, keeps them inline (edge-list quick
+// patterns, 100k vertices, size 4: 3.05 s, 3.42 s this way).
+#define FSM_NEAR_PROBES 16   // the smallest table has 64 slots
+static __device__ __noinline__ int64_t qp_insert_far(unsigned long long *keys, unsigned long long *used, uint64_t mask,
+                                                     unsigned long long max_used, uint64_t key, uint64_t h, int *err) {
+    QPTab t;
+    t.keys = keys;
+    t.used = used;
+    t.mask = mask;
+    t.max_used = max_used;
+    for (uint64_t probe = FSM_NEAR_PROBES; probe <= t.mask && probe < FSM_MAX_PROBES; ++probe) {
+        if ((probe & 15) == 0 && (*(volatile int *)err & FSM_ERR_QP_OVERFLOW)) return -1;
+        if (qp_try(t, key, h, err)) return (int64_t)h;
+        h = (h + 1) & t.mask;
+    }
+    atomicOr(err, FSM_ERR_QP_OVERFLOW);
+    return -1;
+}
+
+__device__ __forceinline__ int64_t qp_insert_near(const QPTab &t, uint64_t key, int *err) {
+    uint64_t h = mix64(key) & t.mask;
+    for (int probe = 0; probe < FSM_NEAR_PROBES; ++probe) {
+        if (qp_try(t, key, h, err)) return (int64_t)h;
+        h = (h + 1) & t.mask;
+    }
+    return qp_insert_far(t.keys, t.used, t.mask, t.max_used, key, h, err);
+}
+
 template <int L, int PASS, bool QUOTA>
 struct Joiner {
     using G = JoinGeo<L>;
@@ -334,7 +366,7 @@ struct Joiner {
     // One-pass level, a key the warm pass did not meet: count the join and leave its bits for after the
     // level, when such keys are resolved in bulk (deferred_bits_kernel).
     __device__ __forceinline__ void defer(const uint32_t *r, uint64_t key, uint32_t r0, uint32_t r1) {
-        const int64_t slot = qp_insert(A.qp, key, A.err);
+        const int64_t slot = qp_insert_near(A.qp, key, A.err);
         if (slot < 0) return;
         atomicAdd(A.qp.count + slot, 1ull);
         const unsigned long long at = atomicAdd(A.defer_top, 1ull);
@@ -365,7 +397,7 @@ struct Joiner {
     __device__ __forceinline__ void accept(const uint32_t *r, int j, uint64_t key, bool centre, int32_t anchor, int32_t x,
                                            uint32_t ainfo, uint32_t xinfo, bool swap) {
         if constexpr (PASS == PASS_COUNT) {
-            const int64_t slot = qp_insert(A.qp, key, A.err);
+            const int64_t slot = qp_insert_near(A.qp, key, A.err);
             if (slot < 0) return;
             count_join(slot);
             if (A.keep) {
