@@ -213,8 +213,8 @@ def kernel_source_sha() -> str:
 
 
 def traffic_for(kernel_pass: str):
-    """DRAM bytes per launch from the committed ncu summary, if it was taken on the current
-    source of the join kernel (else None)."""
+    """DRAM bytes of one launch on a scaled graph, with that graph named, from the committed ncu
+    summary if it was taken on the current source of the join kernel (else None)."""
     path = os.path.join(ROOT, "profiles", "extend_traffic.json")
     if not os.path.exists(path):
         return None
@@ -222,7 +222,7 @@ def traffic_for(kernel_pass: str):
     ent = d.get(kernel_pass)
     if not ent or d.get("source_sha") != kernel_source_sha():
         return None
-    return ent.get("dram_bytes_per_full_launch")
+    return {"dram_bytes": ent["dram_bytes"], "from": ent["capture"]}
 
 
 def issue_roof(dom, ns: float, nl: int, pieces: int):

@@ -89,9 +89,10 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
  *                passes and calls (reported as stat "chunk_l<l>"); 0 = forget tuned values.
  *   "chunk"      pieces per work-stealing chunk (power of two, 32..65536; 0 = default: the largest
  *                power of two from 64 to 8192 that leaves at least 8 chunks per warp, or 2 below
- *                256, and from 8 where units outnumber pieces four to one; where the extension kernel runs -- the ablations, and levels extended from size 6 and 7 -- the
- *                largest from 256 to 16384 that leaves at least 64 chunks per warp and spans at most
- *                about 16 units' pieces).
+ *                256, and from 8 on where units outnumber pieces four to one; where the extension
+ *                kernel runs -- the ablations, and levels extended from size 6 and 7 -- the largest
+ *                from 256 to 16384 that leaves at least 64 chunks per warp and spans at most about 16
+ *                units' pieces).
  *   "batch"      frontier embeddings per batch (>= 1024; 0 = default).
  *   "explore"    0 = two-vertex exploration (default, Section 4.1); 1 = single-vertex
  *                exploration, l -> l+1 (the ablation Section 6 compares against): every level
@@ -121,7 +122,9 @@ int fsm_load_graph(const int32_t *row_ptr, const int32_t *col, const int32_t *la
  *                identical.
  *   "fused"      1 = the last level of exact mining (k <= 7) is enumerated once: each accepted
  *                join is counted under its quick pattern and sets its MNI domain bits at once.  A
- *                sample of the level finds most quick patterns first; they are canonicalised and given
+ *                sample of the level (below 2^26 pieces all of it, so such a level is enumerated once to
+ *                find its keys and once to count them) finds most quick patterns first; they are
+ *                canonicalised and given
  *                their patterns' orbit bitmaps (every pattern gets bitmaps, frequent or not); joins of
  *                the others are put aside and entered after the level.  0 = a count pass,
  *                canonicalisation, then a domain pass for the patterns that can still reach t

@@ -869,7 +869,7 @@ struct Miner {
             // any allocation that needs it.  Whole calls by two passes and by records: size 6 on 1656
             // vertices 23.7 and 16.0 ms, size 7 under ST 8 72 and 54, size 5 on 37k, vertex-induced, 21.5 and
             // 17.1.  Not at l = 1, where enumerating costs no more than the records do (size 3 on 3.7M
-            // vertices 10.3 and 9.9, but three small mines of a 1.1M-vertex graph 3.1 and 3.4).
+            // vertices 10.3 and 9.9, but loading and mining a 1.1M-vertex graph once 3.1 and 3.4).
             if (!fused && !mem.spare && L >= 2 && joins(L) && pre.base && pre.total >= kKeepPieces && in.N < (1ll << 32)) {
                 keep_shards = grid_for(L, PASS_COUNT);
                 A.keep_cap = (uint32_t)std::min<int64_t>((pre.total / 8 * 3) / keep_shards + 1024, 0x7FFFFFFF);
@@ -1124,9 +1124,7 @@ struct Miner {
         s.cadj = mem.get<uint64_t>(NL);
         s.sigma = mem.get<unsigned long long>(NL);
         s.count = mem.get<unsigned long long>(NL);
-        unsigned long long *nf = mem.get<unsigned long long>(1);
-        ck(launch_level1_tables(NL, G->cls_size, t, lnew, s.lab8, s.adj8, s.clab, s.cadj, s.sigma, s.count, nf, st),
-           "level 1");
+        ck(launch_level1_tables(NL, G->cls_size, t, lnew, s.lab8, s.adj8, s.clab, s.cadj, s.sigma, s.count, st), "level 1");
         for (int l = 0; l < NL; ++l)
             if (G->cls_host[l] >= t && G->cls_host[l] > 0) {
                 s.P += 1;

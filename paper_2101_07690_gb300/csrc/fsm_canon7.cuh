@@ -80,7 +80,7 @@ FSM_HD void decode_code7(int K, unsigned long long clab7, uint32_t cadj7, int *l
             if ((cadj7 >> (np - 1 - q)) & 1u) { adj[c1] |= 1u << c2; adj[c2] |= 1u << c1; }
 }
 
-// Orbit representatives (as orbit_reps of fsm_canon.cuh), 
+// Orbit representatives, as orbit_reps of fsm_canon.cuh.
 static __host__ __device__ __noinline__ void orbit_reps7(int K, unsigned long long clab7, uint32_t cadj7, int *rep) {
     int lab[8];
     uint32_t adj[8];

@@ -42,12 +42,11 @@ struct QPTab {
 };
 
 // Key records (one-pass level and domain pass): per key slot, words 0-1 the key and words 2.. the
-// bitmap offset of each local position in units of 1 << off_shift words.  Every word starts as
-// all ones and is written once with its final value, so a reader that sees the key and no all-ones
-// offset has the whole record, whatever the order it saw the words in.
+// bitmap offset of each local position in units of 1 << off_shift words.  Every word starts as all
+// ones; records are written before the pass that reads them (slot_bases_kernel, resolve_keys_kernel).
 FSM_HD constexpr int key_rec_words(int K) { return K <= 6 ? 8 : 16; }
 #define FSM_DEFER_WORDS 8
-#define FSM_OFF_NONE 0xFFFFFFFFu     // word of a key record not yet published, or no bitmaps
+#define FSM_OFF_NONE 0xFFFFFFFFu     // no record, or a pattern without bitmaps
 
 struct ExtArgs {
     DevGraph g;
@@ -150,8 +149,8 @@ FSM_HD int64_t join_chunk(int64_t total, int64_t units, int64_t warps) {
 
 // Warm pass of a one-pass level: the keys of every warm_stride-th chunk of FSM_WARM_CHUNK pieces are
 // counted and resolved in bulk first, so that the level itself meets few keys for the first time.
-// All pieces up to 2^25 (small levels have most keys per piece), then 2^25 of them, from 2^30 on
-// one in 32.  What the sample misses costs a join about ten times the others: with 36 joins a key
+// All pieces below 2^26 (small levels have most keys per piece; they are enumerated twice), then 2^25 to 2^26
+// of them, from 2^30 on one in 32.  What the sample misses costs a join about ten times the others: with 36 joins a key
 // (7400 vertices, size 5, 1.8M keys), one in 15 pieces left 14 % of the joins to be entered after the
 // level; with 1000 joins a key, one in 32 leaves under 1 %.
 #define FSM_WARM_CHUNK 1024
@@ -1016,7 +1015,7 @@ cudaError_t launch_resolve_keys(const ExtArgs &A, int sms, cudaStream_t st);
 cudaError_t launch_kept_bits(int L, const ExtArgs &A, int shards, cudaStream_t st);
 cudaError_t launch_deferred_bits(const ExtArgs &A, int sms, cudaStream_t st);
 cudaError_t occupancy_join(int pass, int L, int V, int *blocks_per_sm);
-// its tables for stored size L: bytes of each, and the kernels that fill them (tmp: join_tmp_bytes)
+// its tables for stored size L: bytes of each, and the kernels that fill them (tmp: scratch of theirs)
 void join_table_bytes(int L, size_t *acc, size_t *any, size_t *tmp);
 cudaError_t launch_join_tables(int L, uint32_t *acc, uint16_t *any, void *tmp, cudaStream_t st);
 

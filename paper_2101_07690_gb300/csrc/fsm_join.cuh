@@ -3,9 +3,9 @@
 // Section 5's quotas).  fsm_extend.cuh states the work of a join and holds the kernel of the other
 // forms; this one does the same joins in another order of steps.
 //
-// What bounds a level is the number of candidate pieces times the instructions each costs (DRAM
-// and L2 are nearly idle), so the steps are ordered by what they reject per instruction, and every
-// step runs with full warps:
+// What bounds a level is the number of candidate pieces times the instructions each costs (DRAM is
+// nearly idle where the bitmaps fit L2), so the steps are ordered by what they reject per instruction,
+// and every step runs with full warps:
 //
 //   tables     Whether smallest-vertex-first dissection (Algorithm 1) returns exactly (t, s) depends
 //              only on the relative order of the l + 2 ids and on the edges among them.  With s
@@ -32,15 +32,15 @@
 // One launch on a GB300 (same graph and output): the extension kernel before, this kernel with a
 // key table per block in shared memory (flushed between chunks) and both new vertices' tests made
 // per survivor, and as it is:
-//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms,  77.7 ms,  19.1 ms
-//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,   110 ms
-//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,   9.4 ms
-//   5 -> 7, count, ST 8 quotas, 6.0e8 pieces, 1.2e8 joins:          248 ms,  60.6 ms,  25.3 ms
-//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   4.2 ms
+//   3 -> 5, one pass, 74k vertices, 1.7e9 pieces, 3.3e8 joins:      475 ms,  77.7 ms,  18.8 ms
+//   2 -> 4, one pass, 100k vertices, 7.5e9 pieces, 3.2e9 joins:     733 ms, 283 ms,    88 ms
+//   4 -> 6, count, 1656 vertices, 1.4e9 pieces, 2.9e8 joins:        265 ms,  18.5 ms,   9.8 ms
+//   5 -> 7, count, ST 8 quotas, 6.0e8 pieces, 1.2e8 joins:          248 ms,  60.6 ms,  27.6 ms
+//   1 -> 3, count, 3.7M vertices, 6.3e8 pieces, 2.0e8 joins:       14.4 ms,   8.1 ms,   4.3 ms
 // The block tables missed 70 to 77 % of the lookups of levels 1 and 2, and their flushes made warps
 // wait for each other; a record read at the L2 costs each join one latency and no barrier.  What is
-// left is bound by issue and dependent loads (3 -> 5, one pass, 370k vertices: 9.3 warp instructions a
-// piece where the extension kernel took 80, 60 % of the issue slots, 21.7 of 32 lanes, DRAM at 3 %), by
+// left is bound by issue and dependent loads (3 -> 5, one pass, 370k vertices: 9.4 warp instructions a
+// piece where the extension kernel took 80, 60 % of the issue slots, 21.5 of 32 lanes, DRAM at 3 %), by
 // scattered requests (2 -> 4: load-store unit 66 %, L2 58 % busy) and, where the body is large, by
 // instruction fetch: one copy of the joins (take) instead of two took 5 -> 7 from 55 to 35 ms.
 #pragma once
@@ -133,8 +133,8 @@ template <int L, bool QUOTA> struct UnitRec {
     // searches they save (3 -> 5 one pass 28.2 ms).
     static constexpr int U = L == 1 ? 16 : 8;
     static constexpr int BLOOM = L <= 3 ? 256 : 512;
-    static constexpr int RP = 0, D = 1, PID = 2, META = 3, CLS = 4, OLAB = 5, OPP = 6, SEG = 7, SLO = 8, RLO = 9,
-                         RHI = 11, NC = 13, SCN = 15, SEO = 16, SS = 17, BND = SS + L, RK = BND + L, OB = RK + L, OE = OB + O, OK = OE + O,
+    static constexpr int RP = 0, D = 1, PID = 2, META = 3, CLS = 4, SCN = 5, OPP = 6, SEG = 7, SLO = 8, RLO = 9,
+                         RHI = 11, NC = 13, SEO = 15, SS = 16, BND = SS + L, RK = BND + L, OB = RK + L, OE = OB + O, OK = OE + O,
                          VB = OK + 6 * O, VE = VB + 1, EI = VE + 1, QA = EI + 1, END = QA + (QUOTA ? 6 : 0);
     static constexpr int UW = END | 1;               // odd stride: lanes on different units hit different banks
 };

@@ -57,7 +57,7 @@ __global__ void validate_kernel(DevGraph g, int32_t num_labels, int *err) {
 
 // Ranks come from one counter per label class.  A block counts its vertices per label in shared
 // memory first and reserves each label's range once: 1.1M vertices of 16 labels made 1.1M atomics on 16
-// addresses (197 us), now one per block and label (75 us).
+// addresses (197 us), now one per block and label (57 us).
 __global__ void __launch_bounds__(kThreads) prepare_kernel(DevGraph g, int64_t *piece_cnt, int32_t *end_off, int32_t *rank,
                                                            int32_t *cls_size, int4 *vinfo) {
     __shared__ int32_t cnt[64], base[64];
@@ -420,7 +420,7 @@ __device__ __forceinline__ bool rec_less(const CodeRec &a, const CodeRec &b) {
 
 // ---- sort by (lab, adj, idx)
 //
-// Up to FSM_SORT_BLOCK records (small graphs and levels, where a launch costs more than the work):
+// Up to kSortBlock records (small graphs and levels, where a launch costs more than the work):
 // one block sorts them in shared memory.  Above: least-significant-digit radix sort of the code as
 // one integer of 6 K + K (K - 1) / 2 bits (labels above pairs), eight bits a pass, stable, so equal
 // codes keep their order.  A pass reads the records twice and writes them once.  Before, a bitonic
@@ -1016,8 +1016,7 @@ cudaError_t launch_level2_frontier(const DevGraph &g, int32_t NL, const int32_t 
 namespace {
 __global__ void level1_tables_kernel(int32_t NL, const int32_t *cls_size, int64_t t, int32_t *label_newid,
                                      uint64_t *lab8, uint64_t *adj8, unsigned long long *clab, uint64_t *cadj,
-                                     unsigned long long *sigma, unsigned long long *count,
-                                     unsigned long long *n_freq) {
+                                     unsigned long long *sigma, unsigned long long *count) {
     if (gtid() != 0) return;
     int32_t id = 0;
     for (int l = 0; l < NL; ++l) {
@@ -1036,7 +1035,6 @@ __global__ void level1_tables_kernel(int32_t NL, const int32_t *cls_size, int64_
             label_newid[l] = -1;
         }
     }
-    *n_freq = (unsigned long long)id;
 }
 
 __global__ void level2_tables_kernel(int32_t NL, const unsigned long long *pair_sigma,
@@ -1068,10 +1066,9 @@ __global__ void level2_tables_kernel(int32_t NL, const unsigned long long *pair_
 
 cudaError_t launch_level1_tables(int32_t NL, const int32_t *cls_size, int64_t t, int32_t *label_newid,
                                  uint64_t *lab8, uint64_t *adj8, unsigned long long *clab, uint64_t *cadj,
-                                 unsigned long long *sigma, unsigned long long *count,
-                                 unsigned long long *n_freq, cudaStream_t st) {
+                                 unsigned long long *sigma, unsigned long long *count, cudaStream_t st) {
     LAUNCHED(1);
-    level1_tables_kernel<<<1, 32, 0, st>>>(NL, cls_size, t, label_newid, lab8, adj8, clab, cadj, sigma, count, n_freq);
+    level1_tables_kernel<<<1, 32, 0, st>>>(NL, cls_size, t, label_newid, lab8, adj8, clab, cadj, sigma, count);
     return cudaGetLastError();
 }
 
@@ -1182,7 +1179,7 @@ __global__ void aut_size_kernel(int K, const unsigned long long *pat_lab, const 
         int lab[FSM_MAXK], perm[FSM_MAXK], seg[FSM_MAXK];
         uint32_t adj[FSM_MAXK];
         decode_code(K, pat_lab[P], pat_adj[P], lab, adj);
-        if (K <= 7) {   // by placing vertices, not by trying every order (98k patterns: 154 -> 12 us)
+        if (K <= 7) {   // by placing vertices, not by trying every order (98k patterns: 154 -> 21 us)
             aut[P] = automorphisms7(K, lab, adj);
             continue;
         }

@@ -129,8 +129,7 @@ cudaError_t launch_level2_frontier(const DevGraph &g, int32_t NL, const int32_t 
 // frequent ids in code order, level tables, codes, supports, counts; *n_freq = frequent count
 cudaError_t launch_level1_tables(int32_t NL, const int32_t *cls_size, int64_t t, int32_t *label_newid,
                                  uint64_t *lab8, uint64_t *adj8, unsigned long long *clab, uint64_t *cadj,
-                                 unsigned long long *sigma, unsigned long long *count,
-                                 unsigned long long *n_freq, cudaStream_t st);
+                                 unsigned long long *sigma, unsigned long long *count, cudaStream_t st);
 cudaError_t launch_level2_tables(int32_t NL, const unsigned long long *pair_sigma,
                                  const unsigned long long *pair_count, int64_t t, int32_t *pair_newid,
                                  uint64_t *lab8, uint64_t *adj8, unsigned long long *clab, uint64_t *cadj,
