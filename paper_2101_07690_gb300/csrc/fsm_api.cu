@@ -564,7 +564,7 @@ struct Miner {
         // Per-pattern launches need the frontier grouped.  The persistent launch groups it from
         // size 3 on (option "group" = 2): consecutive units then share the pattern, and
         // its key records and bitmaps stay in the caches (one-pass level 3 of the 3.7M-vertex graph,
-        // k = 5: at 1/10 scale 165 -> 110 ms, at 3/10 533 -> 439 ms).  Edges keep emission order,
+        // k = 5: at 1/10 scale 183 -> 105 ms, at 3/10 625 -> 343 ms).  Edges keep emission order,
         // whose consecutive units share key vertices (measured faster there).
         const bool grouped = G->launch == 2 || (G->launch == 1 && (G->group == 1 || (G->group == 2 && in.L >= 3)));
         if (!grouped || in.N == 0 || in.P == 0) return off;

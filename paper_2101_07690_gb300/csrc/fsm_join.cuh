@@ -382,7 +382,7 @@ struct Joiner {
     // One more join of key slot `slot`, for the lanes here together: lanes of one key add once.  A few keys
     // that take all of a level's joins (few labels, hubs) queue on their counters otherwise: 30k vertices, 4
     // labels, two hubs of degree 20000, 4e8 joins of 138 keys, 1 -> 3 count 24.6 ms, 6.2 this way; 2 -> 4 one
-    // pass, 3.2e9 joins, whole call 114 and 95 ms.  Where a count pass meets many keys the match only costs
+    // pass, 3.2e9 joins, whole call 114 and 95 ms; 3.7M vertices, 3 -> 5 one pass, 1.6e10 joins, 2410 and 1361 ms.  Where a count pass meets many keys the match only costs
     // (4 -> 6, 2.9e8 joins, whole call 18.5 and 18.9 ms; 1 -> 3, 37 labels, 10.5 and 10.8): ExtArgs::merge.
     __device__ __forceinline__ void count_join(int64_t slot) {
         if (PASS == PASS_FUSED || A.merge) {
