@@ -687,9 +687,11 @@ struct Miner {
             // (108 words), one pass: 154 ms with, 146 ms without; 3.7M vertices, size 3: 9.4 and 7.8 ms
             A.check_bits = (int64_t)G->n < (int64_t)512 * G->NL;
             A.any = G->join_any[L];
-            // few stored patterns and labels: few keys (37 labels, l = 1: 1369; 4 labels: 16; the counts of
-            // both are at count_join)
-            A.merge = in.P * G->NL < 1024;
+            // few stored patterns and labels: few keys.  1 -> 3 count without and with, by labels (patterns times
+            // labels is their square): two hubs of degree 20000, 1: 236 and 8.2 ms, 4: 24.5 and 6.2, 8: 11.7 and
+            // 6.3, 15: 6.46 and 6.35, 16: 6.36 and 6.45; 550k vertices without hubs, 4: 0.376 and 0.378, 15: 0.369
+            // and 0.389
+            A.merge = in.P * G->NL < 256;
             if (piece_freq) {
                 lf = mem.get<unsigned long long>(3 * 4096);
                 ck(launch_label_masks(piece_freq, lf, st), "label masks");
